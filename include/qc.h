@@ -189,8 +189,8 @@ typedef struct {
     int32_t order;             /* -1 auto, 0 row-major tiles, 1 baseline-strip tiles */
     int32_t block_threads;     /* threads per CTA of the accumulate kernel (0: auto) */
     int32_t ctas_per_sm;       /* resident CTAs per SM for its grid (0: auto)        */
-    int32_t kernel;            /* accumulate kernel: 0 auto (3 for chains of <= 2 terms,
-                                  2 otherwise), 1 bulk-copy pipeline with per-warp rings
+    int32_t kernel;            /* accumulate kernel: 0 auto (sums where they cost less, else 3
+                                  for chains of <= 2 terms, 2 otherwise), 1 bulk-copy pipeline with per-warp rings
                                   (chains of <= 2 terms), 2 per-lane cp.async prefetching
                                   kernel, 3 streaming kernel (step-major row table, flags
                                   folded into weights; chains of <= 2 terms), 4 warp-
@@ -206,29 +206,35 @@ typedef struct {
     int32_t div_flag;          /* 1 = flag diverging gains (see below)              */
     int32_t robust;            /* 1 = robust reweighting between epochs (below)     */
     double robust_nu;          /* its degrees of freedom nu (> 0; 0 -> 5)           */
-    int32_t moments;           /* 1 = single-term chains from per-baseline sums (below) */
+    int32_t moments;           /* 1 = terms from per-(interval, pair) sums (below)  */
 } qc_opts;
 
 /*
- * Sufficient statistics (not in the paper), opt-in with qc_opts.moments.  While one
- * term is solved the other terms are fixed, so every sample of a baseline (p, q) in a
- * solution interval enters Eq. jhj_entry_simplified and Eq. jhr_entry_simplified
- * through sums that do not depend on the solved gains.  One pass over the data per
- * term solve forms them per (interval, antenna pair); every iteration forms the blocks
- * from the sums and the current gains.  Two forms (chains of one or two terms, one
- * direction, complex64 model, the solved term not a delay term):
- *  - full form, the solved term (any kind) has no term to its left: with
- *    X = R_p M R_q^H (R the term to its right, X = M without one), per correlation kj
- *    S[kj][u][v] = sum w_kj conj(X_u) X_v, T[kj][u] = sum w_kj conj(X_u) D_kj,
- *    U[kj] = sum w_kj |D_kj|^2 (100 FP32 words per interval and pair);
- *  - diagonal form, a diagonal or phase-only solved term with a term L to its left:
- *    with E_kj,ab = L_p,ka M_ab conj(L_q,jb), S'[u][v] = sum sum_kj w_kj conj(E_kj,u)
- *    E_kj,v, T'[u] = sum sum_kj w_kj conj(E_kj,u) D_kj (28 FP32 words per interval and pair).
- * Other solves (a full-Jones term with a term to its left, longer chains, sums of 2^31
- * or more slots) ignore the option.  qc_stats.vis_iters counts the samples of the
- * active intervals per iteration as without it; qc_stats.acc_bytes counts the pass (the
- * samples' bytes, once) and, per iteration and active interval, the sums read on both
- * sides and the accumulators written; qc_stats.pass_ms the passes' device time.
+ * Sufficient statistics (not in the paper).  While one term is solved the other terms are
+ * fixed, so every sample of a baseline (p, q) in a solution interval enters Eq.
+ * jhj_entry_simplified and Eq. jhr_entry_simplified through sums that do not depend on the
+ * solved gains.  One pass over the data per term solve forms them per (interval, antenna
+ * pair); every iteration forms the blocks from the sums and the current gains.  Three
+ * forms (chains of one or two terms, one direction, the solved term not a delay term):
+ *  - full form, a full-Jones solved term with no term to its left: with X = R_p M R_q^H (R
+ *    the term to its right, X = M without one), per correlation kj
+ *    S[kj][u][v] = sum w_kj conj(X_u) X_v, T[kj][u] = sum w_kj conj(X_u) D_kj (100 FP32
+ *    words per interval and pair, four of them padding);
+ *  - E form, a diagonal or phase-only solved term with a full-Jones term L to its left: with
+ *    E_kj,ab = L_p,ka M_ab conj(L_q,jb), S'[u][v] = sum sum_kj w_kj conj(E_kj,u) E_kj,v,
+ *    T'[u] = sum sum_kj w_kj conj(E_kj,u) D_kj (28 FP32 words, four of them padding);
+ *  - plain diagonal form, any other diagonal or phase-only solved term: with X = O_p M O_q^H
+ *    (O the other term), S_kj = sum w_kj |X_kj|^2, T_kj = sum w_kj conj(X_kj) D_kj (12 words).
+ * qc_opts.moments = 1 asks for the sums (complex64 model); qc_solve also takes them by
+ * itself, with either model, where an iteration on the sums moves at most half the bytes of
+ * one on the samples, unless the options name an accumulate kernel, a tile order or a launch
+ * shape, or ask for divergence flagging or an allreduce.  The steps are the same either way.
+ * Other solves (a full-Jones term with a term to its left, longer chains, sums of 2^31 or
+ * more slots, or more than the device has room for) ignore the option.  qc_stats.vis_iters
+ * counts the samples of the active intervals per iteration however a term was solved; from
+ * sums, qc_stats.acc_bytes counts the pass (the samples' bytes, once) and, per iteration and
+ * active interval, the sums read on both sides and the accumulators written;
+ * qc_stats.pass_ms is the passes' device time when qc_opts.moments asked for them.
  */
 
 /*

@@ -150,6 +150,7 @@ qc_ctx::~qc_ctx()
     for (auto &b : tb) if (b.exec) cudaGraphExecDestroy(b.exec);
     for (void *p : owned) qc_dev_free(p);
     for (auto e : events) cudaEventDestroy(e);
+    for (auto e : sums_events) cudaEventDestroy(e);
     if (own_stream) cudaStreamDestroy(own_stream);
 }
 
@@ -855,7 +856,8 @@ extern "C" int qc_solve(qc_ctx *c, qc_term *terms, int32_t n_terms, const qc_opt
         CK(cudaMemcpyAsync(&S.chi2_before, d_chi2, sizeof(double), cudaMemcpyDeviceToHost, st));
     }
 
-    // per solved term: bin counts and byte weights
+    // per solved term: its route, bin counts and byte weights
+    c->pending.clear();
     const long long b_flag = c->has_flag ? 1 : 0;
     const long long b_unflag = 32 + (c->m16 ? 16 : 32 * c->n_dir) + 16;
     for (int j = 0; j < n_terms; ++j) {
@@ -865,15 +867,21 @@ extern "C" int qc_solve(qc_ctx *c, qc_term *terms, int32_t n_terms, const qc_opt
         const size_t nb = term_nbins(t);
         const size_t KG = t.type == 1 ? KG_FULL : KG_DIAG;
         const size_t nat = c->term_nat(t);
-        if ((rc = c->ensure(B.acc, nbytes<double>(nb * nat * KG)))) return rc;
-        if ((rc = c->ensure(B.active, nb))) return rc;
-        if ((rc = c->ensure(B.cnt, nbytes<int>(t.max_iter + 1)))) return rc;
+        if ((rc = c->plan_sums(xt.data(), n_terms, j, o))) return rc;
+        const bool one_launch = B.sums.one_launch;
+        if (!one_launch) {
+            if ((rc = c->ensure(B.acc, nbytes<double>(nb * nat * KG)))) return rc;
+            if ((rc = c->ensure(B.active, nb))) return rc;
+            if ((rc = c->ensure(B.cnt, nbytes<int>(t.max_iter + 1)))) return rc;
+        }
         if ((rc = c->ensure(B.nvis, nbytes<long long>(3 * nb)))) return rc;
         if ((rc = c->ensure(B.iters, nbytes<int>(nb)))) return rc;
         if ((rc = c->ensure(B.flags, nb * nat))) return rc;
-        CK(cudaMemsetAsync(B.acc.ptr, 0, nbytes<double>(nb * nat * KG), st));
-        CK(cudaMemsetAsync(B.iters.ptr, 0, nbytes<int>(nb), st));
-        CK(cudaMemsetAsync(B.flags.ptr, 0, nb * nat, st));
+        if (!one_launch) {       // the one-launch iterations write every interval's count and flags
+            CK(cudaMemsetAsync(B.acc.ptr, 0, nbytes<double>(nb * nat * KG), st));
+            CK(cudaMemsetAsync(B.iters.ptr, 0, nbytes<int>(nb), st));
+            CK(cudaMemsetAsync(B.flags.ptr, 0, nb * nat, st));
+        }
         // the counts of the previous call stand while the term's maps are the same (FNV-1a
         // over the kernels' view of them)
         uint64_t sig = 1469598103934665603ull;
@@ -946,6 +954,15 @@ extern "C" int qc_solve(qc_ctx *c, qc_term *terms, int32_t n_terms, const qc_opt
             int it_max = 0;
             double acc_ms = 0, pass_ms = 0;
             long long acc_launches = 0;
+            if (c->tb[n].sums.one_launch) {
+                if ((rc = c->solve_term_sums(xt.data(), n_terms, n, chain, o, st, epoch == o->n_epochs - 1))) return rc;
+                if ((int)c->pending.size() == qc_ctx::MAX_PENDING) {
+                    if ((rc = c->copy_pending(st))) return rc;
+                    CK(cudaStreamSynchronize(st));
+                    if ((rc = c->collect_sums(S, n_iter_max))) return rc;
+                }
+                continue;
+            }
             if ((rc = c->solve_term(xt.data(), n_terms, n, chain, o, st, &it_max, &acc_ms, &acc_launches, &pass_ms)))
                 return rc;
             S.acc_ms += acc_ms;
@@ -1006,8 +1023,10 @@ extern "C" int qc_solve(qc_ctx *c, qc_term *terms, int32_t n_terms, const qc_opt
     }
     unsigned long long hc[2];
     CK(cudaMemcpyAsync(hc, d_counters, sizeof hc, cudaMemcpyDeviceToHost, st));
+    if ((rc = c->copy_pending(st))) return rc;
     CK(cudaEventRecord(ev1, st));
     CK(cudaStreamSynchronize(st));
+    if ((rc = c->collect_sums(S, n_iter_max))) return rc;
     float ms = 0;
     CK(cudaEventElapsedTime(&ms, ev0, ev1));
     S.ms = ms;
@@ -1033,6 +1052,225 @@ int qc_ctx::get_event(int i, cudaEvent_t &ev)
         events.push_back(e);
     }
     ev = events[i];
+    return QC_OK;
+}
+
+// ---------------------------------------------------------------------------
+// solving a term from per-(interval, antenna pair) sums
+// ---------------------------------------------------------------------------
+
+// Antennas up to which one CTA keeps an interval's gains and normal equations in shared memory
+// (256 x (32 + 128) B = 40 KB) and walks all of its pairs itself.
+static constexpr int SUMS_ONE_LAUNCH_ANT = 256;
+
+// The route of a solved term: from sums when the caller asks for it (qc_opts.moments), or by itself
+// where that is the cheaper way to the same steps; sets B.sums and sizes its workspace.
+//
+// An iteration on the samples reads 80 B a sample (64 with the FP16 model) and is limited by
+// instruction issue at about 0.64 of the HBM rate; the sums cost one pass, about 1.3 such
+// iterations, and then 2 x 4 x words B per (interval, pair) and iteration, mostly out of L2.  The
+// rule takes the sums when an iteration on them moves at most half the bytes of one on the
+// samples, i.e. from 2.4 (plain diagonal form), 5.6 (E form) or 20 (full form) samples per slot
+// on, and a term may take three iterations or more.  It also bounds the workspace to a quarter of
+// the samples' bytes.  The options that name an accumulate kernel, its tiles or launch shape,
+// divergence flagging and an allreduce (whose buffers are documented per iteration) keep the
+// iterations on the samples.
+int qc_ctx::plan_sums(const qc_term *terms, int n_terms, int n, const qc_opts *o)
+{
+    const qc_term &t = terms[n];
+    TermBufs &B = tb[n];
+    B.sums = SumsPlan();
+    if (n_terms > 2 || delay[n] || n_dir > 1 || n_up == 0) return QC_OK;
+    const size_t nb = term_nbins(t), slots = nb * (size_t)n_up;
+    if (slots >= (size_t)INT32_MAX) return QC_OK;
+    const int lk = kind_of_range(terms, 0, n), rk = kind_of_range(terms, n + 1, n_terms);
+    int form, ok;
+    if (t.type != QC_TERM_FULL && lk != KIND_FULL) { form = FORM_D; ok = lk != KIND_NONE ? lk : rk; }
+    else if (t.type != QC_TERM_FULL) { form = FORM_E; ok = lk; }
+    else if (lk == KIND_NONE) { form = FORM_FULL; ok = rk; }
+    else return QC_OK;
+    const bool asked = o->moments && d_model != nullptr;
+    const bool one_launch = n_ant <= SUMS_ONE_LAUNCH_ANT && !t.reduce && !(o->div_flag && t.max_iter >= 4);
+    if (!asked) {
+        const bool plain = o->kernel == 0 && o->order == -1 && o->block_threads == 0 && o->ctas_per_sm == 0;
+        if (!plain || !one_launch || o->div_flag || t.max_iter < 3) return QC_OK;
+        const double sample_bytes = (m16 ? 64.0 : 80.0) * (double)n_strip_rows * n_chan;
+        if (2.0 * 4.0 * mom_words(form) * (double)slots > 0.5 * sample_bytes) return QC_OK;
+    }
+    const size_t sums_bytes = ((nbytes<float>(slots * mom_words(form)) + 15) / 16) * 16;
+    int rc;
+    if ((rc = ensure(B.mom, sums_bytes + nbytes<long long>(nb)))) {
+        if (asked || rc != QC_ENOMEM) return rc;
+        cudaGetLastError();                    // no room for the sums: iterate on the samples
+        err.clear();
+        return QC_OK;
+    }
+    B.sums.form = form;
+    B.sums.ok = ok;
+    B.sums.asked = asked;
+    B.sums.one_launch = one_launch;
+    return QC_OK;
+}
+
+// Arguments of the pass and of the normal equations of a term solved from sums; builds the
+// context's table of strip rows the first time (a function of the rows and flags staged at create).
+int qc_ctx::sums_args(const qc_term *terms, int n_terms, int n, const Chain &chain, cudaStream_t st, MomArgs &ma,
+                      MomNormArgs &mn)
+{
+    qc_ctx *c = this;
+    const qc_term &t = terms[n];
+    TermBufs &B = tb[n];
+    memset(&ma, 0, sizeof ma);
+    memset(&mn, 0, sizeof mn);
+    int rc;
+    const size_t scale_off = nbytes<int4>(std::max(1L, n_strip_rows));
+    if (!mom_rows_ready) {
+        if ((rc = ensure(mom_rows, scale_off + (m16 ? nbytes<float>(std::max(1L, n_strip_rows)) : 0)))) return rc;
+        CK(mom_launch_rows(n_strip_rows, d_strip_rows, d_rows, d_row_live, d_up_of_bl, d_bl_scale, (int4 *)mom_rows.ptr,
+                           m16 ? (float *)((char *)mom_rows.ptr + scale_off) : nullptr, st));
+        // built on this call's stream: finished before any later call can use it on another one
+        CK(cudaStreamSynchronize(st));
+        mom_rows_ready = true;
+        ++launches;
+    }
+    ma.n_chan = n_chan;
+    ma.n_ant = n_ant;
+    ma.n_up = n_up;
+    ma.vis = d_vis;
+    ma.model = d_model;
+    ma.model16 = d_model16;
+    ma.wf = d_wf;
+    ma.mrows = (const int4 *)mom_rows.ptr;
+    ma.mscale = m16 ? (const float *)((const char *)mom_rows.ptr + scale_off) : nullptr;
+    ma.strip_off = d_strip_off;
+    ma.n_strips = n_strips;
+    ma.n_chunks = (n_chan + 31) / 32;
+    // an interval several times long: the rows inside each chunk keep a lane's key (units of a strip
+    // x one chunk); else a row's chunks inside each row (units of whole rows), so that an interval
+    // one time long flushes once per row.  The rows are cut into blocks until there are about four
+    // units per resident warp, down to 8 rows inside a chunk (a block's end is a flush)
+    ma.chunk_major = t.n_tint < n_time ? 1 : 0;
+    const long max_strip = std::max(1, max_strip_rows);
+    const long want_units = 4L * sm_count * 12;
+    ma.group = ma.chunk_major ? 1 : ma.n_chunks;
+    const long strips = std::max(1L, (long)n_strips * (ma.chunk_major ? ma.n_chunks : 1));
+    const long blocks = std::max(1L, (want_units + strips - 1) / strips);
+    ma.rb = (int)std::min(max_strip, std::max(ma.chunk_major ? 8L : 1L, (max_strip + blocks - 1) / blocks));
+    ma.n_rb = (int)((max_strip + ma.rb - 1) / ma.rb);
+    ma.tn = chain.t[n];
+    ma.to = n_terms == 2 ? chain.t[1 - n] : chain.t[n];
+    ma.mom = (float *)B.mom.ptr;
+    mn.n_bins = (int)term_nbins(t);
+    mn.n_ant = n_ant;
+    mn.n_up = n_up;
+    mn.type = t.type;
+    mn.form = B.sums.form;
+    mn.upair = d_upair;
+    mn.mom = ma.mom;
+    mn.params = (const double *)B.params.ptr;
+    mn.tab = (const float4 *)B.tab.ptr;
+    mn.n_fint = t.n_fint;
+    return QC_OK;
+}
+
+// One term solve from sums with its iterations in one launch; its statistics are collected when the
+// stream is next synchronised (collect_sums).
+int qc_ctx::solve_term_sums(const qc_term *terms, int n_terms, int n, const Chain &chain, const qc_opts *o,
+                            cudaStream_t st, bool last_epoch)
+{
+    qc_ctx *c = this;
+    const qc_term &t = terms[n];
+    TermBufs &B = tb[n];
+    MomArgs ma;
+    MomIterArgs mi;
+    memset(&mi, 0, sizeof mi);
+    int rc;
+    if ((rc = sums_args(terms, n_terms, n, chain, st, ma, mi.n))) return rc;
+    Pending P;
+    P.max_iter = t.max_iter;
+    P.n_bins = mi.n.n_bins;
+    P.last_epoch = last_epoch;
+    P.asked = B.sums.asked;
+    P.off = pending.empty() ? 0 : pending.back().off + pending.back().max_iter + 1;
+    P.ev = 3 * (int)pending.size();
+    while ((int)sums_events.size() < P.ev + 3) {
+        cudaEvent_t e;
+        CK(cudaEventCreate(&e));
+        sums_events.push_back(e);
+    }
+    const cudaEvent_t *ev = sums_events.data() + P.ev;
+    // a counter region per pending term solve; the buffer only grows while nothing is pending
+    const size_t need = nbytes<int>((size_t)MAX_PENDING * (t.max_iter + 1));
+    if (sums_cnt.bytes < need || sums_cnt.bytes < nbytes<int>((size_t)P.off + t.max_iter + 1)) {
+        if (!pending.empty()) {
+            // terms of different max_iter: keep the counts so far, then make room
+            Buf old = sums_cnt;
+            sums_cnt = Buf();
+            if ((rc = ensure(sums_cnt, std::max(need, nbytes<int>((size_t)P.off + need / sizeof(int)))))) {
+                sums_cnt = old;
+                return rc;
+            }
+            CK(cudaMemcpyAsync(sums_cnt.ptr, old.ptr, nbytes<int>(P.off), cudaMemcpyDeviceToDevice, st));
+            CK(cudaStreamSynchronize(st));
+            release(old.ptr);
+        } else if ((rc = ensure(sums_cnt, need))) {
+            return rc;
+        }
+    }
+    int *cnt = (int *)sums_cnt.ptr + P.off;
+    CK(cudaMemsetAsync(cnt, 0, nbytes<int>(t.max_iter + 1), st));
+    CK(cudaMemsetAsync(B.mom.ptr, 0, nbytes<float>((size_t)P.n_bins * n_up * mom_words(B.sums.form)), st));
+    CK(cudaEventRecord(ev[0], st));
+    CK(mom_launch_pass(ma, B.sums.form, B.sums.ok, sm_count, st));
+    CK(cudaEventRecord(ev[1], st));
+    mi.params = (double *)B.params.ptr;
+    mi.tab = (float4 *)B.tab.ptr;
+    mi.gain_flags = (int8_t *)B.flags.ptr;
+    mi.iters = (int *)B.iters.ptr;
+    mi.cnt = cnt;
+    mi.bin_nvis = (const long long *)B.nvis.ptr;
+    mi.bin_nbytes = (const long long *)B.nvis.ptr + 2 * (size_t)P.n_bins;
+    mi.iter_bytes = 2LL * n_up * mom_words(B.sums.form) * 4 + 8LL * n_ant * (t.type == 1 ? KG_FULL : KG_DIAG);
+    mi.vis_iters = (unsigned long long *)scalars.ptr;
+    mi.acc_bytes = (unsigned long long *)scalars.ptr + 1;
+    mi.max_iter = t.max_iter;
+    mi.alternate = o->damping_mode == QC_DAMP_ALTERNATE;
+    mi.damping = o->damping > 0 ? o->damping : 1.0;
+    mi.tol = t.tol;
+    CK(mom_launch_iterate(mi, st));
+    CK(cudaEventRecord(ev[2], st));
+    launches += 2;
+    pending.push_back(P);
+    return QC_OK;
+}
+
+// Host copies of the pending term solves' counters, ordered on the stream.
+int qc_ctx::copy_pending(cudaStream_t st)
+{
+    qc_ctx *c = this;
+    if (pending.empty()) return QC_OK;
+    const size_t n = (size_t)pending.back().off + pending.back().max_iter + 1;
+    pending_cnt.resize(n);
+    CK(cudaMemcpyAsync(pending_cnt.data(), sums_cnt.ptr, nbytes<int>(n), cudaMemcpyDeviceToHost, st));
+    return QC_OK;
+}
+
+// After a synchronisation that followed copy_pending: iteration counts and device times.
+int qc_ctx::collect_sums(qc_stats &S, int &n_iter_max)
+{
+    qc_ctx *c = this;
+    for (const Pending &P : pending) {
+        int its = P.n_bins > 0 ? 1 : 0;
+        while (its > 0 && its < P.max_iter && pending_cnt[P.off + its] > 0) ++its;
+        float ms = 0, pass = 0;
+        CK(cudaEventElapsedTime(&ms, sums_events[P.ev], sums_events[P.ev + 2]));
+        CK(cudaEventElapsedTime(&pass, sums_events[P.ev], sums_events[P.ev + 1]));
+        S.acc_ms += ms;
+        if (P.asked) S.pass_ms += pass;
+        S.acc_launches += its;
+        if (P.last_epoch) n_iter_max = std::max(n_iter_max, its);
+    }
+    pending.clear();
     return QC_OK;
 }
 
@@ -1081,17 +1319,8 @@ int qc_ctx::solve_term(const qc_term *terms, int n_terms, int n, Chain chain, co
     AccLaunch L = acc_launcher(ts, simple, lk, rk, m16);
     const int nat = term_nat(t);
     if (!L.fn && !ddp) return fail(QC_EUNSUPPORTED, "no accumulate kernel for this chain");
-    // the term from per-(interval, pair) sums (qc_moments.cu): one pass over the data, then
-    // every iteration forms the blocks from the sums and the current gains.  No term to the
-    // left: the full form, the term to the right folded into the model; a diagonal or phase-only
-    // term with a term to its left: the diagonal form
-    int mom_form = -1, mom_ok = KIND_NONE;
-    if (o->moments && n_terms <= 2 && !delay[n] && !ddp && d_model != nullptr && n_up > 0 &&
-        (size_t)nb * n_up < (size_t)INT32_MAX) {
-        if (lk == KIND_NONE) { mom_form = FORM_FULL; mom_ok = rk; }
-        else if (t.type != QC_TERM_FULL) { mom_form = FORM_E; mom_ok = lk; }
-    }
-    const bool mom = mom_form >= 0;
+    // the term from per-(interval, pair) sums (qc_moments.cu), iteration by iteration (plan_sums)
+    const bool mom = B.sums.form >= 0;
     // pipelined kernel: shared-memory layout of the per-warp rings for this chain
     PipeArgs pa;
     memset(&pa, 0, sizeof pa);
@@ -1449,57 +1678,14 @@ int qc_ctx::solve_term(const qc_term *terms, int n_terms, int n, Chain chain, co
         dua.tol = ua.tol;
     }
 
-    // sums of the term solve: [bins][unordered pairs][MOM_N or MOM_E] FP32, the per-bin bytes of
-    // one iteration for the byte counter, then the pass's row table
     MomArgs ma;
     MomNormArgs mn;
-    memset(&ma, 0, sizeof ma);
-    memset(&mn, 0, sizeof mn);
-    const int mom_n = mom_form == FORM_E ? MOM_E : MOM_N;
-    const size_t mom_words_all = mom ? (size_t)nb * n_up * mom_n : 0;
+    const int mom_n = mom ? mom_words(B.sums.form) : 0;
+    const size_t mom_words_all = (size_t)nb * n_up * mom_n;
     const size_t mom_cnt_off = ((nbytes<float>(mom_words_all) + 15) / 16) * 16;
-    const size_t mom_rows_off = ((mom_cnt_off + nbytes<long long>(nb) + 15) / 16) * 16;
     if (mom) {
-        if ((rc = ensure(B.mom, mom_rows_off + nbytes<int4>(std::max(1L, n_strip_rows))))) return rc;
-        ma.n_chan = n_chan;
-        ma.n_ant = n_ant;
-        ma.n_up = n_up;
-        ma.vis = d_vis;
-        ma.model = d_model;
-        ma.wf = d_wf;
-        ma.mrows = (const int4 *)((char *)B.mom.ptr + mom_rows_off);
-        ma.strip_off = d_strip_off;
-        ma.n_strips = n_strips;
-        ma.n_chunks = (n_chan + 31) / 32;
-        // an interval several times long: the rows inside each chunk keep a lane's key (units of
-        // a whole strip x one chunk); else a row's chunks inside each row (units of whole rows x
-        // a block of rows), so that an interval one time long flushes once per row.  Either way
-        // about four units per resident warp
-        ma.chunk_major = t.n_tint < n_time ? 1 : 0;
-        const int max_strip = std::max(1, max_strip_rows);
-        const long want_units = 4L * sm_count * 12;
-        if (ma.chunk_major) {
-            ma.group = 1;
-            ma.rb = max_strip;
-        } else {
-            ma.group = ma.n_chunks;
-            const long blocks = std::max(1L, (want_units + std::max(1, n_strips) - 1) / std::max(1, n_strips));
-            ma.rb = (int)std::max(1L, (max_strip + blocks - 1) / blocks);
-        }
-        ma.n_rb = (max_strip + ma.rb - 1) / ma.rb;
-        ma.tn = chain.t[n];
-        ma.to = n_terms == 2 ? chain.t[1 - n] : chain.t[n];
-        ma.mom = (float *)B.mom.ptr;
-        mn.n_bins = nb;
-        mn.n_ant = n_ant;
-        mn.n_up = n_up;
-        mn.type = t.type;
-        mn.form = mom_form;
-        mn.upair = d_upair;
-        mn.mom = ma.mom;
-        mn.params = (const double *)B.params.ptr;
-        mn.tab = (const float4 *)B.tab.ptr;
-        mn.n_fint = t.n_fint;
+        int rc_ = sums_args(terms, n_terms, n, chain, st, ma, mn);
+        if (rc_) return rc_;
         mn.active = (const uint8_t *)B.active.ptr;
         mn.acc = (double *)B.acc.ptr;
         ua.bin_nbytes = (const long long *)((char *)B.mom.ptr + mom_cnt_off);
@@ -1549,11 +1735,9 @@ int qc_ctx::solve_term(const qc_term *terms, int n_terms, int n, Chain chain, co
                     CK(cudaMemsetAsync(B.mom.ptr, 0, nbytes<float>(mom_words_all), st));
                     CK(mom_launch_bytes(nb, (const long long *)B.nvis.ptr + 2 * (size_t)nb, mom_iter_bytes,
                                         (long long *)((char *)B.mom.ptr + mom_cnt_off), ua.acc_bytes, st));
-                    CK(mom_launch_rows(n_strip_rows, d_strip_rows, d_rows, d_row_live, d_up_of_bl,
-                                       const_cast<int4 *>(ma.mrows), st));
                     CK(cudaEventRecordWithFlags(events[ev_pass], st, rec_flags));
                     ma.n_active = cnt;
-                    CK(mom_launch_pass(ma, mom_form, mom_ok, sm_count, st));
+                    CK(mom_launch_pass(ma, B.sums.form, B.sums.ok, sm_count, st));
                     CK(cudaEventRecordWithFlags(events[ev_pass + 1], st, rec_flags));
                 }
                 mn.n_active = cnt + (k - 1);
@@ -1663,7 +1847,7 @@ int qc_ctx::solve_term(const qc_term *terms, int n_terms, int n, Chain chain, co
         ++worked;
         last = k;
     }
-    if (mom && hcnt[0] != 0) {
+    if (mom && B.sums.asked && hcnt[0] != 0) {
         float ms = 0;
         CK(cudaEventElapsedTime(&ms, events[ev_pass], events[ev_pass + 1]));
         *pass_ms = ms;

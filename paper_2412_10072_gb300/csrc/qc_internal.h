@@ -48,13 +48,21 @@ cudaError_t mom_launch_normal(const qc::MomNormArgs &a, cudaStream_t st);
 cudaError_t mom_launch_bytes(int n_bins, const long long *bin_nbytes, long long per_iter, long long *iter_nbytes,
                              unsigned long long *acc_bytes, cudaStream_t st);
 cudaError_t mom_launch_rows(long n, const int *strip_rows, const int4 *rows, const uint8_t *row_live,
-                            const int *up_of_bl, int4 *out, cudaStream_t st);
-size_t mom_words(int form);
+                            const int *up_of_bl, const float *bl_scale, int4 *out, float *scale, cudaStream_t st);
+cudaError_t mom_launch_iterate(const qc::MomIterArgs &a, cudaStream_t st);
 cudaError_t dd_launch_residual(const qc::DDArgs &a, int grid, cudaStream_t st);
 
 struct Buf {
     void *ptr = nullptr;
     size_t bytes = 0;
+};
+
+// How a term of the current call is solved from per-(interval, pair) sums (qc_moments.cu).
+struct SumsPlan {
+    int form = -1;             // FORM_*, or -1: iterations on the samples
+    int ok = 0;                // KIND_* of the fixed term
+    bool asked = false;        // by qc_opts.moments (else the route was chosen by its cost)
+    bool one_launch = false;   // every iteration in one launch (mom_iterate_kernel)
 };
 
 // Device buffers of one chain position, reused across calls while large enough.
@@ -88,7 +96,8 @@ struct TermBufs {
     Buf ws_sb;     // warp-specialised kernel, strip tiles: uint32 [n_chunks][words] active-entry bits
     Buf div;       // divergence flagging: double [bins][ant][2] first / last relative updates
     Buf params0;   // divergence flagging: the FP64 parameters before the solve
-    Buf mom;       // single-term chains: FP64 sums per (interval, unordered baseline)
+    Buf mom;       // a term solved from sums: FP32 sums per (interval, unordered pair), bytes per interval
+    SumsPlan sums; // the route of the current call
     Buf dfmap;     // delay terms: int [n_chan] parameter interval of each channel
     Buf dfr;       // delay terms: int2 [n_fint] first and last channel of each interval
     Buf dnu;       // delay terms: double [n_chan] channel frequencies
@@ -190,6 +199,16 @@ struct qc_ctx {
     Buf mad_out;                      // MAD flagging: uint8 [n_vis] flags (host output staging)
     Buf mad_groups;                   // MAD flagging, per-baseline mode: group offsets, then rows
     Buf resid_stage;
+    // terms solved from sums: the strip rows as the pass reads them (int4, then the FP16 scales)
+    Buf mom_rows;
+    bool mom_rows_ready = false;
+    // term solves whose statistics are read back with the next synchronisation
+    struct Pending { int off, max_iter, n_bins, ev; bool last_epoch, asked; };
+    static constexpr int MAX_PENDING = 16;
+    std::vector<Pending> pending;
+    std::vector<int> pending_cnt;
+    std::vector<cudaEvent_t> sums_events;   // three per pending term solve
+    Buf sums_cnt;                     // int: intervals still active after iteration k, per pending solve
     long long launches = 0;
     std::vector<const void *> configured_fns;   // kernels whose dynamic smem limit was raised
     std::string err;
@@ -218,6 +237,13 @@ struct qc_ctx {
     qc::Data data_desc() const;
     int run_residual(const qc::Chain &chain, float4 *dres, double *d_chi2, cudaStream_t st);
     int pick_order(const qc_term &t, const qc_opts *o) const;
+    int plan_sums(const qc_term *terms, int n_terms, int n, const qc_opts *o);
+    int sums_args(const qc_term *terms, int n_terms, int n, const qc::Chain &chain, cudaStream_t st, qc::MomArgs &ma,
+                  qc::MomNormArgs &mn);
+    int solve_term_sums(const qc_term *terms, int n_terms, int n, const qc::Chain &chain, const qc_opts *o,
+                        cudaStream_t st, bool last_epoch);
+    int copy_pending(cudaStream_t st);
+    int collect_sums(qc_stats &S, int &n_iter_max);
     int solve_term(const qc_term *terms, int n_terms, int n, qc::Chain chain, const qc_opts *o, cudaStream_t st,
                    int *it_max, double *acc_ms, long long *acc_launches, double *pass_ms);
 };

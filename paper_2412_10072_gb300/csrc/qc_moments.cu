@@ -7,28 +7,32 @@
 // D -> D^H, M -> M^H, the cross-hand weights swapped, p and q exchanged); kj = 2k + j indexes the
 // weight and data of correlation (k, j).
 //
-// Full form: the solved term G (any kind) has no term to its left.  With X = R_p M R_q^H, R the
+// Full form: the solved term G is full-Jones with no term to its left.  With X = R_p M R_q^H, R the
 // term to its right (X = M when there is none), and u = 2l + m indexing X_lm:
-//     S[kj][u][v] = sum w_kj conj(X_u) X_v,  T[kj][u] = sum w_kj conj(X_u) D_kj,
-//     U[kj] = sum w_kj |D_kj|^2                                               (100 words)
+//     S[kj][u][v] = sum w_kj conj(X_u) X_v,  T[kj][u] = sum w_kj conj(X_u) D_kj    (96 words of 100)
 //     JHJ_p[(k,l),(k,l')] += sum_j sum_m sum_m' G_q,jm conj(G_q,jm') S[kj][(l,m)][(l',m')]
 //     b_p[(k,l)]          += sum_j sum_m G_q,jm T[kj][(l,m)]
 //     JHJ_q[(k,l),(k,l')] += sum_j sum_m sum_m' G_p,jm conj(G_p,jm') conj(S[jk][(m,l)][(m',l')])
 //     b_q[(k,l)]          += sum_j sum_m G_p,jm conj(T[jk][(m,l)])
-// Diagonal form: the solved term g (diagonal or phase-only) has a term L to its left.  With
+// E form: the solved term g (diagonal or phase-only) has a full term L to its left.  With
 // E_kj,ab = L_p,ka M_ab conj(L_q,jb) and u = 2a + b:
-//     S'[u][v] = sum sum_kj w_kj conj(E_kj,u) E_kj,v,  T'[u] = sum sum_kj w_kj conj(E_kj,u) D_kj,
-//     U = sum sum_kj w_kj |D_kj|^2                                            (25 words)
+//     S'[u][v] = sum sum_kj w_kj conj(E_kj,u) E_kj,v,  T'[u] = sum sum_kj w_kj conj(E_kj,u) D_kj
+//                                                                                  (24 words of 28)
 //     JHJ_p[a][a'] += sum_b sum_b' g_q,b conj(g_q,b') S'[(a,b)][(a',b')],  b_p[a] += sum_b g_q,b T'[(a,b)]
 //     JHJ_q[b][b'] += sum_a sum_a' g_p,a conj(g_p,a') conj(S'[(a,b)][(a',b')]),
 //     b_q[b]       += sum_a g_p,a conj(T'[(a,b)])
-// In both forms JHr = b - JHJ vec(g).  One pass over the data per term solve forms the sums in
+// Plain diagonal form: any other diagonal or phase-only solved term (the other term diagonal, or to
+// its right).  With X = O_p M O_q^H: S_kj = sum w_kj |X_kj|^2, T_kj = sum w_kj conj(X_kj) D_kj (12 words),
+//     JHJ_p[k][k] += sum_j |g_q,j|^2 S_kj,  b_p[k] += sum_j g_q,j T_kj,  and conjugated for q.
+// In all of them JHr = b - JHJ vec(g).  One pass over the data per term solve forms the sums in
 // FP32 (mom_pass_kernel: per-lane register sums, added to the slots by FP32 atomics, a few per
-// slot: a warp covers a whole row, or a whole strip of one chunk); every iteration forms each
-// antenna's blocks from them and the current gains in FP32 (mom_normal_kernel), JHr = b - JHJ g
-// and everything after it in FP64, in the update kernel's accumulator layout (a diagonal or
-// phase-only term of the full form takes the (0, 3) rows and columns).  An iteration then reads
-// 400 or 112 B per (interval, pair) instead of 81 B per sample.
+// slot: a warp covers a whole row, or a strip of one chunk).  The intervals are independent from
+// there on, so one CTA per interval runs all of its iterations (mom_iterate_kernel): an iteration
+// reads 400, 112 or 48 B per (interval, pair) and side out of L2 instead of 80 B per sample out of
+// HBM, with no launch in between.  Measured on the two-term chain (64 antennas, 300 x 512, three
+// epochs of 20 iterations a term): 663 ms with the iterations on the samples, 47.0 ms from sums (passes 6.3
+// ms for G, 6.8 ms for B, 20 iterations 1.5 and 0.9 ms); 27 antennas, 61 x 131, intervals of 5 x 17: 3.80
+// -> 0.36 ms; 7 antennas, 60 x 16: 1.03 -> 0.28 ms.
 #include "qc_internal.h"
 
 #include <algorithm>
@@ -46,9 +50,10 @@ __device__ __forceinline__ void cacc_conj(float &re, float &im, float2 x, float2
 }
 
 // One sample's terms added to a lane's register sums, full form (one lane per sample; words as
-// the slot: S[kj] at 16 kj, T[kj] at MOM_T + 8 kj, U[kj] at MOM_U + kj; all indices compile-time
-// constants after unrolling; X = R_p M R_q^H).
-__device__ __forceinline__ void mom_add(float (&acc)[MOM_N], const J2 &D, const J2 &X, float4 w)
+// the slot: S[kj] at 16 kj, T[kj] at MOM_T + 8 kj; all indices compile-time constants after
+// unrolling; X = R_p M R_q^H).
+constexpr int MOM_FW = 96;
+__device__ __forceinline__ void mom_add(float (&acc)[MOM_FW], const J2 &D, const J2 &X, float4 w)
 {
     const float2 x[4] = { X.a, X.b, X.c, X.d };
     const float2 d[4] = { D.a, D.b, D.c, D.d };
@@ -75,54 +80,87 @@ __device__ __forceinline__ void mom_add(float (&acc)[MOM_N], const J2 &D, const 
         const int t = MOM_T + 8 * kj;
 #pragma unroll
         for (int u = 0; u < 4; ++u) cacc_conj(acc[t + 2 * u], acc[t + 2 * u + 1], x[u], wd);   // conj(x_u) w d
-        acc[MOM_U + kj] = fmaf(wv[kj], cnorm2(d[kj]), acc[MOM_U + kj]);
     }
 }
 
 // The diagonal form, one lane per sample: register words [0, 16) S' packed as the full form's
-// S blocks, [16, 24) T', 24 U.
-constexpr int MOM_EW = 25;
+// S blocks, [16, 24) T'.
+constexpr int MOM_EW = 24;
 
-template <int LK>
+// The plain diagonal form: X_kj = R_p,k M_kj conj(R_q,j) for a diagonal fixed term on either side
+// (or R_p M R_q^H for a full one on the right): words [0, 4) S_kj = sum w |X_kj|^2, [4, 12) T_kj =
+// sum w conj(X_kj) D_kj.
+__device__ __forceinline__ void mom_add_d(float (&acc)[MOM_D], const J2 &D, const J2 &X, float4 w)
+{
+    const float2 x[4] = { X.a, X.b, X.c, X.d };
+    const float2 d[4] = { D.a, D.b, D.c, D.d };
+    const float wv[4] = { w.x, w.y, w.z, w.w };
+#pragma unroll
+    for (int kj = 0; kj < 4; ++kj) {
+        acc[kj] = fmaf(wv[kj], cnorm2(x[kj]), acc[kj]);
+        cacc_conj(acc[4 + 2 * kj], acc[5 + 2 * kj], x[kj], cscale(d[kj], wv[kj]));
+    }
+}
+
+// E form: with E_kj,ab = L_p,ka M_ab conj(L_q,jb), every product conj(E_kj,ab) E_kj,a'b' is conj(M_ab)
+// M_a'b' times a factor of L alone, so the four correlations are summed in those factors first,
+//   K[(a,b)][(a',b')] = sum_k P_k[a][a'] sum_j w_kj Q_j[b][b'],
+//   P_k[a][a'] = conj(L_p,ka) L_p,ka',  Q_j[b][b'] = L_q,jb conj(L_q,jb'),
+// S' += conj(M_ab) M_a'b' K, and T' += conj(M_ab) (L_p^H (w D) L_q)_ab.  Forming the E_kj and adding their
+// products one by one takes 390 instructions a sample, this 236, and each word of the sums is
+// rounded once or twice a sample instead of eight times.
 __device__ __forceinline__ void mom_add_e(float (&acc)[MOM_EW], const J2 &D, const J2 &M, const J2 &Lp,
                                           const J2 &Lq, float4 w)
 {
     const float2 m[4] = { M.a, M.b, M.c, M.d };       // M_ab at 2a + b
     const float2 lp[4] = { Lp.a, Lp.b, Lp.c, Lp.d };  // L_p,ka at 2k + a
     const float2 lq[4] = { Lq.a, Lq.b, Lq.c, Lq.d };
-    const float2 d[4] = { D.a, D.b, D.c, D.d };
     const float wv[4] = { w.x, w.y, w.z, w.w };
+    float kd[4] = { 0.f, 0.f, 0.f, 0.f };             // K on the diagonal
+    float2 ko[6];                                     // K[u][v] at mom_pair(u, v)
 #pragma unroll
-    for (int kj = 0; kj < 4; ++kj) {
-        const int k = kj >> 1, j = kj & 1;
-        if constexpr (LK == KIND_DIAG) {
-            // E_kj,ab is non-zero only at (a, b) = (k, j): S' stays diagonal
-            const float2 e = cmulc(cmul(lp[3 * k], m[kj]), lq[3 * j]);
-            acc[kj] = fmaf(wv[kj], cnorm2(e), acc[kj]);
-            cacc_conj(acc[16 + 2 * kj], acc[17 + 2 * kj], e, cscale(d[kj], wv[kj]));   // conj(e) w d
-        } else {
-            // sqrt(w) E_kj: S' += conj(e_u) e_v, T' += conj(e_u) sqrt(w) d
-            const float sw = sqrtf(wv[kj]);
-            float2 e[4];
+    for (int i = 0; i < 6; ++i) ko[i] = make_float2(0.f, 0.f);
 #pragma unroll
-            for (int a = 0; a < 2; ++a) {
-                const float2 l = cscale(lp[2 * k + a], sw);
-#pragma unroll
-                for (int b = 0; b < 2; ++b) e[2 * a + b] = cmul(l, cmulc(m[2 * a + b], lq[2 * j + b]));
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u) acc[u] = fmaf(e[u].x, e[u].x, fmaf(e[u].y, e[u].y, acc[u]));
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-#pragma unroll
-                for (int v = u + 1; v < 4; ++v)
-                    cacc_conj(acc[4 + 2 * mom_pair(u, v)], acc[5 + 2 * mom_pair(u, v)], e[u], e[v]);
-            const float2 ds = cscale(d[kj], sw);
-#pragma unroll
-            for (int u = 0; u < 4; ++u) cacc_conj(acc[16 + 2 * u], acc[17 + 2 * u], e[u], ds);
-        }
-        acc[24] = fmaf(wv[kj], cnorm2(d[kj]), acc[24]);
+    for (int k = 0; k < 2; ++k) {
+        const float w0 = wv[2 * k], w1 = wv[2 * k + 1];
+        const float r0 = fmaf(w0, cnorm2(lq[0]), w1 * cnorm2(lq[2]));      // sum_j w_kj Q_j[0][0]
+        const float r1 = fmaf(w0, cnorm2(lq[1]), w1 * cnorm2(lq[3]));
+        const float2 qa = cmulc(lq[0], lq[1]), qb = cmulc(lq[2], lq[3]);
+        const float2 r01 = make_float2(fmaf(w0, qa.x, w1 * qb.x), fmaf(w0, qa.y, w1 * qb.y));
+        const float p0 = cnorm2(lp[2 * k]), p1 = cnorm2(lp[2 * k + 1]);
+        const float2 p01 = cmulc(lp[2 * k + 1], lp[2 * k]);                // conj(L_k0) L_k1
+        kd[0] = fmaf(p0, r0, kd[0]);
+        kd[1] = fmaf(p0, r1, kd[1]);
+        kd[2] = fmaf(p1, r0, kd[2]);
+        kd[3] = fmaf(p1, r1, kd[3]);
+        ko[0] = make_float2(fmaf(p0, r01.x, ko[0].x), fmaf(p0, r01.y, ko[0].y));       // (00)(01)
+        ko[5] = make_float2(fmaf(p1, r01.x, ko[5].x), fmaf(p1, r01.y, ko[5].y));       // (10)(11)
+        ko[1] = make_float2(fmaf(r0, p01.x, ko[1].x), fmaf(r0, p01.y, ko[1].y));       // (00)(10)
+        ko[4] = make_float2(fmaf(r1, p01.x, ko[4].x), fmaf(r1, p01.y, ko[4].y));       // (01)(11)
+        // (00)(11): p01 r01;  (01)(10): p01 conj(r01)
+        ko[2] = make_float2(fmaf(p01.x, r01.x, fmaf(-p01.y, r01.y, ko[2].x)),
+                            fmaf(p01.x, r01.y, fmaf(p01.y, r01.x, ko[2].y)));
+        ko[3] = make_float2(fmaf(p01.x, r01.x, fmaf(p01.y, r01.y, ko[3].x)),
+                            fmaf(-p01.x, r01.y, fmaf(p01.y, r01.x, ko[3].y)));
     }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        acc[u] = fmaf(cnorm2(m[u]), kd[u], acc[u]);
+#pragma unroll
+        for (int v = u + 1; v < 4; ++v) {
+            const int i = mom_pair(u, v);
+            const float2 z = cmulc(m[v], m[u]);                             // conj(M_u) M_v
+            acc[4 + 2 * i] = fmaf(z.x, ko[i].x, fmaf(-z.y, ko[i].y, acc[4 + 2 * i]));
+            acc[5 + 2 * i] = fmaf(z.x, ko[i].y, fmaf(z.y, ko[i].x, acc[5 + 2 * i]));
+        }
+    }
+    J2 wd;
+    wd.a = cscale(D.a, w.x); wd.b = cscale(D.b, w.y);
+    wd.c = cscale(D.c, w.z); wd.d = cscale(D.d, w.w);
+    const J2 z = j_mul(j_herm(Lp), j_mul(wd, Lq));
+    const float2 zv[4] = { z.a, z.b, z.c, z.d };
+#pragma unroll
+    for (int u = 0; u < 4; ++u) cacc_conj(acc[16 + 2 * u], acc[17 + 2 * u], m[u], zv[u]);
 }
 
 // Add the warp's register sums (NW words, the slot's order) to the sums of each lane's key
@@ -190,7 +228,7 @@ __device__ __forceinline__ void mom_flush(float (&acc)[NW], int key, int lane, f
 // The rows of the baseline strips in strip order, as the pass reads them: {row (-1: no usable
 // sample), time, pair | conj << 31, p | q << 16} with (p, q) the baseline as the sums orient it.
 static __global__ void mom_rows_kernel(long n, const int *strip_rows, const int4 *rows, const uint8_t *row_live,
-                                       const int *up_of_bl, int4 *out)
+                                       const int *up_of_bl, const float *bl_scale, int4 *out, float *scale)
 {
     const long k = (long)blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= n) return;
@@ -200,6 +238,7 @@ static __global__ void mom_rows_kernel(long n, const int *strip_rows, const int4
     const int p = conj ? r.y : r.x, q = conj ? r.x : r.y;
     out[k] = make_int4(row_live[row] ? row : -1, r.z, (int)((unsigned)up_of_bl[r.w] | (conj ? 0x80000000u : 0u)),
                        p | (q << 16));
+    if (scale) scale[k] = bl_scale[r.w];
 }
 
 template <int K>
@@ -211,13 +250,14 @@ __device__ __forceinline__ J2 fac_jones(const float4 *o)
 }
 
 // Shape of a warp's ring of the pass (one lane per sample, 32-channel chunks): per stage, in
-// float4 units, the chunk's data quads d0 [0, 32), d1 [32, 64), model quads m0 [64, 96),
-// m1 [96, 128), folded weights w [128, 160), then the fixed term's table entries for p and for
+// float4 units, the chunk's data quads d0 [0, 32), d1 [32, 64), model quads m0 [64, 96) and m1
+// (FP16 model: one word), folded weights w, then the fixed term's table entries for p and for
 // q (NO float4 each, per channel, or only the first one when the chunk lies in one of the term's
 // frequency intervals), the lanes' keys (32 ints) and one int4 of meta data.
-template <int FORM, int OK> struct MomRing {
+template <int FORM, int OK, bool M16> struct MomRing {
     static constexpr int NO = OK == KIND_FULL ? 2 : (OK == KIND_DIAG ? 1 : 0);
-    static constexpr int OFF_OP = 160, OFF_OQ = OFF_OP + 32 * NO, OFF_KEY = OFF_OQ + 32 * NO;
+    static constexpr int OFF_W = M16 ? 96 : 128;
+    static constexpr int OFF_OP = OFF_W + 32, OFF_OQ = OFF_OP + 32 * NO, OFF_KEY = OFF_OQ + 32 * NO;
     static constexpr int OFF_META = OFF_KEY + 8;
     static constexpr int STAGE = OFF_META + 1;               // float4 per stage
     // three CTAs of 4 warps per SM (the full form's 100 register sums fit 168 registers); ring
@@ -225,6 +265,14 @@ template <int FORM, int OK> struct MomRing {
     static constexpr int PER_SM = 3;
     static constexpr int DEPTH = NO == 2 ? 3 : (NO == 1 ? 4 : 6);
     static constexpr size_t SMEM = (size_t)4 * DEPTH * STAGE * sizeof(float4);
+    // A lane's sums over a long strip are FP32 sums of terms of one sign, whose rounding grows with
+    // the number of terms and moves the fixed point of all antennas the same way.  The short slots keep
+    // a second set of registers that takes the first one's sums every 8 steps; the full form, which
+    // has no registers left, goes to its slot every 32 (16 with the FP16 model).  Measured over three
+    // epochs of G and B (64 antennas, 40 integrations): B's error against FP64 1.7e-7 without, 3.7e-8
+    // with sums of 8, 3.2e-8 for the iterations on the samples.
+    static constexpr bool TWO_LEVEL = FORM != FORM_FULL;
+    static constexpr int FLUSH_EVERY = TWO_LEVEL ? 1 << 30 : (M16 ? 16 : 32);
 };
 
 constexpr int MOM_END = 2;       // meta: the warp's steps have run out (bit 0: conjugate baseline)
@@ -233,8 +281,8 @@ constexpr int MOM_END = 2;       // meta: the warp's steps have run out (bit 0: 
 // of rb rows of one baseline strip x a group of chunks), each copied into a ring stage by
 // cp.async (zero-filled past the last channel and for rows without usable data, whose weights
 // then read 0).
-template <int FORM, int OK> struct MomCursor {
-    using R = MomRing<FORM, OK>;
+template <int FORM, int OK, bool M16> struct MomCursor {
+    using R = MomRing<FORM, OK, M16>;
     long unit, n_units, stride;
     int n_groups;
     int k0, k1, ch0, ch1, k, ch;
@@ -292,9 +340,13 @@ template <int FORM, int OK> struct MomCursor {
             const uint32_t nb = rd ? 16u : 0u;
             cp_async16(stage + lane, a.vis + 2 * i, nb);
             cp_async16(stage + 32 + lane, a.vis + 2 * i + 1, nb);
-            cp_async16(stage + 64 + lane, a.model + 2 * i, nb);
-            cp_async16(stage + 96 + lane, a.model + 2 * i + 1, nb);
-            cp_async16(stage + 128 + lane, a.wf + i, nb);
+            if constexpr (M16) {
+                cp_async16(stage + 64 + lane, a.model16 + i, nb);
+            } else {
+                cp_async16(stage + 64 + lane, a.model + 2 * i, nb);
+                cp_async16(stage + 96 + lane, a.model + 2 * i + 1, nb);
+            }
+            cp_async16(stage + R::OFF_W + lane, a.wf + i, nb);
             if constexpr (R::NO > 0) {
                 const int ti = __ldg(a.to.t_map + mr.y);
                 const int f_first = __ldg(a.to.f_map + c0);
@@ -324,7 +376,10 @@ template <int FORM, int OK> struct MomCursor {
                 in ? (__ldg(a.tn.t_map + mr.y) * a.tn.n_fint + __ldg(a.tn.f_map + c)) * a.n_up + (mr.z & 0x7fffffff)
                    : -1;
         }
-        if (lane == 0) reinterpret_cast<int *>(stage + R::OFF_META)[0] = meta;
+        if (lane == 0) {
+            reinterpret_cast<int *>(stage + R::OFF_META)[0] = meta;
+            if (M16 && unit < n_units) reinterpret_cast<float *>(stage + R::OFF_META)[1] = __ldg(a.mscale + k);
+        }
         cp_async_commit();
         if (unit < n_units) advance(a);
     }
@@ -337,20 +392,29 @@ template <int FORM, int OK> struct MomCursor {
 // DEPTH - 1 steps ahead of the arithmetic, which adds each lane's sample to its register sums;
 // the sums are flushed when any lane's (interval, pair) key changes.  The fixed term is L
 // (diagonal form) or R (full form) of kind OK.
-template <int FORM, int OK>
-static __global__ void __launch_bounds__(128, MomRing<FORM, OK>::PER_SM) mom_pass_kernel(const MomArgs a)
+template <int FORM, int OK, bool M16>
+static __global__ void __launch_bounds__(128, MomRing<FORM, OK, M16>::PER_SM) mom_pass_kernel(const MomArgs a)
 {
-    using R = MomRing<FORM, OK>;
-    constexpr int NW = FORM == FORM_FULL ? MOM_N : MOM_EW;
-    if (__ldg(a.n_active) == 0) return;
+    using R = MomRing<FORM, OK, M16>;
+    constexpr int NW = FORM == FORM_FULL ? MOM_FW : (FORM == FORM_E ? MOM_EW : MOM_D);
+    if (a.n_active && __ldg(a.n_active) == 0) return;
     extern __shared__ float4 mom_ring[];
     const int lane = threadIdx.x & 31;
     float4 *ring = mom_ring + (size_t)(threadIdx.x >> 5) * R::DEPTH * R::STAGE;
-    const int stride = FORM == FORM_FULL ? MOM_N : MOM_E;
-    float acc[NW];
+    constexpr int stride = mom_words(FORM);
+    float acc[NW], hi[R::TWO_LEVEL ? NW : 1];
 #pragma unroll
-    for (int v = 0; v < NW; ++v) acc[v] = 0.f;
-    MomCursor<FORM, OK> cur;
+    for (int v = 0; v < NW; ++v) {
+        acc[v] = 0.f;
+        if constexpr (R::TWO_LEVEL) hi[v] = 0.f;
+    }
+    auto lift = [&]() {
+        if constexpr (R::TWO_LEVEL) {
+#pragma unroll
+            for (int v = 0; v < NW; ++v) { hi[v] += acc[v]; acc[v] = 0.f; }
+        }
+    };
+    MomCursor<FORM, OK, M16> cur;
     cur.start(a, ((long)blockIdx.x * blockDim.x + threadIdx.x) >> 5, ((long)gridDim.x * blockDim.x) >> 5);
     int is = 0;
 #pragma unroll
@@ -359,16 +423,21 @@ static __global__ void __launch_bounds__(128, MomRing<FORM, OK>::PER_SM) mom_pas
         if (++is == R::DEPTH) is = 0;
     }
     auto add = [&](const float4 *st, int meta) {
-        float4 w = st[128 + lane];
+        float4 w = st[R::OFF_W + lane];
         if (w.x != 0.f || w.y != 0.f || w.z != 0.f || w.w != 0.f) {
-            J2 D = j_from(st[lane], st[32 + lane]), M = j_from(st[64 + lane], st[96 + lane]);
+            J2 D = j_from(st[lane], st[32 + lane]), M;
+            if constexpr (M16)
+                M = load_model16(*reinterpret_cast<const uint4 *>(st + 64 + lane),
+                                 reinterpret_cast<const float *>(st + R::OFF_META)[1]);
+            else
+                M = j_from(st[64 + lane], st[96 + lane]);
             if (meta & 1) {                    // the conjugate baseline: D -> D^H, M -> M^H, w permuted
                 D = j_herm(D);
                 M = j_herm(M);
                 w = make_float4(w.x, w.z, w.y, w.w);
             }
             const int oc = (meta & 4) ? 0 : lane * R::NO;
-            if constexpr (FORM == FORM_FULL) {
+            if constexpr (FORM != FORM_E) {
                 if constexpr (OK == KIND_DIAG) {
                     const float4 rp = st[R::OFF_OP + oc], rq = st[R::OFF_OQ + oc];
                     M = j_muld(j_dmul(make_float2(rp.x, rp.y), make_float2(rp.z, rp.w), M),
@@ -376,15 +445,16 @@ static __global__ void __launch_bounds__(128, MomRing<FORM, OK>::PER_SM) mom_pas
                 } else if constexpr (OK == KIND_FULL) {
                     M = j_mul_h(j_mul(fac_jones<OK>(st + R::OFF_OP + oc), M), fac_jones<OK>(st + R::OFF_OQ + oc));
                 }
-                mom_add(acc, D, M, w);
+                if constexpr (FORM == FORM_FULL) mom_add(acc, D, M, w);
+                else mom_add_d(acc, D, M, w);
             } else {
-                mom_add_e<OK>(acc, D, M, fac_jones<OK>(st + R::OFF_OP + oc), fac_jones<OK>(st + R::OFF_OQ + oc), w);
+                mom_add_e(acc, D, M, fac_jones<OK>(st + R::OFF_OP + oc), fac_jones<OK>(st + R::OFF_OQ + oc), w);
             }
         }
     };
     // runs of steps with unchanged keys: the inner loop only adds; a key change leaves it to
     // flush the sums, then adds the step that changed the key
-    int key_cur = -1, stage = 0;
+    int key_cur = -1, stage = 0, run = 0;
     bool done = false;
     for (;;) {
         const float4 *st;
@@ -399,12 +469,19 @@ static __global__ void __launch_bounds__(128, MomRing<FORM, OK>::PER_SM) mom_pas
             meta = reinterpret_cast<const int *>(st + R::OFF_META)[0];
             if (meta & MOM_END) { done = true; break; }
             key = reinterpret_cast<const int *>(st + R::OFF_KEY)[lane];
-            if (__any_sync(FULL_MASK, key != key_cur)) break;
+            if (__any_sync(FULL_MASK, key != key_cur) || ++run == R::FLUSH_EVERY) break;
+            if (R::TWO_LEVEL && (run & 7) == 0) lift();
             add(st, meta);
             if (++stage == R::DEPTH) stage = 0;
         }
-        mom_flush<NW>(acc, key_cur, lane, a.mom, stride);
+        if constexpr (R::TWO_LEVEL) {
+            lift();
+            mom_flush<NW>(hi, key_cur, lane, a.mom, stride);
+        } else {
+            mom_flush<NW>(acc, key_cur, lane, a.mom, stride);
+        }
         if (done) break;
+        run = 0;
         key_cur = key;
         add(st, meta);
         if (++stage == R::DEPTH) stage = 0;
@@ -413,288 +490,319 @@ static __global__ void __launch_bounds__(128, MomRing<FORM, OK>::PER_SM) mom_pas
 }
 
 // gains of an antenna in a bin as complex FP64 entries (row-major; phase-only: diag(e^{i phi}))
-__device__ __forceinline__ void gains_of(const MomNormArgs &A, int bin, int ant, double2 G[4])
+__device__ __forceinline__ void gains_of(int type, const double *params, size_t pidx, double2 G[4])
 {
-    const size_t pidx = (size_t)bin * A.n_ant + ant;
-    if (A.type == QC_TERM_PHASE) {
+    if (type == QC_TERM_PHASE) {
         double sn, cs;
-        sincos(A.params[2 * pidx], &sn, &cs);
+        sincos(params[2 * pidx], &sn, &cs);
         G[0] = make_double2(cs, sn);
-        sincos(A.params[2 * pidx + 1], &sn, &cs);
+        sincos(params[2 * pidx + 1], &sn, &cs);
         G[3] = make_double2(cs, sn);
         G[1] = G[2] = make_double2(0.0, 0.0);
     } else {
-        const double2 *P = reinterpret_cast<const double2 *>(A.params) + 4 * pidx;
+        const double2 *P = reinterpret_cast<const double2 *>(params) + 4 * pidx;
 #pragma unroll
         for (int e = 0; e < 4; ++e) G[e] = P[e];
     }
 }
 
-__device__ __forceinline__ float2 f2(double2 a) { return make_float2((float)a.x, (float)a.y); }
-
-// a slot's words held in registers (loaded as 16-byte or 8-byte vectors); word i of the slot
-template <int NV> struct SlotRegs {
-    float4 v[NV];
-    __device__ __forceinline__ float at(int i) const
-    {
-        const float4 &x = v[i >> 2];
-        const int c = i & 3;
-        return c == 0 ? x.x : c == 1 ? x.y : c == 2 ? x.z : x.w;
-    }
-    // element (u, v) of the Hermitian S block at word `base` (u, v compile-time after unrolling)
-    __device__ __forceinline__ float2 S(int base, int u, int v) const
-    {
-        if (u == v) return make_float2(at(base + u), 0.f);
-        const int i = base + 4 + 2 * (u < v ? mom_pair(u, v) : mom_pair(v, u));
-        return u < v ? make_float2(at(i), at(i + 1)) : make_float2(at(i), -at(i + 1));
-    }
-    __device__ __forceinline__ float2 C(int i) const { return make_float2(at(i), at(i + 1)); }
+// One antenna's normal equations from its pairs, the register sums of a lane: per block k the
+// Hermitian 2x2 [[h00, h01], [conj(h01), h11]] and b[2] (the full form has two blocks, rows
+// (k, 0), (k, 1) of G; the other forms one, over g_XX and g_YY).
+constexpr int NE_WORDS = 8;      // h00, h11, Re h01, Im h01, b0, b1 of one block
+template <int FORM> struct NormSums {
+    static constexpr int NB = FORM == FORM_FULL ? 2 : 1;
+    static constexpr int NWORD = NB * NE_WORDS;
 };
 
-// the other antenna's gains from the solved term's FP32 table (the update kernel writes it with
-// every update): row-major entries, a diagonal or phase-only term as diag(g_0, g_1)
-__device__ __forceinline__ void gains_f32(const MomNormArgs &A, int bin, int ant, float2 G[4])
+// The pair's contribution of one 4x4 block S (16 packed words), T (8 words) with the other
+// antenna's gain row (g0, g1): with u = 2l + m,
+//   h[l][l2] += sum_m sum_m2 g_m conj(g_m2) S[(l,m)][(l2,m2)],  b[l] += sum_m g_m T[(l,m)].
+// The q side takes conj(S[(m,l)][(m2,l2)]) and conj(T[(m,l)]): indices 1 and 2 exchanged, conjugated.
+__device__ __forceinline__ void pair_block(const float4 *__restrict__ sv, const float4 *__restrict__ tv, bool p_side,
+                                           float2 g0, float2 g1, float *h)
 {
-    const int tint = bin / A.n_fint, fint = bin - tint * A.n_fint;
-    const size_t idx = ((size_t)tint * A.n_ant + ant) * A.n_fint + fint;
-    if (A.type == QC_TERM_FULL) {
-        const float4 lo = __ldg(A.tab + 2 * idx), hi = __ldg(A.tab + 2 * idx + 1);
-        G[0] = make_float2(lo.x, lo.y); G[1] = make_float2(lo.z, lo.w);
-        G[2] = make_float2(hi.x, hi.y); G[3] = make_float2(hi.z, hi.w);
-    } else {
-        const float4 d = __ldg(A.tab + idx);
-        G[0] = make_float2(d.x, d.y); G[3] = make_float2(d.z, d.w);
-        G[1] = G[2] = make_float2(0.f, 0.f);
-    }
+    const float4 a0 = __ldg(sv), a1 = __ldg(sv + 1), a2 = __ldg(sv + 2), a3 = __ldg(sv + 3);
+    const float4 t0 = __ldg(tv), t1 = __ldg(tv + 1);
+    const float sg = p_side ? 1.f : -1.f;
+    const float d1 = p_side ? a0.y : a0.z, d2 = p_side ? a0.z : a0.y;
+    float2 s01 = p_side ? make_float2(a1.x, a1.y) : make_float2(a1.z, a1.w);
+    float2 s02 = p_side ? make_float2(a1.z, a1.w) : make_float2(a1.x, a1.y);
+    float2 s03 = make_float2(a2.x, a2.y);
+    const float2 s12 = make_float2(a2.z, a2.w);             // its own conjugate transpose on the q side
+    float2 s13 = p_side ? make_float2(a3.x, a3.y) : make_float2(a3.z, a3.w);
+    float2 s23 = p_side ? make_float2(a3.z, a3.w) : make_float2(a3.x, a3.y);
+    s01.y *= sg; s02.y *= sg; s03.y *= sg; s13.y *= sg; s23.y *= sg;
+    float2 u0 = make_float2(t0.x, t0.y), u3 = make_float2(t1.z, t1.w);
+    float2 u1 = p_side ? make_float2(t0.z, t0.w) : make_float2(t1.x, t1.y);
+    float2 u2 = p_side ? make_float2(t1.x, t1.y) : make_float2(t0.z, t0.w);
+    u0.y *= sg; u1.y *= sg; u2.y *= sg; u3.y *= sg;
+    const float n0 = cnorm2(g0), n1 = cnorm2(g1);
+    const float2 x = cmulc(g0, g1);                         // g_0 conj(g_1)
+    h[0] += fmaf(n0, a0.x, fmaf(n1, d1, 2.f * fmaf(x.x, s01.x, -x.y * s01.y)));
+    h[1] += fmaf(n0, d2, fmaf(n1, a0.w, 2.f * fmaf(x.x, s23.x, -x.y * s23.y)));
+    // n0 S02 + n1 S13 + x S03 + conj(x) S12
+    h[2] += fmaf(n0, s02.x, fmaf(n1, s13.x, fmaf(x.x, s03.x + s12.x, x.y * (s12.y - s03.y))));
+    h[3] += fmaf(n0, s02.y, fmaf(n1, s13.y, fmaf(x.x, s03.y + s12.y, x.y * (s03.x - s12.x))));
+    h[4] += fmaf(g0.x, u0.x, fmaf(-g0.y, u0.y, fmaf(g1.x, u1.x, -g1.y * u1.y)));
+    h[5] += fmaf(g0.x, u0.y, fmaf(g0.y, u0.x, fmaf(g1.x, u1.y, g1.y * u1.x)));
+    h[6] += fmaf(g0.x, u2.x, fmaf(-g0.y, u2.y, fmaf(g1.x, u3.x, -g1.y * u3.y)));
+    h[7] += fmaf(g0.x, u2.y, fmaf(g0.y, u2.x, fmaf(g1.x, u3.y, g1.y * u3.x)));
 }
 
-// One warp per (interval, antenna a): lanes take the other antennas o, form the contributions
-// of the pair (a, o) to a's block-diagonal J^H W J (the 2x2 blocks k = 0, 1 on rows
-// (k, l), l = 0, 1) and to b, in FP32; a warp reduction sums them; lane 0 forms
-// JHr = b - JHJ vec(G_a) in FP64 and writes the update kernel's accumulator layout.
-static __global__ void __launch_bounds__(128) mom_normal_kernel(const MomNormArgs A)
+// The contribution of pair (a, o) to antenna a's register sums; gains of o from g (full: the two
+// float4 of its table entry; else one, (g_XX, g_YY)).
+template <int FORM>
+__device__ __forceinline__ void pair_add(const float *__restrict__ slot, bool p_side, const float4 *g, float *h)
 {
-    if (__ldg(A.n_active) == 0) return;
-    const long w = ((long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (w >= (long)A.n_bins * A.n_ant) return;
-    const int lane = threadIdx.x & 31;
-    const int bin = (int)(w / A.n_ant), a = (int)(w % A.n_ant);
-    if (!A.active[bin]) return;
-    // h[k][0] = H[(k,0),(k,0)], h[k][1] = H[(k,0),(k,1)], h[k][2] = H[(k,1),(k,1)]; b[(k,l)]
-    float2 h[2][3], b[4];
+    const float4 *s = reinterpret_cast<const float4 *>(slot);
+    if constexpr (FORM == FORM_FULL) {
+        // rows j of G_o; a diagonal term's table entry is diag(g_XX, g_YY)
 #pragma unroll
-    for (int k = 0; k < 2; ++k)
-#pragma unroll
-        for (int i = 0; i < 3; ++i) h[k][i] = make_float2(0.f, 0.f);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) b[i] = make_float2(0.f, 0.f);
-    for (int o = lane; o < A.n_ant; o += 32) {
-        if (o == a) continue;
-        const int up = __ldg(A.upair + (size_t)a * A.n_ant + o);
-        if (up < 0) continue;
-        SlotRegs<MOM_N / 4> sl;
-        const float4 *Mo = reinterpret_cast<const float4 *>(A.mom + ((size_t)bin * A.n_up + up) * MOM_N);
-#pragma unroll
-        for (int i = 0; i < MOM_N / 4; ++i) sl.v[i] = __ldg(Mo + i);
-        float2 G[4];
-        gains_f32(A, bin, o, G);
-        const bool p_side = a < o;           // the sums are oriented with the smaller index first
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-            // gg[m][m2] = G_jm conj(G_jm2)
-            float2 gg[2][2];
-#pragma unroll
-            for (int m = 0; m < 2; ++m)
-#pragma unroll
-                for (int m2 = 0; m2 < 2; ++m2) gg[m][m2] = cmulc(G[2 * j + m], G[2 * j + m2]);
+        for (int j = 0; j < 2; ++j)
 #pragma unroll
             for (int k = 0; k < 2; ++k) {
-                const int kp = 2 * k + j, kq = 2 * j + k;      // the slot block for the p and the q side
-#pragma unroll
-                for (int l = 0; l < 2; ++l)
-#pragma unroll
-                    for (int l2 = l; l2 < 2; ++l2) {
-                        float2 acc = make_float2(0.f, 0.f);
-#pragma unroll
-                        for (int m = 0; m < 2; ++m)
-#pragma unroll
-                            for (int m2 = 0; m2 < 2; ++m2) {
-                                // p side: S[kj][(l,m)][(l2,m2)]; q side: conj(S[jk][(m,l)][(m2,l2)])
-                                const float2 sv = p_side ? sl.S(16 * kp, 2 * l + m, 2 * l2 + m2)
-                                                         : cconj(sl.S(16 * kq, 2 * m + l, 2 * m2 + l2));
-                                const float2 t = cmul(gg[m][m2], sv);
-                                acc.x += t.x;
-                                acc.y += t.y;
-                            }
-                        float2 &hh = h[k][l + l2];
-                        hh.x += acc.x;
-                        hh.y += acc.y;
-                    }
-#pragma unroll
-                for (int l = 0; l < 2; ++l)
-#pragma unroll
-                    for (int m = 0; m < 2; ++m) {
-                        const float2 tv = p_side ? sl.C(MOM_T + 8 * kp + 2 * (2 * l + m))
-                                                 : cconj(sl.C(MOM_T + 8 * kq + 2 * (2 * m + l)));
-                        const float2 t = cmul(G[2 * j + m], tv);
-                        b[2 * k + l].x += t.x;
-                        b[2 * k + l].y += t.y;
-                    }
+                const int blk = p_side ? 2 * k + j : 2 * j + k;
+                pair_block(s + 4 * blk, s + MOM_T / 4 + 2 * blk, p_side, make_float2(g[j].x, g[j].y),
+                           make_float2(g[j].z, g[j].w), h + NE_WORDS * k);
             }
-        }
-    }
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1) {
-#pragma unroll
-        for (int k = 0; k < 2; ++k)
-#pragma unroll
-            for (int i = 0; i < 3; ++i) {
-                h[k][i].x += __shfl_xor_sync(FULL_MASK, h[k][i].x, d);
-                h[k][i].y += __shfl_xor_sync(FULL_MASK, h[k][i].y, d);
-            }
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            b[i].x += __shfl_xor_sync(FULL_MASK, b[i].x, d);
-            b[i].y += __shfl_xor_sync(FULL_MASK, b[i].y, d);
-        }
-    }
-    if (lane != 0) return;
-    // the full 4x4 (zero between the k blocks) in FP64, JHr = b - H g
-    double2 H[4][4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) H[i][j] = make_double2(0.0, 0.0);
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-        H[2 * k][2 * k] = make_double2(h[k][0].x, 0.0);
-        H[2 * k][2 * k + 1] = make_double2(h[k][1].x, h[k][1].y);
-        H[2 * k + 1][2 * k] = make_double2(h[k][1].x, -(double)h[k][1].y);
-        H[2 * k + 1][2 * k + 1] = make_double2(h[k][2].x, 0.0);
-    }
-    double2 G[4];
-    gains_of(A, bin, a, G);
-    double2 r[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        double2 s = make_double2(b[i].x, b[i].y);
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            s.x -= H[i][j].x * G[j].x - H[i][j].y * G[j].y;
-            s.y -= H[i][j].x * G[j].y + H[i][j].y * G[j].x;
-        }
-        r[i] = s;
-    }
-    double *out = A.acc + ((size_t)bin * A.n_ant + a) * (A.type == QC_TERM_FULL ? KG_FULL : KG_DIAG);
-    if (A.type == QC_TERM_FULL) {
-#pragma unroll
-        for (int u = 0; u < 4; ++u) out[u] = H[u][u].x;
-        int o = 4;
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-#pragma unroll
-            for (int v = u + 1; v < 4; ++v) { out[o] = H[u][v].x; out[o + 1] = H[u][v].y; o += 2; }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) { out[16 + 2 * u] = r[u].x; out[17 + 2 * u] = r[u].y; }
+    } else if constexpr (FORM == FORM_E) {
+        pair_block(s, s + MOM_ET / 4, p_side, make_float2(g[0].x, g[0].y), make_float2(g[0].z, g[0].w), h);
     } else {
-        out[0] = H[0][0].x;
-        out[1] = H[3][3].x;
-        out[2] = H[0][3].x;
-        out[3] = H[0][3].y;
-        out[4] = r[0].x; out[5] = r[0].y;
-        out[6] = r[3].x; out[7] = r[3].y;
+        const float4 sv = __ldg(s), t0 = __ldg(s + 1), t1 = __ldg(s + 2);
+        const float sg = p_side ? 1.f : -1.f;
+        const float s01 = p_side ? sv.y : sv.z, s10 = p_side ? sv.z : sv.y;
+        const float2 u01 = p_side ? make_float2(t0.z, t0.w) : make_float2(t1.x, t1.y);
+        const float2 u10 = p_side ? make_float2(t1.x, t1.y) : make_float2(t0.z, t0.w);
+        const float4 q = g[0];
+        const float n0 = fmaf(q.x, q.x, q.y * q.y), n1 = fmaf(q.z, q.z, q.w * q.w);
+        h[0] += fmaf(n0, sv.x, n1 * s01);
+        h[1] += fmaf(n0, s10, n1 * sv.w);
+        h[4] += fmaf(q.x, t0.x, fmaf(-q.y, sg * t0.y, fmaf(q.z, u01.x, -q.w * (sg * u01.y))));
+        h[5] += fmaf(q.x, sg * t0.y, fmaf(q.y, t0.x, fmaf(q.z, sg * u01.y, q.w * u01.x)));
+        h[6] += fmaf(q.x, u10.x, fmaf(-q.y, sg * u10.y, fmaf(q.z, t1.z, -q.w * (sg * t1.w))));
+        h[7] += fmaf(q.x, sg * u10.y, fmaf(q.y, u10.x, fmaf(q.z, sg * t1.w, q.w * t1.z)));
     }
 }
 
-// Diagonal form: one warp per (interval, antenna a); lanes take the other antennas o and form
-// the pair's contributions to a's 2x2 block and right-hand side in FP32 (p side when a < o, q
-// side otherwise); a warp reduction sums them; lane 0 forms JHr = b - JHJ g in FP64 and writes
-// the update kernel's diagonal accumulator layout.
-static __global__ void __launch_bounds__(128) mom_normal_e_kernel(const MomNormArgs A)
+// One warp: antenna a's normal equations of an interval over the other antennas (lanes), in FP32;
+// the totals to out[NWORD].  Antenna o's gains (full: two float4, else one) at gains + o * gstride.
+template <int FORM>
+__device__ __forceinline__ void antenna_sums(const MomNormArgs &A, const float *__restrict__ bin_sums, int a, int lane,
+                                             const float4 *gains, size_t gstride, double *out)
 {
-    if (__ldg(A.n_active) == 0) return;
-    const long w = ((long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (w >= (long)A.n_bins * A.n_ant) return;
-    const int lane = threadIdx.x & 31;
-    const int bin = (int)(w / A.n_ant), a = (int)(w % A.n_ant);
-    if (!A.active[bin]) return;
-    float h00 = 0.f, h11 = 0.f;
-    float2 h01 = make_float2(0.f, 0.f), b0 = h01, b1 = h01;
+    constexpr int N = NormSums<FORM>::NWORD;
+    float h[N];
+#pragma unroll
+    for (int i = 0; i < N; ++i) h[i] = 0.f;
     for (int o = lane; o < A.n_ant; o += 32) {
         if (o == a) continue;
         const int up = __ldg(A.upair + (size_t)a * A.n_ant + o);
         if (up < 0) continue;
-        SlotRegs<MOM_E / 4> sl;
-        const float4 *Mo = reinterpret_cast<const float4 *>(A.mom + ((size_t)bin * A.n_up + up) * MOM_E);
-#pragma unroll
-        for (int i = 0; i < MOM_E / 4; ++i) sl.v[i] = __ldg(Mo + i);
-        float2 Go[4];
-        gains_f32(A, bin, o, Go);
-        const float2 g[2] = { Go[0], Go[3] };
-        const bool p_side = a < o;
-        // the slot's S' entry for this antenna's parameters (x, x') and the other's (y, y'):
-        // p side S'[(x,y)][(x',y')] with the other's gains g_y conj(g_y'); q side
-        // conj(S'[(y,x)][(y',x')]) with the same weights
-        float2 hh[3];
-#pragma unroll
-        for (int i = 0; i < 3; ++i) hh[i] = make_float2(0.f, 0.f);
-        float2 bb[2] = { make_float2(0.f, 0.f), make_float2(0.f, 0.f) };
-#pragma unroll
-        for (int x = 0; x < 2; ++x) {
-#pragma unroll
-            for (int x2 = x; x2 < 2; ++x2)
-#pragma unroll
-                for (int y = 0; y < 2; ++y)
-#pragma unroll
-                    for (int y2 = 0; y2 < 2; ++y2) {
-                        const float2 gg = cmulc(g[y], g[y2]);
-                        const float2 sv = p_side ? sl.S(0, 2 * x + y, 2 * x2 + y2)
-                                                 : cconj(sl.S(0, 2 * y + x, 2 * y2 + x2));
-                        const float2 t = cmul(gg, sv);
-                        hh[x + x2].x += t.x;
-                        hh[x + x2].y += t.y;
-                    }
-#pragma unroll
-            for (int y = 0; y < 2; ++y) {
-                const float2 tf = p_side ? sl.C(MOM_ET + 2 * (2 * x + y)) : cconj(sl.C(MOM_ET + 2 * (2 * y + x)));
-                const float2 t = cmul(g[y], tf);
-                bb[x].x += t.x;
-                bb[x].y += t.y;
-            }
-        }
-        h00 += hh[0].x;
-        h01.x += hh[1].x;
-        h01.y += hh[1].y;
-        h11 += hh[2].x;
-        b0.x += bb[0].x; b0.y += bb[0].y;
-        b1.x += bb[1].x; b1.y += bb[1].y;
+        float4 g[2];
+        g[0] = gains[o * gstride];
+        if constexpr (FORM == FORM_FULL) g[1] = gains[o * gstride + 1];
+        pair_add<FORM>(bin_sums + (size_t)up * mom_words(FORM), a < o, g, h);   // the smaller index is the sums' p
     }
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1) {
-        h00 += __shfl_xor_sync(FULL_MASK, h00, d);
-        h11 += __shfl_xor_sync(FULL_MASK, h11, d);
-        h01.x += __shfl_xor_sync(FULL_MASK, h01.x, d);
-        h01.y += __shfl_xor_sync(FULL_MASK, h01.y, d);
-        b0.x += __shfl_xor_sync(FULL_MASK, b0.x, d);
-        b0.y += __shfl_xor_sync(FULL_MASK, b0.y, d);
-        b1.x += __shfl_xor_sync(FULL_MASK, b1.x, d);
-        b1.y += __shfl_xor_sync(FULL_MASK, b1.y, d);
-    }
+    const double v = reduce_words<N>(h, lane);
+    if (lane % (32 / N) == 0) out[lane / (32 / N)] = v;
+}
+
+// Per-iteration form (more antennas than the one-launch kernel takes, divergence flagging, an
+// allreduce before the update): one warp per (interval, antenna); JHr = b - JHJ vec(G_a) in FP64,
+// written in the update kernel's accumulator layout.
+template <int FORM>
+static __global__ void __launch_bounds__(128) mom_normal_kernel(const MomNormArgs A)
+{
+    constexpr int N = NormSums<FORM>::NWORD, NF4 = FORM == FORM_FULL ? 2 : 1;
+    if (__ldg(A.n_active) == 0) return;
+    __shared__ double s_out[4][N];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const long w = (long)blockIdx.x * 4 + warp;
+    if (w >= (long)A.n_bins * A.n_ant) return;
+    const int bin = (int)(w / A.n_ant), a = (int)(w % A.n_ant);
+    if (!A.active[bin]) return;
+    const int tint = bin / A.n_fint, fint = bin - tint * A.n_fint;
+    antenna_sums<FORM>(A, A.mom + (size_t)bin * A.n_up * mom_words(FORM), a, lane,
+                       A.tab + NF4 * ((size_t)tint * A.n_ant * A.n_fint + fint), (size_t)NF4 * A.n_fint, s_out[warp]);
+    __syncwarp();
     if (lane != 0) return;
     double2 G[4];
-    gains_of(A, bin, a, G);
-    // JHr = b - H g, H = [[h00, h01], [conj(h01), h11]] on (g_0, g_1) = (G[0], G[3])
-    const double r0x = (double)b0.x - (h00 * G[0].x + (h01.x * G[3].x - h01.y * G[3].y));
-    const double r0y = (double)b0.y - (h00 * G[0].y + (h01.x * G[3].y + h01.y * G[3].x));
-    const double r1x = (double)b1.x - ((h01.x * G[0].x + h01.y * G[0].y) + h11 * G[3].x);
-    const double r1y = (double)b1.y - ((h01.x * G[0].y - h01.y * G[0].x) + h11 * G[3].y);
-    double *out = A.acc + ((size_t)bin * A.n_ant + a) * KG_DIAG;
-    out[0] = h00;
-    out[1] = h11;
-    out[2] = h01.x;
-    out[3] = h01.y;
-    out[4] = r0x; out[5] = r0y;
-    out[6] = r1x; out[7] = r1y;
+    gains_of(A.type, A.params, (size_t)bin * A.n_ant + a, G);
+    double *out = A.acc + ((size_t)bin * A.n_ant + a) * (FORM == FORM_FULL ? KG_FULL : KG_DIAG);
+    if constexpr (FORM == FORM_FULL)
+        for (int i = 4; i < 16; ++i) out[i] = 0.0;                  // no coupling between the rows of G
+#pragma unroll
+    for (int k = 0; k < N / NE_WORDS; ++k) {
+        const double *x = s_out[warp] + NE_WORDS * k;
+        const double h00 = x[0], h11 = x[1], hx = x[2], hy = x[3];
+        const double2 g0 = FORM == FORM_FULL ? G[2 * k] : G[0], g1 = FORM == FORM_FULL ? G[2 * k + 1] : G[3];
+        out[2 * k] = h00;
+        out[2 * k + 1] = h11;
+        double *off = out + (FORM == FORM_FULL ? (k ? 14 : 4) : 2);
+        off[0] = hx;
+        off[1] = hy;
+        double *r = out + (FORM == FORM_FULL ? 16 + 4 * k : 4);
+        r[0] = x[4] - (h00 * g0.x + (hx * g1.x - hy * g1.y));
+        r[1] = x[5] - (h00 * g0.y + (hx * g1.y + hy * g1.x));
+        r[2] = x[6] - ((hx * g0.x + hy * g0.y) + h11 * g1.x);
+        r[3] = x[7] - ((hx * g0.y - hy * g0.x) + h11 * g1.y);
+    }
+}
+
+// Solve the Hermitian 2x2 blocks [[h00, h01], [conj(h01), h11]] x = r of one antenna in FP64 with
+// block_solve's singularity tests over the whole block-diagonal matrix (zero trace, zero
+// determinant, reciprocal 1-norm condition number); returns 1 when singular.
+template <int NB>
+__device__ __forceinline__ int solve_blocks(const double (&h00)[NB], const double (&h11)[NB], const double2 (&h01)[NB],
+                                            const double2 (&r)[2 * NB], double2 (&x)[2 * NB])
+{
+    double trace = 0, anorm = 0, inorm = 0;
+#pragma unroll
+    for (int k = 0; k < NB; ++k) trace += h00[k] + h11[k];
+    if (!(trace > 0)) return 1;
+#pragma unroll
+    for (int k = 0; k < NB; ++k) {
+        const double o2 = h01[k].x * h01[k].x + h01[k].y * h01[k].y;
+        const double det = h00[k] * h11[k] - o2;
+        if (!(fabs(det) > 0)) return 1;
+        const double rd = 1.0 / det, o = sqrt(o2);
+        const double big = fmax(fabs(h00[k]), fabs(h11[k])) + o;
+        anorm = fmax(anorm, big);
+        inorm = fmax(inorm, big * fabs(rd));
+        const double2 r0 = r[2 * k], r1 = r[2 * k + 1], z = h01[k];
+        x[2 * k] = make_double2((h11[k] * r0.x - (z.x * r1.x - z.y * r1.y)) * rd,
+                                (h11[k] * r0.y - (z.x * r1.y + z.y * r1.x)) * rd);
+        x[2 * k + 1] = make_double2((h00[k] * r1.x - (z.x * r0.x + z.y * r0.y)) * rd,
+                                    (h00[k] * r1.y - (z.x * r0.y - z.y * r0.x)) * rd);
+    }
+    return !(1.0 / (anorm * inorm) >= 1e-12);
+}
+
+// Every iteration of one solution interval in one CTA: intervals are independent of each other once
+// their sums are formed, so nothing has to be exchanged between CTAs and no launch, graph node
+// or grid-wide counter stands between two iterations.  Per iteration the warps form the antennas'
+// normal equations from the sums (L2), one thread per antenna solves and updates in FP64 exactly as
+// update_kernel does, and the FP64 relative change of the interval ends the loop.
+template <int FORM>
+static __global__ void __launch_bounds__(256, 2) mom_iterate_kernel(const MomIterArgs a)
+{
+    constexpr bool GFULL = FORM == FORM_FULL;
+    constexpr int N = NormSums<FORM>::NWORD, NB = GFULL ? 2 : 1, NF4 = NB;
+    extern __shared__ float4 s_mem[];
+    const MomNormArgs &A = a.n;
+    float4 *g32 = s_mem;                                                       // [n_ant][NF4]
+    double *sums = reinterpret_cast<double *>(s_mem + (size_t)A.n_ant * NF4);  // [n_ant][N]
+    __shared__ double s_num[8], s_den[8];
+    __shared__ int s_done;
+    const int bin = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+    const int tint = bin / A.n_fint, fint = bin - tint * A.n_fint;
+    const float *bin_sums = A.mom + (size_t)bin * A.n_up * mom_words(FORM);
+    auto tab_at = [&](int i) { return a.tab + NF4 * (((size_t)tint * A.n_ant + i / NF4) * A.n_fint + fint) + i % NF4; };
+    for (int i = tid; i < A.n_ant * NF4; i += blockDim.x) g32[i] = *tab_at(i);
+    __syncthreads();
+    int k = 1;
+    for (;; ++k) {
+        for (int ant = warp; ant < A.n_ant; ant += nw)
+            antenna_sums<FORM>(A, bin_sums, ant, lane, g32, NF4, sums + (size_t)ant * N);
+        __syncthreads();
+        const double alpha = a.alternate ? ((k % 2 == 0) ? 0.5 : 1.0) : a.damping;
+        double num = 0, den = 0;
+        for (int ant = tid; ant < A.n_ant; ant += blockDim.x) {
+            const double *h = sums + (size_t)ant * N;
+            const size_t pidx = (size_t)bin * A.n_ant + ant;
+            double2 old[2 * NB], now[2 * NB], r[2 * NB], x[2 * NB], h01[NB];
+            double h00[NB], h11[NB];
+            double phi0 = 0, phi1 = 0;
+            double2 *P = reinterpret_cast<double2 *>(a.params) + 4 * pidx;
+            if constexpr (GFULL) {
+#pragma unroll
+                for (int e = 0; e < 4; ++e) old[e] = P[e];
+            } else if (A.type == QC_TERM_PHASE) {
+                phi0 = a.params[2 * pidx];
+                phi1 = a.params[2 * pidx + 1];
+                sincos(phi0, &old[0].y, &old[0].x);
+                sincos(phi1, &old[1].y, &old[1].x);
+            } else {
+                old[0] = P[0];
+                old[1] = P[3];
+            }
+#pragma unroll
+            for (int b = 0; b < NB; ++b) {
+                const double *w = h + NE_WORDS * b;
+                h00[b] = w[0];
+                h11[b] = w[1];
+                h01[b] = FORM == FORM_D ? make_double2(0, 0) : make_double2(w[2], w[3]);
+                const double2 g0 = old[2 * b], g1 = old[2 * b + 1], z = h01[b];
+                r[2 * b] = make_double2(w[4] - (h00[b] * g0.x + (z.x * g1.x - z.y * g1.y)),
+                                        w[5] - (h00[b] * g0.y + (z.x * g1.y + z.y * g1.x)));
+                r[2 * b + 1] = make_double2(w[6] - ((z.x * g0.x + z.y * g0.y) + h11[b] * g1.x),
+                                            w[7] - ((z.x * g0.y - z.y * g0.x) + h11[b] * g1.y));
+            }
+            int singular;
+            if (!GFULL && A.type == QC_TERM_PHASE) {
+                // chain rule with dg/dphi = i g (Scenario 1): 2 Re(conj(g_u) g_v JHJ), 2 Im(conj(g_u) JHr)
+                const double2 g0 = old[0], g1 = old[1], z = h01[0];
+                const double2 c = make_double2(g0.x * g1.x + g0.y * g1.y, g0.x * g1.y - g0.y * g1.x);
+                double m0[1] = { 2.0 * (g0.x * g0.x + g0.y * g0.y) * h00[0] };
+                double m1[1] = { 2.0 * (g1.x * g1.x + g1.y * g1.y) * h11[0] };
+                double2 mo[1] = { make_double2(2.0 * (c.x * z.x - c.y * z.y), 0.0) }, rb[2], xb[2];
+                rb[0] = make_double2(2.0 * (g0.x * r[0].y - g0.y * r[0].x), 0.0);
+                rb[1] = make_double2(2.0 * (g1.x * r[1].y - g1.y * r[1].x), 0.0);
+                singular = solve_blocks<1>(m0, m1, mo, rb, xb);
+                if (!singular) { phi0 += alpha * xb[0].x; phi1 += alpha * xb[1].x; }
+                a.params[2 * pidx] = phi0;
+                a.params[2 * pidx + 1] = phi1;
+                sincos(phi0, &now[0].y, &now[0].x);
+                sincos(phi1, &now[1].y, &now[1].x);
+            } else {
+                singular = solve_blocks<NB>(h00, h11, h01, r, x);
+#pragma unroll
+                for (int e = 0; e < 2 * NB; ++e)
+                    now[e] = singular ? old[e] : make_double2(old[e].x + alpha * x[e].x, old[e].y + alpha * x[e].y);
+                if constexpr (GFULL) {
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) P[e] = now[e];
+                } else {
+                    P[0] = now[0];
+                    P[3] = now[1];
+                }
+            }
+            a.gain_flags[pidx] = (int8_t)singular;
+#pragma unroll
+            for (int f = 0; f < NF4; ++f)
+                g32[NF4 * ant + f] = make_float4((float)now[2 * f].x, (float)now[2 * f].y, (float)now[2 * f + 1].x,
+                                                 (float)now[2 * f + 1].y);
+#pragma unroll
+            for (int e = 0; e < 2 * NB; ++e) {
+                const double dx = now[e].x - old[e].x, dy = now[e].y - old[e].y;
+                num += dx * dx + dy * dy;
+                den += now[e].x * now[e].x + now[e].y * now[e].y;
+            }
+        }
+        for (int d = 16; d > 0; d >>= 1) {
+            num += __shfl_down_sync(FULL_MASK, num, d);
+            den += __shfl_down_sync(FULL_MASK, den, d);
+        }
+        if (lane == 0) { s_num[warp] = num; s_den[warp] = den; }
+        __syncthreads();
+        if (tid == 0) {
+            double tn = 0, td = 0;
+            for (int i = 0; i < nw; ++i) { tn += s_num[i]; td += s_den[i]; }
+            const double delta = td > 0 ? sqrt(tn / td) : 0.0;
+            const bool conv = delta < a.tol;
+            if (!conv) atomicAdd(a.cnt + k, 1);                      // still active after iteration k
+            s_done = conv || k == a.max_iter;
+        }
+        __syncthreads();
+        if (s_done) break;
+    }
+    for (int i = tid; i < A.n_ant * NF4; i += blockDim.x) *tab_at(i) = g32[i];
+    if (tid == 0) {
+        a.iters[bin] = k;
+        atomicAdd(a.vis_iters, (unsigned long long)a.bin_nvis[bin] * k);
+        atomicAdd(a.acc_bytes, (unsigned long long)(a.bin_nbytes[bin] + a.iter_bytes * k));
+    }
 }
 
 // algorithmic bytes: the pass reads every sample of the bins once (their streaming bytes);
@@ -713,40 +821,42 @@ static __global__ void mom_bytes_kernel(int n_bins, const long long *bin_nbytes,
 
 } // namespace qc
 
-// the pass kernel of a form and fixed-term kind (ok: KIND_* of R in the full form, of L in the
-// diagonal form; the diagonal form needs one)
-template <int FORM, int OK>
+template <int FORM, int OK, bool M16>
 static cudaError_t launch_pass(const qc::MomArgs &a, int sm_count, cudaStream_t st)
 {
-    using R = qc::MomRing<FORM, OK>;
-    static bool configured = false;              // the raised shared-memory limit, once per process
-    if (!configured) {
-        const cudaError_t e = cudaFuncSetAttribute(qc::mom_pass_kernel<FORM, OK>,
-                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)R::SMEM);
-        if (e != cudaSuccess) return e;
-        configured = true;
-    }
+    using R = qc::MomRing<FORM, OK, M16>;
+    // the raised shared-memory limit belongs to the device's copy of the kernel: set on every launch
+    const cudaError_t e = cudaFuncSetAttribute(qc::mom_pass_kernel<FORM, OK, M16>,
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)R::SMEM);
+    if (e != cudaSuccess) return e;
     const int block = 128;
     const int n_groups = (a.n_chunks + a.group - 1) / a.group;
     const long units = (long)a.n_strips * a.n_rb * n_groups;
     const int grid = (int)std::max(1L, std::min((long)sm_count * R::PER_SM, (units * 32 + block - 1) / block));
-    qc::mom_pass_kernel<FORM, OK><<<grid, block, R::SMEM, st>>>(a);
+    qc::mom_pass_kernel<FORM, OK, M16><<<grid, block, R::SMEM, st>>>(a);
     return cudaGetLastError();
 }
 
-// the pass kernel of a form and fixed-term kind (ok: KIND_* of R in the full form, of L in the
-// diagonal form; the diagonal form needs one)
-cudaError_t mom_launch_pass(const qc::MomArgs &a, int form, int ok, int sm_count, cudaStream_t st)
+// the pass kernel of a form and fixed-term kind (ok: KIND_* of the term to the right in the full
+// form, of the one to the left in the E form, of either in the plain diagonal form)
+template <bool M16>
+static cudaError_t launch_pass_any(const qc::MomArgs &a, int form, int ok, int sm_count, cudaStream_t st)
 {
     using namespace qc;
     if (form == FORM_FULL) {
-        if (ok == KIND_NONE) return launch_pass<FORM_FULL, KIND_NONE>(a, sm_count, st);
-        if (ok == KIND_DIAG) return launch_pass<FORM_FULL, KIND_DIAG>(a, sm_count, st);
-        return launch_pass<FORM_FULL, KIND_FULL>(a, sm_count, st);
+        if (ok == KIND_NONE) return launch_pass<FORM_FULL, KIND_NONE, M16>(a, sm_count, st);
+        if (ok == KIND_DIAG) return launch_pass<FORM_FULL, KIND_DIAG, M16>(a, sm_count, st);
+        return launch_pass<FORM_FULL, KIND_FULL, M16>(a, sm_count, st);
     }
-    if (ok == KIND_DIAG) return launch_pass<FORM_E, KIND_DIAG>(a, sm_count, st);
-    if (ok == KIND_FULL) return launch_pass<FORM_E, KIND_FULL>(a, sm_count, st);
-    return cudaErrorInvalidValue;
+    if (form == FORM_E) return ok == KIND_FULL ? launch_pass<FORM_E, KIND_FULL, M16>(a, sm_count, st) : cudaErrorInvalidValue;
+    if (ok == KIND_NONE) return launch_pass<FORM_D, KIND_NONE, M16>(a, sm_count, st);
+    if (ok == KIND_DIAG) return launch_pass<FORM_D, KIND_DIAG, M16>(a, sm_count, st);
+    return launch_pass<FORM_D, KIND_FULL, M16>(a, sm_count, st);
+}
+
+cudaError_t mom_launch_pass(const qc::MomArgs &a, int form, int ok, int sm_count, cudaStream_t st)
+{
+    return a.model16 ? launch_pass_any<true>(a, form, ok, sm_count, st) : launch_pass_any<false>(a, form, ok, sm_count, st);
 }
 
 cudaError_t mom_launch_bytes(int n_bins, const long long *bin_nbytes, long long per_iter, long long *iter_nbytes,
@@ -756,20 +866,42 @@ cudaError_t mom_launch_bytes(int n_bins, const long long *bin_nbytes, long long 
     return cudaGetLastError();
 }
 
-cudaError_t mom_launch_normal(const qc::MomNormArgs &a, cudaStream_t st)
+template <int FORM> static cudaError_t launch_normal(const qc::MomNormArgs &a, cudaStream_t st)
 {
     const long warps = (long)a.n_bins * a.n_ant;
-    if (a.form == qc::FORM_FULL) qc::mom_normal_kernel<<<(int)((warps + 3) / 4), 128, 0, st>>>(a);
-    else qc::mom_normal_e_kernel<<<(int)((warps + 3) / 4), 128, 0, st>>>(a);
+    qc::mom_normal_kernel<FORM><<<(unsigned)((warps + 3) / 4), 128, 0, st>>>(a);
     return cudaGetLastError();
+}
+
+cudaError_t mom_launch_normal(const qc::MomNormArgs &a, cudaStream_t st)
+{
+    if (a.form == qc::FORM_FULL) return launch_normal<qc::FORM_FULL>(a, st);
+    if (a.form == qc::FORM_E) return launch_normal<qc::FORM_E>(a, st);
+    return launch_normal<qc::FORM_D>(a, st);
+}
+
+template <int FORM> static cudaError_t launch_iterate(const qc::MomIterArgs &a, cudaStream_t st)
+{
+    const int n_ant = a.n.n_ant;
+    const int block = n_ant > 16 ? 256 : (n_ant > 8 ? 128 : 64);
+    const size_t smem = (size_t)n_ant * ((FORM == qc::FORM_FULL ? 2 : 1) * sizeof(float4) + qc::NormSums<FORM>::NWORD * sizeof(double));
+    qc::mom_iterate_kernel<FORM><<<a.n.n_bins, block, smem, st>>>(a);
+    return cudaGetLastError();
+}
+
+cudaError_t mom_launch_iterate(const qc::MomIterArgs &a, cudaStream_t st)
+{
+    if (a.n.form == qc::FORM_FULL) return launch_iterate<qc::FORM_FULL>(a, st);
+    if (a.n.form == qc::FORM_E) return launch_iterate<qc::FORM_E>(a, st);
+    return launch_iterate<qc::FORM_D>(a, st);
 }
 
 cudaError_t mom_launch_rows(long n, const int *strip_rows, const int4 *rows, const uint8_t *row_live,
-                            const int *up_of_bl, int4 *out, cudaStream_t st)
+                            const int *up_of_bl, const float *bl_scale, int4 *out, float *scale, cudaStream_t st)
 {
     if (n == 0) return cudaSuccess;
-    qc::mom_rows_kernel<<<(int)((n + 255) / 256), 256, 0, st>>>(n, strip_rows, rows, row_live, up_of_bl, out);
+    qc::mom_rows_kernel<<<(int)((n + 255) / 256), 256, 0, st>>>(n, strip_rows, rows, row_live, up_of_bl, bl_scale, out,
+                                                               scale);
     return cudaGetLastError();
 }
 
-size_t mom_words(int form) { return form == qc::FORM_FULL ? qc::MOM_N : qc::MOM_E; }

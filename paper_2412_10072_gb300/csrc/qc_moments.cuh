@@ -12,7 +12,14 @@ constexpr int MOM_T = 64, MOM_U = 96;
 // Hermitian packed as S), T' 8, U 1, three words of padding (slots of whole 16-byte vectors)
 constexpr int MOM_E = 28;
 constexpr int MOM_ET = 16, MOM_EU = 24;
-constexpr int FORM_FULL = 0, FORM_E = 1;
+// plain diagonal form (a diagonal or phase-only solved term, the other term diagonal or to its
+// right): S 4, T 8
+constexpr int MOM_D = 12;
+constexpr int FORM_FULL = 0, FORM_E = 1, FORM_D = 2;
+__host__ __device__ constexpr int mom_words(int form)
+{
+    return form == FORM_FULL ? MOM_N : (form == FORM_E ? MOM_E : MOM_D);
+}
 
 // Hermitian pairs (u, v), u < v, of the 4x4 S blocks: packed as 4 diagonal reals then 6 (re, im)
 __host__ __device__ constexpr int mom_pair(int u, int v)
@@ -20,9 +27,53 @@ __host__ __device__ constexpr int mom_pair(int u, int v)
     return u == 0 ? (v == 1 ? 0 : v == 2 ? 1 : 2) : u == 1 ? (v == 2 ? 3 : 4) : 5;
 }
 
+// Transposed warp reduction of N = 4, 8 or 16 values per lane: each halving exchanges half of the
+// values a lane holds; the lanes from 32 / N * i on end with the total of value i.  The sum over
+// the lanes is carried as head and tail (Knuth's two-sum, one exact step per level), so the total over
+// the antennas is as good as an FP64 sum of the lanes' terms: rounding the tree in FP32 alone is
+// one unit in the last place of the whole right-hand side, which JHr = b - JHJ g turns into that
+// much of the gains.
+__device__ __forceinline__ void two_sum(float a, float b, float &s, float &e)
+{
+    s = a + b;
+    const float z = s - a;
+    e = (a - (s - z)) + (b - z);
+}
+template <int N> __device__ __forceinline__ double reduce_words(float (&h)[N], int lane)
+{
+    float t[N / 2];
+    int o = 16;
+#pragma unroll
+    for (int n = N / 2; n >= 1; n >>= 1, o >>= 1) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int i = 0; i < n; ++i) {
+            const float send = up ? h[i] : h[i + n], keep = up ? h[i + n] : h[i];
+            float tail = 0.f;
+            if (n < N / 2) {                                   // the tails of the levels before
+                const float ts = up ? t[i] : t[i + n];
+                tail = (up ? t[i + n] : t[i]) + __shfl_xor_sync(0xffffffffu, ts, o);
+            }
+            float e;
+            two_sum(keep, __shfl_xor_sync(0xffffffffu, send, o), h[i], e);
+            t[i] = tail + e;
+        }
+    }
+#pragma unroll
+    for (; o >= 1; o >>= 1) {
+        const float tail = t[0] + __shfl_xor_sync(0xffffffffu, t[0], o);
+        float e;
+        two_sum(h[0], __shfl_xor_sync(0xffffffffu, h[0], o), h[0], e);
+        t[0] = tail + e;
+    }
+    return (double)h[0] + (double)t[0];
+}
+
 struct MomArgs {
     int n_chan, n_ant, n_up;             // n_up: unordered antenna pairs with data
     const float4 *vis, *model, *wf;      // wf: weights with flags and autocorrelations folded in (w = 0)
+    const uint4 *model16;                // FP16 model, or null
+    const float *mscale;                 // [strip rows] its scale, or null
     // [strip rows] {row or -1 (nothing usable), time, pair | conj << 31, p | q << 16}: p, q the
     // antennas of the baseline as oriented in the sums (p < q); conj: the row is (q, p)
     const int4 *mrows;
@@ -33,21 +84,36 @@ struct MomArgs {
     int chunk_major;                     // 1: a unit's rows inside each chunk; 0: a row's chunks inside it
     DevTerm tn;                          // the solved term (maps)
     DevTerm to;                          // the fixed other term of a two-term chain (tables)
-    float *mom;                          // [bins][n_up][MOM_N or MOM_E]
-    const int *n_active;
+    float *mom;                          // [bins][n_up][mom_words(form)]
+    const int *n_active;                 // or null: always
 };
 
 struct MomNormArgs {
     int n_bins, n_ant, n_up, type;       // type: QC_TERM_* (diag, full, phase)
-    int form;                            // FORM_FULL or FORM_E
+    int form;                            // FORM_*
     const int *upair;                    // [n_ant][n_ant] unordered pair index or -1
-    const float *mom;                    // [bins][n_up][MOM_N or MOM_E]
+    const float *mom;                    // [bins][n_up][mom_words(form)]
     const double *params;                // FP64 gains of the solved term
     const float4 *tab;                   // their FP32 table [n_tint][n_ant][n_fint] x (1 | 2)
     int n_fint;
     const uint8_t *active;               // [bins]
     const int *n_active;
-    double *acc;                         // [bins][n_ant][KG] (written)
+    double *acc;                         // [bins][n_ant][KG] (written by the per-iteration form)
+};
+
+// Every iteration in one launch (mom_iterate_kernel).
+struct MomIterArgs {
+    MomNormArgs n;
+    double *params;                      // FP64 master (read and updated)
+    float4 *tab;                         // FP32 table (read at the start, written at the end)
+    int8_t *gain_flags;                  // [bins][n_ant]
+    int *iters;                          // [bins]
+    int *cnt;                            // [max_iter + 1], zeroed: intervals still active after iteration k
+    const long long *bin_nvis, *bin_nbytes;
+    long long iter_bytes;                // algorithmic bytes of an interval's iteration
+    unsigned long long *vis_iters, *acc_bytes;
+    int max_iter, alternate;             // alternate: step 1, 1/2, 1, ...; else `damping`
+    double damping, tol;
 };
 
 } // namespace qc
