@@ -305,6 +305,12 @@ extern "C" int qc_create(const qc_problem *p, qc_ctx **out)
     c->n_strips = n_bl;
     c->n_strip_rows = (long)strip_rows.size();
     for (int b = 0; b < n_bl; ++b) c->max_strip_rows = std::max(c->max_strip_rows, strip_off[b + 1] - strip_off[b]);
+    c->full_grid = n_bl > 0;
+    for (int b = 0; b < n_bl && c->full_grid; ++b) {
+        c->full_grid = strip_off[b + 1] - strip_off[b] == p->n_time;
+        for (int k = strip_off[b]; k < strip_off[b + 1] && c->full_grid; ++k)
+            c->full_grid = rows[strip_rows[k]].z == k - strip_off[b];
+    }
     cudaError_t e;
     qc_ctx *cc = c.get();
     auto dalloc = [&](size_t bytes) -> void * { return cc->alloc(bytes, &e); };
@@ -339,6 +345,7 @@ extern "C" int qc_create(const qc_problem *p, qc_ctx **out)
                 up_of_bl[bl] = slot;
             }
         c->n_up = n_up;
+        c->full_grid = c->full_grid && n_up == n_bl;
         DALLOC(c->d_upair, int, std::max<size_t>(1, upair.size()));
         if (!upair.empty()) HCOPY(c->d_upair, upair.data(), nbytes<int>(upair.size()));
         DALLOC(c->d_up_of_bl, int, up_of_bl.size());
@@ -1112,8 +1119,102 @@ int qc_ctx::plan_sums(const qc_term *terms, int n_terms, int n, const qc_opts *o
     return QC_OK;
 }
 
-// Arguments of the pass and of the normal equations of a term solved from sums; builds the
-// context's table of strip rows the first time (a function of the rows and flags staged at create).
+// The context's table of strip rows as the passes read them, built the first time (a function of the
+// rows and flags staged at create).
+int qc_ctx::ensure_mom_rows(cudaStream_t st)
+{
+    qc_ctx *c = this;
+    if (mom_rows_ready) return QC_OK;
+    const size_t scale_off = nbytes<int4>(std::max(1L, n_strip_rows));
+    const int rc = ensure(mom_rows, scale_off + (m16 ? nbytes<float>(std::max(1L, n_strip_rows)) : 0));
+    if (rc) return rc;
+    CK(mom_launch_rows(n_strip_rows, d_strip_rows, d_rows, d_row_live, d_up_of_bl, d_bl_scale, (int4 *)mom_rows.ptr,
+                       m16 ? (float *)((char *)mom_rows.ptr + scale_off) : nullptr, st));
+    // built on this call's stream: finished before any later call can use it on another one
+    CK(cudaStreamSynchronize(st));
+    mom_rows_ready = true;
+    ++launches;
+    return QC_OK;
+}
+
+// A solved delay term from the products T and H of qc_delay_sums.cu (chains of one or two terms, the
+// other one to the right or diagonal).  The rule: an iteration on T reads 1 KB per (time interval,
+// pair, 32 channels), one on the samples 80 B (64 B with the FP16 model, 32 B more for each further
+// direction) a sample; T is taken when it is at most 0.6 of that, which leaves the pass that forms
+// it paid for after two iterations (measured on 64 antennas, 75 x 512: pass 1.9 iterations on the
+// samples, an iteration on T 0.3).  That also bounds T to 0.6 of the samples' bytes.
+int qc_ctx::plan_delay_sums(const qc_term *terms, int n_terms, int n, const qc_opts *o, bool &use)
+{
+    use = false;
+    const qc_term &t = terms[n];
+    TermBufs &B = tb[n];
+    if (!delay[n] || n_terms > 2 || n_dir > DSUM_MAX_DIR || n_up == 0 || n_ant > 256 || t.reduce || t.max_iter < 3)
+        return QC_OK;
+    if (o->kernel != 0 || o->order != -1 || o->block_threads != 0 || o->ctas_per_sm != 0) return QC_OK;
+    if (n == 1 && kind_of_range(terms, 0, 1) == KIND_FULL) return QC_OK;
+    const size_t n_chunks = (n_chan + 31) / 32;
+    const size_t t_bytes = (size_t)t.n_tint * n_chunks * n_up * 1024;
+    const double sample = 32.0 + 16.0 + (m16 ? 16.0 : 32.0 * n_dir);
+    if ((double)t_bytes > 0.6 * sample * (double)n_strip_rows * n_chan) return QC_OK;
+    int rc = ensure(B.dsum_t, t_bytes);
+    if (!rc) rc = ensure(B.dsum_h, nbytes<double>((size_t)t.n_tint * B.hfr.size() * n_ant * KG_HSUM));
+    if (rc == QC_ENOMEM) {
+        cudaGetLastError();                    // no room for the products: iterate on the samples
+        err.clear();
+        return QC_OK;
+    }
+    use = rc == QC_OK;
+    return rc;
+}
+
+DelaySumsArgs qc_ctx::delay_sums_args(const qc_term *terms, int n_terms, int n, const Chain &chain)
+{
+    const qc_term &t = terms[n];
+    TermBufs &B = tb[n];
+    DelaySumsArgs a;
+    memset(&a, 0, sizeof a);
+    a.n_chan = n_chan;
+    a.n_ant = n_ant;
+    a.n_up = n_up;
+    a.n_dir = n_dir;
+    a.n_fint = (int)B.hfr.size();
+    a.n_chunks = (n_chan + 31) / 32;
+    a.vis = d_vis;
+    a.model = d_model;
+    a.wf = d_wf;
+    a.model16 = m16 ? d_model16 : nullptr;
+    a.mrows = (const int4 *)mom_rows.ptr;
+    a.mscale = m16 ? (const float *)((const char *)mom_rows.ptr + nbytes<int4>(std::max(1L, n_strip_rows))) : nullptr;
+    a.strip_off = d_strip_off;
+    a.n_strips = n_strips;
+    // an interval several times long keeps its slot while the rows run inside a chunk; the blocks of
+    // rows give about four units per resident warp, down to 8 rows inside a chunk
+    a.chunk_major = t.n_tint < n_time ? 1 : 0;
+    const long max_strip = std::max(1, max_strip_rows), want = 4L * sm_count * 16;
+    const long strips = std::max(1L, (long)n_strips * (a.chunk_major ? a.n_chunks : 1));
+    const long blocks = std::max(1L, (want + strips - 1) / strips);
+    a.rb = (int)std::min(max_strip, std::max(a.chunk_major ? 8L : 1L, (max_strip + blocks - 1) / blocks));
+    a.n_rb = (int)((max_strip + a.rb - 1) / a.rb);
+    a.t_map = chain.t[n].t_map;
+    a.to = n_terms == 2 ? chain.t[1 - n] : chain.t[n];
+    a.nd_o = n_terms == 2 ? cur_nd[1 - n] : 1;
+    // one row per (interval, pair): every slot is written exactly once
+    a.store = full_grid && t.n_tint == n_time;
+    for (int i = 0; i < n_time && a.store; ++i) a.store = t.t_map[i] == i;
+    a.active = (const uint8_t *)B.active.ptr;
+    a.fmap = (const int *)B.dfmap.ptr;
+    a.omega = (const float *)B.domega.ptr;
+    a.T = (float4 *)B.dsum_t.ptr;
+    a.hsum = (double *)B.dsum_h.ptr;
+    a.n_tint = t.n_tint;
+    a.upair = d_upair;
+    a.nu = (const double *)B.dnu.ptr;
+    a.params = (const double *)B.params.ptr;
+    a.acc = (double *)B.acc.ptr;
+    return a;
+}
+
+// Arguments of the pass and of the normal equations of a term solved from sums.
 int qc_ctx::sums_args(const qc_term *terms, int n_terms, int n, const Chain &chain, cudaStream_t st, MomArgs &ma,
                       MomNormArgs &mn)
 {
@@ -1122,17 +1223,9 @@ int qc_ctx::sums_args(const qc_term *terms, int n_terms, int n, const Chain &cha
     TermBufs &B = tb[n];
     memset(&ma, 0, sizeof ma);
     memset(&mn, 0, sizeof mn);
-    int rc;
+    const int rc = ensure_mom_rows(st);
+    if (rc) return rc;
     const size_t scale_off = nbytes<int4>(std::max(1L, n_strip_rows));
-    if (!mom_rows_ready) {
-        if ((rc = ensure(mom_rows, scale_off + (m16 ? nbytes<float>(std::max(1L, n_strip_rows)) : 0)))) return rc;
-        CK(mom_launch_rows(n_strip_rows, d_strip_rows, d_rows, d_row_live, d_up_of_bl, d_bl_scale, (int4 *)mom_rows.ptr,
-                           m16 ? (float *)((char *)mom_rows.ptr + scale_off) : nullptr, st));
-        // built on this call's stream: finished before any later call can use it on another one
-        CK(cudaStreamSynchronize(st));
-        mom_rows_ready = true;
-        ++launches;
-    }
     ma.n_chan = n_chan;
     ma.n_ant = n_ant;
     ma.n_up = n_up;
@@ -1343,7 +1436,14 @@ int qc_ctx::solve_term(const qc_term *terms, int n_terms, int n, Chain chain, co
     const bool ded = DL.fn != nullptr;
     // a solved delay term with sums per parameter interval (the streaming kernels), else
     // the per-channel bins
-    const bool psums = ded || (dds && delay[n]);
+    // or, where that is cheaper, products of every (time interval, pair, channel) formed once
+    bool dsum = false;
+    {
+        int rc_;
+        if ((rc_ = plan_delay_sums(terms, n_terms, n, o, dsum))) return rc_;
+        if (dsum && (rc_ = ensure_mom_rows(st))) return rc_;
+    }
+    const bool psums = dsum || ded || (dds && delay[n]);
     DevTerm tnu = chain.t[n];
     const int nbu = delay[n] ? t.n_tint * (int)B.hfr.size() : nb;
     if (psums) {
@@ -1676,7 +1776,13 @@ int qc_ctx::solve_term(const qc_term *terms, int n_terms, int n, Chain chain, co
         dua.vis_iters = ua.vis_iters;
         dua.acc_bytes = ua.acc_bytes;
         dua.tol = ua.tol;
+        if (dsum) {
+            dua.hsum = (const double *)B.dsum_h.ptr;
+            dua.omega = (const float *)B.domega.ptr;
+        }
     }
+    DelaySumsArgs dsa_;
+    if (dsum) dsa_ = delay_sums_args(terms, n_terms, n, chain);
 
     MomArgs ma;
     MomNormArgs mn;
@@ -1696,7 +1802,9 @@ int qc_ctx::solve_term(const qc_term *terms, int n_terms, int n, Chain chain, co
     for (int k = 0; k < 2 * max_iter + 2; ++k) { cudaEvent_t ev; if ((rc = get_event(2 + k, ev))) return rc; }
     const int ev_pass = 2 + 2 * max_iter;     // the sums pass (its own bracket inside iteration 1's)
     // (no graph while a test stalls a stage: a captured graph would keep the stall)
-    const bool use_graph = o->use_graph && !t.reduce && qc_wait_stall_stage() < 0;
+    // (a delay term from products has two short kernels an iteration: launching them costs less than
+    // capturing and instantiating a graph for the one replay of a solve)
+    const bool use_graph = o->use_graph && !t.reduce && qc_wait_stall_stage() < 0 && !dsum;
     const unsigned rec_flags = use_graph ? cudaEventRecordExternal : cudaEventRecordDefault;
 
     auto enqueue = [&]() -> int {
@@ -1710,14 +1818,23 @@ int qc_ctx::solve_term(const qc_term *terms, int n_terms, int n, Chain chain, co
         for (int k = 1; k <= max_iter; ++k) {
             aa.n_active = cnt + (k - 1);
             // inside a capture the record must be an external event node to be timed on replay
-            {
+            if (!dsum) {
                 chunk_active_kernel<<<(ca_threads + 255) / 256, 256, 0, st>>>(aa.tn, n_chan, aa.n_chunks,
                                                                             (const uint8_t *)B.active.ptr, cnt + (k - 1),
                                                                             (uint8_t *)B.chunk_act.ptr);
                 CK(cudaGetLastError());
             }
             CK(cudaEventRecordWithFlags(events[2 + 2 * (k - 1)], st, rec_flags));
-            if (dds) {
+            if (dsum) {
+                dsa_.n_active = cnt + (k - 1);
+                if (k == 1) {
+                    CK(cudaMemsetAsync(B.dsum_h.ptr, 0, nbytes<double>((size_t)nbu * n_ant * KG_HSUM), st));
+                    if (!dsa_.store)
+                        CK(cudaMemsetAsync(B.dsum_t.ptr, 0, (size_t)t.n_tint * dsa_.n_chunks * n_up * 1024, st));
+                    CK(dsum_launch_pass(dsa_, lk != KIND_NONE ? lk : rk, sm_count, st));
+                }
+                CK(dsum_launch_iter(dsa_, st));
+            } else if (dds) {
                 DDStreamArgs x;
                 x.s = sa;
                 x.s.n_active = cnt + (k - 1);
@@ -1798,6 +1915,10 @@ int qc_ctx::solve_term(const qc_term *terms, int n_terms, int n, Chain chain, co
             } else {
                 update_kernel<<<nb, upd_block, 0, st>>>(ua);
             }
+            CK(cudaGetLastError());
+        }
+        if (dsum) {
+            delay_tab_kernel<<<grid_for((long)nb * n_ant, 256, sm_count), 256, 0, st>>>(dua.d);
             CK(cudaGetLastError());
         }
         return QC_OK;

@@ -103,6 +103,10 @@ struct DelayUpdArgs {
     unsigned long long *vis_iters, *acc_bytes;
     int k;                    // iteration (1-based)
     double alpha, tol;
+    // a term solved from products (qc_delay_sums.cu): the h sums [bins][n_ant][6], the same for every
+    // iteration (else null: they are in acc); the channel table is then left to the end of the solve
+    const double *hsum;
+    const float *omega;       // [n_chan] 2 pi nu - omega_ref (with hsum)
 };
 
 // One block per parameter interval (time interval x frequency interval), threads over antennas.
@@ -148,6 +152,10 @@ static __global__ void __launch_bounds__(128) delay_update_kernel(const DelayUpd
             double *A = u.acc + ((size_t)bin * d.n_ant + ant) * KG_SUMS;
             double S[13];
             for (int i = 0; i < 13; ++i) { S[i] = A[i]; A[i] = 0.0; }
+            if (u.hsum) {
+                const double *H = u.hsum + ((size_t)bin * d.n_ant + ant) * 6;
+                for (int i = 0; i < 6; ++i) S[i] = H[i];
+            }
             // sum h w^k with w = w' + w0:  h w = h w' + w0 h,  h w^2 = h w'^2 + 2 w0 h w' + w0^2 h
             const double w0 = d.omega_ref;
             for (int base = 0; base <= 10; base += (base == 3 ? 7 : 3)) {
@@ -219,7 +227,34 @@ static __global__ void __launch_bounds__(128) delay_update_kernel(const DelayUpd
             den += 2.0;
         }
     }
-    if (SUMS) {
+    if (SUMS && u.hsum) {
+        // the change of the gains, (antenna, channel) by (antenna, channel) over the block's threads.
+        // The phase change (d0 + d1 w_ref) + d1 (w - w_ref) is formed in FP64 at the band's centre
+        // and in FP32 away from it: 0.84 ms a launch with FP64 phases and the channel table on the
+        // 300 x 512 x 64 grid
+        __syncthreads();
+        const int nch = fr.y - fr.x + 1;
+        for (int a0 = 0; a0 < d.n_ant; a0 += 128) {
+            __shared__ float4 s_e[128];
+            const int na = min(128, d.n_ant - a0);
+            if ((int)threadIdx.x < na) {
+                double *A = u.acc + ((size_t)bin * d.n_ant + a0 + threadIdx.x) * KG_SUMS;
+                s_e[threadIdx.x] = make_float4((float)(A[0] + A[1] * d.omega_ref), (float)A[1],
+                                               (float)(A[2] + A[3] * d.omega_ref), (float)A[3]);
+                A[0] = A[1] = A[2] = A[3] = 0.0;
+            }
+            __syncthreads();
+            for (int i = threadIdx.x; i < na * nch; i += blockDim.x) {
+                const int ant = i / nch, c = fr.x + (i - ant * nch);
+                const float4 e = s_e[ant];
+                const float om = __ldg(u.omega + c);
+                const float s0 = sinf(0.5f * fmaf(e.y, om, e.x)), s1 = sinf(0.5f * fmaf(e.w, om, e.z));
+                num += 4.0 * (double)fmaf(s0, s0, s1 * s1);
+            }
+            __syncthreads();
+        }
+        if (threadIdx.x == 0) den = 2.0 * d.n_ant * nch;
+    } else if (SUMS) {
         // the channel table and the change of the gains, spread over the block's threads by
         // (antenna, channel)
         __syncthreads();

@@ -13,6 +13,7 @@
 #include "qc_ws.cuh"
 #include "qc_robust.cuh"
 #include "qc_moments.cuh"
+#include "qc_delay_sums.cuh"
 
 // Every device allocation of the library goes through these two calls.  They count the
 // live allocations and honour the test hook of qc_test_fail_alloc (qc.h), so that tests can
@@ -98,6 +99,8 @@ struct TermBufs {
     Buf params0;   // divergence flagging: the FP64 parameters before the solve
     Buf mom;       // a term solved from sums: FP32 sums per (interval, unordered pair), bytes per interval
     SumsPlan sums; // the route of the current call
+    Buf dsum_t;    // delay terms solved from products: T [n_tint][chunks][pairs][2][32] float4
+    Buf dsum_h;    //   double [bins][ant][KG_HSUM]
     Buf dfmap;     // delay terms: int [n_chan] parameter interval of each channel
     Buf dfr;       // delay terms: int2 [n_fint] first and last channel of each interval
     Buf dnu;       // delay terms: double [n_chan] channel frequencies
@@ -172,6 +175,7 @@ struct qc_ctx {
     int n_dir = 1;                    // directions of the model (Eq. baselinemodel)
     long n_strip_rows = 0;            // rows in the baseline strips (cross-correlations)
     int max_strip_rows = 0;           // rows of the longest strip
+    bool full_grid = false;           // every pair in one orientation, each with one row per data time
     bool m16 = false, has_flag = false;
     const float4 *d_vis = nullptr, *d_model = nullptr, *d_weight = nullptr;
     const uint8_t *d_flag = nullptr;
@@ -238,6 +242,9 @@ struct qc_ctx {
     int run_residual(const qc::Chain &chain, float4 *dres, double *d_chi2, cudaStream_t st);
     int pick_order(const qc_term &t, const qc_opts *o) const;
     int plan_sums(const qc_term *terms, int n_terms, int n, const qc_opts *o);
+    int ensure_mom_rows(cudaStream_t st);
+    int plan_delay_sums(const qc_term *terms, int n_terms, int n, const qc_opts *o, bool &use);
+    qc::DelaySumsArgs delay_sums_args(const qc_term *terms, int n_terms, int n, const qc::Chain &chain);
     int sums_args(const qc_term *terms, int n_terms, int n, const qc::Chain &chain, cudaStream_t st, qc::MomArgs &ma,
                   qc::MomNormArgs &mn);
     int solve_term_sums(const qc_term *terms, int n_terms, int n, const qc::Chain &chain, const qc_opts *o,
