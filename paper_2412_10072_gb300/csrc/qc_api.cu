@@ -1077,7 +1077,7 @@ static constexpr int SUMS_ONE_LAUNCH_ANT = 256;
 // instruction issue at about 0.64 of the HBM rate; the sums cost one pass, about 1.3 such
 // iterations, and then 2 x 4 x words B per (interval, pair) and iteration, mostly out of L2.  The
 // rule takes the sums when an iteration on them moves at most half the bytes of one on the
-// samples, i.e. from 2.4 (plain diagonal form), 5.6 (E form) or 20 (full form) samples per slot
+// samples, i.e. from 2.4 (plain diagonal form), 4.6 (two directions), 5.6 (E form) or 20 (full form) samples per slot
 // on, and a term may take three iterations or more.  It also bounds the workspace to a quarter of
 // the samples' bytes.  The options that name an accumulate kernel, its tiles or launch shape,
 // divergence flagging and an allreduce (whose buffers are documented per iteration) keep the
@@ -1087,21 +1087,27 @@ int qc_ctx::plan_sums(const qc_term *terms, int n_terms, int n, const qc_opts *o
     const qc_term &t = terms[n];
     TermBufs &B = tb[n];
     B.sums = SumsPlan();
-    if (n_terms > 2 || delay[n] || n_dir > 1 || n_up == 0) return QC_OK;
+    if (n_terms > 2 || delay[n] || n_up == 0) return QC_OK;
     const size_t nb = term_nbins(t), slots = nb * (size_t)n_up;
     if (slots >= (size_t)INT32_MAX) return QC_OK;
     const int lk = kind_of_range(terms, 0, n), rk = kind_of_range(terms, n + 1, n_terms);
     int form, ok;
-    if (t.type != QC_TERM_FULL && lk != KIND_FULL) { form = FORM_D; ok = lk != KIND_NONE ? lk : rk; }
+    if (n_dir > 1) {
+        // two directions: a direction-dependent diagonal term beside a direction-independent one
+        if (n_dir != 2 || cur_nd[n] != 2 || t.type != QC_TERM_DIAG || lk == KIND_FULL) return QC_OK;
+        if (n_terms == 2 && cur_nd[1 - n] != 1) return QC_OK;
+        form = FORM_DD;
+        ok = lk != KIND_NONE ? lk : rk;
+    } else if (t.type != QC_TERM_FULL && lk != KIND_FULL) { form = FORM_D; ok = lk != KIND_NONE ? lk : rk; }
     else if (t.type != QC_TERM_FULL) { form = FORM_E; ok = lk; }
     else if (lk == KIND_NONE) { form = FORM_FULL; ok = rk; }
     else return QC_OK;
-    const bool asked = o->moments && d_model != nullptr;
+    const bool asked = o->moments && d_model != nullptr && n_dir == 1;
     const bool one_launch = n_ant <= SUMS_ONE_LAUNCH_ANT && !t.reduce && !(o->div_flag && t.max_iter >= 4);
     if (!asked) {
         const bool plain = o->kernel == 0 && o->order == -1 && o->block_threads == 0 && o->ctas_per_sm == 0;
         if (!plain || !one_launch || o->div_flag || t.max_iter < 3) return QC_OK;
-        const double sample_bytes = (m16 ? 64.0 : 80.0) * (double)n_strip_rows * n_chan;
+        const double sample_bytes = (m16 ? 64.0 : 48.0 + 32.0 * n_dir) * (double)n_strip_rows * n_chan;
         if (2.0 * 4.0 * mom_words(form) * (double)slots > 0.5 * sample_bytes) return QC_OK;
     }
     const size_t sums_bytes = ((nbytes<float>(slots * mom_words(form)) + 15) / 16) * 16;
@@ -1323,7 +1329,7 @@ int qc_ctx::solve_term_sums(const qc_term *terms, int n_terms, int n, const Chai
     mi.cnt = cnt;
     mi.bin_nvis = (const long long *)B.nvis.ptr;
     mi.bin_nbytes = (const long long *)B.nvis.ptr + 2 * (size_t)P.n_bins;
-    mi.iter_bytes = 2LL * n_up * mom_words(B.sums.form) * 4 + 8LL * n_ant * (t.type == 1 ? KG_FULL : KG_DIAG);
+    mi.iter_bytes = 2LL * n_up * mom_words(B.sums.form) * 4 + 8LL * term_nat(t) * (t.type == 1 ? KG_FULL : KG_DIAG);
     mi.vis_iters = (unsigned long long *)scalars.ptr;
     mi.acc_bytes = (unsigned long long *)scalars.ptr + 1;
     mi.max_iter = t.max_iter;

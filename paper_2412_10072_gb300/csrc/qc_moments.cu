@@ -109,6 +109,26 @@ __device__ __forceinline__ void mom_add_d(float (&acc)[MOM_D], const J2 &D, cons
 // S' += conj(M_ab) M_a'b' K, and T' += conj(M_ab) (L_p^H (w D) L_q)_ab.  Forming the E_kj and adding their
 // products one by one takes 390 instructions a sample, this 236, and each word of the sums is
 // rounded once or twice a sample instead of eight times.
+// Two directions, E_d the model of direction d with the fixed term folded in:
+// S_de,kj = sum w conj(E_d,kj) E_e,kj (de = 00, 11 real, 01), T_d,kj = sum w conj(E_d,kj) D_kj.
+__device__ __forceinline__ void mom_add_dd(float (&acc)[MOM_DD], const J2 &D, const J2 &X0, const J2 &X1, float4 w)
+{
+    const float2 x0[4] = { X0.a, X0.b, X0.c, X0.d }, x1[4] = { X1.a, X1.b, X1.c, X1.d };
+    const float2 d[4] = { D.a, D.b, D.c, D.d };
+    const float wv[4] = { w.x, w.y, w.z, w.w };
+#pragma unroll
+    for (int kj = 0; kj < 4; ++kj) {
+        acc[kj] = fmaf(wv[kj], cnorm2(x0[kj]), acc[kj]);
+        acc[4 + kj] = fmaf(wv[kj], cnorm2(x1[kj]), acc[4 + kj]);
+        const float2 z = cmulc(x1[kj], x0[kj]);
+        acc[8 + 2 * kj] = fmaf(wv[kj], z.x, acc[8 + 2 * kj]);
+        acc[9 + 2 * kj] = fmaf(wv[kj], z.y, acc[9 + 2 * kj]);
+        const float2 wd = cscale(d[kj], wv[kj]);
+        cacc_conj(acc[16 + 2 * kj], acc[17 + 2 * kj], x0[kj], wd);
+        cacc_conj(acc[24 + 2 * kj], acc[25 + 2 * kj], x1[kj], wd);
+    }
+}
+
 __device__ __forceinline__ void mom_add_e(float (&acc)[MOM_EW], const J2 &D, const J2 &M, const J2 &Lp,
                                           const J2 &Lq, float4 w)
 {
@@ -256,14 +276,15 @@ __device__ __forceinline__ J2 fac_jones(const float4 *o)
 // frequency intervals), the lanes' keys (32 ints) and one int4 of meta data.
 template <int FORM, int OK, bool M16> struct MomRing {
     static constexpr int NO = OK == KIND_FULL ? 2 : (OK == KIND_DIAG ? 1 : 0);
-    static constexpr int OFF_W = M16 ? 96 : 128;
+    static constexpr int ND = FORM == FORM_DD ? 2 : 1;       // directions of the model
+    static constexpr int OFF_W = M16 ? 96 : 64 + 64 * ND;
     static constexpr int OFF_OP = OFF_W + 32, OFF_OQ = OFF_OP + 32 * NO, OFF_KEY = OFF_OQ + 32 * NO;
     static constexpr int OFF_META = OFF_KEY + 8;
     static constexpr int STAGE = OFF_META + 1;               // float4 per stage
     // three CTAs of 4 warps per SM (the full form's 100 register sums fit 168 registers); ring
     // depth as the shared memory of three CTAs allows
     static constexpr int PER_SM = 3;
-    static constexpr int DEPTH = NO == 2 ? 3 : (NO == 1 ? 4 : 6);
+    static constexpr int DEPTH = NO == 2 || ND == 2 ? 3 : (NO == 1 ? 4 : 6);
     static constexpr size_t SMEM = (size_t)4 * DEPTH * STAGE * sizeof(float4);
     // A lane's sums over a long strip are FP32 sums of terms of one sign, whose rounding grows with
     // the number of terms and moves the fixed point of all antennas the same way.  The short slots keep
@@ -343,8 +364,9 @@ template <int FORM, int OK, bool M16> struct MomCursor {
             if constexpr (M16) {
                 cp_async16(stage + 64 + lane, a.model16 + i, nb);
             } else {
-                cp_async16(stage + 64 + lane, a.model + 2 * i, nb);
-                cp_async16(stage + 96 + lane, a.model + 2 * i + 1, nb);
+#pragma unroll
+                for (int v = 0; v < 2 * R::ND; ++v)
+                    cp_async16(stage + 64 + 32 * v + lane, a.model + 2 * R::ND * i + v, nb);
             }
             cp_async16(stage + R::OFF_W + lane, a.wf + i, nb);
             if constexpr (R::NO > 0) {
@@ -396,7 +418,7 @@ template <int FORM, int OK, bool M16>
 static __global__ void __launch_bounds__(128, MomRing<FORM, OK, M16>::PER_SM) mom_pass_kernel(const MomArgs a)
 {
     using R = MomRing<FORM, OK, M16>;
-    constexpr int NW = FORM == FORM_FULL ? MOM_FW : (FORM == FORM_E ? MOM_EW : MOM_D);
+    constexpr int NW = FORM == FORM_FULL ? MOM_FW : (FORM == FORM_E ? MOM_EW : (FORM == FORM_D ? MOM_D : MOM_DD));
     if (a.n_active && __ldg(a.n_active) == 0) return;
     extern __shared__ float4 mom_ring[];
     const int lane = threadIdx.x & 31;
@@ -437,7 +459,22 @@ static __global__ void __launch_bounds__(128, MomRing<FORM, OK, M16>::PER_SM) mo
                 w = make_float4(w.x, w.z, w.y, w.w);
             }
             const int oc = (meta & 4) ? 0 : lane * R::NO;
-            if constexpr (FORM != FORM_E) {
+            if constexpr (FORM == FORM_DD) {
+                J2 M1 = j_from(st[128 + lane], st[160 + lane]);
+                if (meta & 1) M1 = j_herm(M1);
+                if constexpr (OK == KIND_DIAG) {
+                    const float4 rp = st[R::OFF_OP + oc], rq = st[R::OFF_OQ + oc];
+                    const float2 p0 = make_float2(rp.x, rp.y), p1 = make_float2(rp.z, rp.w);
+                    const float2 q0 = make_float2(rq.x, -rq.y), q1 = make_float2(rq.z, -rq.w);
+                    M = j_muld(j_dmul(p0, p1, M), q0, q1);
+                    M1 = j_muld(j_dmul(p0, p1, M1), q0, q1);
+                } else if constexpr (OK == KIND_FULL) {
+                    const J2 rp = fac_jones<OK>(st + R::OFF_OP + oc), rq = fac_jones<OK>(st + R::OFF_OQ + oc);
+                    M = j_mul_h(j_mul(rp, M), rq);
+                    M1 = j_mul_h(j_mul(rp, M1), rq);
+                }
+                mom_add_dd(acc, D, M, M1, w);
+            } else if constexpr (FORM != FORM_E) {
                 if constexpr (OK == KIND_DIAG) {
                     const float4 rp = st[R::OFF_OP + oc], rq = st[R::OFF_OQ + oc];
                     M = j_muld(j_dmul(make_float2(rp.x, rp.y), make_float2(rp.z, rp.w), M),
@@ -805,6 +842,146 @@ static __global__ void __launch_bounds__(256, 2) mom_iterate_kernel(const MomIte
     }
 }
 
+// The same for a direction-dependent diagonal term over two directions (its gains are stored over
+// (antenna, direction) pairs).  With S_de and T_d of the pair (a, q) as antenna a sees them,
+//   h_d,k = sum_q sum_j |g_q,d,j|^2 S_dd,kj,  C_k = sum_q sum_j g_q,0,j conj(g_q,1,j) S_01,kj,
+//   b_d,k = sum_q sum_j g_q,d,j T_d,kj,
+//   JHr_0,k = b_0,k - h_0,k g_a,0,k - C_k g_a,1,k,  JHr_1,k = b_1,k - h_1,k g_a,1,k - conj(C_k) g_a,0,k,
+// and the block of (a, d) is diag(h_d,0, h_d,1): the blocks between directions are left out, as in
+// the iterations on the samples, but the residual holds every direction.
+static __global__ void __launch_bounds__(256, 2) mom_iterate_dd_kernel(const MomIterArgs a)
+{
+    constexpr int N = 16;     // h_00 h_01 h_10 h_11, C_0, C_1, b_00, b_01, b_10, b_11 (d, k)
+    extern __shared__ float4 s_mem[];
+    const MomNormArgs &A = a.n;
+    const int na = A.n_ant;
+    float4 *g32 = s_mem;                                             // [n_ant][2 directions] (g_XX, g_YY)
+    double *sums = reinterpret_cast<double *>(s_mem + (size_t)na * 2);   // [n_ant][N]
+    __shared__ double s_num[8], s_den[8];
+    __shared__ int s_done;
+    const int bin = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+    const int tint = bin / A.n_fint, fint = bin - tint * A.n_fint;
+    const float *bin_sums = A.mom + (size_t)bin * A.n_up * MOM_DD;
+    auto tab_at = [&](int i) { return a.tab + ((size_t)tint * na * 2 + i) * A.n_fint + fint; };
+    for (int i = tid; i < na * 2; i += blockDim.x) g32[i] = *tab_at(i);
+    __syncthreads();
+    int k = 1;
+    for (;; ++k) {
+        for (int ant = warp; ant < na; ant += nw) {
+            float h[N];
+#pragma unroll
+            for (int i = 0; i < N; ++i) h[i] = 0.f;
+            for (int o = lane; o < na; o += 32) {
+                if (o == ant) continue;
+                const int up = __ldg(A.upair + (size_t)ant * na + o);
+                if (up < 0) continue;
+                const float4 *s = reinterpret_cast<const float4 *>(bin_sums + (size_t)up * MOM_DD);
+                const bool p_side = ant < o;
+                const float sg = p_side ? 1.f : -1.f;
+                const float4 g[2] = { g32[2 * o], g32[2 * o + 1] };
+                // entries (k, j) of the antenna's own view: (0,1) and (1,0) exchanged on the q side
+                auto entry = [&](const float4 &lo, const float4 &hi, float2 (&v)[4]) {
+                    v[0] = make_float2(lo.x, sg * lo.y);
+                    v[3] = make_float2(hi.z, sg * hi.w);
+                    v[1] = p_side ? make_float2(lo.z, lo.w) : make_float2(hi.x, -hi.y);
+                    v[2] = p_side ? make_float2(hi.x, hi.y) : make_float2(lo.z, -lo.w);
+                };
+#pragma unroll
+                for (int d = 0; d < 2; ++d) {
+                    const float4 sd = __ldg(s + d);
+                    const float n0 = fmaf(g[d].x, g[d].x, g[d].y * g[d].y), n1 = fmaf(g[d].z, g[d].z, g[d].w * g[d].w);
+                    h[2 * d] += fmaf(n0, sd.x, n1 * (p_side ? sd.y : sd.z));
+                    h[2 * d + 1] += fmaf(n0, p_side ? sd.z : sd.y, n1 * sd.w);
+                    float2 t[4];
+                    entry(__ldg(s + 4 + 2 * d), __ldg(s + 5 + 2 * d), t);
+                    const float2 g0 = make_float2(g[d].x, g[d].y), g1 = make_float2(g[d].z, g[d].w);
+#pragma unroll
+                    for (int r = 0; r < 2; ++r) {
+                        const float2 v = cdot(g0, t[2 * r], g1, t[2 * r + 1]);
+                        h[8 + 4 * d + 2 * r] += v.x;
+                        h[9 + 4 * d + 2 * r] += v.y;
+                    }
+                }
+                float2 c[4];
+                entry(__ldg(s + 2), __ldg(s + 3), c);
+                const float2 y0 = cmulc(make_float2(g[0].x, g[0].y), make_float2(g[1].x, g[1].y));
+                const float2 y1 = cmulc(make_float2(g[0].z, g[0].w), make_float2(g[1].z, g[1].w));
+#pragma unroll
+                for (int r = 0; r < 2; ++r) {
+                    const float2 v = cdot(y0, c[2 * r], y1, c[2 * r + 1]);
+                    h[4 + 2 * r] += v.x;
+                    h[5 + 2 * r] += v.y;
+                }
+            }
+            const double v = reduce_words<N>(h, lane);
+            if ((lane & 1) == 0) sums[(size_t)ant * N + lane / 2] = v;
+        }
+        __syncthreads();
+        const double alpha = a.alternate ? ((k % 2 == 0) ? 0.5 : 1.0) : a.damping;
+        // JHr in the place of b, from both directions' gains of the antenna (FP64 master) ...
+        for (int i = tid; i < na * 2; i += blockDim.x) {
+            const int ant = i >> 1, d = i & 1;
+            double *h = sums + (size_t)ant * N;
+            const double2 *P = reinterpret_cast<const double2 *>(a.params) + 4 * ((size_t)bin * na * 2 + i);
+            const double2 *O = reinterpret_cast<const double2 *>(a.params) + 4 * ((size_t)bin * na * 2 + (i ^ 1));
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const double2 g = P[3 * e], o = O[3 * e];
+                const double cx = h[4 + 2 * e], cy = d ? -h[5 + 2 * e] : h[5 + 2 * e], hd = h[2 * d + e];
+                h[8 + 4 * d + 2 * e] -= hd * g.x + (cx * o.x - cy * o.y);
+                h[9 + 4 * d + 2 * e] -= hd * g.y + (cx * o.y + cy * o.x);
+            }
+        }
+        __syncthreads();
+        // ... then every (antenna, direction) steps
+        double num = 0, den = 0;
+        for (int i = tid; i < na * 2; i += blockDim.x) {
+            const int ant = i >> 1, d = i & 1;
+            const double *h = sums + (size_t)ant * N;
+            double2 *P = reinterpret_cast<double2 *>(a.params) + 4 * ((size_t)bin * na * 2 + i);
+            const double2 old[2] = { P[0], P[3] };
+            const double h00[1] = { h[2 * d] }, h11[1] = { h[2 * d + 1] };
+            const double2 z[1] = { make_double2(0, 0) };
+            const double2 r[2] = { make_double2(h[8 + 4 * d], h[9 + 4 * d]), make_double2(h[10 + 4 * d], h[11 + 4 * d]) };
+            double2 x[2], now[2];
+            const int singular = solve_blocks<1>(h00, h11, z, r, x);
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                now[e] = singular ? old[e] : make_double2(old[e].x + alpha * x[e].x, old[e].y + alpha * x[e].y);
+                const double dx = now[e].x - old[e].x, dy = now[e].y - old[e].y;
+                num += dx * dx + dy * dy;
+                den += now[e].x * now[e].x + now[e].y * now[e].y;
+            }
+            P[0] = now[0];
+            P[3] = now[1];
+            a.gain_flags[(size_t)bin * na * 2 + i] = (int8_t)singular;
+            g32[i] = make_float4((float)now[0].x, (float)now[0].y, (float)now[1].x, (float)now[1].y);
+        }
+        for (int d = 16; d > 0; d >>= 1) {
+            num += __shfl_down_sync(FULL_MASK, num, d);
+            den += __shfl_down_sync(FULL_MASK, den, d);
+        }
+        if (lane == 0) { s_num[warp] = num; s_den[warp] = den; }
+        __syncthreads();
+        if (tid == 0) {
+            double tn = 0, td = 0;
+            for (int i = 0; i < nw; ++i) { tn += s_num[i]; td += s_den[i]; }
+            const double delta = td > 0 ? sqrt(tn / td) : 0.0;
+            const bool conv = delta < a.tol;
+            if (!conv) atomicAdd(a.cnt + k, 1);
+            s_done = conv || k == a.max_iter;
+        }
+        __syncthreads();
+        if (s_done) break;
+    }
+    for (int i = tid; i < na * 2; i += blockDim.x) *tab_at(i) = g32[i];
+    if (tid == 0) {
+        a.iters[bin] = k;
+        atomicAdd(a.vis_iters, (unsigned long long)a.bin_nvis[bin] * k);
+        atomicAdd(a.acc_bytes, (unsigned long long)(a.bin_nbytes[bin] + a.iter_bytes * k));
+    }
+}
+
 // algorithmic bytes: the pass reads every sample of the bins once (their streaming bytes);
 // an iteration reads each bin's sums twice (once per side) and writes its accumulators
 static __global__ void mom_bytes_kernel(int n_bins, const long long *bin_nbytes, long long per_iter,
@@ -849,6 +1026,12 @@ static cudaError_t launch_pass_any(const qc::MomArgs &a, int form, int ok, int s
         return launch_pass<FORM_FULL, KIND_FULL, M16>(a, sm_count, st);
     }
     if (form == FORM_E) return ok == KIND_FULL ? launch_pass<FORM_E, KIND_FULL, M16>(a, sm_count, st) : cudaErrorInvalidValue;
+    if constexpr (!M16)
+        if (form == FORM_DD) {
+            if (ok == KIND_NONE) return launch_pass<FORM_DD, KIND_NONE, false>(a, sm_count, st);
+            if (ok == KIND_DIAG) return launch_pass<FORM_DD, KIND_DIAG, false>(a, sm_count, st);
+            return launch_pass<FORM_DD, KIND_FULL, false>(a, sm_count, st);
+        }
     if (ok == KIND_NONE) return launch_pass<FORM_D, KIND_NONE, M16>(a, sm_count, st);
     if (ok == KIND_DIAG) return launch_pass<FORM_D, KIND_DIAG, M16>(a, sm_count, st);
     return launch_pass<FORM_D, KIND_FULL, M16>(a, sm_count, st);
@@ -893,6 +1076,11 @@ cudaError_t mom_launch_iterate(const qc::MomIterArgs &a, cudaStream_t st)
 {
     if (a.n.form == qc::FORM_FULL) return launch_iterate<qc::FORM_FULL>(a, st);
     if (a.n.form == qc::FORM_E) return launch_iterate<qc::FORM_E>(a, st);
+    if (a.n.form == qc::FORM_DD) {
+        const size_t smem = (size_t)a.n.n_ant * (2 * sizeof(float4) + 16 * sizeof(double));
+        qc::mom_iterate_dd_kernel<<<a.n.n_bins, 256, smem, st>>>(a);
+        return cudaGetLastError();
+    }
     return launch_iterate<qc::FORM_D>(a, st);
 }
 

@@ -15,10 +15,12 @@ constexpr int MOM_ET = 16, MOM_EU = 24;
 // plain diagonal form (a diagonal or phase-only solved term, the other term diagonal or to its
 // right): S 4, T 8
 constexpr int MOM_D = 12;
-constexpr int FORM_FULL = 0, FORM_E = 1, FORM_D = 2;
+// two directions, a direction-dependent diagonal solved term: S_00 4, S_11 4, S_01 8, T_0 8, T_1 8
+constexpr int MOM_DD = 32;
+constexpr int FORM_FULL = 0, FORM_E = 1, FORM_D = 2, FORM_DD = 3;
 __host__ __device__ constexpr int mom_words(int form)
 {
-    return form == FORM_FULL ? MOM_N : (form == FORM_E ? MOM_E : MOM_D);
+    return form == FORM_FULL ? MOM_N : (form == FORM_E ? MOM_E : (form == FORM_D ? MOM_D : MOM_DD));
 }
 
 // Hermitian pairs (u, v), u < v, of the 4x4 S blocks: packed as 4 diagonal reals then 6 (re, im)
