@@ -513,8 +513,12 @@ typedef struct {
 int qc_batch_create(const qc_batch_problem *p, qc_batch **out);
 
 /*
- * Solve every problem of the batch with Algorithm 1 in one persistent
- * kernel launch: each CTA takes whole problems (longest first, or as the
+ * Solve every problem of the batch with Algorithm 1.  With default launch
+ * options, no tuned shape for the batch's class, no fallback start, max_iter >= 3
+ * and about two samples or more per antenna pair, from sums as
+ * qc_batch_solve_moments does (any number of antennas); stats then report the
+ * grid of one CTA per problem, depth 0, and the one data pass in `bytes`.
+ * Otherwise in one persistent kernel launch: each CTA takes whole problems (longest first, or as the
  * schedule says) and iterates them to convergence or max_iter on chip;
  * per iteration it forms the residual of every sample, accumulates the
  * per-antenna diagonal JHJ / JHr blocks (Eq. jhj_entry_simplified,
@@ -540,8 +544,8 @@ int qc_batch_solve(qc_batch *b, void *gains, int8_t *gain_flags, int32_t *iters,
  * baseline enter JHJ and JHr (Eq. jhj_entry_simplified, Eq. jhr_entry_simplified)
  * only through S_c = sum w_c |m_c|^2 and T_c = sum w_c conj(m_c) d_c per
  * correlation, and chi^2 (Eq. min) through them and U = sum_c w_c |d_c|^2.  One
- * pass over the samples forms them (float32 sums in shared memory); the
- * iterations then form the normal equations from them, with the update and
+ * pass over the samples forms them (a warp per antenna pair, float32); the
+ * iterations, one CTA per problem, then form the normal equations from them, with the update and
  * convergence test of qc_batch_solve.  With a fallback start, chi^2 at the
  * starting and at the fallback gains both come from the sums (fallback_chi2 must
  * be given but is not read) and the rule of qc_batch_opts applies.  Arguments and

@@ -28,6 +28,7 @@
 cudaError_t qc_dev_malloc(void **p, size_t bytes);   // counted allocation (qc_api.cu)
 void qc_dev_free(void *p);
 #include "qc_jones.cuh"
+#include "qc_sums.cuh"
 
 namespace {
 
@@ -748,103 +749,144 @@ __global__ void unflag_count_kernel(const uint8_t *flag, const BProb *probs, con
 // ---------------------------------------------------------------------------
 // Not in the paper.  A problem of the batch is one solution interval of one diagonal term,
 // so a baseline's samples enter JHJ and JHr only through two weighted sums per correlation c,
-// S_c = sum w_c |m_c|^2 and T_c = sum w_c conj(m_c) d_c.  One pass over the problem's samples
-// forms them per baseline in shared memory; every iteration then forms the normal equations
-// from them in FP64 (correlations XX XY YX YY = 0 1 2 3):
+// S_c = sum w_c |m_c|^2 and T_c = sum w_c conj(m_c) d_c (correlations XX XY YX YY = 0 1 2 3):
 //   antenna p of (p, q):  h0 = S0 |gq0|^2 + S1 |gq1|^2,   h1 = S2 |gq0|^2 + S3 |gq1|^2,
-//                         j0 = gq0 T0 + gq1 T1 - gp0 h0,  j1 = gq0 T2 + gq1 T3 - gp1 h1;
+//                         b0 = gq0 T0 + gq1 T1,           b1 = gq0 T2 + gq1 T3,  JHr = b - h g;
 //   antenna q through the conjugate baseline: S1 <-> S2, T -> conj(T) with T1 <-> T2, p <-> q.
-// The update and the convergence test are those of batch_kernel.
+// Two launches: batch_sums_kernel forms the sums of every (problem, pair) -- the work of the
+// whole batch spread evenly over the GPU whatever the sizes of the problems -- and
+// batch_iterate_kernel runs all iterations of a problem in one CTA on them.  One CTA per problem
+// for both (the pass into shared memory) left the large problems' pass to a single SM and shared
+// atomics between its warps: 14.6 ms for 512 problems of up to 64 antennas (1.2e8 samples) against
+// 9.9 GB / 6.8 TB/s = 1.5 ms.
 
-constexpr int MOM_MAX_ANT = 64;   // baselines x 13 floats must fit in shared memory
-constexpr int MOM_W = 13;         // S[4], T[4] as (re, im), U = sum_c w_c |d_c|^2
+constexpr int MOM_MAX_ANT = 64;   // antennas qc_batch_solve_moments accepts
+constexpr int MOM_W = 16;         // S[4], T[4] as (re, im), U = sum_c w_c |d_c|^2, 3 words of padding
+constexpr int SUMS_SEG = 8192;    // samples of a segment, where a problem's pairs are cut into several
 
 __host__ __device__ constexpr int mom_bl(int p, int q, int n) { return p * (2 * n - p - 1) / 2 + (q - p - 1); }
 
-__host__ __device__ inline size_t mom_smem_bytes(int max_ant)
-{
-    const size_t m = ((size_t)max_ant * (max_ant - 1) / 2 * MOM_W * sizeof(float) + 15) / 16 * 16;
-    return m + (size_t)max_ant * 2 * sizeof(double2) + (size_t)max_ant * 6 * sizeof(double) +
-           (size_t)max_ant * 2 * sizeof(float2);
-}
+// pairs [pair0, pair0 + n_pair) of a problem; with n_seg > 1 only their segments seg, seg + n_seg, ...
+struct SumsTile { int prob, pair0, n_pair, seg, n_seg; };
 
-template <bool M16>
-__global__ void __launch_bounds__(256) batch_moments_kernel(const BatchArgs a)
+struct SumsArgs {
+    BatchArgs b;
+    const SumsTile *tiles;
+    const long long *pair_base;   // [n_prob + 1] pairs of the problems before this one
+    const int *pair_off;          // [pair_base + prob + pair] first entry of the pair in strip (n_pair + 1 each)
+    const int *strip;             // [rows] the problem's rows grouped by pair: row | conj << 31
+    float *sums;                  // [pairs][MOM_W]
+};
+
+// Rows of each problem grouped by unordered antenna pair (autocorrelations left out).
+__global__ void __launch_bounds__(256) batch_strips_kernel(const BProb *probs, const int2 *ants,
+                                                           const long long *pair_base, int *pair_off, int *strip)
 {
-    extern __shared__ __align__(16) unsigned char msm[];
-    const size_t mom_bytes = ((size_t)a.max_ant * (a.max_ant - 1) / 2 * MOM_W * sizeof(float) + 15) / 16 * 16;
-    float *mom = reinterpret_cast<float *>(msm);                                  // [n_bl][MOM_W]
-    double2 *g64 = reinterpret_cast<double2 *>(msm + mom_bytes);                 // [max_ant][2]
-    double *acc = reinterpret_cast<double *>(g64 + 2 * a.max_ant);               // [max_ant][6]
-    float2 *g32 = reinterpret_cast<float2 *>(acc + 6 * a.max_ant);               // [max_ant][2]
-    __shared__ double red[2][8];
-    __shared__ int s_done;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, n_warps = blockDim.x >> 5;
-    const int pi = a.order[blockIdx.x];
-    const BProb P = a.probs[pi];
-    const int na = P.n_ant, nc = P.n_chan, n_bl = na * (na - 1) / 2;
-    for (int i = tid; i < n_bl * MOM_W; i += blockDim.x) mom[i] = 0.f;
-    for (int i = tid; i < na; i += blockDim.x) {
-        const float2 g0 = a.gains[(size_t)(P.gain_off + i) * 2], g1 = a.gains[(size_t)(P.gain_off + i) * 2 + 1];
-        g64[2 * i] = make_double2(g0.x, g0.y);
-        g64[2 * i + 1] = make_double2(g1.x, g1.y);
+    extern __shared__ int s_cnt[];                 // [n_pair] counts, then cursors
+    __shared__ int s_part[256];
+    const int pi = blockIdx.x, tid = threadIdx.x;
+    const BProb P = probs[pi];
+    const int n_pair = P.n_ant * (P.n_ant - 1) / 2;
+    int *off = pair_off + pair_base[pi] + pi;
+    auto slot_of = [&](int r, bool &conj) {
+        const int2 pq = ants[P.row_off + r];
+        conj = pq.x > pq.y;
+        return pq.x == pq.y ? -1 : (conj ? mom_bl(pq.y, pq.x, P.n_ant) : mom_bl(pq.x, pq.y, P.n_ant));
+    };
+    for (int i = tid; i < n_pair; i += blockDim.x) s_cnt[i] = 0;
+    __syncthreads();
+    bool conj;
+    for (int r = tid; r < P.n_rows; r += blockDim.x) {
+        const int k = slot_of(r, conj);
+        if (k >= 0) atomicAdd(&s_cnt[k], 1);
     }
     __syncthreads();
-    // one pass over the samples: the baseline sums.  The lanes of a warp take consecutive
-    // samples, two groups of 32 per step with both groups' loads issued first; where a group's
-    // samples all belong to one baseline (a row of 32 channels or more) a transposed reduction
-    // leaves one total per sum and one shared add each, otherwise every lane adds its own (short
-    // runs of equal baselines: few conflicts).  Sample indices are 32-bit within a problem.
-    const long long n_samp = (long long)P.n_rows * nc;
-    struct Samp {
-        int key;                 // the row's baseline slot (flagged samples too: keeps runs whole)
-        bool use;                // unflagged cross-correlation sample
-        float4 w, d0, d1, m0, m1;
-        uint4 h;
-        float sc;
-        bool conj;
-    };
-    auto load = [&](long long s) {
-        Samp x;
-        x.key = -1;
-        x.use = false;
-        x.conj = false;
-        if (s < n_samp) {
-            const int si = (int)s, row = si / nc;
-            const int2 pq = a.ants[P.row_off + row];
-            const long long sg = P.vis_off + s;
-            if (pq.x != pq.y) {
-                x.conj = pq.x > pq.y;
-                x.key = x.conj ? mom_bl(pq.y, pq.x, na) : mom_bl(pq.x, pq.y, na);
-                x.use = !(a.flag && a.flag[sg]);
-            }
-            if (x.use) {
-                x.d0 = a.vis[2 * sg];
-                x.d1 = a.vis[2 * sg + 1];
-                if constexpr (M16) {
-                    x.h = a.model16[sg];
-                    x.sc = a.row_scale[P.row_off + row];
-                } else {
-                    x.m0 = a.model[2 * sg];
-                    x.m1 = a.model[2 * sg + 1];
-                }
-                x.w = a.weight[sg];
-            }
-        }
-        return x;
-    };
-    auto add = [&](const Samp &x) {
+    // exclusive scan: each thread a contiguous share of the pairs
+    const int per = (n_pair + (int)blockDim.x - 1) / (int)blockDim.x;
+    const int i0 = min(n_pair, tid * per), i1 = min(n_pair, i0 + per);
+    int sum = 0;
+    for (int i = i0; i < i1; ++i) sum += s_cnt[i];
+    s_part[tid] = sum;
+    __syncthreads();
+    if (tid == 0) {
+        int run = 0;
+        for (int t = 0; t < (int)blockDim.x; ++t) { const int v = s_part[t]; s_part[t] = run; run += v; }
+        off[n_pair] = run;
+    }
+    __syncthreads();
+    int run = s_part[tid];
+    for (int i = i0; i < i1; ++i) {
+        const int v = s_cnt[i];
+        off[i] = run;
+        s_cnt[i] = run;
+        run += v;
+    }
+    __syncthreads();
+    for (int r = tid; r < P.n_rows; r += blockDim.x) {
+        const int k = slot_of(r, conj);
+        if (k >= 0) strip[P.row_off + atomicAdd(&s_cnt[k], 1)] = (int)((unsigned)r | (conj ? 0x80000000u : 0u));
+    }
+}
+
+// The sums of a tile's pairs: a warp per pair, lanes over its samples (its rows' channels one after
+// the other), two samples a lane in flight; 13 register sums, one transposed reduction and one
+// plain store per pair (an atomic add per word where a pair is cut into segments).  Bound by HBM:
+// every sample is read once (flagged ones too: they share their DRAM bursts with read neighbours,
+// and a select keeps what they hold out).
+template <bool M16>
+__global__ void __launch_bounds__(256) batch_sums_kernel(const SumsArgs a)
+{
+    const SumsTile T = a.tiles[blockIdx.x];
+    const BProb P = a.b.probs[T.prob];
+    const int lane = threadIdx.x & 31, nc = P.n_chan;
+    const int *off = a.pair_off + a.pair_base[T.prob] + T.prob;
+    const int *strip = a.strip + P.row_off;
+    const int q32 = 32 / nc, r32 = 32 - q32 * nc;
+    const uint8_t *flag = a.b.flag ? a.b.flag + P.vis_off : nullptr;
+    for (int j = threadIdx.x >> 5; j < T.n_pair; j += blockDim.x >> 5) {
+        const int pair = T.pair0 + j;
+        const int o0 = __ldg(off + pair);
+        const long long n = (long long)(__ldg(off + pair + 1) - o0) * nc;
+        if (T.seg > 0 && (long long)T.seg * SUMS_SEG >= n) continue;
         float v[16];
 #pragma unroll
         for (int i = 0; i < 16; ++i) v[i] = 0.f;
-        if (x.use) {
-            J2 D = j_from(x.d0, x.d1);
-            J2 M;
+        int k = 0, c = 0;                      // (row, channel) of the lane's sample, 32 samples at a time
+        struct Samp { float4 d0, d1, m0, m1, w; bool use, conj; float sc; };
+        auto load = [&](bool in) {
+            Samp x;
+            x.use = false;
+            if (in) {
+                const int rr = __ldg(strip + o0 + k), row = rr & 0x7fffffff;
+                const size_t l = (size_t)row * nc + c, sg = (size_t)P.vis_off + l;
+                x.conj = rr < 0;
+                x.use = !(flag && __ldg(flag + l));
+                x.d0 = __ldg(a.b.vis + 2 * sg);
+                x.d1 = __ldg(a.b.vis + 2 * sg + 1);
+                if constexpr (M16) {
+                    const uint4 h = __ldg(a.b.model16 + sg);
+                    x.m0 = *reinterpret_cast<const float4 *>(&h);
+                    x.sc = __ldg(a.b.row_scale + P.row_off + row);
+                } else {
+                    x.m0 = __ldg(a.b.model + 2 * sg);
+                    x.m1 = __ldg(a.b.model + 2 * sg + 1);
+                }
+                x.w = __ldg(a.b.weight + sg);
+            }
+            c += r32;
+            k += q32;
+            if (c >= nc) { c -= nc; ++k; }
+            return x;
+        };
+        auto add = [&](const Samp &x) {
+            if (!x.use) return;
+            J2 D = j_from(x.d0, x.d1), M;
             if constexpr (M16) {
-                M.a = cscale(h2f(*reinterpret_cast<const __half2 *>(&x.h.x)), x.sc);
-                M.b = cscale(h2f(*reinterpret_cast<const __half2 *>(&x.h.y)), x.sc);
-                M.c = cscale(h2f(*reinterpret_cast<const __half2 *>(&x.h.z)), x.sc);
-                M.d = cscale(h2f(*reinterpret_cast<const __half2 *>(&x.h.w)), x.sc);
+                const uint4 h = *reinterpret_cast<const uint4 *>(&x.m0);
+                M.a = cscale(h2f(*reinterpret_cast<const __half2 *>(&h.x)), x.sc);
+                M.b = cscale(h2f(*reinterpret_cast<const __half2 *>(&h.y)), x.sc);
+                M.c = cscale(h2f(*reinterpret_cast<const __half2 *>(&h.z)), x.sc);
+                M.d = cscale(h2f(*reinterpret_cast<const __half2 *>(&h.w)), x.sc);
             } else {
                 M = j_from(x.m0, x.m1);
             }
@@ -857,68 +899,56 @@ __global__ void __launch_bounds__(256) batch_moments_kernel(const BatchArgs a)
             const float2 Mv[4] = { M.a, M.b, M.c, M.d }, Dv[4] = { D.a, D.b, D.c, D.d };
             const float wv[4] = { w.x, w.y, w.z, w.w };
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                v[c] = wv[c] * cnorm2(Mv[c]);
-                const float2 t = cscale(cmulc(Dv[c], Mv[c]), wv[c]);      // w conj(m) d
-                v[4 + 2 * c] = t.x;
-                v[5 + 2 * c] = t.y;
-                v[12] = fmaf(wv[c], cnorm2(Dv[c]), v[12]);                 // w |d|^2 (chi^2 from the sums)
+            for (int e = 0; e < 4; ++e) {
+                v[e] = fmaf(wv[e], cnorm2(Mv[e]), v[e]);
+                const float2 t = cfma_conj(Mv[e], cscale(Dv[e], wv[e]), make_float2(v[4 + 2 * e], v[5 + 2 * e]));
+                v[4 + 2 * e] = t.x;                                            // w conj(m) d
+                v[5 + 2 * e] = t.y;
+                v[12] = fmaf(wv[e], cnorm2(Dv[e]), v[12]);                     // w |d|^2 (chi^2 from the sums)
             }
+        };
+        for (long long s0 = (long long)T.seg * SUMS_SEG; s0 < n; s0 += (long long)T.n_seg * SUMS_SEG) {
+            const long long s1 = T.n_seg > 1 ? min(n, s0 + SUMS_SEG) : n;
+            k = (int)((s0 + lane) / nc);
+            c = (int)((s0 + lane) - (long long)k * nc);
+            for (long long i = s0 + lane; i - lane < s1; i += 64) {
+                const Samp x0 = load(i < s1);
+                const Samp x1 = load(i + 32 < s1);
+                add(x0);
+                add(x1);
+            }
+            if (T.n_seg == 1) break;
         }
-        const int key = x.key;
-        const int k0 = __shfl_sync(0xffffffffu, key, 0);
-        if (__all_sync(0xffffffffu, key == k0)) {
-            if (k0 >= 0) {
-                // 16 slots (13 sums + 3 zeros) over 32 lanes: four halving exchanges, then a
-                // butterfly; lane l holds the total of slot l >> 1
-                int idx = 0;
-#pragma unroll
-                for (int lev = 0; lev < 4; ++lev) {
-                    const int d = 16 >> lev, h = 8 >> lev;
-                    const bool up = (lane & d) != 0;
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        if (i < h) {
-                            const float send = up ? v[i] : v[i + h];
-                            const float keep = up ? v[i + h] : v[i];
-                            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, d);
-                        }
-                    }
-                    if (up) idx += h;
-                }
-                v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
-                if ((lane & 1) == 0 && idx < MOM_W) atomicAdd(&mom[(size_t)k0 * MOM_W + idx], v[0]);
-            }
-        } else {
-            // runs of equal keys (the samples of one row, when rows are shorter than 32): a
-            // segmented reduction per sum, one shared add per run; keys that repeat apart (two
-            // rows of one baseline in a group) add per lane
-            const unsigned m = __match_any_sync(0xffffffffu, key);
-            const unsigned lo = m & (0u - m);
-            const bool contig = ((m + lo) & m) == 0;          // the set bits of m are one run
-            if (__all_sync(0xffffffffu, contig)) {
-                const int seg_end = 32 - __clz(m);
-                const bool head = lane == __ffs(m) - 1;
-#pragma unroll
-                for (int i = 0; i < MOM_W; ++i) {
-                    float t = v[i];
-#pragma unroll
-                    for (int d = 1; d < 32; d <<= 1) {
-                        const float o = __shfl_down_sync(0xffffffffu, t, d);
-                        if (lane + d < seg_end) t += o;
-                    }
-                    if (head && key >= 0) atomicAdd(&mom[(size_t)key * MOM_W + i], t);
-                }
-            } else if (key >= 0) {
-#pragma unroll
-                for (int i = 0; i < MOM_W; ++i) atomicAdd(&mom[(size_t)key * MOM_W + i], v[i]);
-            }
+        const double tot = reduce_words<16>(v, lane);
+        if ((lane & 1) == 0 && lane / 2 < 13) {
+            float *dst = a.sums + ((size_t)a.pair_base[T.prob] + pair) * MOM_W + lane / 2;
+            if (T.n_seg > 1 && n > SUMS_SEG) atomicAdd(dst, (float)tot);
+            else *dst = (float)tot;
         }
-    };
-    for (long long base = (long long)warp * 64; base < n_samp; base += 2LL * blockDim.x) {
-        const Samp x0 = load(base + lane), x1 = load(base + 32 + lane);
-        add(x0);
-        add(x1);
+    }
+}
+
+// All iterations of one problem in one CTA: warps over the antennas, lanes over the others, the
+// cross-antenna sums compensated (reduce_words), JHr = b - h g, the update and the convergence test
+// in FP64 as batch_kernel's.  The sums come out of L2 (48 of the 64 B per pair and side).
+__global__ void __launch_bounds__(256) batch_iterate_kernel(const SumsArgs s)
+{
+    const BatchArgs &a = s.b;
+    extern __shared__ __align__(16) unsigned char msm[];
+    double2 *g64 = reinterpret_cast<double2 *>(msm);                              // [max_ant][2]
+    double *acc = reinterpret_cast<double *>(g64 + 2 * a.max_ant);               // [max_ant][6]
+    float4 *g32 = reinterpret_cast<float4 *>(acc + 6 * a.max_ant);               // [max_ant] (g_XX, g_YY)
+    __shared__ double red[2][8];
+    __shared__ int s_done;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, n_warps = blockDim.x >> 5;
+    const int pi = a.order[blockIdx.x];
+    const BProb P = a.probs[pi];
+    const int na = P.n_ant;
+    const float *mom = s.sums + (size_t)s.pair_base[pi] * MOM_W;
+    for (int i = tid; i < na; i += blockDim.x) {
+        const float2 g0 = a.gains[(size_t)(P.gain_off + i) * 2], g1 = a.gains[(size_t)(P.gain_off + i) * 2 + 1];
+        g64[2 * i] = make_double2(g0.x, g0.y);
+        g64[2 * i + 1] = make_double2(g1.x, g1.y);
     }
     __syncthreads();
     // a fallback start: chi^2 at the starting and at the fallback gains from the sums (per
@@ -972,49 +1002,30 @@ __global__ void __launch_bounds__(256) batch_moments_kernel(const BatchArgs a)
         }
         __syncthreads();
     }
+    for (int i = tid; i < na; i += blockDim.x) {
+        const double2 G0 = g64[2 * i], G1 = g64[2 * i + 1];
+        g32[i] = make_float4((float)G0.x, (float)G0.y, (float)G1.x, (float)G1.y);
+    }
+    __syncthreads();
     int k;
     for (k = 1; k <= a.max_iter; ++k) {
-        // the normal equations of each antenna from the sums of its baselines (no atomics: one
-        // thread per antenna, float32 sums as batch_kernel's accumulators)
-        for (int i = tid; i < 2 * na; i += blockDim.x) g32[i] = make_float2((float)g64[i].x, (float)g64[i].y);
-        __syncthreads();
-        for (int ant = tid; ant < na; ant += blockDim.x) {
-            const float2 ga0 = g32[2 * ant], ga1 = g32[2 * ant + 1];
-            float h0 = 0.f, h1 = 0.f;
-            float2 j0 = make_float2(0.f, 0.f), j1 = j0;
-            for (int o = 0; o < na; ++o) {
+        for (int ant = warp; ant < na; ant += n_warps) {
+            float h[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) h[i] = 0.f;
+            for (int o = lane; o < na; o += 32) {
                 if (o == ant) continue;
-                const float2 go0 = g32[2 * o], go1 = g32[2 * o + 1];
-                const float ao0 = cnorm2(go0), ao1 = cnorm2(go1);
-                if (ant < o) {      // antenna p of (ant, o)
-                    const float *m = mom + (size_t)mom_bl(ant, o, na) * MOM_W;
-                    const float e0 = m[0] * ao0 + m[1] * ao1, e1 = m[2] * ao0 + m[3] * ao1;
-                    const float2 T0 = make_float2(m[4], m[5]), T1 = make_float2(m[6], m[7]);
-                    const float2 T2 = make_float2(m[8], m[9]), T3 = make_float2(m[10], m[11]);
-                    h0 += e0;
-                    h1 += e1;
-                    j0 = cadd(j0, csub(cadd(cmul(go0, T0), cmul(go1, T1)), cscale(ga0, e0)));
-                    j1 = cadd(j1, csub(cadd(cmul(go0, T2), cmul(go1, T3)), cscale(ga1, e1)));
-                } else {            // antenna q of (o, ant), through the conjugate baseline
-                    const float *m = mom + (size_t)mom_bl(o, ant, na) * MOM_W;
-                    const float e0 = m[0] * ao0 + m[2] * ao1, e1 = m[1] * ao0 + m[3] * ao1;
-                    const float2 T0 = make_float2(m[4], m[5]), T1 = make_float2(m[6], m[7]);
-                    const float2 T2 = make_float2(m[8], m[9]), T3 = make_float2(m[10], m[11]);
-                    h0 += e0;
-                    h1 += e1;
-                    j0 = cadd(j0, csub(cadd(cmulc(go0, T0), cmulc(go1, T2)), cscale(ga0, e0)));
-                    j1 = cadd(j1, csub(cadd(cmulc(go0, T1), cmulc(go1, T3)), cscale(ga1, e1)));
-                }
+                const bool p_side = ant < o;
+                const float4 *m = reinterpret_cast<const float4 *>(
+                    mom + (size_t)(p_side ? mom_bl(ant, o, na) : mom_bl(o, ant, na)) * MOM_W);
+                diag_pair_add(__ldg(m), __ldg(m + 1), __ldg(m + 2), p_side, g32[o], h);
             }
-            acc[ant * 6 + 0] = h0;
-            acc[ant * 6 + 1] = h1;
-            acc[ant * 6 + 2] = j0.x;
-            acc[ant * 6 + 3] = j0.y;
-            acc[ant * 6 + 4] = j1.x;
-            acc[ant * 6 + 5] = j1.y;
+            // h[2], h[3] (no coupling between the parameters) stay zero
+            const double v = reduce_words<8>(h, lane);
+            const int w = lane >> 2;
+            if ((lane & 3) == 0 && w != 2 && w != 3) acc[ant * 6 + (w < 2 ? w : w - 2)] = v;
         }
         __syncthreads();
-        // FP64 per-antenna solve and update, as batch_kernel
         const double alpha = a.damping_mode == QC_DAMP_ALTERNATE ? ((k % 2 == 0) ? 0.5 : 1.0)
                                                                   : (a.damping > 0 ? a.damping : 1.0);
         double num = 0, den = 0;
@@ -1022,15 +1033,17 @@ __global__ void __launch_bounds__(256) batch_moments_kernel(const BatchArgs a)
             const double h0 = acc[ant * 6], h1 = acc[ant * 6 + 1];
             const double hmax = fmax(h0, h1), hmin = fmin(h0, h1);
             const bool singular = !(h0 + h1 > 0) || !(hmin / hmax >= 1e-12);
+            double2 G0 = g64[2 * ant], G1 = g64[2 * ant + 1];
             double2 d0 = make_double2(0, 0), d1 = d0;
             if (!singular) {
-                d0 = make_double2(alpha * acc[ant * 6 + 2] / h0, alpha * acc[ant * 6 + 3] / h0);
-                d1 = make_double2(alpha * acc[ant * 6 + 4] / h1, alpha * acc[ant * 6 + 5] / h1);
+                const double r0 = alpha / h0, r1 = alpha / h1;
+                d0 = make_double2((acc[ant * 6 + 2] - h0 * G0.x) * r0, (acc[ant * 6 + 3] - h0 * G0.y) * r0);
+                d1 = make_double2((acc[ant * 6 + 4] - h1 * G1.x) * r1, (acc[ant * 6 + 5] - h1 * G1.y) * r1);
             }
-            double2 G0 = g64[2 * ant], G1 = g64[2 * ant + 1];
             G0.x += d0.x; G0.y += d0.y; G1.x += d1.x; G1.y += d1.y;
             g64[2 * ant] = G0;
             g64[2 * ant + 1] = G1;
+            g32[ant] = make_float4((float)G0.x, (float)G0.y, (float)G1.x, (float)G1.y);
             if (a.gain_flags) a.gain_flags[P.gain_off + ant] = singular ? 1 : 0;
             num += d0.x * d0.x + d0.y * d0.y + d1.x * d1.x + d1.y * d1.y;
             den += G0.x * G0.x + G0.y * G0.y + G1.x * G1.x + G1.y * G1.y;
@@ -1058,10 +1071,10 @@ __global__ void __launch_bounds__(256) batch_moments_kernel(const BatchArgs a)
     }
     if (tid == 0) {
         if (a.iters) a.iters[pi] = done_iters;
-        const unsigned long long ns = (unsigned long long)n_samp;
+        const unsigned long long ns = (unsigned long long)P.n_rows * P.n_chan;
         atomicAdd(a.vis_iters, ns * done_iters);
         // one pass over the data
-        atomicAdd(a.bytes, (a.flag ? ns : 0ull) + (unsigned long long)P.n_unflag * (M16 ? 64ull : 80ull));
+        atomicAdd(a.bytes, (a.flag ? ns : 0ull) + (unsigned long long)P.n_unflag * (a.model16 ? 64ull : 80ull));
     }
 }
 
@@ -1088,6 +1101,14 @@ struct qc_batch {
     unsigned long long *counters = nullptr;
     void *gstage = nullptr;       // device staging for host gains/flags/iters
     std::vector<BProb> hprobs;
+    // the solve from sums, staged by its first use: tiles, rows grouped by pair, the sums
+    long long n_pairs = 0;        // antenna pairs over all problems
+    long long max_samples = 0;    // of one problem
+    int n_tiles = 0;
+    SumsTile *tiles = nullptr;
+    long long *pair_base = nullptr;
+    int *pair_off = nullptr, *strip = nullptr;
+    float *sums = nullptr;
     std::vector<long long> lpt_samples;   // samples of the problems in LPT order (non-increasing)
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     cudaStream_t aux_stream = nullptr;    // the small-problem class's launch
@@ -1174,6 +1195,8 @@ extern "C" int qc_batch_create(const qc_batch_problem *p, qc_batch **out)
         P.gain_off = (int)gain_off;
         P.n_unflag = 0;
         gain_off += na;
+        b->n_pairs += (long long)na * (na - 1) / 2;
+        b->max_samples = std::max(b->max_samples, v1 - v0);
         b->max_ant = std::max(b->max_ant, na);
     }
     b->n_rows = p->row_offset[p->n_prob];
@@ -1474,6 +1497,97 @@ static int launch_shape(qc_batch *b, const qc_batch_opts *o, qc_batch::Shape &sh
     return QC_OK;
 }
 
+// Stage the solve from sums: the work tiles, the rows of every problem grouped by antenna pair and room
+// for the sums.  On failure nothing is kept.
+static int stage_sums(qc_batch *b)
+{
+    if (b->sums) return QC_OK;
+    std::vector<SumsTile> tiles;
+    std::vector<long long> base(b->n_prob + 1, 0);
+    for (int i = 0; i < b->n_prob; ++i) {
+        const BProb &P = b->hprobs[i];
+        const int n_pair = P.n_ant * (P.n_ant - 1) / 2;
+        base[i + 1] = base[i] + n_pair;
+        // eight warps a tile and at least 4096 samples a warp where the problem has as many
+        const double per_pair = std::max(1.0, (double)P.n_rows * P.n_chan / n_pair);
+        const int take = (int)std::min<double>(n_pair, 8.0 * std::max(1.0, std::ceil(4096.0 / per_pair)));
+        // cut where the mean pair is longer than a segment, at most into a few per SM
+        const int segs = (int)std::min<double>(4.0 * b->sm_count, std::max(1.0, std::ceil(per_pair / SUMS_SEG)));
+        for (int p0 = 0; p0 < n_pair; p0 += take)
+            for (int sg = 0; sg < segs; ++sg) tiles.push_back({ i, p0, std::min(take, n_pair - p0), sg, segs });
+    }
+    const size_t n0 = b->owned.size();
+    cudaError_t e = cudaSuccess;
+    auto get = [&](size_t bytes) -> void * { return e == cudaSuccess ? b->alloc(std::max<size_t>(bytes, 16), &e) : nullptr; };
+    SumsTile *tl = (SumsTile *)get(sizeof(SumsTile) * tiles.size());
+    long long *pb = (long long *)get(sizeof(long long) * base.size());
+    int *po = (int *)get(sizeof(int) * ((size_t)b->n_pairs + b->n_prob));
+    int *st = (int *)get(sizeof(int) * (size_t)std::max(1LL, b->n_rows));
+    float *sm = (float *)get(sizeof(float) * MOM_W * (size_t)b->n_pairs);
+    cudaStream_t cs = b->own_stream;
+    if (e == cudaSuccess) e = cudaMemcpyAsync(tl, tiles.data(), sizeof(SumsTile) * tiles.size(), cudaMemcpyHostToDevice, cs);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(pb, base.data(), sizeof(long long) * base.size(), cudaMemcpyHostToDevice, cs);
+    if (e == cudaSuccess) {
+        const int smem = std::max(16, b->max_ant * (b->max_ant - 1) / 2 * (int)sizeof(int));
+        e = cudaFuncSetAttribute(batch_strips_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e == cudaSuccess) {
+            batch_strips_kernel<<<b->n_prob, 256, smem, cs>>>(b->probs, b->ants, pb, po, st);
+            e = cudaGetLastError();
+        }
+    }
+    // every later call, on whatever stream, finds the tables complete
+    if (e == cudaSuccess) e = cudaStreamSynchronize(cs);
+    if (e != cudaSuccess) {
+        while (b->owned.size() > n0) { qc_dev_free(b->owned.back()); b->owned.pop_back(); }
+        return b->cuda_fail(e, "sums of the batch");
+    }
+    b->n_tiles = (int)tiles.size();
+    b->tiles = tl;
+    b->pair_base = pb;
+    b->pair_off = po;
+    b->strip = st;
+    b->sums = sm;
+    return QC_OK;
+}
+
+// The two launches of a solve from sums.
+static int enqueue_sums(qc_batch *b, const BatchArgs &a, cudaStream_t st)
+{
+    SumsArgs s;
+    s.b = a;
+    s.tiles = b->tiles;
+    s.pair_base = b->pair_base;
+    s.pair_off = b->pair_off;
+    s.strip = b->strip;
+    s.sums = b->sums;
+    if (b->max_samples > SUMS_SEG)             // only then a pair can be cut
+        BCK(cudaMemsetAsync(b->sums, 0, sizeof(float) * MOM_W * (size_t)b->n_pairs, st));
+    if (b->m16) batch_sums_kernel<true><<<b->n_tiles, 256, 0, st>>>(s);
+    else batch_sums_kernel<false><<<b->n_tiles, 256, 0, st>>>(s);
+    BCK(cudaGetLastError());
+    const size_t smem = (size_t)b->max_ant * (2 * sizeof(double2) + 6 * sizeof(double) + sizeof(float4));
+    const int threads = b->max_ant > 8 ? 256 : 64;
+    batch_iterate_kernel<<<b->n_prob, threads, smem, st>>>(s);
+    BCK(cudaGetLastError());
+    return QC_OK;
+}
+
+// Whether qc_batch_solve takes the sums by itself: no launch option of the persistent kernel named or
+// tuned, no fallback start (its bound comes from the caller's chi^2), three iterations or more, and
+// room for the sums in half the samples' bytes (about two samples a pair).  The persistent kernel
+// reads every sample each iteration and flushes its register sums to shared memory at each change
+// of baseline: 180 ms for 1024 problems of up to 64 antennas (2.0e8 samples) against 3.5 from sums.
+static bool sums_pay(const qc_batch *b, const qc_batch_opts *o)
+{
+    qc_batch::Shape t;
+    return o->threads == 0 && o->ctas_per_sm == 0 && o->schedule == QC_SCHED_AUTO && o->depth == 0 && o->split == 0 &&
+           o->small_threads == 0 && o->small_ctas_per_sm == 0 && !o->fallback_gains && o->max_iter >= 3 &&
+           4.0 * MOM_W * (double)b->n_pairs <= 0.5 * 80.0 * (double)b->n_vis && !tuned_shape(b, t);
+}
+
+static int batch_solve_sums(qc_batch *b, void *gains, int8_t *gain_flags, int32_t *iters, int32_t mem,
+                            const qc_batch_opts *o, qc_batch_stats *stats);
+
 static int batch_solve_impl(qc_batch *b, void *gains, int8_t *gain_flags, int32_t *iters, int32_t mem,
                             const qc_batch_opts *o, qc_batch_stats *stats, bool tuning)
 {
@@ -1487,6 +1601,13 @@ static int batch_solve_impl(qc_batch *b, void *gains, int8_t *gain_flags, int32_
     if (o->damping_mode != QC_DAMP_CONST && o->damping_mode != QC_DAMP_ALTERNATE) return b->fail(QC_EINVAL, "damping_mode");
     qc_batch::Shape sh;
     int rc;
+    if (!tuning && sums_pay(b, o)) {
+        rc = stage_sums(b);
+        if (rc == QC_OK) return batch_solve_sums(b, gains, gain_flags, iters, mem, o, stats);
+        if (rc != QC_ENOMEM) return rc;
+        cudaGetLastError();                    // no room for the sums: iterate on the samples
+        b->err.clear();
+    }
     if ((rc = launch_shape(b, o, sh))) return rc;
     const int threads = sh.threads, per_sm = sh.per_sm, schedule = sh.schedule, depth = sh.depth;
     cudaStream_t st = o->stream ? (cudaStream_t)o->stream : b->own_stream;
@@ -1627,6 +1748,14 @@ extern "C" int qc_batch_solve_moments(qc_batch *b, void *gains, int8_t *gain_fla
     if (o->damping_mode != QC_DAMP_CONST && o->damping_mode != QC_DAMP_ALTERNATE) return b->fail(QC_EINVAL, "damping_mode");
     if (!o->fallback_gains != !o->fallback_chi2) return b->fail(QC_EINVAL, "fallback_gains and fallback_chi2: both or neither");
     if (b->max_ant > MOM_MAX_ANT) return b->fail(QC_EUNSUPPORTED, "the moments solve takes at most 64 antennas");
+    const int rc = stage_sums(b);
+    return rc ? rc : batch_solve_sums(b, gains, gain_flags, iters, mem, o, stats);
+}
+
+// A solve from sums (staged); the options have been checked.
+static int batch_solve_sums(qc_batch *b, void *gains, int8_t *gain_flags, int32_t *iters, int32_t mem,
+                            const qc_batch_opts *o, qc_batch_stats *stats)
+{
     cudaStream_t st = o->stream ? (cudaStream_t)o->stream : b->own_stream;
     const size_t gbytes = (size_t)b->total_ant * 2 * sizeof(float2);
     unsigned char *stage = (unsigned char *)b->gstage;
@@ -1646,16 +1775,12 @@ extern "C" int qc_batch_solve_moments(qc_batch *b, void *gains, int8_t *gain_fla
     a.fb_gains = (const float2 *)o->fallback_gains;
     a.fb_chi2 = o->fallback_chi2;
     a.n_fallback = b->counters + 2 + b->n_prob;
-    const size_t smem = mom_smem_bytes(std::max(2, b->max_ant));
-    const void *fn = b->m16 ? (const void *)batch_moments_kernel<true> : (const void *)batch_moments_kernel<false>;
-    BCK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     BCK(cudaEventRecord(b->ev0, st));
     if (mem == QC_MEM_HOST) BCK(cudaMemcpyAsync(dg, gains, gbytes, cudaMemcpyHostToDevice, st));
     BCK(cudaMemsetAsync(b->counters, 0, 2 * sizeof(unsigned long long), st));
     BCK(cudaMemsetAsync(b->counters + 2 + b->n_prob, 0, sizeof(unsigned long long), st));
-    if (b->m16) batch_moments_kernel<true><<<b->n_prob, 256, smem, st>>>(a);
-    else batch_moments_kernel<false><<<b->n_prob, 256, smem, st>>>(a);
-    BCK(cudaGetLastError());
+    const int rc = enqueue_sums(b, a, st);
+    if (rc) return rc;
     if (mem == QC_MEM_HOST) {
         BCK(cudaMemcpyAsync(gains, dg, gbytes, cudaMemcpyDeviceToHost, st));
         if (gain_flags) BCK(cudaMemcpyAsync(gain_flags, dflags, (size_t)b->total_ant, cudaMemcpyDeviceToHost, st));

@@ -606,19 +606,7 @@ __device__ __forceinline__ void pair_add(const float *__restrict__ slot, bool p_
     } else if constexpr (FORM == FORM_E) {
         pair_block(s, s + MOM_ET / 4, p_side, make_float2(g[0].x, g[0].y), make_float2(g[0].z, g[0].w), h);
     } else {
-        const float4 sv = __ldg(s), t0 = __ldg(s + 1), t1 = __ldg(s + 2);
-        const float sg = p_side ? 1.f : -1.f;
-        const float s01 = p_side ? sv.y : sv.z, s10 = p_side ? sv.z : sv.y;
-        const float2 u01 = p_side ? make_float2(t0.z, t0.w) : make_float2(t1.x, t1.y);
-        const float2 u10 = p_side ? make_float2(t1.x, t1.y) : make_float2(t0.z, t0.w);
-        const float4 q = g[0];
-        const float n0 = fmaf(q.x, q.x, q.y * q.y), n1 = fmaf(q.z, q.z, q.w * q.w);
-        h[0] += fmaf(n0, sv.x, n1 * s01);
-        h[1] += fmaf(n0, s10, n1 * sv.w);
-        h[4] += fmaf(q.x, t0.x, fmaf(-q.y, sg * t0.y, fmaf(q.z, u01.x, -q.w * (sg * u01.y))));
-        h[5] += fmaf(q.x, sg * t0.y, fmaf(q.y, t0.x, fmaf(q.z, sg * u01.y, q.w * u01.x)));
-        h[6] += fmaf(q.x, u10.x, fmaf(-q.y, sg * u10.y, fmaf(q.z, t1.z, -q.w * (sg * t1.w))));
-        h[7] += fmaf(q.x, sg * u10.y, fmaf(q.y, u10.x, fmaf(q.z, sg * t1.w, q.w * t1.z)));
+        diag_pair_add(__ldg(s), __ldg(s + 1), __ldg(s + 2), p_side, g[0], h);
     }
 }
 

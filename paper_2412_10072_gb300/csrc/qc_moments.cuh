@@ -3,6 +3,7 @@
 #pragma once
 
 #include "qc_kernels.cuh"
+#include "qc_sums.cuh"
 
 namespace qc {
 
@@ -27,48 +28,6 @@ __host__ __device__ constexpr int mom_words(int form)
 __host__ __device__ constexpr int mom_pair(int u, int v)
 {
     return u == 0 ? (v == 1 ? 0 : v == 2 ? 1 : 2) : u == 1 ? (v == 2 ? 3 : 4) : 5;
-}
-
-// Transposed warp reduction of N = 4, 8 or 16 values per lane: each halving exchanges half of the
-// values a lane holds; the lanes from 32 / N * i on end with the total of value i.  The sum over
-// the lanes is carried as head and tail (Knuth's two-sum, one exact step per level), so the total over
-// the antennas is as good as an FP64 sum of the lanes' terms: rounding the tree in FP32 alone is
-// one unit in the last place of the whole right-hand side, which JHr = b - JHJ g turns into that
-// much of the gains.
-__device__ __forceinline__ void two_sum(float a, float b, float &s, float &e)
-{
-    s = a + b;
-    const float z = s - a;
-    e = (a - (s - z)) + (b - z);
-}
-template <int N> __device__ __forceinline__ double reduce_words(float (&h)[N], int lane)
-{
-    float t[N / 2];
-    int o = 16;
-#pragma unroll
-    for (int n = N / 2; n >= 1; n >>= 1, o >>= 1) {
-        const bool up = (lane & o) != 0;
-#pragma unroll
-        for (int i = 0; i < n; ++i) {
-            const float send = up ? h[i] : h[i + n], keep = up ? h[i + n] : h[i];
-            float tail = 0.f;
-            if (n < N / 2) {                                   // the tails of the levels before
-                const float ts = up ? t[i] : t[i + n];
-                tail = (up ? t[i + n] : t[i]) + __shfl_xor_sync(0xffffffffu, ts, o);
-            }
-            float e;
-            two_sum(keep, __shfl_xor_sync(0xffffffffu, send, o), h[i], e);
-            t[i] = tail + e;
-        }
-    }
-#pragma unroll
-    for (; o >= 1; o >>= 1) {
-        const float tail = t[0] + __shfl_xor_sync(0xffffffffu, t[0], o);
-        float e;
-        two_sum(h[0], __shfl_xor_sync(0xffffffffu, h[0], o), h[0], e);
-        t[0] = tail + e;
-    }
-    return (double)h[0] + (double)t[0];
 }
 
 struct MomArgs {

@@ -1,0 +1,67 @@
+// qc_sums.cuh -- device code shared by the solves from per-(interval, pair) sums.
+#pragma once
+#include "qc_jones.cuh"
+
+namespace qc {
+
+// Transposed warp reduction of N = 4, 8 or 16 values per lane: each halving exchanges half of the
+// values a lane holds; the lanes from 32 / N * i on end with the total of value i.  The sum over
+// the lanes is carried as head and tail (Knuth's two-sum, one exact step per level), so the total over
+// the antennas is as good as an FP64 sum of the lanes' terms: rounding the tree in FP32 alone is
+// one unit in the last place of the whole right-hand side, which JHr = b - JHJ g turns into that
+// much of the gains.
+__device__ __forceinline__ void two_sum(float a, float b, float &s, float &e)
+{
+    s = a + b;
+    const float z = s - a;
+    e = (a - (s - z)) + (b - z);
+}
+template <int N> __device__ __forceinline__ double reduce_words(float (&h)[N], int lane)
+{
+    float t[N / 2];
+    int o = 16;
+#pragma unroll
+    for (int n = N / 2; n >= 1; n >>= 1, o >>= 1) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int i = 0; i < n; ++i) {
+            const float send = up ? h[i] : h[i + n], keep = up ? h[i + n] : h[i];
+            float tail = 0.f;
+            if (n < N / 2) {                                   // the tails of the levels before
+                const float ts = up ? t[i] : t[i + n];
+                tail = (up ? t[i + n] : t[i]) + __shfl_xor_sync(0xffffffffu, ts, o);
+            }
+            float e;
+            two_sum(keep, __shfl_xor_sync(0xffffffffu, send, o), h[i], e);
+            t[i] = tail + e;
+        }
+    }
+#pragma unroll
+    for (; o >= 1; o >>= 1) {
+        const float tail = t[0] + __shfl_xor_sync(0xffffffffu, t[0], o);
+        float e;
+        two_sum(h[0], __shfl_xor_sync(0xffffffffu, h[0], o), h[0], e);
+        t[0] = tail + e;
+    }
+    return (double)h[0] + (double)t[0];
+}
+
+// The contribution of one pair's plain diagonal sums S_kj (s), T_kj (t0, t1) to one of its antennas:
+// h_k += sum_j |g_j|^2 S_kj into h[0], h[1] and b_k += sum_j g_j T_kj into h[4..7], with the other
+// antenna's gains q = (g_XX, g_YY); the q side takes S_jk and conj(T_jk).
+__device__ __forceinline__ void diag_pair_add(float4 sv, float4 t0, float4 t1, bool p_side, float4 q, float *h)
+{
+    const float sg = p_side ? 1.f : -1.f;
+    const float s01 = p_side ? sv.y : sv.z, s10 = p_side ? sv.z : sv.y;
+    const float2 u01 = p_side ? make_float2(t0.z, t0.w) : make_float2(t1.x, t1.y);
+    const float2 u10 = p_side ? make_float2(t1.x, t1.y) : make_float2(t0.z, t0.w);
+    const float n0 = fmaf(q.x, q.x, q.y * q.y), n1 = fmaf(q.z, q.z, q.w * q.w);
+    h[0] += fmaf(n0, sv.x, n1 * s01);
+    h[1] += fmaf(n0, s10, n1 * sv.w);
+    h[4] += fmaf(q.x, t0.x, fmaf(-q.y, sg * t0.y, fmaf(q.z, u01.x, -q.w * (sg * u01.y))));
+    h[5] += fmaf(q.x, sg * t0.y, fmaf(q.y, t0.x, fmaf(q.z, sg * u01.y, q.w * u01.x)));
+    h[6] += fmaf(q.x, u10.x, fmaf(-q.y, sg * u10.y, fmaf(q.z, t1.z, -q.w * (sg * t1.w))));
+    h[7] += fmaf(q.x, sg * u10.y, fmaf(q.y, u10.x, fmaf(q.z, sg * t1.w, q.w * t1.z)));
+}
+
+} // namespace qc
