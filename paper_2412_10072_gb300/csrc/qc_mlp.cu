@@ -40,73 +40,137 @@ __device__ __forceinline__ float gelu_d(float z)
 // so the layers learn the correction to them)
 // ---------------------------------------------------------------------------
 
-constexpr int FR = 64;            // rows per CTA tile
+// Both kernels take tiles of 32 rows and keep the two 128 x 128 matrices in shared memory with rows of
+// 132 floats, which makes every 16-byte access below conflict-free: eight lanes of a quarter of a
+// warp touch eight matrix rows 4 banks apart, or 128 contiguous bytes.  A warp computes 16 rows x 32
+// columns of a layer, a thread 4 x 4, from float4s along the summed index: 64 FMAs for eight 16-byte
+// shared loads of one wavefront each, so the FMA pipe and not shared memory is the limit.  (One
+// thread's four columns a matrix row apart, read word by word, put all lanes on one bank.)  32
+// rows give 128 tiles for the usual mini-batch of 4096 rows on 152 SMs.  Training step, 4096
+// rows: 315 us before, 81 us now (forward 23, backward 60 of them on the device).
+constexpr int TR = 32;            // rows per CTA tile
 constexpr int FT = 256;           // threads
+constexpr int LD = HID + 4;       // row stride of matrices and activations in shared memory
+constexpr int LD1 = IN + 1;       // row stride of W1 and of the input tile
 
-// out[r][j] = sum_k in[r][k] W[j][k] + b[j] for a tile of FR rows and HID outputs;
-// thread t computes rows 8*(t/32) .. +8 and outputs 4*(t%32) .. +4.
-__device__ __forceinline__ void dense_tile(const float *in, int in_dim, int in_ld, const float *W, const float *b,
-                                           float *out, int out_ld, int n_rows, float *z_store, size_t z_ld,
-                                           long row0, bool act)
+// rows x HID floats from global memory (row-major) to shared rows of LD floats
+__device__ __forceinline__ void stage_rows(float *dst, const float *__restrict__ src, int rows)
 {
-    static_assert(FR == 8 * (FT / 32) && HID == 4 * 32, "thread tile covers the CTA tile");
-    const int t = threadIdx.x;
-    const int r0 = 8 * (t >> 5), j0 = 4 * (t & 31);
-    float acc[8][4];
+    if (((uintptr_t)src & 15) == 0) {
+        for (int i = threadIdx.x; i < rows * (HID / 4); i += blockDim.x) {
+            const int r = i / (HID / 4), c = i % (HID / 4);
+            *reinterpret_cast<float4 *>(dst + r * LD + 4 * c) = __ldg(reinterpret_cast<const float4 *>(src) + i);
+        }
+    } else {
+        for (int i = threadIdx.x; i < rows * HID; i += blockDim.x) dst[(i / HID) * LD + i % HID] = __ldg(src + i);
+    }
+}
+
+// the thread's rows and columns of a layer's 32 x 128 outputs
+struct TileMap {
+    int r0, c0;                   // first row (then +4 i), first column
+    __device__ __forceinline__ TileMap()
+    {
+        const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+        r0 = 16 * (w & 1) + (lane >> 3);
+        c0 = 32 * (w >> 1) + (lane & 7);
+    }
+};
+
+__device__ __forceinline__ float at4(const float4 &v, int i) { return i == 0 ? v.x : i == 1 ? v.y : i == 2 ? v.z : v.w; }
+
+// out = GELU(in W^T + b) for the tile (sums over k in ascending order from the bias); z (nullable)
+// receives the pre-activations
+__device__ __forceinline__ void dense_tile(const float *in, const float *W, const float *__restrict__ b, float *out,
+                                           float *z, long row0, int nr)
+{
+    const TileMap m;              // columns c0 + 8 j
+    float acc[4][4];
 #pragma unroll
-    for (int i = 0; i < 8; ++i)
+    for (int j = 0; j < 4; ++j) {
+        const float bj = __ldg(b + m.c0 + 8 * j);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = b[j0 + j];
-    for (int k = 0; k < in_dim; ++k) {
-        float xv[8], wv[4];
+        for (int i = 0; i < 4; ++i) acc[i][j] = bj;
+    }
+#pragma unroll 2
+    for (int k = 0; k < HID; k += 4) {
+        float4 x[4], w[4];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) xv[i] = in[(r0 + i) * in_ld + k];
+        for (int i = 0; i < 4; ++i) x[i] = *reinterpret_cast<const float4 *>(in + (m.r0 + 4 * i) * LD + k);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) wv[j] = W[(j0 + j) * in_dim + k];
+        for (int j = 0; j < 4; ++j) w[j] = *reinterpret_cast<const float4 *>(W + (m.c0 + 8 * j) * LD + k);
 #pragma unroll
-        for (int i = 0; i < 8; ++i)
+        for (int e = 0; e < 4; ++e)
 #pragma unroll
-            for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(xv[i], wv[j], acc[i][j]);
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(at4(x[i], e), at4(w[j], e), acc[i][j]);
     }
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const int r = r0 + i;
+    for (int i = 0; i < 4; ++i) {
+        const int r = m.r0 + 4 * i;
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            if (z_store && r < n_rows) z_store[(size_t)(row0 + r) * z_ld + j0 + j] = acc[i][j];
-            out[r * out_ld + j0 + j] = act ? gelu(acc[i][j]) : acc[i][j];
+            if (z && r < nr) z[(size_t)(row0 + r) * 3 * HID + m.c0 + 8 * j] = acc[i][j];
+            out[r * LD + m.c0 + 8 * j] = gelu(acc[i][j]);
         }
     }
 }
 
-__global__ void __launch_bounds__(FT) mlp_forward_kernel(const float *__restrict__ P, const float *__restrict__ x,
-                                                         long n, float *__restrict__ y, float *__restrict__ z)
+__global__ void __launch_bounds__(FT, 1) mlp_forward_kernel(const float *__restrict__ P, const float *__restrict__ x,
+                                                            long n, float *__restrict__ y, float *__restrict__ z)
 {
-    extern __shared__ float sm[];
-    float *w = sm;                                   // all parameters
-    float *h0 = w + NPARAM;                          // [FR][HID]
-    float *h1 = h0 + FR * HID;                       // [FR][HID]
-    for (int i = threadIdx.x; i < NPARAM; i += blockDim.x) w[i] = P[i];
-    for (long row0 = (long)blockIdx.x * FR; row0 < n; row0 += (long)gridDim.x * FR) {
-        const int nr = (int)min((long)FR, n - row0);
+    extern __shared__ __align__(16) float sm[];
+    float *w2 = sm, *w3 = w2 + HID * LD, *h0 = w3 + HID * LD, *h1 = h0 + TR * LD, *w4 = h1 + TR * LD;
+    float *w1 = w4 + OUT * HID, *xs = w1 + HID * LD1;
+    stage_rows(w2, P + W2, HID);
+    stage_rows(w3, P + W3, HID);
+    for (int i = threadIdx.x; i < HID * IN; i += blockDim.x) w1[(i / IN) * LD1 + i % IN] = __ldg(P + W1 + i);
+    for (int i = threadIdx.x; i < OUT * HID; i += blockDim.x) w4[i] = __ldg(P + W4 + i);
+    for (long row0 = (long)blockIdx.x * TR; row0 < n; row0 += (long)gridDim.x * TR) {
+        const int nr = (int)min((long)TR, n - row0);
         __syncthreads();
-        for (int i = threadIdx.x; i < FR * IN; i += blockDim.x) {
-            const int r = i / IN, k = i % IN;
-            h1[r * IN + k] = r < nr ? x[(row0 + r) * IN + k] : 0.f;
+        for (int i = threadIdx.x; i < TR * IN; i += blockDim.x) {
+            const int r = i / IN;
+            xs[r * LD1 + i % IN] = r < nr ? __ldg(x + row0 * IN + i) : 0.f;
         }
         __syncthreads();
-        dense_tile(h1, IN, IN, w + W1, w + B1, h0, HID, nr, z, 3 * HID, row0, true);
+        {
+            const TileMap m;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int c = m.c0 + 8 * j;
+                const float bj = __ldg(P + B1 + c);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int r = m.r0 + 4 * i;
+                    float s = bj;
+#pragma unroll
+                    for (int k = 0; k < IN; ++k) s = fmaf(xs[r * LD1 + k], w1[c * LD1 + k], s);
+                    if (z && r < nr) z[(size_t)(row0 + r) * 3 * HID + c] = s;
+                    h0[r * LD + c] = gelu(s);
+                }
+            }
+        }
         __syncthreads();
-        dense_tile(h0, HID, HID, w + W2, w + B2, h1, HID, nr, z ? z + HID : nullptr, 3 * HID, row0, true);
+        dense_tile(h0, w2, P + B2, h1, z ? z + HID : nullptr, row0, nr);
         __syncthreads();
-        dense_tile(h1, HID, HID, w + W3, w + B3, h0, HID, nr, z ? z + 2 * HID : nullptr, 3 * HID, row0, true);
+        dense_tile(h1, w3, P + B3, h0, z ? z + 2 * HID : nullptr, row0, nr);
         __syncthreads();
-        for (int i = threadIdx.x; i < FR * OUT; i += blockDim.x) {
-            const int r = i / OUT, j = i % OUT;
-            if (r >= nr) continue;
-            float s = w[B4 + j] + x[(row0 + r) * IN + SKIP + j];
-            for (int k = 0; k < HID; ++k) s = fmaf(h0[r * HID + k], w[W4 + j * HID + k], s);
-            y[(row0 + r) * OUT + j] = s;
+        // one thread per output (32 rows x 4): h0's rows are 4 banks apart, w4 is a broadcast
+        if (threadIdx.x < TR * OUT) {
+            const int r = threadIdx.x % TR, j = threadIdx.x / TR;
+            float s = __ldg(P + B4 + j) + xs[r * LD1 + SKIP + j];
+#pragma unroll 8
+            for (int k = 0; k < HID; k += 4) {
+                const float4 h = *reinterpret_cast<const float4 *>(h0 + r * LD + k);
+                const float4 w = *reinterpret_cast<const float4 *>(w4 + j * HID + k);
+                s = fmaf(h.x, w.x, s);
+                s = fmaf(h.y, w.y, s);
+                s = fmaf(h.z, w.z, s);
+                s = fmaf(h.w, w.w, s);
+            }
+            if (r < nr) y[(row0 + r) * OUT + j] = s;
         }
     }
 }
@@ -115,102 +179,225 @@ __global__ void __launch_bounds__(FT) mlp_forward_kernel(const float *__restrict
 // backward of the mean squared error over n rows x OUT outputs
 // ---------------------------------------------------------------------------
 
-constexpr int BR = 32;            // rows per CTA tile
-
-// dW[j][k] += sum_r d[r][j] a[r][k] over the tile (rows r < nr), db[j] += sum_r d[r][j]
-__device__ __forceinline__ void grad_tile(const float *d, int out_dim, const float *a, int in_dim, int in_ld, int nr,
-                                          float *dW, float *db)
+// dst = (d W) * gelu'(z) for the tile: the deltas of a layer from those of the next one
+__device__ __forceinline__ void delta_tile(const float *d, const float *W, const float *__restrict__ z, float *dst,
+                                           long row0, int nr)
 {
-    for (int i = threadIdx.x; i < out_dim * in_dim; i += blockDim.x) {
-        const int j = i / in_dim, k = i % in_dim;
-        float s = 0.f;
-        for (int r = 0; r < nr; ++r) s = fmaf(d[r * HID + j], a[r * in_ld + k], s);
-        atomicAdd(dW + i, s);
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int r0 = 16 * (w & 1) + (lane >> 3), c0 = 32 * (w >> 1) + 4 * (lane & 7);   // columns c0 .. c0 + 3
+    float acc[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+#pragma unroll 2
+    for (int k = 0; k < HID; k += 4) {
+        float4 x[4], v[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) x[i] = *reinterpret_cast<const float4 *>(d + (r0 + 4 * i) * LD + k);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) v[e] = *reinterpret_cast<const float4 *>(W + (k + e) * LD + c0);
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(at4(x[i], e), at4(v[e], j), acc[i][j]);
     }
-    for (int j = threadIdx.x; j < out_dim; j += blockDim.x) {
-        float s = 0.f;
-        for (int r = 0; r < nr; ++r) s += d[r * HID + j];
-        atomicAdd(db + j, s);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int r = r0 + 4 * i;
+        float o[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            o[j] = r < nr ? acc[i][j] * gelu_d(__ldg(z + (size_t)(row0 + r) * 3 * HID + c0 + j)) : 0.f;
+        *reinterpret_cast<float4 *>(dst + r * LD + c0) = make_float4(o[0], o[1], o[2], o[3]);
     }
 }
 
-__global__ void __launch_bounds__(FT) mlp_backward_kernel(const float *__restrict__ P, const float *__restrict__ x,
-                                                          const float *__restrict__ z, const float *__restrict__ y,
-                                                          const float *__restrict__ target, long n,
-                                                          float *__restrict__ G, double *__restrict__ loss)
+// the thread's 8 x 8 part of a 128 x 128 weight gradient: rows j0 .. j0 + 7, columns k0 .. k0 + 3 and
+// k0 + 32 .. k0 + 35
+struct GradMap {
+    int j0, k0;
+    __device__ __forceinline__ GradMap()
+    {
+        const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+        j0 = 32 * (w >> 1) + 8 * (lane >> 3);
+        k0 = 64 * (w & 1) + 4 * (lane & 7);
+    }
+};
+
+// acc += d^T a over the tile's rows (64 FMAs for four 16-byte shared loads)
+__device__ __forceinline__ void grad_tile(float (&acc)[8][8], const float *d, const float *a)
 {
-    extern __shared__ float sm[];
-    float *w2 = sm, *w3 = w2 + HID * HID, *w4 = w3 + HID * HID;
-    float *xa = w4 + OUT * HID;                      // [BR][IN]
-    float *a1 = xa + BR * IN, *a2 = a1 + BR * HID, *a3 = a2 + BR * HID;   // activations [BR][HID]
-    float *dA = a3 + BR * HID, *dB = dA + BR * HID;  // deltas [BR][HID]
+    const GradMap m;
+#pragma unroll 2
+    for (int r = 0; r < TR; ++r) {
+        const float4 d0 = *reinterpret_cast<const float4 *>(d + r * LD + m.j0);
+        const float4 d1 = *reinterpret_cast<const float4 *>(d + r * LD + m.j0 + 4);
+        const float4 a0 = *reinterpret_cast<const float4 *>(a + r * LD + m.k0);
+        const float4 a1 = *reinterpret_cast<const float4 *>(a + r * LD + m.k0 + 32);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const float dj = j < 4 ? at4(d0, j) : at4(d1, j - 4);
+#pragma unroll
+            for (int k = 0; k < 8; ++k) acc[j][k] = fmaf(dj, k < 4 ? at4(a0, k) : at4(a1, k - 4), acc[j][k]);
+        }
+    }
+}
+
+__device__ __forceinline__ void grad_add(float *G, const float (&acc)[8][8])
+{
+    const GradMap m;
+    const bool al = ((uintptr_t)G & 15) == 0;
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            float *p = G + (m.j0 + j) * HID + m.k0 + 32 * h;
+            const float *v = &acc[j][4 * h];
+            if (al) {
+                asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(__cvta_generic_to_global(p)), "f"(v[0]),
+                             "f"(v[1]), "f"(v[2]), "f"(v[3])
+                             : "memory");
+            } else {
+                for (int e = 0; e < 4; ++e) atomicAdd(p + e, v[e]);
+            }
+        }
+}
+
+// A CTA keeps its part of every gradient in registers over all of its tiles (the two 128 x 128
+// matrices 64 words a thread each) and adds it to the result once.
+__global__ void __launch_bounds__(FT, 1) mlp_backward_kernel(const float *__restrict__ P, const float *__restrict__ x,
+                                                             const float *__restrict__ z, const float *__restrict__ y,
+                                                             const float *__restrict__ target, long n,
+                                                             float *__restrict__ G, double *__restrict__ loss)
+{
+    extern __shared__ __align__(16) float sm[];
+    float *w2 = sm, *w3 = w2 + HID * LD;
+    float *a1 = w3 + HID * LD, *a2 = a1 + TR * LD, *a3 = a2 + TR * LD;      // activations
+    float *dA = a3 + TR * LD, *dB = dA + TR * LD;                            // deltas
+    float *w4 = dB + TR * LD, *dout = w4 + OUT * HID, *xs = dout + TR * OUT;
     __shared__ double red[FT / 32];
-    for (int i = threadIdx.x; i < HID * HID; i += blockDim.x) { w2[i] = P[W2 + i]; w3[i] = P[W3 + i]; }
-    for (int i = threadIdx.x; i < OUT * HID; i += blockDim.x) w4[i] = P[W4 + i];
+    const int tid = threadIdx.x;
+    stage_rows(w2, P + W2, HID);
+    stage_rows(w3, P + W3, HID);
+    for (int i = tid; i < OUT * HID; i += blockDim.x) w4[i] = __ldg(P + W4 + i);
     const float scale = 2.f / (float)((double)n * OUT);
     double lsum = 0;
-    for (long row0 = (long)blockIdx.x * BR; row0 < n; row0 += (long)gridDim.x * BR) {
-        const int nr = (int)min((long)BR, n - row0);
+    float g2[8][8], g3[8][8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+#pragma unroll
+        for (int k = 0; k < 8; ++k) { g2[j][k] = 0.f; g3[j][k] = 0.f; }
+    float g1[HID * IN / FT], g4[OUT * HID / FT], gb[2], gb4 = 0.f;   // W1, W4, b1..b3, b4
+#pragma unroll
+    for (int i = 0; i < HID * IN / FT; ++i) g1[i] = 0.f;
+#pragma unroll
+    for (int i = 0; i < OUT * HID / FT; ++i) g4[i] = 0.f;
+    gb[0] = gb[1] = 0.f;
+    // bias sums: thread t < 128 takes b3[t] then b1[t], the others b2[t - 128]
+    auto bias = [&](const float *d, int slot) {
+        const int c = tid & (HID - 1);
+        float s = 0.f;
+#pragma unroll 8
+        for (int r = 0; r < TR; ++r) s += d[r * LD + c];
+        gb[slot] += s;
+    };
+    for (long row0 = (long)blockIdx.x * TR; row0 < n; row0 += (long)gridDim.x * TR) {
+        const int nr = (int)min((long)TR, n - row0);
         __syncthreads();
-        for (int i = threadIdx.x; i < BR * HID; i += blockDim.x) {
+        for (int i = tid; i < TR * HID; i += blockDim.x) {
             const int r = i / HID, k = i % HID;
             const bool ok = r < nr;
             const float *zr = z + (size_t)(row0 + r) * 3 * HID;
-            a1[i] = ok ? gelu(zr[k]) : 0.f;
-            a2[i] = ok ? gelu(zr[HID + k]) : 0.f;
-            a3[i] = ok ? gelu(zr[2 * HID + k]) : 0.f;
+            a1[r * LD + k] = ok ? gelu(__ldg(zr + k)) : 0.f;
+            a2[r * LD + k] = ok ? gelu(__ldg(zr + HID + k)) : 0.f;
+            a3[r * LD + k] = ok ? gelu(__ldg(zr + 2 * HID + k)) : 0.f;
         }
-        for (int i = threadIdx.x; i < BR * IN; i += blockDim.x) {
+        for (int i = tid; i < TR * IN; i += blockDim.x) {
             const int r = i / IN;
-            xa[i] = r < nr ? x[row0 * IN + i] : 0.f;
+            xs[r * LD1 + i % IN] = r < nr ? __ldg(x + row0 * IN + i) : 0.f;
         }
-        // output deltas (in dB, columns 0..OUT-1)
-        for (int i = threadIdx.x; i < BR * OUT; i += blockDim.x) {
-            const int r = i / OUT, j = i % OUT;
+        if (tid < TR * OUT) {
+            const int r = tid / OUT;
             float d = 0.f;
             if (r < nr) {
-                const float e = y[(row0 + r) * OUT + j] - target[(row0 + r) * OUT + j];
+                const float e = __ldg(y + row0 * OUT + tid) - __ldg(target + row0 * OUT + tid);
                 lsum += (double)e * e;
                 d = scale * e;
             }
-            dB[r * HID + j] = d;
+            dout[tid] = d;
         }
         __syncthreads();
-        grad_tile(dB, OUT, a3, HID, HID, nr, G + W4, G + B4);
-        // delta of layer 3: (d_out W4) * g'(z3)
-        for (int i = threadIdx.x; i < BR * HID; i += blockDim.x) {
+        // output layer: its gradient, and delta 3 = (d_out W4) * gelu'(z3) into dA
+#pragma unroll
+        for (int i = 0; i < OUT * HID / FT; ++i) {
+            const int e = tid + FT * i, j = e / HID, k = e % HID;
+            float s = 0.f;
+#pragma unroll 8
+            for (int r = 0; r < TR; ++r) s = fmaf(dout[r * OUT + j], a3[r * LD + k], s);
+            g4[i] += s;
+        }
+        if (tid < OUT) {
+            float s = 0.f;
+            for (int r = 0; r < TR; ++r) s += dout[r * OUT + tid];
+            gb4 += s;
+        }
+        for (int i = tid; i < TR * HID; i += blockDim.x) {
             const int r = i / HID, k = i % HID;
             float s = 0.f;
-            for (int j = 0; j < OUT; ++j) s = fmaf(dB[r * HID + j], w4[j * HID + k], s);
-            dA[i] = r < nr ? s * gelu_d(z[(size_t)(row0 + r) * 3 * HID + 2 * HID + k]) : 0.f;
+#pragma unroll
+            for (int j = 0; j < OUT; ++j) s = fmaf(dout[r * OUT + j], w4[j * HID + k], s);
+            dA[r * LD + k] = r < nr ? s * gelu_d(__ldg(z + (size_t)(row0 + r) * 3 * HID + 2 * HID + k)) : 0.f;
         }
         __syncthreads();
-        grad_tile(dA, HID, a2, HID, HID, nr, G + W3, G + B3);
-        for (int i = threadIdx.x; i < BR * HID; i += blockDim.x) {
-            const int r = i / HID, k = i % HID;
+        grad_tile(g3, dA, a2);
+        if (tid < HID) bias(dA, 0);
+        delta_tile(dA, w3, z + HID, dB, row0, nr);
+        __syncthreads();
+        grad_tile(g2, dB, a1);
+        if (tid >= HID) bias(dB, 0);
+        delta_tile(dB, w2, z, dA, row0, nr);
+        __syncthreads();
+        if (tid < HID) bias(dA, 1);
+#pragma unroll
+        for (int i = 0; i < HID * IN / FT; ++i) {
+            const int e = tid + FT * i, j = e / IN, k = e % IN;
             float s = 0.f;
-            for (int j = 0; j < HID; ++j) s = fmaf(dA[r * HID + j], w3[j * HID + k], s);
-            dB[i] = r < nr ? s * gelu_d(z[(size_t)(row0 + r) * 3 * HID + HID + k]) : 0.f;
+#pragma unroll 8
+            for (int r = 0; r < TR; ++r) s = fmaf(dA[r * LD + j], xs[r * LD1 + k], s);
+            g1[i] += s;
         }
-        __syncthreads();
-        grad_tile(dB, HID, a1, HID, HID, nr, G + W2, G + B2);
-        for (int i = threadIdx.x; i < BR * HID; i += blockDim.x) {
-            const int r = i / HID, k = i % HID;
-            float s = 0.f;
-            for (int j = 0; j < HID; ++j) s = fmaf(dB[r * HID + j], w2[j * HID + k], s);
-            dA[i] = r < nr ? s * gelu_d(z[(size_t)(row0 + r) * 3 * HID + k]) : 0.f;
-        }
-        __syncthreads();
-        grad_tile(dA, HID, xa, IN, IN, nr, G + W1, G + B1);
     }
+    grad_add(G + W3, g3);
+    grad_add(G + W2, g2);
+#pragma unroll
+    for (int i = 0; i < HID * IN / FT; ++i) atomicAdd(G + W1 + tid + FT * i, g1[i]);
+#pragma unroll
+    for (int i = 0; i < OUT * HID / FT; ++i) atomicAdd(G + W4 + tid + FT * i, g4[i]);
+    if (tid < HID) {
+        atomicAdd(G + B3 + tid, gb[0]);
+        atomicAdd(G + B1 + tid, gb[1]);
+    } else {
+        atomicAdd(G + B2 + tid - HID, gb[0]);
+    }
+    if (tid < OUT) atomicAdd(G + B4 + tid, gb4);
     for (int d = 16; d > 0; d >>= 1) lsum += __shfl_down_sync(0xffffffffu, lsum, d);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = lsum;
+    if ((tid & 31) == 0) red[tid >> 5] = lsum;
     __syncthreads();
-    if (threadIdx.x == 0) {
+    if (tid == 0) {
         double t = 0;
         for (int i = 0; i < (int)blockDim.x / 32; ++i) t += red[i];
         atomicAdd(loss, t / ((double)n * OUT));
     }
+}
+
+__global__ void mlp_zero_kernel(float *grad, double *loss)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < NPARAM) grad[i] = 0.f;
+    if (i == 0) *loss = 0.0;
 }
 
 __global__ void adam_kernel(float *p, const float *g, float *m, float *v, int n, float lr, float b1, float b2,
@@ -234,8 +421,8 @@ int cerr(cudaError_t e, const char *what)
     return e == cudaErrorMemoryAllocation ? QC_ENOMEM : QC_ECUDA;
 }
 
-size_t fwd_smem() { return sizeof(float) * (NPARAM + 2 * FR * HID); }
-size_t bwd_smem() { return sizeof(float) * (2 * HID * HID + OUT * HID + BR * IN + 5 * BR * HID); }
+size_t fwd_smem() { return sizeof(float) * (2 * HID * LD + 2 * TR * LD + OUT * HID + HID * LD1 + TR * LD1); }
+size_t bwd_smem() { return sizeof(float) * (2 * HID * LD + 5 * TR * LD + OUT * HID + TR * OUT + TR * LD1); }
 
 int sm_count()
 {
@@ -254,7 +441,7 @@ extern "C" int qc_mlp_forward(const float *params, const float *x, int64_t n, fl
     if (n == 0) return QC_OK;
     cudaError_t e = cudaFuncSetAttribute(mlp_forward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fwd_smem());
     if (e != cudaSuccess) return cerr(e, "cudaFuncSetAttribute");
-    const long tiles = (n + FR - 1) / FR;
+    const long tiles = (n + TR - 1) / TR;
     const int grid = (int)std::min<long>(tiles, (long)sm_count());
     mlp_forward_kernel<<<grid, FT, fwd_smem(), (cudaStream_t)stream>>>(params, x, n, y, z);
     e = cudaGetLastError();
@@ -267,12 +454,12 @@ extern "C" int qc_mlp_backward(const float *params, const float *x, const float 
     g_mlp_error.clear();
     if (!params || !x || !z || !y || !target || !grad || !loss || n < 1) { g_mlp_error = "invalid arguments"; return QC_EINVAL; }
     cudaStream_t st = (cudaStream_t)stream;
-    cudaError_t e = cudaMemsetAsync(grad, 0, sizeof(float) * NPARAM, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(loss, 0, sizeof(double), st);
+    mlp_zero_kernel<<<(NPARAM + 255) / 256, 256, 0, st>>>(grad, loss);
+    cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaFuncSetAttribute(mlp_backward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bwd_smem());
     if (e != cudaSuccess) return cerr(e, "mlp backward setup");
-    const long tiles = (n + BR - 1) / BR;
-    const int grid = (int)std::min<long>(tiles, 2L * sm_count());
+    const long tiles = (n + TR - 1) / TR;
+    const int grid = (int)std::min<long>(tiles, (long)sm_count());
     mlp_backward_kernel<<<grid, FT, bwd_smem(), st>>>(params, x, z, y, target, n, grad, loss);
     e = cudaGetLastError();
     return e == cudaSuccess ? QC_OK : cerr(e, "mlp backward");
