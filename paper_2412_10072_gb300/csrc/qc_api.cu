@@ -345,6 +345,11 @@ extern "C" int qc_create(const qc_problem *p, qc_ctx **out)
                 up_of_bl[bl] = slot;
             }
         c->n_up = n_up;
+        c->pair_strips.assign(n_up, make_int2(-1, -1));
+        for (int bl = 0; bl < n_bl; ++bl) {
+            int2 &g = c->pair_strips[up_of_bl[bl]];
+            (g.x < 0 ? g.x : g.y) = bl;
+        }
         c->full_grid = c->full_grid && n_up == n_bl;
         DALLOC(c->d_upair, int, std::max<size_t>(1, upair.size()));
         if (!upair.empty()) HCOPY(c->d_upair, upair.data(), nbytes<int>(upair.size()));
@@ -525,7 +530,17 @@ int qc_ctx::expand_terms(const qc_term *terms, int n_terms, std::vector<qc_term>
         for (int ch = 0; ch < n_chan; ++ch) mean_nu += t.chan_freq[ch];
         B.omega_ref = n_chan ? DELAY_TWO_PI * (mean_nu / n_chan) : 0.0;
         std::vector<float> om(n_chan);
-        for (int ch = 0; ch < n_chan; ++ch) om[ch] = (float)(DELAY_TWO_PI * t.chan_freq[ch] - B.omega_ref);
+        B.hom_sums.assign(t.n_fint, make_double2(0.0, 0.0));
+        B.om_max = 0.f;
+        for (int ch = 0; ch < n_chan; ++ch) {
+            om[ch] = (float)(DELAY_TWO_PI * t.chan_freq[ch] - B.omega_ref);
+            B.om_max = std::max(B.om_max, std::fabs(om[ch]));
+            double2 &m = B.hom_sums[t.f_map[ch]];
+            m.x += om[ch];
+            m.y += (double)om[ch] * om[ch];
+        }
+        if ((rc = ensure(B.dom_sums, nbytes<double2>(t.n_fint)))) return rc;
+        CK(cudaMemcpyAsync(B.dom_sums.ptr, B.hom_sums.data(), nbytes<double2>(t.n_fint), cudaMemcpyHostToDevice, st));
         if (n_chan) {
             CK(cudaMemcpyAsync(B.dfmap.ptr, t.f_map, nbytes<int>(n_chan), cudaMemcpyHostToDevice, st));
             CK(cudaMemcpyAsync(B.dnu.ptr, t.chan_freq, nbytes<double>(n_chan), cudaMemcpyHostToDevice, st));
@@ -794,11 +809,7 @@ int qc_ctx::run_residual(const Chain &chain, float4 *dres, double *d_chi2, cudaS
     ra.C = chain;
     ra.resid = dres;
     ra.chi2 = d_chi2;
-    const long warps = (long)n_row * ((n_chan + 31) / 32);
-    const int grid = grid_for(warps * 32, 256, sm_count);
-    if (m16) residual_kernel<true><<<grid, 256, 0, st>>>(ra);
-    else residual_kernel<false><<<grid, 256, 0, st>>>(ra);
-    CK(cudaGetLastError());
+    CK(residual_launch(ra, m16, sm_count, st));
     ++launches;
     return QC_OK;
 }
@@ -1077,7 +1088,7 @@ static constexpr int SUMS_ONE_LAUNCH_ANT = 256;
 // instruction issue at about 0.64 of the HBM rate; the sums cost one pass, about 1.3 such
 // iterations, and then 2 x 4 x words B per (interval, pair) and iteration, mostly out of L2.  The
 // rule takes the sums when an iteration on them moves at most half the bytes of one on the
-// samples, i.e. from 2.4 (plain diagonal form), 4.6 (two directions), 5.6 (E form) or 20 (full form) samples per slot
+// samples, i.e. from 2.4 (plain diagonal form), 5.6 (E form) or 20 (full form) samples per slot
 // on, and a term may take three iterations or more.  It also bounds the workspace to a quarter of
 // the samples' bytes.  The options that name an accumulate kernel, its tiles or launch shape,
 // divergence flagging and an allreduce (whose buffers are documented per iteration) keep the
@@ -1087,27 +1098,21 @@ int qc_ctx::plan_sums(const qc_term *terms, int n_terms, int n, const qc_opts *o
     const qc_term &t = terms[n];
     TermBufs &B = tb[n];
     B.sums = SumsPlan();
-    if (n_terms > 2 || delay[n] || n_up == 0) return QC_OK;
+    if (n_terms > 2 || delay[n] || n_dir > 1 || n_up == 0) return QC_OK;
     const size_t nb = term_nbins(t), slots = nb * (size_t)n_up;
     if (slots >= (size_t)INT32_MAX) return QC_OK;
     const int lk = kind_of_range(terms, 0, n), rk = kind_of_range(terms, n + 1, n_terms);
     int form, ok;
-    if (n_dir > 1) {
-        // two directions: a direction-dependent diagonal term beside a direction-independent one
-        if (n_dir != 2 || cur_nd[n] != 2 || t.type != QC_TERM_DIAG || lk == KIND_FULL) return QC_OK;
-        if (n_terms == 2 && cur_nd[1 - n] != 1) return QC_OK;
-        form = FORM_DD;
-        ok = lk != KIND_NONE ? lk : rk;
-    } else if (t.type != QC_TERM_FULL && lk != KIND_FULL) { form = FORM_D; ok = lk != KIND_NONE ? lk : rk; }
+    if (t.type != QC_TERM_FULL && lk != KIND_FULL) { form = FORM_D; ok = lk != KIND_NONE ? lk : rk; }
     else if (t.type != QC_TERM_FULL) { form = FORM_E; ok = lk; }
     else if (lk == KIND_NONE) { form = FORM_FULL; ok = rk; }
     else return QC_OK;
-    const bool asked = o->moments && d_model != nullptr && n_dir == 1;
+    const bool asked = o->moments && d_model != nullptr;
     const bool one_launch = n_ant <= SUMS_ONE_LAUNCH_ANT && !t.reduce && !(o->div_flag && t.max_iter >= 4);
     if (!asked) {
         const bool plain = o->kernel == 0 && o->order == -1 && o->block_threads == 0 && o->ctas_per_sm == 0;
         if (!plain || !one_launch || o->div_flag || t.max_iter < 3) return QC_OK;
-        const double sample_bytes = (m16 ? 64.0 : 48.0 + 32.0 * n_dir) * (double)n_strip_rows * n_chan;
+        const double sample_bytes = (m16 ? 64.0 : 80.0) * (double)n_strip_rows * n_chan;
         if (2.0 * 4.0 * mom_words(form) * (double)slots > 0.5 * sample_bytes) return QC_OK;
     }
     const size_t sums_bytes = ((nbytes<float>(slots * mom_words(form)) + 15) / 16) * 16;
@@ -1145,8 +1150,7 @@ int qc_ctx::ensure_mom_rows(cudaStream_t st)
 
 // A solved delay term from the products T and H of qc_delay_sums.cu (chains of one or two terms, the
 // other one to the right or diagonal).  The rule: an iteration on T reads 1 KB per (time interval,
-// pair, 32 channels), one on the samples 80 B (64 B with the FP16 model, 32 B more for each further
-// direction) a sample; T is taken when it is at most 0.6 of that, which leaves the pass that forms
+// pair, 32 channels), one on the samples 80 B (64 B with the FP16 model) a sample; T is taken when it is at most 0.6 of that, which leaves the pass that forms
 // it paid for after two iterations (measured on 64 antennas, 75 x 512: pass 1.9 iterations on the
 // samples, an iteration on T 0.3).  That also bounds T to 0.6 of the samples' bytes.
 int qc_ctx::plan_delay_sums(const qc_term *terms, int n_terms, int n, const qc_opts *o, bool &use)
@@ -1154,13 +1158,13 @@ int qc_ctx::plan_delay_sums(const qc_term *terms, int n_terms, int n, const qc_o
     use = false;
     const qc_term &t = terms[n];
     TermBufs &B = tb[n];
-    if (!delay[n] || n_terms > 2 || n_dir > DSUM_MAX_DIR || n_up == 0 || n_ant > 256 || t.reduce || t.max_iter < 3)
+    if (!delay[n] || n_terms > 2 || n_dir > 1 || n_up == 0 || n_ant > 256 || t.reduce || t.max_iter < 3)
         return QC_OK;
     if (o->kernel != 0 || o->order != -1 || o->block_threads != 0 || o->ctas_per_sm != 0) return QC_OK;
     if (n == 1 && kind_of_range(terms, 0, 1) == KIND_FULL) return QC_OK;
     const size_t n_chunks = (n_chan + 31) / 32;
     const size_t t_bytes = (size_t)t.n_tint * n_chunks * n_up * 1024;
-    const double sample = 32.0 + 16.0 + (m16 ? 16.0 : 32.0 * n_dir);
+    const double sample = m16 ? 64.0 : 80.0;
     if ((double)t_bytes > 0.6 * sample * (double)n_strip_rows * n_chan) return QC_OK;
     int rc = ensure(B.dsum_t, t_bytes);
     if (!rc) rc = ensure(B.dsum_h, nbytes<double>((size_t)t.n_tint * B.hfr.size() * n_ant * KG_HSUM));
@@ -1182,7 +1186,6 @@ DelaySumsArgs qc_ctx::delay_sums_args(const qc_term *terms, int n_terms, int n, 
     a.n_chan = n_chan;
     a.n_ant = n_ant;
     a.n_up = n_up;
-    a.n_dir = n_dir;
     a.n_fint = (int)B.hfr.size();
     a.n_chunks = (n_chan + 31) / 32;
     a.vis = d_vis;
@@ -1203,7 +1206,6 @@ DelaySumsArgs qc_ctx::delay_sums_args(const qc_term *terms, int n_terms, int n, 
     a.n_rb = (int)((max_strip + a.rb - 1) / a.rb);
     a.t_map = chain.t[n].t_map;
     a.to = n_terms == 2 ? chain.t[1 - n] : chain.t[n];
-    a.nd_o = n_terms == 2 ? cur_nd[1 - n] : 1;
     // one row per (interval, pair): every slot is written exactly once
     a.store = full_grid && t.n_tint == n_time;
     for (int i = 0; i < n_time && a.store; ++i) a.store = t.t_map[i] == i;
@@ -1243,6 +1245,7 @@ int qc_ctx::sums_args(const qc_term *terms, int n_terms, int n, const Chain &cha
     ma.mscale = m16 ? (const float *)((const char *)mom_rows.ptr + scale_off) : nullptr;
     ma.strip_off = d_strip_off;
     ma.n_strips = n_strips;
+    ma.n_time = n_time;
     ma.n_chunks = (n_chan + 31) / 32;
     // an interval several times long: the rows inside each chunk keep a lane's key (units of a strip
     // x one chunk); else a row's chunks inside each row (units of whole rows), so that an interval
@@ -1785,6 +1788,8 @@ int qc_ctx::solve_term(const qc_term *terms, int n_terms, int n, Chain chain, co
         if (dsum) {
             dua.hsum = (const double *)B.dsum_h.ptr;
             dua.omega = (const float *)B.domega.ptr;
+            dua.om_sums = (const double2 *)B.dom_sums.ptr;
+            dua.om_max = B.om_max;
         }
     }
     DelaySumsArgs dsa_;
@@ -1994,190 +1999,8 @@ int qc_ctx::solve_term(const qc_term *terms, int n_terms, int n, Chain chain, co
 // multiply-add) in a fixed order.  Median and MAD are exact order statistics (the
 // floor((n - 1) / 2)-th smallest value), found by a radix select over the float bit
 // patterns, which order like the values for non-negative floats.  A sample is flagged when
-// |z - median| > fl32(threshold * 1.4826) * MAD in float32.
-
-namespace {
-
-constexpr unsigned MAD_SENTINEL = 0x7f800000u;   // +inf: excluded samples sort after the rest
-
-__device__ __forceinline__ bool mad_use(const int4 *rows, const uint8_t *flag, long i, int n_chan)
-{
-    const int4 r = rows[i / n_chan];
-    return r.x != r.y && !(flag && flag[i]);
-}
-
-__global__ void mad_z_kernel(long n_vis, int n_chan, const float4 *resid, const float4 *weight, const uint8_t *flag,
-                             const int4 *rows, unsigned *keys, unsigned long long *n_used)
-{
-    unsigned cnt = 0;
-    for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n_vis; i += (long)gridDim.x * blockDim.x) {
-        unsigned key = MAD_SENTINEL;
-        if (mad_use(rows, flag, i, n_chan)) {
-            const float4 lo = resid[2 * i], hi = resid[2 * i + 1];
-            const float4 w = weight[i];
-            const float t0 = __fadd_rn(__fmul_rn(lo.x, lo.x), __fmul_rn(lo.y, lo.y));
-            const float t1 = __fadd_rn(__fmul_rn(lo.z, lo.z), __fmul_rn(lo.w, lo.w));
-            const float t2 = __fadd_rn(__fmul_rn(hi.x, hi.x), __fmul_rn(hi.y, hi.y));
-            const float t3 = __fadd_rn(__fmul_rn(hi.z, hi.z), __fmul_rn(hi.w, hi.w));
-            float acc = __fmul_rn(w.x, t0);
-            acc = __fadd_rn(acc, __fmul_rn(w.y, t1));
-            acc = __fadd_rn(acc, __fmul_rn(w.z, t2));
-            acc = __fadd_rn(acc, __fmul_rn(w.w, t3));
-            key = __float_as_uint(__fsqrt_rn(acc));
-            ++cnt;
-        }
-        keys[i] = key;
-    }
-    for (int d = 16; d > 0; d >>= 1) cnt += __shfl_down_sync(0xffffffffu, cnt, d);
-    if ((threadIdx.x & 31) == 0 && cnt) atomicAdd(n_used, (unsigned long long)cnt);
-}
-
-// histogram of the 8 bits at `shift` of the keys whose bits above them equal `prefix`
-__global__ void mad_hist_kernel(long n, const unsigned *keys, unsigned prefix, unsigned mask, int shift, unsigned *hist)
-{
-    __shared__ unsigned h[256];
-    for (int t = threadIdx.x; t < 256; t += blockDim.x) h[t] = 0;
-    __syncthreads();
-    for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
-        const unsigned k = keys[i];
-        if ((k & mask) == prefix) atomicAdd(&h[(k >> shift) & 0xffu], 1u);
-    }
-    __syncthreads();
-    for (int t = threadIdx.x; t < 256; t += blockDim.x)
-        if (h[t]) atomicAdd(&hist[t], h[t]);
-}
-
-// keys of the used samples become the bits of |z - median|
-__global__ void mad_dev_kernel(long n_vis, int n_chan, const uint8_t *flag, const int4 *rows, float med, unsigned *keys)
-{
-    for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n_vis; i += (long)gridDim.x * blockDim.x)
-        if (mad_use(rows, flag, i, n_chan)) keys[i] = __float_as_uint(fabsf(__fsub_rn(__uint_as_float(keys[i]), med)));
-}
-
-__global__ void mad_flag_kernel(long n_vis, int n_chan, const uint8_t *flag, const int4 *rows, const unsigned *keys,
-                                float thr, uint8_t *out, unsigned long long *n_flagged)
-{
-    unsigned cnt = 0;
-    for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n_vis; i += (long)gridDim.x * blockDim.x) {
-        const bool f = mad_use(rows, flag, i, n_chan) && __uint_as_float(keys[i]) > thr;
-        out[i] = f ? 1 : 0;
-        cnt += f ? 1u : 0u;
-    }
-    for (int d = 16; d > 0; d >>= 1) cnt += __shfl_down_sync(0xffffffffu, cnt, d);
-    if ((threadIdx.x & 31) == 0 && cnt) atomicAdd(n_flagged, (unsigned long long)cnt);
-}
-
-// per-baseline mode: one block per group of rows (the rows of one baseline in either
-// orientation); two exact order statistics of its used samples by four 8-bit radix passes
-// with a shared-memory histogram, then its flags
-__device__ __forceinline__ unsigned mad_block_select(const unsigned *keys, const int *grows, int n_grow, int n_chan,
-                                                     const uint8_t *flag, unsigned long long k, unsigned *hist,
-                                                     unsigned *s_res)
-{
-    unsigned prefix = 0, mask = 0;
-    const long n = (long)n_grow * n_chan;
-    for (int shift = 24; shift >= 0; shift -= 8) {
-        for (int t = threadIdx.x; t < 256; t += blockDim.x) hist[t] = 0;
-        __syncthreads();
-        for (long i = threadIdx.x; i < n; i += blockDim.x) {
-            const long sidx = (long)grows[i / n_chan] * n_chan + (i % n_chan);
-            if (flag && flag[sidx]) continue;
-            const unsigned kk = keys[sidx];
-            if ((kk & mask) == prefix) atomicAdd(&hist[(kk >> shift) & 0xffu], 1u);
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            unsigned long long cum = 0;
-            int b = 0;
-            for (; b < 255; ++b) {
-                if (cum + hist[b] > k) break;
-                cum += hist[b];
-            }
-            s_res[0] = (unsigned)b;
-            s_res[1] = (unsigned)(k - cum);
-        }
-        __syncthreads();
-        prefix |= s_res[0] << shift;
-        mask |= 0xffu << shift;
-        k = s_res[1];
-        __syncthreads();
-    }
-    return prefix;
-}
-
-__global__ void __launch_bounds__(256) mad_group_kernel(int n_chan, const int *goff, const int *grows,
-                                                        const uint8_t *flag, unsigned *keys, float factor,
-                                                        uint8_t *out, unsigned long long *n_flagged)
-{
-    __shared__ unsigned hist[256];
-    __shared__ unsigned s_res[2];
-    __shared__ unsigned long long s_cnt;
-    const int g = blockIdx.x;
-    const int *rows = grows + goff[g];
-    const int n_grow = goff[g + 1] - goff[g];
-    const long n = (long)n_grow * n_chan;
-    if (threadIdx.x == 0) s_cnt = 0;
-    __syncthreads();
-    unsigned long long used = 0;
-    for (long i = threadIdx.x; i < n; i += blockDim.x) {
-        const long sidx = (long)rows[i / n_chan] * n_chan + (i % n_chan);
-        if (!(flag && flag[sidx])) ++used;
-    }
-    atomicAdd(&s_cnt, used);
-    __syncthreads();
-    const unsigned long long n_used = s_cnt;
-    float thr = INFINITY;
-    if (n_used > 0) {
-        const unsigned long long k = (n_used - 1) / 2;
-        const unsigned med_bits = mad_block_select(keys, rows, n_grow, n_chan, flag, k, hist, s_res);
-        const float med = __uint_as_float(med_bits);
-        for (long i = threadIdx.x; i < n; i += blockDim.x) {
-            const long sidx = (long)rows[i / n_chan] * n_chan + (i % n_chan);
-            if (!(flag && flag[sidx])) keys[sidx] = __float_as_uint(fabsf(__fsub_rn(__uint_as_float(keys[sidx]), med)));
-        }
-        __syncthreads();
-        const unsigned mad_bits = mad_block_select(keys, rows, n_grow, n_chan, flag, k, hist, s_res);
-        thr = __fmul_rn(factor, __uint_as_float(mad_bits));
-    }
-    unsigned cnt = 0;
-    for (long i = threadIdx.x; i < n; i += blockDim.x) {
-        const long sidx = (long)rows[i / n_chan] * n_chan + (i % n_chan);
-        const bool f = !(flag && flag[sidx]) && __uint_as_float(keys[sidx]) > thr;
-        out[sidx] = f ? 1 : 0;
-        cnt += f ? 1u : 0u;
-    }
-    for (int d = 16; d > 0; d >>= 1) cnt += __shfl_down_sync(0xffffffffu, cnt, d);
-    if ((threadIdx.x & 31) == 0 && cnt) atomicAdd(n_flagged, (unsigned long long)cnt);
-}
-
-} // namespace
-
-// the k-th smallest of n keys (0-based), k < n: four 8-bit radix passes from the top bits
-static int mad_select(qc_ctx *c, const unsigned *keys, long n, unsigned long long k, unsigned *hist, cudaStream_t st,
-                      unsigned &out)
-{
-    unsigned prefix = 0, mask = 0;
-    unsigned h[256];
-    for (int shift = 24; shift >= 0; shift -= 8) {
-        CK(cudaMemsetAsync(hist, 0, 256 * sizeof(unsigned), st));
-        mad_hist_kernel<<<grid_for(n, 256, c->sm_count), 256, 0, st>>>(n, keys, prefix, mask, shift, hist);
-        CK(cudaGetLastError());
-        CK(cudaMemcpyAsync(h, hist, sizeof h, cudaMemcpyDeviceToHost, st));
-        CK(cudaStreamSynchronize(st));
-        unsigned long long cum = 0;
-        int b = 0;
-        for (; b < 256; ++b) {
-            if (cum + h[b] > k) break;
-            cum += h[b];
-        }
-        if (b == 256) return c->fail(QC_ECUDA, "radix select lost its element");
-        k -= cum;
-        prefix |= (unsigned)b << shift;
-        mask |= 0xffu << shift;
-    }
-    out = prefix;
-    return QC_OK;
-}
+// |z - median| > fl32(threshold * 1.4826) * MAD in float32.  The whole sequence runs on the
+// stream (qc_residual.cu): the digits are picked on the device, so that nothing waits for the host.
 
 extern "C" int qc_mad_flag(qc_ctx *c, const qc_term *terms, int32_t n_terms, double threshold, int32_t per_baseline,
                            uint8_t *flags_out, int32_t out_memory, int64_t *n_flagged)
@@ -2196,15 +2019,10 @@ extern "C" int qc_mad_flag(qc_ctx *c, const qc_term *terms, int32_t n_terms, dou
     Chain chain;
     if ((rc = c->stage_terms(xt.data(), n_terms, st, chain))) return rc;
     const long n_vis = (long)c->n_row * c->n_chan;
-    if ((rc = c->ensure(c->scalars, 64))) return rc;
-    if ((rc = c->ensure(c->resid_stage, nbytes<float4>(2 * (size_t)std::max(1L, n_vis))))) return rc;
     if ((rc = c->ensure(c->mad_keys, nbytes<unsigned>((size_t)std::max(1L, n_vis))))) return rc;
-    if ((rc = c->ensure(c->mad_hist, 256 * sizeof(unsigned) + 2 * sizeof(unsigned long long)))) return rc;
-    double *d_chi2 = (double *)c->scalars.ptr;
-    float4 *dres = (float4 *)c->resid_stage.ptr;
+    if ((rc = c->ensure(c->mad_state, sizeof(MadState)))) return rc;
     unsigned *keys = (unsigned *)c->mad_keys.ptr;
-    unsigned *hist = (unsigned *)c->mad_hist.ptr;
-    unsigned long long *cnt = (unsigned long long *)((char *)c->mad_hist.ptr + 256 * sizeof(unsigned));
+    MadState *state = (MadState *)c->mad_state.ptr;
     uint8_t *dout = (uint8_t *)flags_out;
     if (out_memory == QC_MEM_HOST) {
         if ((rc = c->ensure(c->mad_out, (size_t)std::max(1L, n_vis)))) return rc;
@@ -2214,72 +2032,31 @@ extern "C" int qc_mad_flag(qc_ctx *c, const qc_term *terms, int32_t n_terms, dou
         if (n_flagged) *n_flagged = 0;
         return QC_OK;
     }
-    if ((rc = c->run_residual(chain, dres, d_chi2, st))) return rc;
-    CK(cudaMemsetAsync(cnt, 0, 2 * sizeof(unsigned long long), st));
-    const int grid = grid_for(n_vis, 256, c->sm_count);
-    mad_z_kernel<<<grid, 256, 0, st>>>(n_vis, c->n_chan, dres, c->d_weight, c->d_flag, c->d_rows, keys, cnt);
-    CK(cudaGetLastError());
-    unsigned long long hc[2];
-    CK(cudaMemcpyAsync(hc, cnt, sizeof hc, cudaMemcpyDeviceToHost, st));
-    CK(cudaStreamSynchronize(st));
+    const float factor = (float)(threshold * 1.4826);
+    CK(cudaMemsetAsync(state, 0, sizeof(MadState), st));
+    ResArgs ra;
+    ra.D = c->data_desc();
+    ra.C = chain;
+    ra.resid = nullptr;
+    ra.chi2 = nullptr;
+    CK(mad_keys_launch(ra, c->m16, keys, state, c->sm_count, st));
     if (per_baseline) {
-        // groups: the rows of each unordered antenna pair (cross-correlations only)
-        std::vector<int4> hrows(c->n_row);
-        CK(cudaMemcpyAsync(hrows.data(), c->d_rows, nbytes<int4>(c->n_row), cudaMemcpyDeviceToHost, st));
-        CK(cudaStreamSynchronize(st));
-        std::vector<int> gid((size_t)c->n_ant * c->n_ant, -1), count;
-        std::vector<int> row_g(c->n_row, -1);
-        for (int r = 0; r < c->n_row; ++r) {
-            const int a1 = hrows[r].x, a2 = hrows[r].y;
-            if (a1 == a2) continue;
-            int &slot = gid[(size_t)std::min(a1, a2) * c->n_ant + std::max(a1, a2)];
-            if (slot < 0) { slot = (int)count.size(); count.push_back(0); }
-            row_g[r] = slot;
-            ++count[slot];
+        if (!c->mad_groups.ptr && !c->pair_strips.empty()) {
+            // the strips of each unordered antenna pair, staged by the first call
+            if ((rc = c->ensure(c->mad_groups, nbytes<int2>(c->pair_strips.size())))) return rc;
+            CK(cudaMemcpyAsync(c->mad_groups.ptr, c->pair_strips.data(), nbytes<int2>(c->pair_strips.size()),
+                               cudaMemcpyHostToDevice, st));
         }
-        const int n_groups = (int)count.size();
-        std::vector<int> goff(n_groups + 1, 0), grows;
-        for (int gi = 0; gi < n_groups; ++gi) goff[gi + 1] = goff[gi] + count[gi];
-        grows.resize(goff[n_groups]);
-        std::vector<int> fill(goff.begin(), goff.end() - 1);
-        for (int r = 0; r < c->n_row; ++r) if (row_g[r] >= 0) grows[fill[row_g[r]]++] = r;
         CK(cudaMemsetAsync(dout, 0, (size_t)n_vis, st));
-        if (n_groups > 0) {
-            if ((rc = c->ensure(c->mad_groups, nbytes<int>(goff.size() + grows.size())))) return rc;
-            int *dgoff = (int *)c->mad_groups.ptr, *dgrows = dgoff + goff.size();
-            CK(cudaMemcpyAsync(dgoff, goff.data(), nbytes<int>(goff.size()), cudaMemcpyHostToDevice, st));
-            CK(cudaMemcpyAsync(dgrows, grows.data(), nbytes<int>(grows.size()), cudaMemcpyHostToDevice, st));
-            mad_group_kernel<<<n_groups, 256, 0, st>>>(c->n_chan, dgoff, dgrows, c->d_flag, keys,
-                                                      (float)(threshold * 1.4826), dout, cnt + 1);
-            CK(cudaGetLastError());
-        }
-        if (out_memory == QC_MEM_HOST) CK(cudaMemcpyAsync(flags_out, dout, (size_t)n_vis, cudaMemcpyDeviceToHost, st));
-        CK(cudaMemcpyAsync(hc + 1, cnt + 1, sizeof(unsigned long long), cudaMemcpyDeviceToHost, st));
-        CK(cudaStreamSynchronize(st));
-        if (n_flagged) *n_flagged = (int64_t)hc[1];
-        return QC_OK;
+        CK(mad_group_launch((int)c->pair_strips.size(), (const int2 *)c->mad_groups.ptr, c->d_strip_off, c->d_strip_rows,
+                            c->n_chan, keys, factor, state, dout, st));
+    } else {
+        CK(mad_global_launch(n_vis, keys, factor, state, dout, c->sm_count, st));
     }
-    float thr = 0.f;
-    if (hc[0] > 0) {
-        const unsigned long long k = (hc[0] - 1) / 2;
-        unsigned med_bits = 0, mad_bits = 0;
-        if ((rc = mad_select(c, keys, n_vis, k, hist, st, med_bits))) return rc;
-        float med;
-        memcpy(&med, &med_bits, sizeof med);
-        mad_dev_kernel<<<grid, 256, 0, st>>>(n_vis, c->n_chan, c->d_flag, c->d_rows, med, keys);
-        CK(cudaGetLastError());
-        if ((rc = mad_select(c, keys, n_vis, k, hist, st, mad_bits))) return rc;
-        float mad;
-        memcpy(&mad, &mad_bits, sizeof mad);
-        const float factor = (float)(threshold * 1.4826);
-        thr = factor * mad;
-    }
-    mad_flag_kernel<<<grid, 256, 0, st>>>(n_vis, c->n_chan, hc[0] > 0 ? c->d_flag : nullptr, c->d_rows, keys,
-                                         hc[0] > 0 ? thr : INFINITY, dout, cnt + 1);
-    CK(cudaGetLastError());
+    unsigned long long hc = 0;
     if (out_memory == QC_MEM_HOST) CK(cudaMemcpyAsync(flags_out, dout, (size_t)n_vis, cudaMemcpyDeviceToHost, st));
-    CK(cudaMemcpyAsync(hc + 1, cnt + 1, sizeof(unsigned long long), cudaMemcpyDeviceToHost, st));
+    CK(cudaMemcpyAsync(&hc, &state->n_flagged, sizeof hc, cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
-    if (n_flagged) *n_flagged = (int64_t)hc[1];
+    if (n_flagged) *n_flagged = (int64_t)hc;
     return QC_OK;
 }

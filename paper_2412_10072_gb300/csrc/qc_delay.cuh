@@ -106,7 +106,9 @@ struct DelayUpdArgs {
     // a term solved from products (qc_delay_sums.cu): the h sums [bins][n_ant][6], the same for every
     // iteration (else null: they are in acc); the channel table is then left to the end of the solve
     const double *hsum;
-    const float *omega;       // [n_chan] 2 pi nu - omega_ref (with hsum)
+    const float *omega;       // [n_chan] omega' = 2 pi nu - omega_ref (with hsum)
+    const double2 *om_sums;   // [n_fint] sum of omega', of omega'^2 over the interval's channels (with hsum)
+    float om_max;             // largest |omega'|
 };
 
 // One block per parameter interval (time interval x frequency interval), threads over antennas.
@@ -119,6 +121,26 @@ struct DelayUpdArgs {
 // one frequency gives the exactly proportional phase and delay columns of the oracle (a
 // singular block) rather than FP32 rounding; activity per interval.
 constexpr int KG_SUMS = 16;
+
+// Two real symmetric 2x2 systems [[a0, a1], [a1, a2]] (y0, y1) = (r0, r1) and [[c0, c1], [c1, c2]] (y2, y3) =
+// (r2, r3) under block_solve's tests over the whole block-diagonal matrix (zero trace, zero
+// determinant, reciprocal 1-norm condition number); returns 1 when singular.
+__device__ __forceinline__ int delay_solve_pair(double a0, double a1, double a2, double c0, double c1, double c2, double r0,
+                                                double r1, double r2, double r3, double (&y)[4])
+{
+    y[0] = y[1] = y[2] = y[3] = 0.0;
+    if (!(a0 + a2 + c0 + c2 > 0)) return 1;
+    const double da = a0 * a2 - a1 * a1, dc = c0 * c2 - c1 * c1;
+    if (!(fabs(da) > 0) || !(fabs(dc) > 0)) return 1;
+    const double ia = 1.0 / da, ic = 1.0 / dc;
+    const double na = fmax(fabs(a0), fabs(a2)) + fabs(a1), nc = fmax(fabs(c0), fabs(c2)) + fabs(c1);
+    if (!(1.0 / (fmax(na, nc) * fmax(na * fabs(ia), nc * fabs(ic))) >= 1e-12)) return 1;
+    y[0] = (a2 * r0 - a1 * r1) * ia;
+    y[1] = (a0 * r1 - a1 * r0) * ia;
+    y[2] = (c2 * r2 - c1 * r3) * ic;
+    y[3] = (c0 * r3 - c1 * r2) * ic;
+    return 0;
+}
 
 template <bool SUMS>
 static __global__ void __launch_bounds__(128) delay_update_kernel(const DelayUpdArgs u)
@@ -202,7 +224,17 @@ static __global__ void __launch_bounds__(128) delay_update_kernel(const DelayUpd
                 b[2 + i].x += 2.0 * ry * f[i];
             }
         }
-        const int singular = block_solve<4>(M, b, x);
+        int singular;
+        if (SUMS && u.hsum) {
+            // no coupling between X and Y: two real 2x2 solves (64 threads through the general 4x4
+            // complex elimination took 0.1 of the update's 0.13 ms)
+            double y[4];
+            singular = delay_solve_pair(M[0][0].x, M[0][1].x, M[1][1].x, M[2][2].x, M[2][3].x, M[3][3].x, b[0].x, b[1].x,
+                                        b[2].x, b[3].x, y);
+            for (int e = 0; e < 4; ++e) x[e] = make_double2(y[e], 0.0);
+        } else {
+            singular = block_solve<4>(M, b, x);
+        }
         if (!singular)
             for (int e = 0; e < 4; ++e) P[e] += u.alpha * x[e].x;
         if (u.gain_flags) u.gain_flags[(size_t)bin * d.n_ant + ant] = (int8_t)singular;
@@ -244,6 +276,24 @@ static __global__ void __launch_bounds__(128) delay_update_kernel(const DelayUpd
                 A[0] = A[1] = A[2] = A[3] = 0.0;
             }
             __syncthreads();
+            // phase changes below 1e-3 over the whole interval (all but the first iterations): 4 sin^2
+            // of half the change is its square to 1e-7, and the sum over the channels is closed
+            bool small = true;
+            if ((int)threadIdx.x < na) {
+                const float4 e = s_e[threadIdx.x];
+                const float wmax = u.om_max;
+                small = fabsf(e.x) + fabsf(e.y) * wmax < 1e-3f && fabsf(e.z) + fabsf(e.w) * wmax < 1e-3f;
+            }
+            if (__syncthreads_and(small)) {
+                if ((int)threadIdx.x < na) {
+                    const float4 e = s_e[threadIdx.x];
+                    const double2 m = u.om_sums[fu];
+                    const double x0 = e.x, x1 = e.y, y0 = e.z, y1 = e.w;
+                    num += x0 * x0 * nch + 2.0 * x0 * x1 * m.x + x1 * x1 * m.y;
+                    num += y0 * y0 * nch + 2.0 * y0 * y1 * m.x + y1 * y1 * m.y;
+                }
+                continue;
+            }
             for (int i = threadIdx.x; i < na * nch; i += blockDim.x) {
                 const int ant = i / nch, c = fr.x + (i - ant * nch);
                 const float4 e = s_e[ant];

@@ -1,15 +1,15 @@
 // qc_delay_sums.cu -- the solve of a delay term from products formed once (not in the paper).
 //
 // The gains of a delay term have unit modulus, so with the other term fixed and X = O_p M O_q^H (the
-// other term folded into the model, summed over the directions) the blocks of one sample are
+// other term folded into the model) the blocks of one sample are
 //   h_p,k = sum_j w_kj |X_kj|^2 |g_q,j|^2 = sum_j w_kj |X_kj|^2              (no gains in it), and
 //   Im(conj(g_p,k) JHr_p,k) = sum_j Im z_kj,   z_kj = conj(g_p,k) g_q,j w_kj conj(X_kj) D_kj
 // (the terms h |g_p|^2 are real), for antenna q h_q,j = sum_k w_kj |X_kj|^2 and -sum_k Im z_kj.  One pass
 // over the samples forms
 //   T[time interval][pair][channel]_kj = sum w_kj conj(X_kj) D_kj   (four complex FP32, 32 B), and
 //   H[interval][antenna] = sum h (1, omega', omega'^2) per correlation (FP64),
-// and every iteration reads T alone: 32 B a sample and about 45 instructions instead of 80 B (112 B
-// with two directions) and about 300.
+// and every iteration reads T alone: 32 B a sample and about 45 instructions instead of 80 B and
+// about 300.
 #include "qc_internal.h"
 
 #include <algorithm>
@@ -34,11 +34,11 @@ __device__ __forceinline__ void red_add_v4(float4 *p, float4 v)
 // inside each row or, with chunk_major, its rows inside one chunk), DEPTH - 1 steps ahead through a
 // cp.async ring.  A lane (one channel) keeps T of its slot until the time interval or chunk
 // changes and H until its parameter interval or the pair changes.  HBM-bound: it reads the samples once
-// and writes T (80 + 32 B a sample with one direction and one integration an interval).
-template <int OK, int ND, bool M16>
+// and writes T (80 + 32 B a sample with one integration an interval).
+template <int OK, bool M16>
 static __global__ void __launch_bounds__(128, 4) delay_sums_pass_kernel(const DelaySumsArgs a)
 {
-    constexpr int NM = M16 ? 1 : 2 * ND, V4 = 3 + NM, DEPTH = ND > 2 ? 3 : 4;
+    constexpr int V4 = M16 ? 4 : 5, DEPTH = 4;
     extern __shared__ float4 s_ring[];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     float4 *ring = s_ring + (size_t)wib * DEPTH * (V4 * 32 + 2);
@@ -49,6 +49,13 @@ static __global__ void __launch_bounds__(128, 4) delay_sums_pass_kernel(const De
     // issue cursor
     long unit = ((long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     int k0 = 0, k1 = 0, k = 0, ch = 0, ch0 = 0, ch1 = 0;
+    // the current row's entry, loaded a step before its copies are issued (their addresses depend on it)
+    int4 mr = make_int4(-1, 0, 0, 0);
+    float msc = 0.f;
+    auto load_row = [&]() {
+        mr = __ldg(a.mrows + k);
+        if constexpr (M16) msc = __ldg(a.mscale + k);
+    };
     auto unit_start = [&]() {
         for (; unit < n_units; unit += stride) {
             const int g = (int)(unit % groups);
@@ -63,6 +70,7 @@ static __global__ void __launch_bounds__(128, 4) delay_sums_pass_kernel(const De
         }
         k = k0;
         ch = ch0;
+        if (unit < n_units) load_row();
     };
     unit_start();
     int is = 0;
@@ -71,7 +79,6 @@ static __global__ void __launch_bounds__(128, 4) delay_sums_pass_kernel(const De
         if (++is == DEPTH) is = 0;
         int4 m0 = make_int4(-1, 0, 0, 0), m1 = make_int4(0, 0, 0, 0);
         if (unit < n_units) {
-            const int4 mr = __ldg(a.mrows + k);
             const int c = ch * 32 + lane;
             const bool rd = mr.x >= 0 && c < n_chan;
             const size_t s = rd ? (size_t)mr.x * n_chan + c : 0;
@@ -82,12 +89,12 @@ static __global__ void __launch_bounds__(128, 4) delay_sums_pass_kernel(const De
             if constexpr (M16) {
                 cp_async16(stage + 96 + lane, a.model16 + s, nb);
             } else {
-#pragma unroll
-                for (int i = 0; i < NM; ++i) cp_async16(stage + 96 + 32 * i + lane, a.model + NM * s + i, nb);
+                cp_async16(stage + 96 + lane, a.model + 2 * s, nb);
+                cp_async16(stage + 128 + lane, a.model + 2 * s + 1, nb);
             }
             m0 = make_int4(__ldg(a.t_map + mr.y), ch, mr.z, mr.w);
             if constexpr (OK != KIND_NONE) m1.x = __ldg(a.to.t_map + mr.y);
-            if constexpr (M16) m1.y = __float_as_int(__ldg(a.mscale + k));
+            if constexpr (M16) m1.y = __float_as_int(msc);
         }
         if (lane == 0) {
             reinterpret_cast<int4 *>(stage + V4 * 32)[0] = m0;
@@ -96,11 +103,14 @@ static __global__ void __launch_bounds__(128, 4) delay_sums_pass_kernel(const De
         cp_async_commit();
         if (unit < n_units) {
             bool done;
+            const int kp = k;
             if (a.chunk_major) done = ++k == k1;
             else { if (++ch == ch1) { ch = ch0; ++k; } done = k >= k1; }
             if (done) {
                 unit += stride;
                 unit_start();
+            } else if (k != kp) {
+                load_row();
             }
         }
     };
@@ -159,21 +169,15 @@ static __global__ void __launch_bounds__(128, 4) delay_sums_pass_kernel(const De
             const bool conj = m0.z < 0;     // the row is (q, p): D -> D^H, M -> M^H, w permuted
             const int p = pq & 0xffff, q = (int)((unsigned)pq >> 16);
             J2 X;
-#pragma unroll
-            for (int d = 0; d < ND; ++d) {
-                J2 M;
-                if constexpr (M16) M = load_model16(*reinterpret_cast<const uint4 *>(st + 96 + lane), __int_as_float(m1.y));
-                else M = j_from(st[96 + 64 * d + lane], st[128 + 64 * d + lane]);
-                if (conj) M = j_herm(M);
-                if constexpr (OK != KIND_NONE) {
-                    const int fo = __ldg(a.to.f_map + cc), no = a.n_ant * a.nd_o, od = a.nd_o > 1 ? d : 0;
-                    const J2 Op = fetch_k<OK>(a.to, no, m1.x, fo, p * a.nd_o + od);
-                    const J2 Oq = fetch_k<OK>(a.to, no, m1.x, fo, q * a.nd_o + od);
-                    if constexpr (OK == KIND_DIAG) M = j_muld(j_dmul(Op.a, Op.d, M), cconj(Oq.a), cconj(Oq.d));
-                    else M = j_mul_h(j_mul(Op, M), Oq);
-                }
-                if (d == 0) X = M;
-                else { X.a = cadd(X.a, M.a); X.b = cadd(X.b, M.b); X.c = cadd(X.c, M.c); X.d = cadd(X.d, M.d); }
+            if constexpr (M16) X = load_model16(*reinterpret_cast<const uint4 *>(st + 96 + lane), __int_as_float(m1.y));
+            else X = j_from(st[96 + lane], st[128 + lane]);
+            if (conj) X = j_herm(X);
+            if constexpr (OK != KIND_NONE) {
+                const int fo = __ldg(a.to.f_map + cc);
+                const J2 Op = fetch_k<OK>(a.to, a.n_ant, m1.x, fo, p);
+                const J2 Oq = fetch_k<OK>(a.to, a.n_ant, m1.x, fo, q);
+                if constexpr (OK == KIND_DIAG) X = j_muld(j_dmul(Op.a, Op.d, X), cconj(Oq.a), cconj(Oq.d));
+                else X = j_mul_h(j_mul(Op, X), Oq);
             }
             if (conj) {
                 D = j_herm(D);
@@ -318,32 +322,25 @@ static __global__ void __launch_bounds__(256, 2) delay_sums_iter_kernel(const De
 
 } // namespace qc
 
-template <int OK, int ND, bool M16>
+template <int OK, bool M16>
 static cudaError_t launch_dsum_pass(const qc::DelaySumsArgs &a, int sm_count, cudaStream_t st)
 {
-    constexpr int V4 = 3 + (M16 ? 1 : 2 * ND), DEPTH = ND > 2 ? 3 : 4;
+    constexpr int V4 = M16 ? 4 : 5, DEPTH = 4;
     const int smem = 4 * DEPTH * (V4 * 32 + 2) * (int)sizeof(float4);
-    const void *fn = (const void *)qc::delay_sums_pass_kernel<OK, ND, M16>;
+    const void *fn = (const void *)qc::delay_sums_pass_kernel<OK, M16>;
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     int occ = 0;
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, 128, smem);
     if (e != cudaSuccess) return e;
     const long units = (long)a.n_strips * a.n_rb * (a.chunk_major ? a.n_chunks : 1);
     const int grid = (int)std::max(1L, std::min((long)sm_count * std::max(1, occ), (units + 3) / 4));
-    qc::delay_sums_pass_kernel<OK, ND, M16><<<grid, 128, smem, st>>>(a);
+    qc::delay_sums_pass_kernel<OK, M16><<<grid, 128, smem, st>>>(a);
     return cudaGetLastError();
 }
 
 template <int OK> static cudaError_t launch_dsum_pass_ok(const qc::DelaySumsArgs &a, int sm_count, cudaStream_t st)
 {
-    if (a.model16) return launch_dsum_pass<OK, 1, true>(a, sm_count, st);
-    switch (a.n_dir) {
-    case 1: return launch_dsum_pass<OK, 1, false>(a, sm_count, st);
-    case 2: return launch_dsum_pass<OK, 2, false>(a, sm_count, st);
-    case 3: return launch_dsum_pass<OK, 3, false>(a, sm_count, st);
-    case 4: return launch_dsum_pass<OK, 4, false>(a, sm_count, st);
-    default: return cudaErrorInvalidValue;
-    }
+    return a.model16 ? launch_dsum_pass<OK, true>(a, sm_count, st) : launch_dsum_pass<OK, false>(a, sm_count, st);
 }
 
 cudaError_t dsum_launch_pass(const qc::DelaySumsArgs &a, int ok, int sm_count, cudaStream_t st)

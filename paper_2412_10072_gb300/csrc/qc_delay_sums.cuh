@@ -7,10 +7,9 @@
 namespace qc {
 
 constexpr int KG_HSUM = 6;           // FP64 words of the constant sums per (interval, antenna)
-constexpr int DSUM_MAX_DIR = 4;      // directions of the model (as the streaming kernel)
 
 struct DelaySumsArgs {
-    int n_chan, n_ant, n_up, n_dir, n_fint, n_chunks;
+    int n_chan, n_ant, n_up, n_fint, n_chunks;
     // pass
     const float4 *vis, *model, *wf;
     const uint4 *model16;            // FP16 model, or null
@@ -21,7 +20,6 @@ struct DelaySumsArgs {
     int chunk_major;
     const int *t_map;                // [n_time] time interval of the delay term
     DevTerm to;                      // the other term (a copy of anything when there is none)
-    int nd_o;                        // directions in its table
     int store;                       // every slot is written exactly once: plain stores, no zeroing
     const uint8_t *active;           // [bins], all set when the pass runs
     // both

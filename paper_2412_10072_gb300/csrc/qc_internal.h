@@ -14,6 +14,7 @@
 #include "qc_robust.cuh"
 #include "qc_moments.cuh"
 #include "qc_delay_sums.cuh"
+#include "qc_residual.cuh"
 
 // Every device allocation of the library goes through these two calls.  They count the
 // live allocations and honour the test hook of qc_test_fail_alloc (qc.h), so that tests can
@@ -105,6 +106,9 @@ struct TermBufs {
     Buf dfr;       // delay terms: int2 [n_fint] first and last channel of each interval
     Buf dnu;       // delay terms: double [n_chan] channel frequencies
     Buf domega;    // delay terms: float [n_chan] 2 pi nu - omega_ref
+    Buf dom_sums;  // delay terms: double2 [n_fint] sums of omega' and omega'^2 over the channels
+    std::vector<double2> hom_sums;
+    float om_max = 0;
     double omega_ref = 0;     // delay terms: 2 pi times the mean channel frequency
     std::vector<int2> hfr;    // host copy of dfr (its size is the term's n_fint)
     std::vector<int> hufmap;  // delay terms: host copy of the term's own f_map
@@ -199,9 +203,10 @@ struct qc_ctx {
     TermBufs tb[QC_MAX_TERMS];
     Buf scalars;                      // counters and chi^2 scratch
     Buf mad_keys;                     // MAD flagging: uint32 [n_vis] statistic keys
-    Buf mad_hist;                     // MAD flagging: uint32 [256] histogram + counters
+    Buf mad_state;                    // MAD flagging: the selection's state (MadState)
     Buf mad_out;                      // MAD flagging: uint8 [n_vis] flags (host output staging)
-    Buf mad_groups;                   // MAD flagging, per-baseline mode: group offsets, then rows
+    Buf mad_groups;                   // MAD flagging, per-baseline mode: pair_strips on the device
+    std::vector<int2> pair_strips;    // strips (one per orientation, -1: none) of each unordered pair
     Buf resid_stage;
     // terms solved from sums: the strip rows as the pass reads them (int4, then the FP16 scales)
     Buf mom_rows;

@@ -943,80 +943,6 @@ static __global__ void __launch_bounds__(128) update_kernel(const UpdArgs u)
 }
 
 // ---------------------------------------------------------------------------
-// residual and chi^2 (Eq. min): full chain, row tiles, FP64 block sums
-// ---------------------------------------------------------------------------
-
-struct ResArgs {
-    Data D;
-    Chain C;              // n = -1: product of all terms
-    float4 *resid;        // [n_row][n_chan] x 2, or nullptr
-    double *chi2;         // one double
-};
-
-template <bool M16>
-__global__ void __launch_bounds__(256) residual_kernel(const ResArgs a)
-{
-    const Data &D = a.D;
-    const Chain &C = a.C;
-    const int lane = threadIdx.x & 31;
-    const long warp = ((long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const long n_warps = ((long)gridDim.x * blockDim.x) >> 5;
-    const int n_chunks = (D.n_chan + 31) / 32;
-    double tot = 0.0;
-    for (long u = warp; u < (long)D.n_row * n_chunks; u += n_warps) {
-        const int row = (int)(u / n_chunks);
-        const int c = (int)(u % n_chunks) * 32 + lane;
-        if (c >= D.n_chan) continue;
-        const int4 meta = __ldg(D.rows + row);
-        const size_t s = (size_t)row * D.n_chan + c;
-        bool ok = meta.x != meta.y;
-        if (ok && D.flag) ok = __ldg(D.flag + s) == 0;
-        if (!ok) {
-            if (a.resid) { a.resid[2 * s] = make_float4(0, 0, 0, 0); a.resid[2 * s + 1] = make_float4(0, 0, 0, 0); }
-            continue;
-        }
-        J2 Cp = j_identity(), Cq = j_identity();
-        for (int j = 0; j < C.n_terms; ++j) {
-            const DevTerm &T = C.t[j];
-            const int tint = __ldg(T.t_map + meta.z), fint = __ldg(T.f_map + c);
-            Cp = j_mul(Cp, fetch_jones(T, C.n_ant, tint, fint, meta.x));
-            Cq = j_mul(Cq, fetch_jones(T, C.n_ant, tint, fint, meta.y));
-        }
-        J2 M;
-        if constexpr (M16) {
-            const uint4 h = __ldg(D.model16 + s);
-            const float sc = __ldg(D.bl_scale + meta.w);
-            M.a = cscale(h2f(*reinterpret_cast<const __half2 *>(&h.x)), sc);
-            M.b = cscale(h2f(*reinterpret_cast<const __half2 *>(&h.y)), sc);
-            M.c = cscale(h2f(*reinterpret_cast<const __half2 *>(&h.z)), sc);
-            M.d = cscale(h2f(*reinterpret_cast<const __half2 *>(&h.w)), sc);
-        } else {
-            M = j_from(__ldg(D.model + 2 * s), __ldg(D.model + 2 * s + 1));
-        }
-        const J2 V = j_mul_h(j_mul(Cp, M), Cq);
-        const J2 Dm = j_from(__ldg(D.vis + 2 * s), __ldg(D.vis + 2 * s + 1));
-        J2 r;
-        r.a = csub(Dm.a, V.a); r.b = csub(Dm.b, V.b); r.c = csub(Dm.c, V.c); r.d = csub(Dm.d, V.d);
-        const float4 w = __ldg(D.weight + s);
-        tot += (double)(w.x * cnorm2(r.a)) + (double)(w.y * cnorm2(r.b)) + (double)(w.z * cnorm2(r.c)) +
-               (double)(w.w * cnorm2(r.d));
-        if (a.resid) {
-            a.resid[2 * s] = make_float4(r.a.x, r.a.y, r.b.x, r.b.y);
-            a.resid[2 * s + 1] = make_float4(r.c.x, r.c.y, r.d.x, r.d.y);
-        }
-    }
-    for (int d = 16; d > 0; d >>= 1) tot += __shfl_down_sync(0xffffffffu, tot, d);
-    __shared__ double part[8];
-    if (lane == 0) part[threadIdx.x >> 5] = tot;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double t = 0;
-        for (int i = 0; i < (int)blockDim.x / 32; ++i) t += part[i];
-        atomicAdd(a.chi2, t);
-    }
-}
-
-// ---------------------------------------------------------------------------
 // per-bin sample counts of a term (for the throughput and byte accounting)
 // ---------------------------------------------------------------------------
 

@@ -109,26 +109,6 @@ __device__ __forceinline__ void mom_add_d(float (&acc)[MOM_D], const J2 &D, cons
 // S' += conj(M_ab) M_a'b' K, and T' += conj(M_ab) (L_p^H (w D) L_q)_ab.  Forming the E_kj and adding their
 // products one by one takes 390 instructions a sample, this 236, and each word of the sums is
 // rounded once or twice a sample instead of eight times.
-// Two directions, E_d the model of direction d with the fixed term folded in:
-// S_de,kj = sum w conj(E_d,kj) E_e,kj (de = 00, 11 real, 01), T_d,kj = sum w conj(E_d,kj) D_kj.
-__device__ __forceinline__ void mom_add_dd(float (&acc)[MOM_DD], const J2 &D, const J2 &X0, const J2 &X1, float4 w)
-{
-    const float2 x0[4] = { X0.a, X0.b, X0.c, X0.d }, x1[4] = { X1.a, X1.b, X1.c, X1.d };
-    const float2 d[4] = { D.a, D.b, D.c, D.d };
-    const float wv[4] = { w.x, w.y, w.z, w.w };
-#pragma unroll
-    for (int kj = 0; kj < 4; ++kj) {
-        acc[kj] = fmaf(wv[kj], cnorm2(x0[kj]), acc[kj]);
-        acc[4 + kj] = fmaf(wv[kj], cnorm2(x1[kj]), acc[4 + kj]);
-        const float2 z = cmulc(x1[kj], x0[kj]);
-        acc[8 + 2 * kj] = fmaf(wv[kj], z.x, acc[8 + 2 * kj]);
-        acc[9 + 2 * kj] = fmaf(wv[kj], z.y, acc[9 + 2 * kj]);
-        const float2 wd = cscale(d[kj], wv[kj]);
-        cacc_conj(acc[16 + 2 * kj], acc[17 + 2 * kj], x0[kj], wd);
-        cacc_conj(acc[24 + 2 * kj], acc[25 + 2 * kj], x1[kj], wd);
-    }
-}
-
 __device__ __forceinline__ void mom_add_e(float (&acc)[MOM_EW], const J2 &D, const J2 &M, const J2 &Lp,
                                           const J2 &Lq, float4 w)
 {
@@ -276,15 +256,14 @@ __device__ __forceinline__ J2 fac_jones(const float4 *o)
 // frequency intervals), the lanes' keys (32 ints) and one int4 of meta data.
 template <int FORM, int OK, bool M16> struct MomRing {
     static constexpr int NO = OK == KIND_FULL ? 2 : (OK == KIND_DIAG ? 1 : 0);
-    static constexpr int ND = FORM == FORM_DD ? 2 : 1;       // directions of the model
-    static constexpr int OFF_W = M16 ? 96 : 64 + 64 * ND;
+    static constexpr int OFF_W = M16 ? 96 : 128;
     static constexpr int OFF_OP = OFF_W + 32, OFF_OQ = OFF_OP + 32 * NO, OFF_KEY = OFF_OQ + 32 * NO;
     static constexpr int OFF_META = OFF_KEY + 8;
     static constexpr int STAGE = OFF_META + 1;               // float4 per stage
     // three CTAs of 4 warps per SM (the full form's 100 register sums fit 168 registers); ring
     // depth as the shared memory of three CTAs allows
     static constexpr int PER_SM = 3;
-    static constexpr int DEPTH = NO == 2 || ND == 2 ? 3 : (NO == 1 ? 4 : 6);
+    static constexpr int DEPTH = NO == 2 ? 3 : (NO == 1 ? 4 : 6);
     static constexpr size_t SMEM = (size_t)4 * DEPTH * STAGE * sizeof(float4);
     // A lane's sums over a long strip are FP32 sums of terms of one sign, whose rounding grows with
     // the number of terms and moves the fixed point of all antennas the same way.  The short slots keep
@@ -308,6 +287,18 @@ template <int FORM, int OK, bool M16> struct MomCursor {
     int n_groups;
     int k0, k1, ch0, ch1, k, ch;
     bool cm;
+    // the current row's entry, loaded when the cursor reaches it, a step before its copies are
+    // issued: the addresses of the copies depend on it, and a warp that waited for it in L2 then
+    // would wait once a step
+    int4 mr = make_int4(-1, 0, 0, 0);
+    float msc = 0.f;
+    const int *tmap_n, *tmap_o;           // time maps of the solved and the fixed term (shared memory)
+
+    __device__ __forceinline__ void load_row(const MomArgs &a)
+    {
+        mr = __ldg(a.mrows + k);
+        if constexpr (M16) msc = __ldg(a.mscale + k);
+    }
 
     __device__ __forceinline__ void bounds(const MomArgs &a)
     {
@@ -325,10 +316,13 @@ template <int FORM, int OK, bool M16> struct MomCursor {
         }
         k = k0;
         ch = ch0;
+        if (unit < n_units) load_row(a);
     }
 
-    __device__ __forceinline__ void start(const MomArgs &a, long first, long step)
+    __device__ __forceinline__ void start(const MomArgs &a, long first, long step, const int *tn, const int *to)
     {
+        tmap_n = tn;
+        tmap_o = to;
         n_groups = (a.n_chunks + a.group - 1) / a.group;
         n_units = (long)a.n_strips * a.n_rb * n_groups;
         stride = step;
@@ -340,11 +334,14 @@ template <int FORM, int OK, bool M16> struct MomCursor {
     __device__ __forceinline__ void advance(const MomArgs &a)
     {
         bool done;
+        const int kp = k;
         if (cm) { if (++k == k1) { k = k0; ++ch; } done = ch >= ch1; }
         else { if (++ch == ch1) { ch = ch0; ++k; } done = k >= k1; }
         if (done) {
             unit += stride;
             bounds(a);
+        } else if (k != kp) {
+            load_row(a);
         }
     }
 
@@ -352,7 +349,6 @@ template <int FORM, int OK, bool M16> struct MomCursor {
     {
         int meta = MOM_END;
         if (unit < n_units) {
-            const int4 mr = __ldg(a.mrows + k);
             const int c0 = ch * 32, c = c0 + lane;
             const bool in = c < a.n_chan;
             const bool rd = mr.x >= 0 && in;
@@ -364,13 +360,12 @@ template <int FORM, int OK, bool M16> struct MomCursor {
             if constexpr (M16) {
                 cp_async16(stage + 64 + lane, a.model16 + i, nb);
             } else {
-#pragma unroll
-                for (int v = 0; v < 2 * R::ND; ++v)
-                    cp_async16(stage + 64 + 32 * v + lane, a.model + 2 * R::ND * i + v, nb);
+                cp_async16(stage + 64 + lane, a.model + 2 * i, nb);
+                cp_async16(stage + 96 + lane, a.model + 2 * i + 1, nb);
             }
             cp_async16(stage + R::OFF_W + lane, a.wf + i, nb);
             if constexpr (R::NO > 0) {
-                const int ti = __ldg(a.to.t_map + mr.y);
+                const int ti = tmap_o[mr.y];
                 const int f_first = __ldg(a.to.f_map + c0);
                 const int f_last = __ldg(a.to.f_map + min(a.n_chan, c0 + 32) - 1);
                 const bool uni = f_first == f_last;       // f_map is non-decreasing
@@ -395,12 +390,12 @@ template <int FORM, int OK, bool M16> struct MomCursor {
                 }
             }
             reinterpret_cast<int *>(stage + R::OFF_KEY)[lane] =
-                in ? (__ldg(a.tn.t_map + mr.y) * a.tn.n_fint + __ldg(a.tn.f_map + c)) * a.n_up + (mr.z & 0x7fffffff)
+                in ? (tmap_n[mr.y] * a.tn.n_fint + __ldg(a.tn.f_map + c)) * a.n_up + (mr.z & 0x7fffffff)
                    : -1;
         }
         if (lane == 0) {
             reinterpret_cast<int *>(stage + R::OFF_META)[0] = meta;
-            if (M16 && unit < n_units) reinterpret_cast<float *>(stage + R::OFF_META)[1] = __ldg(a.mscale + k);
+            if (M16 && unit < n_units) reinterpret_cast<float *>(stage + R::OFF_META)[1] = msc;
         }
         cp_async_commit();
         if (unit < n_units) advance(a);
@@ -418,7 +413,7 @@ template <int FORM, int OK, bool M16>
 static __global__ void __launch_bounds__(128, MomRing<FORM, OK, M16>::PER_SM) mom_pass_kernel(const MomArgs a)
 {
     using R = MomRing<FORM, OK, M16>;
-    constexpr int NW = FORM == FORM_FULL ? MOM_FW : (FORM == FORM_E ? MOM_EW : (FORM == FORM_D ? MOM_D : MOM_DD));
+    constexpr int NW = FORM == FORM_FULL ? MOM_FW : (FORM == FORM_E ? MOM_EW : MOM_D);
     if (a.n_active && __ldg(a.n_active) == 0) return;
     extern __shared__ float4 mom_ring[];
     const int lane = threadIdx.x & 31;
@@ -436,8 +431,19 @@ static __global__ void __launch_bounds__(128, MomRing<FORM, OK, M16>::PER_SM) mo
             for (int v = 0; v < NW; ++v) { hi[v] += acc[v]; acc[v] = 0.f; }
         }
     };
+    const int *tmap_n = a.tn.t_map, *tmap_o = a.to.t_map;
+    if (a.stage_maps) {
+        int *s_map = reinterpret_cast<int *>(mom_ring + (size_t)4 * R::DEPTH * R::STAGE);
+        for (int i = threadIdx.x; i < a.n_time; i += blockDim.x) {
+            s_map[i] = __ldg(a.tn.t_map + i);
+            s_map[a.n_time + i] = __ldg(a.to.t_map + i);
+        }
+        __syncthreads();
+        tmap_n = s_map;
+        tmap_o = s_map + a.n_time;
+    }
     MomCursor<FORM, OK, M16> cur;
-    cur.start(a, ((long)blockIdx.x * blockDim.x + threadIdx.x) >> 5, ((long)gridDim.x * blockDim.x) >> 5);
+    cur.start(a, ((long)blockIdx.x * blockDim.x + threadIdx.x) >> 5, ((long)gridDim.x * blockDim.x) >> 5, tmap_n, tmap_o);
     int is = 0;
 #pragma unroll
     for (int d = 0; d < R::DEPTH - 1; ++d) {
@@ -459,22 +465,7 @@ static __global__ void __launch_bounds__(128, MomRing<FORM, OK, M16>::PER_SM) mo
                 w = make_float4(w.x, w.z, w.y, w.w);
             }
             const int oc = (meta & 4) ? 0 : lane * R::NO;
-            if constexpr (FORM == FORM_DD) {
-                J2 M1 = j_from(st[128 + lane], st[160 + lane]);
-                if (meta & 1) M1 = j_herm(M1);
-                if constexpr (OK == KIND_DIAG) {
-                    const float4 rp = st[R::OFF_OP + oc], rq = st[R::OFF_OQ + oc];
-                    const float2 p0 = make_float2(rp.x, rp.y), p1 = make_float2(rp.z, rp.w);
-                    const float2 q0 = make_float2(rq.x, -rq.y), q1 = make_float2(rq.z, -rq.w);
-                    M = j_muld(j_dmul(p0, p1, M), q0, q1);
-                    M1 = j_muld(j_dmul(p0, p1, M1), q0, q1);
-                } else if constexpr (OK == KIND_FULL) {
-                    const J2 rp = fac_jones<OK>(st + R::OFF_OP + oc), rq = fac_jones<OK>(st + R::OFF_OQ + oc);
-                    M = j_mul_h(j_mul(rp, M), rq);
-                    M1 = j_mul_h(j_mul(rp, M1), rq);
-                }
-                mom_add_dd(acc, D, M, M1, w);
-            } else if constexpr (FORM != FORM_E) {
+            if constexpr (FORM != FORM_E) {
                 if constexpr (OK == KIND_DIAG) {
                     const float4 rp = st[R::OFF_OP + oc], rq = st[R::OFF_OQ + oc];
                     M = j_muld(j_dmul(make_float2(rp.x, rp.y), make_float2(rp.z, rp.w), M),
@@ -830,146 +821,6 @@ static __global__ void __launch_bounds__(256, 2) mom_iterate_kernel(const MomIte
     }
 }
 
-// The same for a direction-dependent diagonal term over two directions (its gains are stored over
-// (antenna, direction) pairs).  With S_de and T_d of the pair (a, q) as antenna a sees them,
-//   h_d,k = sum_q sum_j |g_q,d,j|^2 S_dd,kj,  C_k = sum_q sum_j g_q,0,j conj(g_q,1,j) S_01,kj,
-//   b_d,k = sum_q sum_j g_q,d,j T_d,kj,
-//   JHr_0,k = b_0,k - h_0,k g_a,0,k - C_k g_a,1,k,  JHr_1,k = b_1,k - h_1,k g_a,1,k - conj(C_k) g_a,0,k,
-// and the block of (a, d) is diag(h_d,0, h_d,1): the blocks between directions are left out, as in
-// the iterations on the samples, but the residual holds every direction.
-static __global__ void __launch_bounds__(256, 2) mom_iterate_dd_kernel(const MomIterArgs a)
-{
-    constexpr int N = 16;     // h_00 h_01 h_10 h_11, C_0, C_1, b_00, b_01, b_10, b_11 (d, k)
-    extern __shared__ float4 s_mem[];
-    const MomNormArgs &A = a.n;
-    const int na = A.n_ant;
-    float4 *g32 = s_mem;                                             // [n_ant][2 directions] (g_XX, g_YY)
-    double *sums = reinterpret_cast<double *>(s_mem + (size_t)na * 2);   // [n_ant][N]
-    __shared__ double s_num[8], s_den[8];
-    __shared__ int s_done;
-    const int bin = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
-    const int tint = bin / A.n_fint, fint = bin - tint * A.n_fint;
-    const float *bin_sums = A.mom + (size_t)bin * A.n_up * MOM_DD;
-    auto tab_at = [&](int i) { return a.tab + ((size_t)tint * na * 2 + i) * A.n_fint + fint; };
-    for (int i = tid; i < na * 2; i += blockDim.x) g32[i] = *tab_at(i);
-    __syncthreads();
-    int k = 1;
-    for (;; ++k) {
-        for (int ant = warp; ant < na; ant += nw) {
-            float h[N];
-#pragma unroll
-            for (int i = 0; i < N; ++i) h[i] = 0.f;
-            for (int o = lane; o < na; o += 32) {
-                if (o == ant) continue;
-                const int up = __ldg(A.upair + (size_t)ant * na + o);
-                if (up < 0) continue;
-                const float4 *s = reinterpret_cast<const float4 *>(bin_sums + (size_t)up * MOM_DD);
-                const bool p_side = ant < o;
-                const float sg = p_side ? 1.f : -1.f;
-                const float4 g[2] = { g32[2 * o], g32[2 * o + 1] };
-                // entries (k, j) of the antenna's own view: (0,1) and (1,0) exchanged on the q side
-                auto entry = [&](const float4 &lo, const float4 &hi, float2 (&v)[4]) {
-                    v[0] = make_float2(lo.x, sg * lo.y);
-                    v[3] = make_float2(hi.z, sg * hi.w);
-                    v[1] = p_side ? make_float2(lo.z, lo.w) : make_float2(hi.x, -hi.y);
-                    v[2] = p_side ? make_float2(hi.x, hi.y) : make_float2(lo.z, -lo.w);
-                };
-#pragma unroll
-                for (int d = 0; d < 2; ++d) {
-                    const float4 sd = __ldg(s + d);
-                    const float n0 = fmaf(g[d].x, g[d].x, g[d].y * g[d].y), n1 = fmaf(g[d].z, g[d].z, g[d].w * g[d].w);
-                    h[2 * d] += fmaf(n0, sd.x, n1 * (p_side ? sd.y : sd.z));
-                    h[2 * d + 1] += fmaf(n0, p_side ? sd.z : sd.y, n1 * sd.w);
-                    float2 t[4];
-                    entry(__ldg(s + 4 + 2 * d), __ldg(s + 5 + 2 * d), t);
-                    const float2 g0 = make_float2(g[d].x, g[d].y), g1 = make_float2(g[d].z, g[d].w);
-#pragma unroll
-                    for (int r = 0; r < 2; ++r) {
-                        const float2 v = cdot(g0, t[2 * r], g1, t[2 * r + 1]);
-                        h[8 + 4 * d + 2 * r] += v.x;
-                        h[9 + 4 * d + 2 * r] += v.y;
-                    }
-                }
-                float2 c[4];
-                entry(__ldg(s + 2), __ldg(s + 3), c);
-                const float2 y0 = cmulc(make_float2(g[0].x, g[0].y), make_float2(g[1].x, g[1].y));
-                const float2 y1 = cmulc(make_float2(g[0].z, g[0].w), make_float2(g[1].z, g[1].w));
-#pragma unroll
-                for (int r = 0; r < 2; ++r) {
-                    const float2 v = cdot(y0, c[2 * r], y1, c[2 * r + 1]);
-                    h[4 + 2 * r] += v.x;
-                    h[5 + 2 * r] += v.y;
-                }
-            }
-            const double v = reduce_words<N>(h, lane);
-            if ((lane & 1) == 0) sums[(size_t)ant * N + lane / 2] = v;
-        }
-        __syncthreads();
-        const double alpha = a.alternate ? ((k % 2 == 0) ? 0.5 : 1.0) : a.damping;
-        // JHr in the place of b, from both directions' gains of the antenna (FP64 master) ...
-        for (int i = tid; i < na * 2; i += blockDim.x) {
-            const int ant = i >> 1, d = i & 1;
-            double *h = sums + (size_t)ant * N;
-            const double2 *P = reinterpret_cast<const double2 *>(a.params) + 4 * ((size_t)bin * na * 2 + i);
-            const double2 *O = reinterpret_cast<const double2 *>(a.params) + 4 * ((size_t)bin * na * 2 + (i ^ 1));
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                const double2 g = P[3 * e], o = O[3 * e];
-                const double cx = h[4 + 2 * e], cy = d ? -h[5 + 2 * e] : h[5 + 2 * e], hd = h[2 * d + e];
-                h[8 + 4 * d + 2 * e] -= hd * g.x + (cx * o.x - cy * o.y);
-                h[9 + 4 * d + 2 * e] -= hd * g.y + (cx * o.y + cy * o.x);
-            }
-        }
-        __syncthreads();
-        // ... then every (antenna, direction) steps
-        double num = 0, den = 0;
-        for (int i = tid; i < na * 2; i += blockDim.x) {
-            const int ant = i >> 1, d = i & 1;
-            const double *h = sums + (size_t)ant * N;
-            double2 *P = reinterpret_cast<double2 *>(a.params) + 4 * ((size_t)bin * na * 2 + i);
-            const double2 old[2] = { P[0], P[3] };
-            const double h00[1] = { h[2 * d] }, h11[1] = { h[2 * d + 1] };
-            const double2 z[1] = { make_double2(0, 0) };
-            const double2 r[2] = { make_double2(h[8 + 4 * d], h[9 + 4 * d]), make_double2(h[10 + 4 * d], h[11 + 4 * d]) };
-            double2 x[2], now[2];
-            const int singular = solve_blocks<1>(h00, h11, z, r, x);
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                now[e] = singular ? old[e] : make_double2(old[e].x + alpha * x[e].x, old[e].y + alpha * x[e].y);
-                const double dx = now[e].x - old[e].x, dy = now[e].y - old[e].y;
-                num += dx * dx + dy * dy;
-                den += now[e].x * now[e].x + now[e].y * now[e].y;
-            }
-            P[0] = now[0];
-            P[3] = now[1];
-            a.gain_flags[(size_t)bin * na * 2 + i] = (int8_t)singular;
-            g32[i] = make_float4((float)now[0].x, (float)now[0].y, (float)now[1].x, (float)now[1].y);
-        }
-        for (int d = 16; d > 0; d >>= 1) {
-            num += __shfl_down_sync(FULL_MASK, num, d);
-            den += __shfl_down_sync(FULL_MASK, den, d);
-        }
-        if (lane == 0) { s_num[warp] = num; s_den[warp] = den; }
-        __syncthreads();
-        if (tid == 0) {
-            double tn = 0, td = 0;
-            for (int i = 0; i < nw; ++i) { tn += s_num[i]; td += s_den[i]; }
-            const double delta = td > 0 ? sqrt(tn / td) : 0.0;
-            const bool conv = delta < a.tol;
-            if (!conv) atomicAdd(a.cnt + k, 1);
-            s_done = conv || k == a.max_iter;
-        }
-        __syncthreads();
-        if (s_done) break;
-    }
-    for (int i = tid; i < na * 2; i += blockDim.x) *tab_at(i) = g32[i];
-    if (tid == 0) {
-        a.iters[bin] = k;
-        atomicAdd(a.vis_iters, (unsigned long long)a.bin_nvis[bin] * k);
-        atomicAdd(a.acc_bytes, (unsigned long long)(a.bin_nbytes[bin] + a.iter_bytes * k));
-    }
-}
-
 // algorithmic bytes: the pass reads every sample of the bins once (their streaming bytes);
 // an iteration reads each bin's sums twice (once per side) and writes its accumulators
 static __global__ void mom_bytes_kernel(int n_bins, const long long *bin_nbytes, long long per_iter,
@@ -991,14 +842,18 @@ static cudaError_t launch_pass(const qc::MomArgs &a, int sm_count, cudaStream_t 
 {
     using R = qc::MomRing<FORM, OK, M16>;
     // the raised shared-memory limit belongs to the device's copy of the kernel: set on every launch
+    // time maps of up to 1024 integrations fit beside the rings of three CTAs
+    qc::MomArgs b = a;
+    b.stage_maps = a.n_time <= 1024;
+    const int smem = (int)R::SMEM + (b.stage_maps ? 2 * a.n_time * (int)sizeof(int) : 0);
     const cudaError_t e = cudaFuncSetAttribute(qc::mom_pass_kernel<FORM, OK, M16>,
-                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)R::SMEM);
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     const int block = 128;
     const int n_groups = (a.n_chunks + a.group - 1) / a.group;
     const long units = (long)a.n_strips * a.n_rb * n_groups;
     const int grid = (int)std::max(1L, std::min((long)sm_count * R::PER_SM, (units * 32 + block - 1) / block));
-    qc::mom_pass_kernel<FORM, OK, M16><<<grid, block, R::SMEM, st>>>(a);
+    qc::mom_pass_kernel<FORM, OK, M16><<<grid, block, smem, st>>>(b);
     return cudaGetLastError();
 }
 
@@ -1014,12 +869,6 @@ static cudaError_t launch_pass_any(const qc::MomArgs &a, int form, int ok, int s
         return launch_pass<FORM_FULL, KIND_FULL, M16>(a, sm_count, st);
     }
     if (form == FORM_E) return ok == KIND_FULL ? launch_pass<FORM_E, KIND_FULL, M16>(a, sm_count, st) : cudaErrorInvalidValue;
-    if constexpr (!M16)
-        if (form == FORM_DD) {
-            if (ok == KIND_NONE) return launch_pass<FORM_DD, KIND_NONE, false>(a, sm_count, st);
-            if (ok == KIND_DIAG) return launch_pass<FORM_DD, KIND_DIAG, false>(a, sm_count, st);
-            return launch_pass<FORM_DD, KIND_FULL, false>(a, sm_count, st);
-        }
     if (ok == KIND_NONE) return launch_pass<FORM_D, KIND_NONE, M16>(a, sm_count, st);
     if (ok == KIND_DIAG) return launch_pass<FORM_D, KIND_DIAG, M16>(a, sm_count, st);
     return launch_pass<FORM_D, KIND_FULL, M16>(a, sm_count, st);
@@ -1064,11 +913,6 @@ cudaError_t mom_launch_iterate(const qc::MomIterArgs &a, cudaStream_t st)
 {
     if (a.n.form == qc::FORM_FULL) return launch_iterate<qc::FORM_FULL>(a, st);
     if (a.n.form == qc::FORM_E) return launch_iterate<qc::FORM_E>(a, st);
-    if (a.n.form == qc::FORM_DD) {
-        const size_t smem = (size_t)a.n.n_ant * (2 * sizeof(float4) + 16 * sizeof(double));
-        qc::mom_iterate_dd_kernel<<<a.n.n_bins, 256, smem, st>>>(a);
-        return cudaGetLastError();
-    }
     return launch_iterate<qc::FORM_D>(a, st);
 }
 

@@ -16,12 +16,10 @@ constexpr int MOM_ET = 16, MOM_EU = 24;
 // plain diagonal form (a diagonal or phase-only solved term, the other term diagonal or to its
 // right): S 4, T 8
 constexpr int MOM_D = 12;
-// two directions, a direction-dependent diagonal solved term: S_00 4, S_11 4, S_01 8, T_0 8, T_1 8
-constexpr int MOM_DD = 32;
-constexpr int FORM_FULL = 0, FORM_E = 1, FORM_D = 2, FORM_DD = 3;
+constexpr int FORM_FULL = 0, FORM_E = 1, FORM_D = 2;
 __host__ __device__ constexpr int mom_words(int form)
 {
-    return form == FORM_FULL ? MOM_N : (form == FORM_E ? MOM_E : (form == FORM_D ? MOM_D : MOM_DD));
+    return form == FORM_FULL ? MOM_N : (form == FORM_E ? MOM_E : MOM_D);
 }
 
 // Hermitian pairs (u, v), u < v, of the 4x4 S blocks: packed as 4 diagonal reals then 6 (re, im)
@@ -42,6 +40,7 @@ struct MomArgs {
     int n_strips, n_chunks;              // n_chunks: 32-channel chunks of a row
     int group;                           // chunks per unit of work
     int rb, n_rb;                        // rows of a strip per unit of work, blocks per strip
+    int n_time, stage_maps;              // data times; time maps read from shared memory (set at the launch)
     int chunk_major;                     // 1: a unit's rows inside each chunk; 0: a row's chunks inside it
     DevTerm tn;                          // the solved term (maps)
     DevTerm to;                          // the fixed other term of a two-term chain (tables)
