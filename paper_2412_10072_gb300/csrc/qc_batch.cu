@@ -1031,8 +1031,7 @@ __global__ void __launch_bounds__(256) batch_iterate_kernel(const SumsArgs s)
         double num = 0, den = 0;
         for (int ant = tid; ant < na; ant += blockDim.x) {
             const double h0 = acc[ant * 6], h1 = acc[ant * 6 + 1];
-            const double hmax = fmax(h0, h1), hmin = fmin(h0, h1);
-            const bool singular = !(h0 + h1 > 0) || !(hmin / hmax >= 1e-12);
+            const bool singular = !(h0 + h1 > 0) || !(fmin(h0, h1) >= 1e-12 * fmax(h0, h1));
             double2 G0 = g64[2 * ant], G1 = g64[2 * ant + 1];
             double2 d0 = make_double2(0, 0), d1 = d0;
             if (!singular) {
@@ -1057,8 +1056,8 @@ __global__ void __launch_bounds__(256) batch_iterate_kernel(const SumsArgs s)
         if (tid == 0) {
             double tn = 0, td = 0;
             for (int i = 0; i < n_warps; ++i) { tn += red[0][i]; td += red[1][i]; }
-            const double delta = td > 0 ? sqrt(tn / td) : 0.0;
-            s_done = delta < a.tol ? 1 : 0;
+            // sqrt(tn / td) < tol without the root and the division; 0 where there are no gains
+            s_done = (td > 0 ? tn < a.tol * a.tol * td : 0.0 < a.tol) ? 1 : 0;
         }
         __syncthreads();
         if (s_done) break;

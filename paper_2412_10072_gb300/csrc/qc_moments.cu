@@ -668,8 +668,15 @@ static __global__ void __launch_bounds__(128) mom_normal_kernel(const MomNormArg
 
 // Solve the Hermitian 2x2 blocks [[h00, h01], [conj(h01), h11]] x = r of one antenna in FP64 with
 // block_solve's singularity tests over the whole block-diagonal matrix (zero trace, zero
-// determinant, reciprocal 1-norm condition number); returns 1 when singular.
-template <int NB>
+// determinant, 1-norm condition number above 1e12); returns 1 when singular.  FP64 runs at two
+// lanes a cycle and SM with long latencies, and this chain is most of an iteration on few antennas:
+// one division a block, the condition number tested without one, |h01| (for that test alone)
+// from an FP32 root where FP32 holds it.
+__device__ __forceinline__ double root_of(double v)
+{
+    return v > 1e-30 && v < 1e30 ? (double)sqrtf((float)v) : sqrt(v);
+}
+template <int NB, bool OFF>
 __device__ __forceinline__ int solve_blocks(const double (&h00)[NB], const double (&h11)[NB], const double2 (&h01)[NB],
                                             const double2 (&r)[2 * NB], double2 (&x)[2 * NB])
 {
@@ -679,20 +686,26 @@ __device__ __forceinline__ int solve_blocks(const double (&h00)[NB], const doubl
     if (!(trace > 0)) return 1;
 #pragma unroll
     for (int k = 0; k < NB; ++k) {
-        const double o2 = h01[k].x * h01[k].x + h01[k].y * h01[k].y;
+        const double o2 = OFF ? h01[k].x * h01[k].x + h01[k].y * h01[k].y : 0.0;
         const double det = h00[k] * h11[k] - o2;
         if (!(fabs(det) > 0)) return 1;
-        const double rd = 1.0 / det, o = sqrt(o2);
-        const double big = fmax(fabs(h00[k]), fabs(h11[k])) + o;
+        const double rd = 1.0 / det;
+        const double big = fmax(fabs(h00[k]), fabs(h11[k])) + (OFF ? root_of(o2) : 0.0);
         anorm = fmax(anorm, big);
         inorm = fmax(inorm, big * fabs(rd));
         const double2 r0 = r[2 * k], r1 = r[2 * k + 1], z = h01[k];
-        x[2 * k] = make_double2((h11[k] * r0.x - (z.x * r1.x - z.y * r1.y)) * rd,
-                                (h11[k] * r0.y - (z.x * r1.y + z.y * r1.x)) * rd);
-        x[2 * k + 1] = make_double2((h00[k] * r1.x - (z.x * r0.x + z.y * r0.y)) * rd,
-                                    (h00[k] * r1.y - (z.x * r0.y - z.y * r0.x)) * rd);
+        if constexpr (OFF) {
+            x[2 * k] = make_double2((h11[k] * r0.x - (z.x * r1.x - z.y * r1.y)) * rd,
+                                    (h11[k] * r0.y - (z.x * r1.y + z.y * r1.x)) * rd);
+            x[2 * k + 1] = make_double2((h00[k] * r1.x - (z.x * r0.x + z.y * r0.y)) * rd,
+                                        (h00[k] * r1.y - (z.x * r0.y - z.y * r0.x)) * rd);
+        } else {
+            const double a = h11[k] * rd, b = h00[k] * rd;
+            x[2 * k] = make_double2(a * r0.x, a * r0.y);
+            x[2 * k + 1] = make_double2(b * r1.x, b * r1.y);
+        }
     }
-    return !(1.0 / (anorm * inorm) >= 1e-12);
+    return !(anorm * inorm <= 1e12);
 }
 
 // Every iteration of one solution interval in one CTA: intervals are independent of each other once
@@ -709,6 +722,8 @@ static __global__ void __launch_bounds__(256, 2) mom_iterate_kernel(const MomIte
     const MomNormArgs &A = a.n;
     float4 *g32 = s_mem;                                                       // [n_ant][NF4]
     double *sums = reinterpret_cast<double *>(s_mem + (size_t)A.n_ant * NF4);  // [n_ant][N]
+    double2 *g64 = reinterpret_cast<double2 *>(sums + (size_t)A.n_ant * N);    // [n_ant][2 NB] the FP64 master
+    const bool phase = !GFULL && A.type == QC_TERM_PHASE;
     __shared__ double s_num[8], s_den[8];
     __shared__ int s_done;
     const int bin = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
@@ -716,6 +731,13 @@ static __global__ void __launch_bounds__(256, 2) mom_iterate_kernel(const MomIte
     const float *bin_sums = A.mom + (size_t)bin * A.n_up * mom_words(FORM);
     auto tab_at = [&](int i) { return a.tab + NF4 * (((size_t)tint * A.n_ant + i / NF4) * A.n_fint + fint) + i % NF4; };
     for (int i = tid; i < A.n_ant * NF4; i += blockDim.x) g32[i] = *tab_at(i);
+    // phase-only: (phi_X, phi_Y) in the first entry; diagonal: entries 0 and 3 of the four kept
+    const double2 *P0 = reinterpret_cast<const double2 *>(a.params) + (size_t)bin * A.n_ant * (phase ? 1 : 4);
+    for (int i = tid; i < A.n_ant * 2 * NB; i += blockDim.x) {
+        const int ant = i / (2 * NB), e = i % (2 * NB);
+        if (phase) { if (e == 0) g64[2 * ant] = P0[ant]; }
+        else g64[i] = P0[4 * ant + (GFULL ? e : 3 * e)];
+    }
     __syncthreads();
     int k = 1;
     for (;; ++k) {
@@ -726,22 +748,15 @@ static __global__ void __launch_bounds__(256, 2) mom_iterate_kernel(const MomIte
         double num = 0, den = 0;
         for (int ant = tid; ant < A.n_ant; ant += blockDim.x) {
             const double *h = sums + (size_t)ant * N;
-            const size_t pidx = (size_t)bin * A.n_ant + ant;
             double2 old[2 * NB], now[2 * NB], r[2 * NB], x[2 * NB], h01[NB];
             double h00[NB], h11[NB];
-            double phi0 = 0, phi1 = 0;
-            double2 *P = reinterpret_cast<double2 *>(a.params) + 4 * pidx;
-            if constexpr (GFULL) {
-#pragma unroll
-                for (int e = 0; e < 4; ++e) old[e] = P[e];
-            } else if (A.type == QC_TERM_PHASE) {
-                phi0 = a.params[2 * pidx];
-                phi1 = a.params[2 * pidx + 1];
-                sincos(phi0, &old[0].y, &old[0].x);
-                sincos(phi1, &old[1].y, &old[1].x);
+            double2 *G = g64 + (size_t)ant * 2 * NB;
+            if (phase) {
+                sincos(G[0].x, &old[0].y, &old[0].x);
+                sincos(G[0].y, &old[1].y, &old[1].x);
             } else {
-                old[0] = P[0];
-                old[1] = P[3];
+#pragma unroll
+                for (int e = 0; e < 2 * NB; ++e) old[e] = G[e];
             }
 #pragma unroll
             for (int b = 0; b < NB; ++b) {
@@ -756,7 +771,7 @@ static __global__ void __launch_bounds__(256, 2) mom_iterate_kernel(const MomIte
                                             w[7] - ((z.x * g0.y - z.y * g0.x) + h11[b] * g1.y));
             }
             int singular;
-            if (!GFULL && A.type == QC_TERM_PHASE) {
+            if (phase) {
                 // chain rule with dg/dphi = i g (Scenario 1): 2 Re(conj(g_u) g_v JHJ), 2 Im(conj(g_u) JHr)
                 const double2 g0 = old[0], g1 = old[1], z = h01[0];
                 const double2 c = make_double2(g0.x * g1.x + g0.y * g1.y, g0.x * g1.y - g0.y * g1.x);
@@ -765,26 +780,21 @@ static __global__ void __launch_bounds__(256, 2) mom_iterate_kernel(const MomIte
                 double2 mo[1] = { make_double2(2.0 * (c.x * z.x - c.y * z.y), 0.0) }, rb[2], xb[2];
                 rb[0] = make_double2(2.0 * (g0.x * r[0].y - g0.y * r[0].x), 0.0);
                 rb[1] = make_double2(2.0 * (g1.x * r[1].y - g1.y * r[1].x), 0.0);
-                singular = solve_blocks<1>(m0, m1, mo, rb, xb);
-                if (!singular) { phi0 += alpha * xb[0].x; phi1 += alpha * xb[1].x; }
-                a.params[2 * pidx] = phi0;
-                a.params[2 * pidx + 1] = phi1;
-                sincos(phi0, &now[0].y, &now[0].x);
-                sincos(phi1, &now[1].y, &now[1].x);
+                singular = solve_blocks<1, FORM != FORM_D>(m0, m1, mo, rb, xb);
+                double2 phi = G[0];
+                if (!singular) { phi.x += alpha * xb[0].x; phi.y += alpha * xb[1].x; }
+                G[0] = phi;
+                sincos(phi.x, &now[0].y, &now[0].x);
+                sincos(phi.y, &now[1].y, &now[1].x);
             } else {
-                singular = solve_blocks<NB>(h00, h11, h01, r, x);
+                singular = solve_blocks<NB, FORM != FORM_D>(h00, h11, h01, r, x);
 #pragma unroll
-                for (int e = 0; e < 2 * NB; ++e)
+                for (int e = 0; e < 2 * NB; ++e) {
                     now[e] = singular ? old[e] : make_double2(old[e].x + alpha * x[e].x, old[e].y + alpha * x[e].y);
-                if constexpr (GFULL) {
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) P[e] = now[e];
-                } else {
-                    P[0] = now[0];
-                    P[3] = now[1];
+                    G[e] = now[e];
                 }
             }
-            a.gain_flags[pidx] = (int8_t)singular;
+            a.gain_flags[(size_t)bin * A.n_ant + ant] = (int8_t)singular;
 #pragma unroll
             for (int f = 0; f < NF4; ++f)
                 g32[NF4 * ant + f] = make_float4((float)now[2 * f].x, (float)now[2 * f].y, (float)now[2 * f + 1].x,
@@ -805,8 +815,8 @@ static __global__ void __launch_bounds__(256, 2) mom_iterate_kernel(const MomIte
         if (tid == 0) {
             double tn = 0, td = 0;
             for (int i = 0; i < nw; ++i) { tn += s_num[i]; td += s_den[i]; }
-            const double delta = td > 0 ? sqrt(tn / td) : 0.0;
-            const bool conv = delta < a.tol;
+            // sqrt(tn / td) < tol without the root and the division; 0 where there are no gains
+            const bool conv = td > 0 ? tn < a.tol * a.tol * td : 0.0 < a.tol;
             if (!conv) atomicAdd(a.cnt + k, 1);                      // still active after iteration k
             s_done = conv || k == a.max_iter;
         }
@@ -814,6 +824,12 @@ static __global__ void __launch_bounds__(256, 2) mom_iterate_kernel(const MomIte
         if (s_done) break;
     }
     for (int i = tid; i < A.n_ant * NF4; i += blockDim.x) *tab_at(i) = g32[i];
+    double2 *P1 = reinterpret_cast<double2 *>(a.params) + (size_t)bin * A.n_ant * (phase ? 1 : 4);
+    for (int i = tid; i < A.n_ant * 2 * NB; i += blockDim.x) {
+        const int ant = i / (2 * NB), e = i % (2 * NB);
+        if (phase) { if (e == 0) P1[ant] = g64[2 * ant]; }
+        else P1[4 * ant + (GFULL ? e : 3 * e)] = g64[i];
+    }
     if (tid == 0) {
         a.iters[bin] = k;
         atomicAdd(a.vis_iters, (unsigned long long)a.bin_nvis[bin] * k);
@@ -904,7 +920,12 @@ template <int FORM> static cudaError_t launch_iterate(const qc::MomIterArgs &a, 
 {
     const int n_ant = a.n.n_ant;
     const int block = n_ant > 16 ? 256 : (n_ant > 8 ? 128 : 64);
-    const size_t smem = (size_t)n_ant * ((FORM == qc::FORM_FULL ? 2 : 1) * sizeof(float4) + qc::NormSums<FORM>::NWORD * sizeof(double));
+    constexpr int NB = FORM == qc::FORM_FULL ? 2 : 1;
+    const size_t smem = (size_t)n_ant * (NB * sizeof(float4) + qc::NormSums<FORM>::NWORD * sizeof(double) + 2 * NB * sizeof(double2));
+    if (smem > 48 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(qc::mom_iterate_kernel<FORM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+    }
     qc::mom_iterate_kernel<FORM><<<a.n.n_bins, block, smem, st>>>(a);
     return cudaGetLastError();
 }
