@@ -148,10 +148,66 @@ int grid_for(long n, int block, int sm)
 qc_ctx::~qc_ctx()
 {
     for (auto &b : tb) if (b.exec) cudaGraphExecDestroy(b.exec);
+    if (pin_open && pin_stream) cudaStreamSynchronize(pin_stream);
     for (void *p : owned) qc_dev_free(p);
+    for (auto &b : pin_blocks) cudaFreeHost(b.ptr);
     for (auto e : events) cudaEventDestroy(e);
     for (auto e : sums_events) cudaEventDestroy(e);
     if (own_stream) cudaStreamDestroy(own_stream);
+}
+
+cudaError_t qc_ctx::pin_begin(cudaStream_t st)
+{
+    cudaError_t e = cudaSuccess;
+    if (pin_open) e = cudaStreamSynchronize(pin_stream);
+    pin_block = pin_used = 0;
+    pin_outs.clear();
+    pin_open = true;
+    pin_stream = st;
+    return e;
+}
+
+void *qc_ctx::pin_get(size_t bytes)
+{
+    bytes = (bytes + 63) / 64 * 64;
+    for (; pin_block < pin_blocks.size(); ++pin_block, pin_used = 0)
+        if (pin_used + bytes <= pin_blocks[pin_block].bytes) {
+            void *p = pin_blocks[pin_block].ptr + pin_used;
+            pin_used += bytes;
+            return p;
+        }
+    const size_t size = std::max<size_t>(bytes, 256u << 10);
+    if (pin_total + size > PIN_MAX) return nullptr;
+    void *p = nullptr;
+    if (cudaHostAlloc(&p, size, cudaHostAllocDefault) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    pin_blocks.push_back({ (char *)p, size });
+    pin_total += size;
+    pin_used = bytes;
+    return p;
+}
+
+cudaError_t qc_ctx::to_device(void *dst, const void *src, size_t bytes, cudaStream_t st)
+{
+    void *p = pin_get(bytes);
+    if (p) memcpy(p, src, bytes);
+    return cudaMemcpyAsync(dst, p ? p : src, bytes, cudaMemcpyHostToDevice, st);
+}
+
+cudaError_t qc_ctx::to_host(void *dst, const void *src, size_t bytes, cudaStream_t st)
+{
+    void *p = pin_get(bytes);
+    if (p) pin_outs.push_back({ dst, p, bytes });
+    return cudaMemcpyAsync(p ? p : dst, src, bytes, cudaMemcpyDeviceToHost, st);
+}
+
+void qc_ctx::pin_end()
+{
+    for (const PinOut &o : pin_outs) memcpy(o.dst, o.src, o.bytes);
+    pin_outs.clear();
+    pin_open = false;
 }
 
 int qc_ctx::fail(int code, const std::string &msg)
@@ -540,14 +596,13 @@ int qc_ctx::expand_terms(const qc_term *terms, int n_terms, std::vector<qc_term>
             m.y += (double)om[ch] * om[ch];
         }
         if ((rc = ensure(B.dom_sums, nbytes<double2>(t.n_fint)))) return rc;
-        CK(cudaMemcpyAsync(B.dom_sums.ptr, B.hom_sums.data(), nbytes<double2>(t.n_fint), cudaMemcpyHostToDevice, st));
+        CK(to_device(B.dom_sums.ptr, B.hom_sums.data(), nbytes<double2>(t.n_fint), st));
         if (n_chan) {
-            CK(cudaMemcpyAsync(B.dfmap.ptr, t.f_map, nbytes<int>(n_chan), cudaMemcpyHostToDevice, st));
-            CK(cudaMemcpyAsync(B.dnu.ptr, t.chan_freq, nbytes<double>(n_chan), cudaMemcpyHostToDevice, st));
-            CK(cudaMemcpyAsync(B.domega.ptr, om.data(), nbytes<float>(n_chan), cudaMemcpyHostToDevice, st));
-            CK(cudaStreamSynchronize(st));      // om is a local staging vector
+            CK(to_device(B.dfmap.ptr, t.f_map, nbytes<int>(n_chan), st));
+            CK(to_device(B.dnu.ptr, t.chan_freq, nbytes<double>(n_chan), st));
+            CK(to_device(B.domega.ptr, om.data(), nbytes<float>(n_chan), st));
         }
-        CK(cudaMemcpyAsync(B.dfr.ptr, B.hfr.data(), nbytes<int2>(t.n_fint), cudaMemcpyHostToDevice, st));
+        CK(to_device(B.dfr.ptr, B.hfr.data(), nbytes<int2>(t.n_fint), st));
         xt[j].type = QC_TERM_DIAG;
         xt[j].n_fint = n_chan;
         xt[j].f_map = fid.data();
@@ -593,14 +648,14 @@ int qc_ctx::stage_terms(const qc_term *terms, int n_terms, cudaStream_t st, Chai
         if ((rc = ensure(B.stage, nent * (t.type == 2 ? 8 : 32)))) return rc;
         B.hmaps.assign(t.t_map, t.t_map + n_time);
         B.hmaps.insert(B.hmaps.end(), t.f_map, t.f_map + n_chan);
-        CK(cudaMemcpyAsync(B.maps.ptr, B.hmaps.data(), nbytes<int>(n_time + n_chan), cudaMemcpyHostToDevice, st));
+        CK(to_device(B.maps.ptr, B.hmaps.data(), nbytes<int>(n_time + n_chan), st));
         if (delay[j]) {
             // parameters [n_tint][n_fint][n_ant][4] (float32) -> FP64 master; table per channel
             const DelayArgs da = delay_args(j, t);
             const size_t nvals = (size_t)da.n_tint * da.n_fint * n_ant * 4;
             const void *src = t.gains;
             if (t.memory == QC_MEM_HOST) {
-                CK(cudaMemcpyAsync(B.stage.ptr, t.gains, nbytes<float>(nvals), cudaMemcpyHostToDevice, st));
+                CK(to_device(B.stage.ptr, t.gains, nbytes<float>(nvals), st));
                 src = B.stage.ptr;
             }
             delay_params_in_kernel<<<grid_for((long)nvals, 256, sm_count), 256, 0, st>>>((long)nvals, (const float *)src,
@@ -612,7 +667,7 @@ int qc_ctx::stage_terms(const qc_term *terms, int n_terms, cudaStream_t st, Chai
         } else {
             const void *src = t.gains;
             if (t.memory == QC_MEM_HOST) {
-                CK(cudaMemcpyAsync(B.stage.ptr, t.gains, nent * (t.type == 2 ? 8 : 32), cudaMemcpyHostToDevice, st));
+                CK(to_device(B.stage.ptr, t.gains, nent * (t.type == 2 ? 8 : 32), st));
                 src = B.stage.ptr;
             }
             gains_in_kernel<<<grid_for((long)nent, 256, sm_count), 256, 0, st>>>(t.type, t.n_tint, t.n_fint, term_nat(t), src,
@@ -663,6 +718,7 @@ extern "C" int qc_residual(qc_ctx *c, const qc_term *terms, int32_t n_terms, voi
     int rc = c->validate_terms(terms, n_terms, false);
     if (rc) return rc;
     cudaStream_t st = c->own_stream;
+    CK(c->pin_begin(st));
     std::vector<qc_term> xt;
     if ((rc = c->expand_terms(terms, n_terms, xt, st))) return rc;
     Chain chain;
@@ -679,10 +735,11 @@ extern "C" int qc_residual(qc_ctx *c, const qc_term *terms, int32_t n_terms, voi
         }
     }
     if ((rc = c->run_residual(chain, dres, d_chi2, st))) return rc;
-    CK(cudaMemcpyAsync(chi2, d_chi2, sizeof(double), cudaMemcpyDeviceToHost, st));
+    CK(c->to_host(chi2, d_chi2, sizeof(double), st));
     if (resid && resid_memory != QC_MEM_DEVICE)
         CK(cudaMemcpyAsync(resid, dres, nbytes<float4>(2 * n_vis), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
+    c->pin_end();
     return QC_OK;
 }
 
@@ -861,6 +918,7 @@ extern "C" int qc_solve(qc_ctx *c, qc_term *terms, int32_t n_terms, const qc_opt
     cudaEvent_t ev0, ev1;
     if ((rc = c->get_event(0, ev0)) || (rc = c->get_event(1, ev1))) return rc;
     CK(cudaEventRecord(ev0, st));
+    CK(c->pin_begin(st));
     std::vector<qc_term> xt;     // the kernels' view of the terms (delay terms per channel)
     if ((rc = c->expand_terms(terms, n_terms, xt, st))) return rc;
     Chain chain;
@@ -871,7 +929,7 @@ extern "C" int qc_solve(qc_ctx *c, qc_term *terms, int32_t n_terms, const qc_opt
     CK(cudaMemsetAsync(d_counters, 0, 2 * sizeof(unsigned long long), st));
     if (o->want_chi2) {
         if ((rc = c->run_residual(chain, nullptr, d_chi2, st))) return rc;
-        CK(cudaMemcpyAsync(&S.chi2_before, d_chi2, sizeof(double), cudaMemcpyDeviceToHost, st));
+        CK(c->to_host(&S.chi2_before, d_chi2, sizeof(double), st));
     }
 
     // per solved term: its route, bin counts and byte weights
@@ -977,6 +1035,8 @@ extern "C" int qc_solve(qc_ctx *c, qc_term *terms, int32_t n_terms, const qc_opt
                 if ((int)c->pending.size() == qc_ctx::MAX_PENDING) {
                     if ((rc = c->copy_pending(st))) return rc;
                     CK(cudaStreamSynchronize(st));
+                    c->pin_end();
+                    CK(c->pin_begin(st));
                     if ((rc = c->collect_sums(S, n_iter_max))) return rc;
                 }
                 continue;
@@ -1012,7 +1072,7 @@ extern "C" int qc_solve(qc_ctx *c, qc_term *terms, int32_t n_terms, const qc_opt
     }
     if (o->want_chi2) {
         if ((rc = c->run_residual(chain, nullptr, d_chi2, st))) return rc;
-        CK(cudaMemcpyAsync(&S.chi2_after, d_chi2, sizeof(double), cudaMemcpyDeviceToHost, st));
+        CK(c->to_host(&S.chi2_after, d_chi2, sizeof(double), st));
     }
     // write back solved gains, flags, iteration counts
     for (int j = 0; j < n_terms; ++j) {
@@ -1031,19 +1091,20 @@ extern "C" int qc_solve(qc_ctx *c, qc_term *terms, int32_t n_terms, const qc_opt
         CK(cudaGetLastError());
         ++c->launches;
         if (t.memory == QC_MEM_HOST) {
-            CK(cudaMemcpyAsync(t.gains, B.stage.ptr, gbytes, cudaMemcpyDeviceToHost, st));
-            if (t.gain_flags) CK(cudaMemcpyAsync(t.gain_flags, B.flags.ptr, nent, cudaMemcpyDeviceToHost, st));
-            if (t.iters) CK(cudaMemcpyAsync(t.iters, B.iters.ptr, nbytes<int>(nb), cudaMemcpyDeviceToHost, st));
+            CK(c->to_host(t.gains, B.stage.ptr, gbytes, st));
+            if (t.gain_flags) CK(c->to_host(t.gain_flags, B.flags.ptr, nent, st));
+            if (t.iters) CK(c->to_host(t.iters, B.iters.ptr, nbytes<int>(nb), st));
         } else {
             if (t.gain_flags) CK(cudaMemcpyAsync(t.gain_flags, B.flags.ptr, nent, cudaMemcpyDeviceToDevice, st));
             if (t.iters) CK(cudaMemcpyAsync(t.iters, B.iters.ptr, nbytes<int>(nb), cudaMemcpyDeviceToDevice, st));
         }
     }
     unsigned long long hc[2];
-    CK(cudaMemcpyAsync(hc, d_counters, sizeof hc, cudaMemcpyDeviceToHost, st));
+    CK(c->to_host(hc, d_counters, sizeof hc, st));
     if ((rc = c->copy_pending(st))) return rc;
     CK(cudaEventRecord(ev1, st));
     CK(cudaStreamSynchronize(st));
+    c->pin_end();
     if ((rc = c->collect_sums(S, n_iter_max))) return rc;
     float ms = 0;
     CK(cudaEventElapsedTime(&ms, ev0, ev1));
@@ -1320,7 +1381,13 @@ int qc_ctx::solve_term_sums(const qc_term *terms, int n_terms, int n, const Chai
         }
     }
     int *cnt = (int *)sums_cnt.ptr + P.off;
-    CK(cudaMemsetAsync(cnt, 0, nbytes<int>(t.max_iter + 1), st));
+    // one clearing for the solves of terms with equal max_iter
+    if (pending.empty()) sums_zeroed = 0;
+    if (sums_zeroed < (size_t)P.off + t.max_iter + 1) {
+        const size_t upto = std::max((size_t)P.off + t.max_iter + 1, pending.empty() ? need / sizeof(int) : 0);
+        CK(cudaMemsetAsync(cnt, 0, nbytes<int>(upto - P.off), st));
+        sums_zeroed = upto;
+    }
     CK(cudaMemsetAsync(B.mom.ptr, 0, nbytes<float>((size_t)P.n_bins * n_up * mom_words(B.sums.form)), st));
     CK(cudaEventRecord(ev[0], st));
     CK(mom_launch_pass(ma, B.sums.form, B.sums.ok, sm_count, st));
@@ -1353,7 +1420,7 @@ int qc_ctx::copy_pending(cudaStream_t st)
     if (pending.empty()) return QC_OK;
     const size_t n = (size_t)pending.back().off + pending.back().max_iter + 1;
     pending_cnt.resize(n);
-    CK(cudaMemcpyAsync(pending_cnt.data(), sums_cnt.ptr, nbytes<int>(n), cudaMemcpyDeviceToHost, st));
+    CK(to_host(pending_cnt.data(), sums_cnt.ptr, nbytes<int>(n), st));
     return QC_OK;
 }
 
@@ -2014,6 +2081,7 @@ extern "C" int qc_mad_flag(qc_ctx *c, const qc_term *terms, int32_t n_terms, dou
     int rc = c->validate_terms(terms, n_terms, false);
     if (rc) return rc;
     cudaStream_t st = c->own_stream;
+    CK(c->pin_begin(st));
     std::vector<qc_term> xt;
     if ((rc = c->expand_terms(terms, n_terms, xt, st))) return rc;
     Chain chain;
@@ -2055,8 +2123,9 @@ extern "C" int qc_mad_flag(qc_ctx *c, const qc_term *terms, int32_t n_terms, dou
     }
     unsigned long long hc = 0;
     if (out_memory == QC_MEM_HOST) CK(cudaMemcpyAsync(flags_out, dout, (size_t)n_vis, cudaMemcpyDeviceToHost, st));
-    CK(cudaMemcpyAsync(&hc, &state->n_flagged, sizeof hc, cudaMemcpyDeviceToHost, st));
+    CK(c->to_host(&hc, &state->n_flagged, sizeof hc, st));
     CK(cudaStreamSynchronize(st));
+    c->pin_end();
     if (n_flagged) *n_flagged = (int64_t)hc;
     return QC_OK;
 }

@@ -218,6 +218,24 @@ struct qc_ctx {
     std::vector<int> pending_cnt;
     std::vector<cudaEvent_t> sums_events;   // three per pending term solve
     Buf sums_cnt;                     // int: intervals still active after iteration k, per pending solve
+    size_t sums_zeroed = 0;           // ints of it zeroed for the solves now pending
+    // Pinned staging of one call's small copies: a copy from or to pageable memory holds the host
+    // until it is done, and a small solve makes about ten.  Blocks are kept for the context's life
+    // (at most PIN_MAX in all; larger copies go directly); a call ends synchronised, so the next one
+    // starts from the beginning.
+    static constexpr size_t PIN_MAX = 16u << 20;
+    struct PinBlock { char *ptr; size_t bytes; };
+    struct PinOut { void *dst; const void *src; size_t bytes; };
+    std::vector<PinBlock> pin_blocks;
+    size_t pin_block = 0, pin_used = 0, pin_total = 0;
+    bool pin_open = false;            // a call that did not reach its end left copies on pin_stream
+    cudaStream_t pin_stream = nullptr;
+    std::vector<PinOut> pin_outs;
+    cudaError_t pin_begin(cudaStream_t st);
+    void *pin_get(size_t bytes);
+    cudaError_t to_device(void *dst, const void *src, size_t bytes, cudaStream_t st);
+    cudaError_t to_host(void *dst, const void *src, size_t bytes, cudaStream_t st);   // valid after pin_end
+    void pin_end();                   // after the synchronisation: the staged results to the caller
     long long launches = 0;
     std::vector<const void *> configured_fns;   // kernels whose dynamic smem limit was raised
     std::string err;
