@@ -1198,10 +1198,15 @@ int qc_ctx::ensure_mom_rows(cudaStream_t st)
     qc_ctx *c = this;
     if (mom_rows_ready) return QC_OK;
     const size_t scale_off = nbytes<int4>(std::max(1L, n_strip_rows));
-    const int rc = ensure(mom_rows, scale_off + (m16 ? nbytes<float>(std::max(1L, n_strip_rows)) : 0));
+    const size_t bytes = scale_off + (m16 ? nbytes<float>(std::max(1L, n_strip_rows)) : 0);
+    int rc = ensure(mom_rows, bytes);
+    if (!rc) rc = ensure(mom_live, bytes);
+    if (!rc) rc = ensure(mom_end, nbytes<int>(std::max(1, n_strips)));
     if (rc) return rc;
+    auto scales = [&](const Buf &b) { return m16 ? (float *)((char *)b.ptr + scale_off) : nullptr; };
     CK(mom_launch_rows(n_strip_rows, d_strip_rows, d_rows, d_row_live, d_up_of_bl, d_bl_scale, (int4 *)mom_rows.ptr,
-                       m16 ? (float *)((char *)mom_rows.ptr + scale_off) : nullptr, st));
+                       scales(mom_rows), n_strips, d_strip_off, (int4 *)mom_live.ptr, scales(mom_live), (int *)mom_end.ptr,
+                       st));
     // built on this call's stream: finished before any later call can use it on another one
     CK(cudaStreamSynchronize(st));
     mom_rows_ready = true;
@@ -1302,9 +1307,22 @@ int qc_ctx::sums_args(const qc_term *terms, int n_terms, int n, const Chain &cha
     ma.model = d_model;
     ma.model16 = d_model16;
     ma.wf = d_wf;
-    ma.mrows = (const int4 *)mom_rows.ptr;
-    ma.mscale = m16 ? (const float *)((const char *)mom_rows.ptr + scale_off) : nullptr;
+    ma.mrows = (const int4 *)mom_live.ptr;
+    ma.mscale = m16 ? (const float *)((const char *)mom_live.ptr + scale_off) : nullptr;
     ma.strip_off = d_strip_off;
+    ma.strip_end = (const int *)mom_end.ptr;
+    auto map_kind = [&](const qc_term &x) {
+        if (x.n_fint == 1) return (int)MAP_ONE;
+        bool id = true, chunk = true;
+        for (int ch = 0; ch < n_chan; ++ch) {
+            id = id && x.f_map[ch] == ch;
+            chunk = chunk && x.f_map[ch] == x.f_map[ch / 32 * 32];
+        }
+        return (int)(id ? MAP_IDENTITY : (chunk ? MAP_CHUNK : MAP_ANY));
+    };
+    ma.tn_map = map_kind(t);
+    ma.to_map = n_terms == 2 ? map_kind(terms[1 - n]) : (int)MAP_ONE;
+    if (ma.to_map == MAP_ONE) ma.to_map = MAP_CHUNK;
     ma.n_strips = n_strips;
     ma.n_time = n_time;
     ma.n_chunks = (n_chan + 31) / 32;

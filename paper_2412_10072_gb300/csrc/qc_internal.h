@@ -50,7 +50,8 @@ cudaError_t mom_launch_normal(const qc::MomNormArgs &a, cudaStream_t st);
 cudaError_t mom_launch_bytes(int n_bins, const long long *bin_nbytes, long long per_iter, long long *iter_nbytes,
                              unsigned long long *acc_bytes, cudaStream_t st);
 cudaError_t mom_launch_rows(long n, const int *strip_rows, const int4 *rows, const uint8_t *row_live,
-                            const int *up_of_bl, const float *bl_scale, int4 *out, float *scale, cudaStream_t st);
+                            const int *up_of_bl, const float *bl_scale, int4 *out, float *scale, int n_strips,
+                            const int *strip_off, int4 *live, float *live_scale, int *strip_end, cudaStream_t st);
 cudaError_t mom_launch_iterate(const qc::MomIterArgs &a, cudaStream_t st);
 cudaError_t dd_launch_residual(const qc::DDArgs &a, int grid, cudaStream_t st);
 
@@ -210,6 +211,7 @@ struct qc_ctx {
     Buf resid_stage;
     // terms solved from sums: the strip rows as the pass reads them (int4, then the FP16 scales)
     Buf mom_rows;
+    Buf mom_live, mom_end;            // the same without the rows of no usable sample; strip ends
     bool mom_rows_ready = false;
     // term solves whose statistics are read back with the next synchronisation
     struct Pending { int off, max_iter, n_bins, ev; bool last_epoch, asked; };

@@ -165,37 +165,36 @@ __device__ __forceinline__ void mom_add_e(float (&acc)[MOM_EW], const J2 &D, con
 
 // Add the warp's register sums (NW words, the slot's order) to the sums of each lane's key
 // (-1: nothing) and zero them:
-//  - one key for the warp: a reduce-scatter (words padded to P = a power of two; after the
-//    halvings at lane offsets 16 .. 1 lane L holds words F L .. F L + F - 1, F = P / 32), then
-//    one atomic per word;
+//  - one key for the warp: a reduce-scatter of 32 words at a time (after the halvings at lane
+//    offsets 16 .. 1 lane L holds word L of the group), then one coalesced atomic per group;
 //  - 32 distinct keys: each lane adds its own words;
 //  - otherwise: a segmented reduction per word over the run of equal keys (channel intervals
 //    are contiguous, so a run is a range of lanes), added by the run's first lane.
 template <int NW>
 __device__ __forceinline__ void mom_flush(float (&acc)[NW], int key, int lane, float *mom, int stride)
 {
-    constexpr int P = NW <= 32 ? 32 : (NW <= 64 ? 64 : 128);
-    constexpr int F = P / 32;
+    constexpr int F = (NW + 31) / 32, P = 32;    // groups of 32 words, one exchange tree each
     const int k0 = __shfl_sync(FULL_MASK, key, 0);
     if (__all_sync(FULL_MASK, key == k0)) {
         if (k0 >= 0) {
-            // in place: after the halving at offset o the live words are acc[0 .. h)
+            // in place, group by group: after the halving at offset o the live words are [0 .. h)
+            float *dst = mom + (size_t)k0 * stride + lane;
 #pragma unroll
-            for (int h = P / 2, o = 16; o >= 1; h >>= 1, o >>= 1) {
-                const bool up = (lane & o) != 0;
+            for (int f = 0; f < F; ++f) {
 #pragma unroll
-                for (int i = 0; i < h; ++i) {
-                    const float lo = i < NW ? acc[i] : 0.f;
-                    const float hi = i + h < NW ? acc[i + h] : 0.f;
-                    const float send = up ? lo : hi;
-                    const float keep = up ? hi : lo;
-                    if (i < NW) acc[i] = keep + __shfl_xor_sync(FULL_MASK, send, o);
+                for (int h = P / 2, o = 16; o >= 1; h >>= 1, o >>= 1) {
+                    const bool up = (lane & o) != 0;
+#pragma unroll
+                    for (int i = 0; i < h; ++i) {
+                        const float lo = 32 * f + i < NW ? acc[32 * f + i] : 0.f;
+                        const float hi = 32 * f + i + h < NW ? acc[32 * f + i + h] : 0.f;
+                        const float send = up ? lo : hi;
+                        const float keep = up ? hi : lo;
+                        if (32 * f + i < NW) acc[32 * f + i] = keep + __shfl_xor_sync(FULL_MASK, send, o);
+                    }
                 }
+                if (32 * f + lane < NW) atomicAdd(dst + 32 * f, acc[32 * f]);
             }
-            float *dst = mom + (size_t)k0 * stride + F * lane;
-#pragma unroll
-            for (int j = 0; j < F; ++j)
-                if (F * lane + j < NW) atomicAdd(dst + j, acc[j]);
         }
     } else {
         const unsigned m = __match_any_sync(FULL_MASK, key);
@@ -241,6 +240,29 @@ static __global__ void mom_rows_kernel(long n, const int *strip_rows, const int4
     if (scale) scale[k] = bl_scale[r.w];
 }
 
+// The strips without their rows of no usable sample (one warp per strip): the entries kept, from the
+// strip's offset on, and where they end.
+static __global__ void mom_live_kernel(int n_strips, const int *strip_off, const int4 *rows, const float *scale, int4 *live,
+                                       float *live_scale, int *strip_end)
+{
+    const int s = (int)(((long)blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+    if (s >= n_strips) return;
+    const int k1 = strip_off[s + 1];
+    int at = strip_off[s];
+    for (int k0 = at; k0 < k1; k0 += 32) {
+        const int k = k0 + lane;
+        const int4 r = k < k1 ? rows[k] : make_int4(-1, 0, 0, 0);
+        const unsigned m = __ballot_sync(FULL_MASK, r.x >= 0);
+        if (r.x >= 0) {
+            const int to = at + __popc(m & ((1u << lane) - 1));
+            live[to] = r;
+            if (live_scale) live_scale[to] = scale[k];
+        }
+        at += __popc(m);
+    }
+    if (lane == 0) strip_end[s] = at;
+}
+
 template <int K>
 __device__ __forceinline__ J2 fac_jones(const float4 *o)
 {
@@ -279,25 +301,28 @@ constexpr int MOM_END = 2;       // meta: the warp's steps have run out (bit 0: 
 
 // The issuing side of a warp: its steps in order, unit by unit (grid stride; a unit is a block
 // of rb rows of one baseline strip x a group of chunks), each copied into a ring stage by
-// cp.async (zero-filled past the last channel and for rows without usable data, whose weights
-// then read 0).
+// cp.async (zero-filled past the last channel).  Rows without usable data are not in the table.  What
+// belongs to a row is computed once a row: row-major units take all chunks of it one after the
+// other, and the bookkeeping of a step was as long as its arithmetic.
 template <int FORM, int OK, bool M16> struct MomCursor {
     using R = MomRing<FORM, OK, M16>;
     long unit, n_units, stride;
     int n_groups;
     int k0, k1, ch0, ch1, k, ch;
     bool cm;
-    // the current row's entry, loaded when the cursor reaches it, a step before its copies are
-    // issued: the addresses of the copies depend on it, and a warp that waited for it in L2 then
-    // would wait once a step
+    // the next row's entry, loaded when the cursor reaches the row (a step before its first use)
     int4 mr = make_int4(-1, 0, 0, 0);
     float msc = 0.f;
+    bool fresh = false;                   // mr has not been turned into the values below
+    size_t base = 0;                      // first sample of the row
+    int key0 = 0, tab_p = 0, tab_q = 0, meta = 0;   // key, table entries (first interval), conjugate flag
     const int *tmap_n, *tmap_o;           // time maps of the solved and the fixed term (shared memory)
 
     __device__ __forceinline__ void load_row(const MomArgs &a)
     {
         mr = __ldg(a.mrows + k);
         if constexpr (M16) msc = __ldg(a.mscale + k);
+        fresh = true;
     }
 
     __device__ __forceinline__ void bounds(const MomArgs &a)
@@ -311,7 +336,7 @@ template <int FORM, int OK, bool M16> struct MomCursor {
             ch1 = min(a.n_chunks, ch0 + a.group);
             const int kb = __ldg(a.strip_off + s);
             k0 = kb + b * a.rb;
-            k1 = min(__ldg(a.strip_off + s + 1), k0 + a.rb);
+            k1 = min(__ldg(a.strip_end + s), k0 + a.rb);
             if (k0 < k1) break;
         }
         k = k0;
@@ -333,72 +358,86 @@ template <int FORM, int OK, bool M16> struct MomCursor {
 
     __device__ __forceinline__ void advance(const MomArgs &a)
     {
-        bool done;
-        const int kp = k;
-        if (cm) { if (++k == k1) { k = k0; ++ch; } done = ch >= ch1; }
-        else { if (++ch == ch1) { ch = ch0; ++k; } done = k >= k1; }
-        if (done) {
-            unit += stride;
-            bounds(a);
-        } else if (k != kp) {
-            load_row(a);
+        if (cm) {
+            // chunk-major units hold one chunk
+            if (++k < k1) { load_row(a); return; }
+        } else {
+            if (++ch < ch1) return;
+            ch = ch0;
+            if (++k < k1) { load_row(a); return; }
         }
+        unit += stride;
+        bounds(a);
     }
 
     __device__ __forceinline__ void issue(const MomArgs &a, int lane, float4 *stage)
     {
-        int meta = MOM_END;
-        if (unit < n_units) {
-            const int c0 = ch * 32, c = c0 + lane;
-            const bool in = c < a.n_chan;
-            const bool rd = mr.x >= 0 && in;
+        if (unit >= n_units) {
+            if (lane == 0) reinterpret_cast<int *>(stage + R::OFF_META)[0] = MOM_END;
+            cp_async_commit();
+            return;
+        }
+        if (fresh) {
+            fresh = false;
+            base = (size_t)mr.x * a.n_chan;
+            key0 = tmap_n[mr.y] * a.tn.n_fint * a.n_up + (mr.z & 0x7fffffff);
             meta = mr.z < 0 ? 1 : 0;
-            const size_t i = rd ? (size_t)mr.x * a.n_chan + c : 0;
-            const uint32_t nb = rd ? 16u : 0u;
-            cp_async16(stage + lane, a.vis + 2 * i, nb);
-            cp_async16(stage + 32 + lane, a.vis + 2 * i + 1, nb);
-            if constexpr (M16) {
-                cp_async16(stage + 64 + lane, a.model16 + i, nb);
-            } else {
-                cp_async16(stage + 64 + lane, a.model + 2 * i, nb);
-                cp_async16(stage + 96 + lane, a.model + 2 * i + 1, nb);
-            }
-            cp_async16(stage + R::OFF_W + lane, a.wf + i, nb);
             if constexpr (R::NO > 0) {
-                const int ti = tmap_o[mr.y];
-                const int f_first = __ldg(a.to.f_map + c0);
-                const int f_last = __ldg(a.to.f_map + min(a.n_chan, c0 + 32) - 1);
-                const bool uni = f_first == f_last;       // f_map is non-decreasing
-                if (uni) meta |= 4;
-                const int pa = mr.w & 0xffff, qa = mr.w >> 16;
-                if (uni) {
-                    if (lane < 2 * R::NO) {
-                        const int side = lane / R::NO, part = lane % R::NO;
-                        const size_t idx = ((size_t)ti * a.n_ant + (side ? qa : pa)) * a.to.n_fint + f_first;
-                        cp_async16(stage + (side ? R::OFF_OQ : R::OFF_OP) + part, a.to.tab + R::NO * idx + part,
-                                   mr.x >= 0 ? 16u : 0u);
-                    }
-                } else {
-                    const int fi = in ? __ldg(a.to.f_map + c) : 0;
-                    const size_t ip = ((size_t)ti * a.n_ant + pa) * a.to.n_fint + fi;
-                    const size_t iq = ((size_t)ti * a.n_ant + qa) * a.to.n_fint + fi;
+                const int t = tmap_o[mr.y] * a.n_ant;
+                tab_p = (t + (mr.w & 0xffff)) * a.to.n_fint;
+                tab_q = (t + (mr.w >> 16)) * a.to.n_fint;
+            }
+        }
+        const int c = ch * 32 + lane;
+        const bool in = c < a.n_chan;
+        const size_t i = in ? base + c : 0;
+        const uint32_t nb = in ? 16u : 0u;
+        cp_async16(stage + lane, a.vis + 2 * i, nb);
+        cp_async16(stage + 32 + lane, a.vis + 2 * i + 1, nb);
+        if constexpr (M16) {
+            cp_async16(stage + 64 + lane, a.model16 + i, nb);
+        } else {
+            cp_async16(stage + 64 + lane, a.model + 2 * i, nb);
+            cp_async16(stage + 96 + lane, a.model + 2 * i + 1, nb);
+        }
+        cp_async16(stage + R::OFF_W + lane, a.wf + i, nb);
+        int flags = meta;
+        if constexpr (R::NO > 0) {
+            // the fixed term's entries: one per chunk where the chunk lies in one of its frequency intervals
+            int fi;
+            bool uni;
+            if (a.to_map == MAP_IDENTITY) {
+                fi = in ? c : 0;
+                uni = false;
+            } else {
+                fi = __ldg(a.to.f_map + (a.to_map == MAP_CHUNK ? ch * 32 : min(c, a.n_chan - 1)));
+                uni = a.to_map == MAP_CHUNK || __all_sync(FULL_MASK, fi == __shfl_sync(FULL_MASK, fi, 0));
+            }
+            if (uni) {
+                flags |= 4;
+                if (lane < 2 * R::NO) {
+                    const int side = lane / R::NO, part = lane % R::NO;
+                    cp_async16(stage + (side ? R::OFF_OQ : R::OFF_OP) + part,
+                               a.to.tab + (size_t)R::NO * ((side ? tab_q : tab_p) + fi) + part, 16u);
+                }
+            } else {
 #pragma unroll
-                    for (int part = 0; part < R::NO; ++part) {
-                        cp_async16(stage + R::OFF_OP + R::NO * lane + part, a.to.tab + R::NO * ip + part, nb);
-                        cp_async16(stage + R::OFF_OQ + R::NO * lane + part, a.to.tab + R::NO * iq + part, nb);
-                    }
+                for (int part = 0; part < R::NO; ++part) {
+                    cp_async16(stage + R::OFF_OP + R::NO * lane + part, a.to.tab + (size_t)R::NO * (tab_p + fi) + part, nb);
+                    cp_async16(stage + R::OFF_OQ + R::NO * lane + part, a.to.tab + (size_t)R::NO * (tab_q + fi) + part, nb);
                 }
             }
-            reinterpret_cast<int *>(stage + R::OFF_KEY)[lane] =
-                in ? (tmap_n[mr.y] * a.tn.n_fint + __ldg(a.tn.f_map + c)) * a.n_up + (mr.z & 0x7fffffff)
-                   : -1;
         }
+        int key = key0;
+        if (a.tn_map == MAP_IDENTITY) key += c * a.n_up;
+        else if (a.tn_map != MAP_ONE) key += __ldg(a.tn.f_map + min(c, a.n_chan - 1)) * a.n_up;
+        reinterpret_cast<int *>(stage + R::OFF_KEY)[lane] = in ? key : -1;
         if (lane == 0) {
-            reinterpret_cast<int *>(stage + R::OFF_META)[0] = meta;
-            if (M16 && unit < n_units) reinterpret_cast<float *>(stage + R::OFF_META)[1] = msc;
+            reinterpret_cast<int *>(stage + R::OFF_META)[0] = flags;
+            if constexpr (M16) reinterpret_cast<float *>(stage + R::OFF_META)[1] = msc;
         }
         cp_async_commit();
-        if (unit < n_units) advance(a);
+        advance(a);
     }
 };
 
@@ -452,7 +491,8 @@ static __global__ void __launch_bounds__(128, MomRing<FORM, OK, M16>::PER_SM) mo
     }
     auto add = [&](const float4 *st, int meta) {
         float4 w = st[R::OFF_W + lane];
-        if (w.x != 0.f || w.y != 0.f || w.z != 0.f || w.w != 0.f) {
+        // any weight other than +-0
+        if ((__float_as_uint(w.x) | __float_as_uint(w.y) | __float_as_uint(w.z) | __float_as_uint(w.w)) & 0x7fffffffu) {
             J2 D = j_from(st[lane], st[32 + lane]), M;
             if constexpr (M16)
                 M = load_model16(*reinterpret_cast<const uint4 *>(st + 64 + lane),
@@ -938,11 +978,13 @@ cudaError_t mom_launch_iterate(const qc::MomIterArgs &a, cudaStream_t st)
 }
 
 cudaError_t mom_launch_rows(long n, const int *strip_rows, const int4 *rows, const uint8_t *row_live,
-                            const int *up_of_bl, const float *bl_scale, int4 *out, float *scale, cudaStream_t st)
+                            const int *up_of_bl, const float *bl_scale, int4 *out, float *scale, int n_strips,
+                            const int *strip_off, int4 *live, float *live_scale, int *strip_end, cudaStream_t st)
 {
     if (n == 0) return cudaSuccess;
     qc::mom_rows_kernel<<<(int)((n + 255) / 256), 256, 0, st>>>(n, strip_rows, rows, row_live, up_of_bl, bl_scale, out,
                                                                scale);
+    qc::mom_live_kernel<<<(n_strips + 7) / 8, 256, 0, st>>>(n_strips, strip_off, out, scale, live, live_scale, strip_end);
     return cudaGetLastError();
 }
 

@@ -28,15 +28,20 @@ __host__ __device__ constexpr int mom_pair(int u, int v)
     return u == 0 ? (v == 1 ? 0 : v == 2 ? 1 : 2) : u == 1 ? (v == 2 ? 3 : 4) : 5;
 }
 
+// what is known of a channel map: nothing, one interval, one interval per channel, or each 32-channel
+// chunk in one interval
+enum { MAP_ANY = 0, MAP_ONE = 1, MAP_IDENTITY = 2, MAP_CHUNK = 3 };
+
 struct MomArgs {
     int n_chan, n_ant, n_up;             // n_up: unordered antenna pairs with data
     const float4 *vis, *model, *wf;      // wf: weights with flags and autocorrelations folded in (w = 0)
     const uint4 *model16;                // FP16 model, or null
     const float *mscale;                 // [strip rows] its scale, or null
-    // [strip rows] {row or -1 (nothing usable), time, pair | conj << 31, p | q << 16}: p, q the
+    // [strip rows] {row, time, pair | conj << 31, p | q << 16}, rows with usable samples: p, q the
     // antennas of the baseline as oriented in the sums (p < q); conj: the row is (q, p)
     const int4 *mrows;
-    const int *strip_off;                // rows of each ordered baseline (offsets into mrows)
+    const int *strip_off, *strip_end;    // first and past-the-last row of each ordered baseline in mrows
+    int tn_map, to_map;                  // MAP_* of the channel maps of the solved and the fixed term
     int n_strips, n_chunks;              // n_chunks: 32-channel chunks of a row
     int group;                           // chunks per unit of work
     int rb, n_rb;                        // rows of a strip per unit of work, blocks per strip
