@@ -981,7 +981,11 @@ extern "C" int qc_solve(qc_ctx *c, qc_term *terms, int32_t n_terms, const qc_opt
         ca.nvis = nvis;
         ca.nunflag = nvis + nb;
         if (c->n_row) {
-            count_kernel<<<grid_for((long)c->n_row * 32, 256, c->sm_count), 256, 0, st>>>(ca);
+            // about 64 warps an SM, up to 128 rows each (small data: one row a warp)
+            const long cells = (long)c->n_row * ((c->n_chan + 31) / 32);
+            ca.rb = (int)std::min(128L, std::max(1L, cells / (64L * c->sm_count)));
+            const long units = ((c->n_row + ca.rb - 1) / ca.rb) * (long)((c->n_chan + 31) / 32);
+            count_kernel<<<grid_for(units * 32, 256, c->sm_count), 256, 0, st>>>(ca);
             CK(cudaGetLastError());
             ++c->launches;
         }
@@ -1178,7 +1182,9 @@ int qc_ctx::plan_sums(const qc_term *terms, int n_terms, int n, const qc_opts *o
     }
     const size_t sums_bytes = ((nbytes<float>(slots * mom_words(form)) + 15) / 16) * 16;
     int rc;
-    if ((rc = ensure(B.mom, sums_bytes + nbytes<long long>(nb)))) {
+    rc = ensure(B.mom, sums_bytes + nbytes<long long>(nb));
+    if (!rc) rc = size_mom_rows();
+    if (rc) {
         if (asked || rc != QC_ENOMEM) return rc;
         cudaGetLastError();                    // no room for the sums: iterate on the samples
         err.clear();
@@ -1191,6 +1197,15 @@ int qc_ctx::plan_sums(const qc_term *terms, int n_terms, int n, const qc_opts *o
     return QC_OK;
 }
 
+int qc_ctx::size_mom_rows()
+{
+    const size_t bytes = nbytes<int4>(std::max(1L, n_strip_rows)) + (m16 ? nbytes<float>(std::max(1L, n_strip_rows)) : 0);
+    int rc = ensure(mom_rows, bytes);
+    if (!rc) rc = ensure(mom_live, bytes);
+    if (!rc) rc = ensure(mom_end, nbytes<int>(std::max(1, n_strips)));
+    return rc;
+}
+
 // The context's table of strip rows as the passes read them, built the first time (a function of the
 // rows and flags staged at create).
 int qc_ctx::ensure_mom_rows(cudaStream_t st)
@@ -1198,10 +1213,7 @@ int qc_ctx::ensure_mom_rows(cudaStream_t st)
     qc_ctx *c = this;
     if (mom_rows_ready) return QC_OK;
     const size_t scale_off = nbytes<int4>(std::max(1L, n_strip_rows));
-    const size_t bytes = scale_off + (m16 ? nbytes<float>(std::max(1L, n_strip_rows)) : 0);
-    int rc = ensure(mom_rows, bytes);
-    if (!rc) rc = ensure(mom_live, bytes);
-    if (!rc) rc = ensure(mom_end, nbytes<int>(std::max(1, n_strips)));
+    const int rc = size_mom_rows();
     if (rc) return rc;
     auto scales = [&](const Buf &b) { return m16 ? (float *)((char *)b.ptr + scale_off) : nullptr; };
     CK(mom_launch_rows(n_strip_rows, d_strip_rows, d_rows, d_row_live, d_up_of_bl, d_bl_scale, (int4 *)mom_rows.ptr,
@@ -1234,6 +1246,7 @@ int qc_ctx::plan_delay_sums(const qc_term *terms, int n_terms, int n, const qc_o
     if ((double)t_bytes > 0.6 * sample * (double)n_strip_rows * n_chan) return QC_OK;
     int rc = ensure(B.dsum_t, t_bytes);
     if (!rc) rc = ensure(B.dsum_h, nbytes<double>((size_t)t.n_tint * B.hfr.size() * n_ant * KG_HSUM));
+    if (!rc) rc = size_mom_rows();
     if (rc == QC_ENOMEM) {
         cudaGetLastError();                    // no room for the products: iterate on the samples
         err.clear();

@@ -267,6 +267,7 @@ struct qc_ctx {
     int run_residual(const qc::Chain &chain, float4 *dres, double *d_chi2, cudaStream_t st);
     int pick_order(const qc_term &t, const qc_opts *o) const;
     int plan_sums(const qc_term *terms, int n_terms, int n, const qc_opts *o);
+    int size_mom_rows();
     int ensure_mom_rows(cudaStream_t st);
     int plan_delay_sums(const qc_term *terms, int n_terms, int n, const qc_opts *o, bool &use);
     qc::DelaySumsArgs delay_sums_args(const qc_term *terms, int n_terms, int n, const qc::Chain &chain);

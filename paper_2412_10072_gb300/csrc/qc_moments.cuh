@@ -8,11 +8,11 @@
 namespace qc {
 
 constexpr int MOM_N = 100;          // FP32 words per (interval, pair), full form: S 64, T 32, U 4
-constexpr int MOM_T = 64, MOM_U = 96;
+constexpr int MOM_T = 64;
 // diagonal form (a diagonal or phase-only solved term with a term to its left): S' 16 (4x4
 // Hermitian packed as S), T' 8, U 1, three words of padding (slots of whole 16-byte vectors)
 constexpr int MOM_E = 28;
-constexpr int MOM_ET = 16, MOM_EU = 24;
+constexpr int MOM_ET = 16;
 // plain diagonal form (a diagonal or phase-only solved term, the other term diagonal or to its
 // right): S 4, T 8
 constexpr int MOM_D = 12;
