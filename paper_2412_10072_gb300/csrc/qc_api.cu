@@ -1335,7 +1335,6 @@ int qc_ctx::sums_args(const qc_term *terms, int n_terms, int n, const Chain &cha
     };
     ma.tn_map = map_kind(t);
     ma.to_map = n_terms == 2 ? map_kind(terms[1 - n]) : (int)MAP_ONE;
-    if (ma.to_map == MAP_ONE) ma.to_map = MAP_CHUNK;
     ma.n_strips = n_strips;
     ma.n_time = n_time;
     ma.n_chunks = (n_chan + 31) / 32;

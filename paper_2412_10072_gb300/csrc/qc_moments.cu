@@ -317,6 +317,19 @@ template <int FORM, int OK, bool M16> struct MomCursor {
     size_t base = 0;                      // first sample of the row
     int key0 = 0, tab_p = 0, tab_q = 0, meta = 0;   // key, table entries (first interval), conjugate flag
     const int *tmap_n, *tmap_o;           // time maps of the solved and the fixed term (shared memory)
+    // frequency intervals of the lane's channel (fixed term: of the chunk's first channel where one
+    // stands for all), loaded when the cursor reaches the chunk, a step before their use
+    int fn = 0, fo = 0;
+
+    __device__ __forceinline__ void load_chunk(const MomArgs &a, int lane)
+    {
+        const int c = min(ch * 32 + lane, a.n_chan - 1);
+        if (a.tn_map == MAP_ANY || a.tn_map == MAP_CHUNK) fn = __ldg(a.tn.f_map + c);
+        if constexpr (R::NO > 0) {
+            if (a.to_map == MAP_CHUNK) fo = __ldg(a.to.f_map + ch * 32);
+            else if (a.to_map == MAP_ANY) fo = __ldg(a.to.f_map + c);
+        }
+    }
 
     __device__ __forceinline__ void load_row(const MomArgs &a)
     {
@@ -325,7 +338,7 @@ template <int FORM, int OK, bool M16> struct MomCursor {
         fresh = true;
     }
 
-    __device__ __forceinline__ void bounds(const MomArgs &a)
+    __device__ __forceinline__ void bounds(const MomArgs &a, int lane)
     {
         // the first unit from here on with rows (or none: unit >= n_units)
         for (; unit < n_units; unit += stride) {
@@ -341,10 +354,13 @@ template <int FORM, int OK, bool M16> struct MomCursor {
         }
         k = k0;
         ch = ch0;
-        if (unit < n_units) load_row(a);
+        if (unit < n_units) {
+            load_row(a);
+            load_chunk(a, lane);
+        }
     }
 
-    __device__ __forceinline__ void start(const MomArgs &a, long first, long step, const int *tn, const int *to)
+    __device__ __forceinline__ void start(const MomArgs &a, int lane, long first, long step, const int *tn, const int *to)
     {
         tmap_n = tn;
         tmap_o = to;
@@ -353,21 +369,25 @@ template <int FORM, int OK, bool M16> struct MomCursor {
         stride = step;
         unit = first;
         cm = a.chunk_major != 0;
-        bounds(a);
+        bounds(a, lane);
     }
 
-    __device__ __forceinline__ void advance(const MomArgs &a)
+    __device__ __forceinline__ void advance(const MomArgs &a, int lane)
     {
         if (cm) {
             // chunk-major units hold one chunk
             if (++k < k1) { load_row(a); return; }
         } else {
-            if (++ch < ch1) return;
+            if (++ch < ch1) { load_chunk(a, lane); return; }
             ch = ch0;
-            if (++k < k1) { load_row(a); return; }
+            if (++k < k1) {
+                load_row(a);
+                if (ch1 - ch0 > 1) load_chunk(a, lane);
+                return;
+            }
         }
         unit += stride;
-        bounds(a);
+        bounds(a, lane);
     }
 
     __device__ __forceinline__ void issue(const MomArgs &a, int lane, float4 *stage)
@@ -404,15 +424,9 @@ template <int FORM, int OK, bool M16> struct MomCursor {
         int flags = meta;
         if constexpr (R::NO > 0) {
             // the fixed term's entries: one per chunk where the chunk lies in one of its frequency intervals
-            int fi;
-            bool uni;
-            if (a.to_map == MAP_IDENTITY) {
-                fi = in ? c : 0;
-                uni = false;
-            } else {
-                fi = __ldg(a.to.f_map + (a.to_map == MAP_CHUNK ? ch * 32 : min(c, a.n_chan - 1)));
-                uni = a.to_map == MAP_CHUNK || __all_sync(FULL_MASK, fi == __shfl_sync(FULL_MASK, fi, 0));
-            }
+            const int fi = a.to_map == MAP_IDENTITY ? (in ? c : 0) : fo;
+            const bool uni = a.to_map == MAP_ONE || a.to_map == MAP_CHUNK ||
+                             (a.to_map == MAP_ANY && __all_sync(FULL_MASK, fi == __shfl_sync(FULL_MASK, fi, 0)));
             if (uni) {
                 flags |= 4;
                 if (lane < 2 * R::NO) {
@@ -430,14 +444,14 @@ template <int FORM, int OK, bool M16> struct MomCursor {
         }
         int key = key0;
         if (a.tn_map == MAP_IDENTITY) key += c * a.n_up;
-        else if (a.tn_map != MAP_ONE) key += __ldg(a.tn.f_map + min(c, a.n_chan - 1)) * a.n_up;
+        else key += fn * a.n_up;
         reinterpret_cast<int *>(stage + R::OFF_KEY)[lane] = in ? key : -1;
         if (lane == 0) {
             reinterpret_cast<int *>(stage + R::OFF_META)[0] = flags;
             if constexpr (M16) reinterpret_cast<float *>(stage + R::OFF_META)[1] = msc;
         }
         cp_async_commit();
-        advance(a);
+        advance(a, lane);
     }
 };
 
@@ -482,7 +496,7 @@ static __global__ void __launch_bounds__(128, MomRing<FORM, OK, M16>::PER_SM) mo
         tmap_o = s_map + a.n_time;
     }
     MomCursor<FORM, OK, M16> cur;
-    cur.start(a, ((long)blockIdx.x * blockDim.x + threadIdx.x) >> 5, ((long)gridDim.x * blockDim.x) >> 5, tmap_n, tmap_o);
+    cur.start(a, lane, ((long)blockIdx.x * blockDim.x + threadIdx.x) >> 5, ((long)gridDim.x * blockDim.x) >> 5, tmap_n, tmap_o);
     int is = 0;
 #pragma unroll
     for (int d = 0; d < R::DEPTH - 1; ++d) {
@@ -490,15 +504,26 @@ static __global__ void __launch_bounds__(128, MomRing<FORM, OK, M16>::PER_SM) mo
         if (++is == R::DEPTH) is = 0;
     }
     auto add = [&](const float4 *st, int meta) {
-        float4 w = st[R::OFF_W + lane];
+        float4 w = st[R::OFF_W + lane], d0, d1, m0, m1;
+        auto load = [&]() {
+            d0 = st[lane];
+            d1 = st[32 + lane];
+            m0 = st[64 + lane];
+            if constexpr (!M16) m1 = st[96 + lane];
+        };
+        // all loads of the sample together, one shared-memory latency for the step (the full form has
+        // no registers for it: 1.87 ms a pass with, 1.84 without; the left-full form 1.69 and 1.77)
+        if constexpr (FORM != FORM_FULL) load();
         // any weight other than +-0
         if ((__float_as_uint(w.x) | __float_as_uint(w.y) | __float_as_uint(w.z) | __float_as_uint(w.w)) & 0x7fffffffu) {
-            J2 D = j_from(st[lane], st[32 + lane]), M;
+            if constexpr (FORM == FORM_FULL) load();
+            J2 D = j_from(d0, d1), M;
             if constexpr (M16)
-                M = load_model16(*reinterpret_cast<const uint4 *>(st + 64 + lane),
+                M = load_model16(make_uint4(__float_as_uint(m0.x), __float_as_uint(m0.y), __float_as_uint(m0.z),
+                                            __float_as_uint(m0.w)),
                                  reinterpret_cast<const float *>(st + R::OFF_META)[1]);
             else
-                M = j_from(st[64 + lane], st[96 + lane]);
+                M = j_from(m0, m1);
             if (meta & 1) {                    // the conjugate baseline: D -> D^H, M -> M^H, w permuted
                 D = j_herm(D);
                 M = j_herm(M);
@@ -522,8 +547,18 @@ static __global__ void __launch_bounds__(128, MomRing<FORM, OK, M16>::PER_SM) mo
     };
     // runs of steps with unchanged keys: the inner loop only adds; a key change leaves it to
     // flush the sums, then adds the step that changed the key
-    int key_cur = -1, stage = 0, run = 0;
+    int key_cur = -1, stage = 0, next = 0, run = 0;
     bool done = false;
+    // the key and flags of a step are read a step ahead (they were written with its issue, DEPTH - 1
+    // steps ago), so that the loop's decisions wait on no load
+    auto peek = [&](int s, int &m, int &k) {
+        const float4 *p = ring + (size_t)s * R::STAGE;
+        m = reinterpret_cast<const int *>(p + R::OFF_META)[0];
+        k = reinterpret_cast<const int *>(p + R::OFF_KEY)[lane];
+    };
+    int meta_next, key_next;
+    __syncwarp();
+    peek(0, meta_next, key_next);
     for (;;) {
         const float4 *st;
         int meta = 0, key = -1;
@@ -534,13 +569,15 @@ static __global__ void __launch_bounds__(128, MomRing<FORM, OK, M16>::PER_SM) mo
             cp_async_wait<R::DEPTH - 1>();
             __syncwarp();
             st = ring + (size_t)stage * R::STAGE;
-            meta = reinterpret_cast<const int *>(st + R::OFF_META)[0];
+            next = stage + 1 == R::DEPTH ? 0 : stage + 1;
+            meta = meta_next;
+            key = key_next;
+            peek(next, meta_next, key_next);
             if (meta & MOM_END) { done = true; break; }
-            key = reinterpret_cast<const int *>(st + R::OFF_KEY)[lane];
             if (__any_sync(FULL_MASK, key != key_cur) || ++run == R::FLUSH_EVERY) break;
             if (R::TWO_LEVEL && (run & 7) == 0) lift();
             add(st, meta);
-            if (++stage == R::DEPTH) stage = 0;
+            stage = next;
         }
         if constexpr (R::TWO_LEVEL) {
             lift();
@@ -552,7 +589,7 @@ static __global__ void __launch_bounds__(128, MomRing<FORM, OK, M16>::PER_SM) mo
         run = 0;
         key_cur = key;
         add(st, meta);
-        if (++stage == R::DEPTH) stage = 0;
+        stage = next;
     }
     cp_async_wait<0>();
 }
