@@ -2018,7 +2018,17 @@ int qc_ctx::solve_term(const qc_term *terms, int n_terms, int n, Chain chain, co
                 dua.alpha = ua.alpha;
                 dua.n_active_prev = ua.n_active_prev;
                 dua.n_active_next = ua.n_active_next;
-                if (psums) delay_update_kernel<true><<<dua.d.n_tint * dua.d.n_fint, 128, 0, st>>>(dua);
+                if (psums) {
+                    delay_update_kernel<true><<<dua.d.n_tint * dua.d.n_fint, 128, 0, st>>>(dua);
+                    if (!dsum) {
+                        // about four CTAs an SM, none below 512 (antenna, channel) pairs
+                        CK(cudaGetLastError());
+                        const long n_int = (long)dua.d.n_tint * dua.d.n_fint;
+                        const long by_size = ((long)n_ant * n_chan / dua.d.n_fint + 511) / 512;
+                        const unsigned split = (unsigned)std::max(1L, std::min(by_size, 4L * sm_count / n_int));
+                        delay_chan_kernel<<<dim3((unsigned)n_int, split), 128, 0, st>>>(dua);
+                    }
+                }
                 else delay_update_kernel<false><<<dua.d.n_tint * dua.d.n_fint, upd_block, 0, st>>>(dua);
             } else {
                 update_kernel<<<nb, upd_block, 0, st>>>(ua);
@@ -2054,7 +2064,7 @@ int qc_ctx::solve_term(const qc_term *terms, int n_terms, int n, Chain chain, co
     } else {
         if ((rc = enqueue())) return rc;
     }
-    launches += 1 + 3 * (long long)max_iter + (mom ? 3 : 0);
+    launches += 1 + (delay[n] && psums && !dsum ? 4 : 3) * (long long)max_iter + (mom ? 3 : 0);
     // iteration bookkeeping: which accumulate launches did work, and their device time
     std::vector<int> hcnt(max_iter + 1);
     int herr = 0;

@@ -142,6 +142,32 @@ __device__ __forceinline__ int delay_solve_pair(double a0, double a1, double a2,
     return 0;
 }
 
+// Counts and convergence of an interval, by the whole block (one thread adding up the counts of 512
+// channels was 0.1 of the update's 0.13 ms on 75 intervals); tn, td (thread 0): the squared change
+// of the gains and their squared norm.
+template <bool SUMS>
+__device__ __forceinline__ void delay_finish(const DelayUpdArgs &u, int bin, int2 fr, size_t cb0, double tn, double td)
+{
+    unsigned long long nv = 0, nb = 0;
+    for (int c = fr.x + (int)threadIdx.x; c <= fr.y; c += blockDim.x) {
+        nv += (unsigned long long)u.bin_nvis[cb0 + c];
+        nb += (unsigned long long)u.bin_nbytes[cb0 + c];
+    }
+    if (nv) atomicAdd(u.vis_iters, nv);
+    if (nb) atomicAdd(u.acc_bytes, nb);
+    if (threadIdx.x == 0) {
+        const double delta = td > 0 ? sqrt(tn / td) : 0.0;
+        if (u.iters) u.iters[bin] = u.k;
+        if (delta < u.tol) {
+            if (SUMS) u.active[bin] = 0;
+            else
+                for (int c = fr.x; c <= fr.y; ++c) u.active[cb0 + c] = 0;
+        } else {
+            atomicAdd(u.n_active_next, 1);
+        }
+    }
+}
+
 template <bool SUMS>
 static __global__ void __launch_bounds__(128) delay_update_kernel(const DelayUpdArgs u)
 {
@@ -226,8 +252,7 @@ static __global__ void __launch_bounds__(128) delay_update_kernel(const DelayUpd
         }
         int singular;
         if (SUMS && u.hsum) {
-            // no coupling between X and Y: two real 2x2 solves (64 threads through the general 4x4
-            // complex elimination took 0.1 of the update's 0.13 ms)
+            // no coupling between X and Y: two real 2x2 solves
             double y[4];
             singular = delay_solve_pair(M[0][0].x, M[0][1].x, M[1][1].x, M[2][2].x, M[2][3].x, M[3][3].x, b[0].x, b[1].x,
                                         b[2].x, b[3].x, y);
@@ -259,7 +284,8 @@ static __global__ void __launch_bounds__(128) delay_update_kernel(const DelayUpd
             den += 2.0;
         }
     }
-    if (SUMS && u.hsum) {
+    if (SUMS && !u.hsum) return;       // delay_chan_kernel follows
+    if (SUMS) {
         // the change of the gains, (antenna, channel) by (antenna, channel) over the block's threads.
         // The phase change (d0 + d1 w_ref) + d1 (w - w_ref) is formed in FP64 at the band's centre
         // and in FP32 away from it: 0.84 ms a launch with FP64 phases and the channel table on the
@@ -304,27 +330,6 @@ static __global__ void __launch_bounds__(128) delay_update_kernel(const DelayUpd
             __syncthreads();
         }
         if (threadIdx.x == 0) den = 2.0 * d.n_ant * nch;
-    } else if (SUMS) {
-        // the channel table and the change of the gains, spread over the block's threads by
-        // (antenna, channel)
-        __syncthreads();
-        const int nch = fr.y - fr.x + 1;
-        const long n = (long)d.n_ant * nch;
-        for (long i = threadIdx.x; i < n; i += blockDim.x) {
-            const int ant = (int)(i / nch), c = fr.x + (int)(i - (long)ant * nch);
-            const double *P = d.params + ((size_t)bin * d.n_ant + ant) * 4;
-            const double *A = u.acc + ((size_t)bin * d.n_ant + ant) * KG_SUMS;
-            const double w = DELAY_TWO_PI * d.nu[c];
-            const float2 nx = delay_gain_f32(P[0], P[1], w), ny = delay_gain_f32(P[2], P[3], w);
-            d.tab[((size_t)tint * d.n_ant + ant) * d.n_chan + c] = make_float4(nx.x, nx.y, ny.x, ny.y);
-            num += delay_change2(A[0] + A[1] * w) + delay_change2(A[2] + A[3] * w);
-            den += 2.0;
-        }
-        __syncthreads();
-        for (int ant = threadIdx.x; ant < d.n_ant; ant += blockDim.x) {
-            double *A = u.acc + ((size_t)bin * d.n_ant + ant) * KG_SUMS;
-            A[0] = A[1] = A[2] = A[3] = 0.0;
-        }
     }
     __shared__ double s_num[4], s_den[4];
     for (int dd = 16; dd > 0; dd >>= 1) {
@@ -334,26 +339,63 @@ static __global__ void __launch_bounds__(128) delay_update_kernel(const DelayUpd
     const int wi = threadIdx.x >> 5;
     if ((threadIdx.x & 31) == 0) { s_num[wi] = num; s_den[wi] = den; }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double tn = 0, td = 0;
+    double tn = 0, td = 0;
+    if (threadIdx.x == 0)
         for (int i = 0; i < (int)(blockDim.x + 31) / 32; ++i) { tn += s_num[i]; td += s_den[i]; }
-        const double delta = td > 0 ? sqrt(tn / td) : 0.0;
-        if (u.iters) u.iters[bin] = u.k;
-        unsigned long long nv = 0, nb = 0;
-        for (int c = fr.x; c <= fr.y; ++c) {
-            nv += (unsigned long long)u.bin_nvis[cb0 + c];
-            nb += (unsigned long long)u.bin_nbytes[cb0 + c];
-        }
-        atomicAdd(u.vis_iters, nv);
-        atomicAdd(u.acc_bytes, nb);
-        if (delta < u.tol) {
-            if (SUMS) u.active[bin] = 0;
-            else
-                for (int c = fr.x; c <= fr.y; ++c) u.active[cb0 + c] = 0;
-        } else {
-            atomicAdd(u.n_active_next, 1);
-        }
+    delay_finish<SUMS>(u, bin, fr, cb0, tn, td);
+}
+
+// The channel table and the change of the gains of the active intervals (SUMS without the products),
+// an interval's (antenna, channel) pairs split over gridDim.y CTAs, the last of which tests
+// convergence.  FP64 throughput bounds it (phases formed and reduced in FP64); one CTA an interval
+// inside the update kept 64 of 152 SMs busy where there are 64 intervals: 490 us an iteration with 64
+// antennas and 512 channels, 38 us the update and 166 us this like so.
+static __global__ void __launch_bounds__(128) delay_chan_kernel(const DelayUpdArgs u)
+{
+    if (*u.n_active_prev == 0) return;
+    const DelayArgs &d = u.d;
+    const int bin = blockIdx.x, tint = bin / d.n_fint;
+    const int2 fr = d.frange[bin % d.n_fint];
+    if (fr.x < 0 || !u.active[bin]) return;
+    const int nch = fr.y - fr.x + 1, n = d.n_ant * nch;
+    const int per = (n + gridDim.y - 1) / gridDim.y, i0 = min(n, (int)blockIdx.y * per), i1 = min(n, i0 + per);
+    double num = 0;
+    for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
+        const int ant = i / nch, c = fr.x + (i - ant * nch);
+        const double *P = d.params + ((size_t)bin * d.n_ant + ant) * 4;
+        const double *A = u.acc + ((size_t)bin * d.n_ant + ant) * KG_SUMS;
+        const double w = DELAY_TWO_PI * d.nu[c];
+        const float2 nx = delay_gain_f32(P[0], P[1], w), ny = delay_gain_f32(P[2], P[3], w);
+        d.tab[((size_t)tint * d.n_ant + ant) * d.n_chan + c] = make_float4(nx.x, nx.y, ny.x, ny.y);
+        num += delay_change2(A[0] + A[1] * w) + delay_change2(A[2] + A[3] * w);
     }
+    __shared__ double s_num[4];
+    __shared__ bool s_last;
+    for (int dd = 16; dd > 0; dd >>= 1) num += __shfl_down_sync(0xffffffffu, num, dd);
+    if ((threadIdx.x & 31) == 0) s_num[threadIdx.x >> 5] = num;
+    __syncthreads();                                  // every thread has read its changes
+    // the interval's sum and the number of its CTAs that are done: spare words of the first antenna's sums
+    double *A0 = u.acc + (size_t)bin * d.n_ant * KG_SUMS;
+    unsigned long long *count = reinterpret_cast<unsigned long long *>(A0 + 14);
+    if (threadIdx.x == 0) {
+        atomicAdd(A0 + 13, s_num[0] + s_num[1] + s_num[2] + s_num[3]);
+        __threadfence();
+        s_last = atomicAdd(count, 1ull) == gridDim.y - 1;
+    }
+    __syncthreads();
+    if (!s_last) return;
+    double tn = 0;
+    if (threadIdx.x == 0) {
+        __threadfence();
+        tn = atomicAdd(A0 + 13, 0.0);
+        A0[13] = 0.0;
+        *count = 0ull;
+    }
+    for (int ant = threadIdx.x; ant < d.n_ant; ant += blockDim.x) {
+        double *A = u.acc + ((size_t)bin * d.n_ant + ant) * KG_SUMS;
+        A[0] = A[1] = A[2] = A[3] = 0.0;
+    }
+    delay_finish<true>(u, bin, fr, (size_t)tint * d.n_chan, tn, 2.0 * n);
 }
 
 } // namespace qc

@@ -511,8 +511,9 @@ static __global__ void __launch_bounds__(128, MomRing<FORM, OK, M16>::PER_SM) mo
             m0 = st[64 + lane];
             if constexpr (!M16) m1 = st[96 + lane];
         };
-        // all loads of the sample together, one shared-memory latency for the step (the full form has
-        // no registers for it: 1.87 ms a pass with, 1.84 without; the left-full form 1.69 and 1.77)
+        // all loads of the sample together, one shared-memory latency for the step (with the keys read
+        // ahead 1.77 -> 1.66 ms a pass for the left-full form on 64 antennas, 85 x 512; the full form
+        // gains nothing from it and has no registers to spare)
         if constexpr (FORM != FORM_FULL) load();
         // any weight other than +-0
         if ((__float_as_uint(w.x) | __float_as_uint(w.y) | __float_as_uint(w.z) | __float_as_uint(w.w)) & 0x7fffffffu) {
