@@ -146,9 +146,12 @@ typedef struct {
  *                 every sample of the interval (Eq. jhj_case2, Eq. jhwr_case2);
  *                 convergence uses the gains over the interval's channels.
  *                 Delay terms are accepted by qc_solve and qc_residual.  A
- *                 solved delay term in a chain of one or two terms (kernel 0
- *                 or 3) has its own streaming kernel, which applies the chain
- *                 rule per sample; otherwise the accumulate kernels form
+ *                 solved delay term in a chain of one or two terms with the
+ *                 default options iterates on per-(time interval, pair,
+ *                 channel) products formed in one pass, where those are at most
+ *                 0.6 of the samples and the other term is diagonal or to its
+ *                 right; else (or with kernel 3) a streaming kernel applies the
+ *                 chain rule per sample; otherwise the accumulate kernels form
  *                 diagonal blocks per (time interval, channel) bin and the
  *                 update reduces them over the interval's channels.
  *   dd          : 1 = direction-dependent: with n_dir > 1 the gains (and
