@@ -936,6 +936,9 @@ extern "C" int qc_solve(qc_ctx *c, qc_term *terms, int32_t n_terms, const qc_opt
     c->pending.clear();
     const long long b_flag = c->has_flag ? 1 : 0;
     const long long b_unflag = 32 + (c->m16 ? 16 : 32 * c->n_dir) + 16;
+    for (int j = 0; j < n_terms; ++j)
+        if (terms[j].solve && (rc = c->plan_sums(xt.data(), n_terms, j, o))) return rc;
+    if ((rc = c->plan_counters(xt.data(), n_terms, o->n_epochs))) return rc;
     for (int j = 0; j < n_terms; ++j) {
         if (!terms[j].solve) continue;
         const qc_term &t = xt[j];
@@ -943,7 +946,6 @@ extern "C" int qc_solve(qc_ctx *c, qc_term *terms, int32_t n_terms, const qc_opt
         const size_t nb = term_nbins(t);
         const size_t KG = t.type == 1 ? KG_FULL : KG_DIAG;
         const size_t nat = c->term_nat(t);
-        if ((rc = c->plan_sums(xt.data(), n_terms, j, o))) return rc;
         const bool one_launch = B.sums.one_launch;
         if (!one_launch) {
             if ((rc = c->ensure(B.acc, nbytes<double>(nb * nat * KG)))) return rc;
@@ -1197,6 +1199,43 @@ int qc_ctx::plan_sums(const qc_term *terms, int n_terms, int n, const qc_opts *o
     return QC_OK;
 }
 
+// Counters of the term solves pending together from the call's `first`-th one on: max_iter + 1 each.
+size_t qc_ctx::sums_window(long long first) const
+{
+    size_t n = 0;
+    const long long end = std::min(sums_total, first + MAX_PENDING);
+    for (long long i = first; i < end; ++i) n += (size_t)sums_iters[i % sums_iters.size()] + 1;
+    return n;
+}
+
+// Room for the counters of the call's one-launch term solves (`terms` in the order of an epoch), before
+// the first of them: the buffer stays where it is while solves are pending.  A term that took the
+// sums by itself goes back to the samples where there is no room.
+int qc_ctx::plan_counters(const qc_term *terms, int n_terms, int n_epochs)
+{
+    sums_done = 0;
+    for (;;) {
+        sums_iters.clear();
+        for (int j = 0; j < n_terms; ++j)
+            if (terms[j].solve && tb[j].sums.one_launch) sums_iters.push_back(terms[j].max_iter);
+        sums_total = (long long)n_epochs * (long long)sums_iters.size();
+        size_t most = 0;
+        for (size_t i = 0; i < sums_iters.size(); ++i) most = std::max(most, sums_window((long long)i));
+        if (most == 0) return QC_OK;
+        const int rc = ensure(sums_cnt, nbytes<int>(most));
+        if (rc != QC_ENOMEM) return rc;
+        bool left = false;
+        for (int j = 0; j < n_terms; ++j)
+            if (terms[j].solve && tb[j].sums.one_launch && !tb[j].sums.asked) {
+                tb[j].sums = SumsPlan();
+                left = true;
+            }
+        if (!left) return rc;
+        cudaGetLastError();
+        err.clear();
+    }
+}
+
 int qc_ctx::size_mom_rows()
 {
     const size_t bytes = nbytes<int4>(std::max(1L, n_strip_rows)) + (m16 ? nbytes<float>(std::max(1L, n_strip_rows)) : 0);
@@ -1392,32 +1431,10 @@ int qc_ctx::solve_term_sums(const qc_term *terms, int n_terms, int n, const Chai
         sums_events.push_back(e);
     }
     const cudaEvent_t *ev = sums_events.data() + P.ev;
-    // a counter region per pending term solve; the buffer only grows while nothing is pending
-    const size_t need = nbytes<int>((size_t)MAX_PENDING * (t.max_iter + 1));
-    if (sums_cnt.bytes < need || sums_cnt.bytes < nbytes<int>((size_t)P.off + t.max_iter + 1)) {
-        if (!pending.empty()) {
-            // terms of different max_iter: keep the counts so far, then make room
-            Buf old = sums_cnt;
-            sums_cnt = Buf();
-            if ((rc = ensure(sums_cnt, std::max(need, nbytes<int>((size_t)P.off + need / sizeof(int)))))) {
-                sums_cnt = old;
-                return rc;
-            }
-            CK(cudaMemcpyAsync(sums_cnt.ptr, old.ptr, nbytes<int>(P.off), cudaMemcpyDeviceToDevice, st));
-            CK(cudaStreamSynchronize(st));
-            release(old.ptr);
-        } else if ((rc = ensure(sums_cnt, need))) {
-            return rc;
-        }
-    }
+    // a counter region per pending term solve, all of those up to the next collection cleared together
     int *cnt = (int *)sums_cnt.ptr + P.off;
-    // one clearing for the solves of terms with equal max_iter
-    if (pending.empty()) sums_zeroed = 0;
-    if (sums_zeroed < (size_t)P.off + t.max_iter + 1) {
-        const size_t upto = std::max((size_t)P.off + t.max_iter + 1, pending.empty() ? need / sizeof(int) : 0);
-        CK(cudaMemsetAsync(cnt, 0, nbytes<int>(upto - P.off), st));
-        sums_zeroed = upto;
-    }
+    if (pending.empty()) CK(cudaMemsetAsync(cnt, 0, nbytes<int>(sums_window(sums_done)), st));
+    ++sums_done;
     CK(cudaMemsetAsync(B.mom.ptr, 0, nbytes<float>((size_t)P.n_bins * n_up * mom_words(B.sums.form)), st));
     CK(cudaEventRecord(ev[0], st));
     CK(mom_launch_pass(ma, B.sums.form, B.sums.ok, sm_count, st));

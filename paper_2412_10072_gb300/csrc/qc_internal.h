@@ -220,7 +220,8 @@ struct qc_ctx {
     std::vector<int> pending_cnt;
     std::vector<cudaEvent_t> sums_events;   // three per pending term solve
     Buf sums_cnt;                     // int: intervals still active after iteration k, per pending solve
-    size_t sums_zeroed = 0;           // ints of it zeroed for the solves now pending
+    std::vector<int> sums_iters;      // max_iter of an epoch's one-launch term solves, in their order
+    long long sums_total = 0, sums_done = 0;   // one-launch term solves of the call, those enqueued so far
     // Pinned staging of one call's small copies: a copy from or to pageable memory holds the host
     // until it is done, and a small solve makes about ten.  Blocks are kept for the context's life
     // (at most PIN_MAX in all; larger copies go directly); a call ends synchronised, so the next one
@@ -267,6 +268,8 @@ struct qc_ctx {
     int run_residual(const qc::Chain &chain, float4 *dres, double *d_chi2, cudaStream_t st);
     int pick_order(const qc_term &t, const qc_opts *o) const;
     int plan_sums(const qc_term *terms, int n_terms, int n, const qc_opts *o);
+    size_t sums_window(long long first) const;
+    int plan_counters(const qc_term *terms, int n_terms, int n_epochs);
     int size_mom_rows();
     int ensure_mom_rows(cudaStream_t st);
     int plan_delay_sums(const qc_term *terms, int n_terms, int n, const qc_opts *o, bool &use);
