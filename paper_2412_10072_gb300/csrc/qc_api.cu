@@ -407,6 +407,16 @@ extern "C" int qc_create(const qc_problem *p, qc_ctx **out)
             (g.x < 0 ? g.x : g.y) = bl;
         }
         c->full_grid = c->full_grid && n_up == n_bl;
+        // the last pair that had a row at each time; a pair's rows are in two strips at most
+        c->pair_time_once = true;
+        std::vector<int> last(p->n_time, -1);
+        for (int u = 0; u < n_up; ++u)
+            for (int b : { c->pair_strips[u].x, c->pair_strips[u].y })
+                for (int k = b < 0 ? 0 : strip_off[b]; b >= 0 && k < strip_off[b + 1]; ++k) {
+                    int &l = last[rows[strip_rows[k]].z];
+                    if (l == u) c->pair_time_once = false;
+                    l = u;
+                }
         DALLOC(c->d_upair, int, std::max<size_t>(1, upair.size()));
         if (!upair.empty()) HCOPY(c->d_upair, upair.data(), nbytes<int>(upair.size()));
         DALLOC(c->d_up_of_bl, int, up_of_bl.size());
@@ -1147,6 +1157,13 @@ int qc_ctx::get_event(int i, cudaEvent_t &ev)
 // Antennas up to which one CTA keeps an interval's gains and normal equations in shared memory
 // (256 x (32 + 128) B = 40 KB) and walks all of its pairs itself.
 static constexpr int SUMS_ONE_LAUNCH_ANT = 256;
+// Antennas from which the full and left-full forms' slots are rounded to their heads: a slot's rounding
+// averages out over the pairs.  Error of three chains and single terms against FP64 (rounding the result
+// alone 2.4e-8): 20 antennas 3.6e-8 heads only, 3.2e-8 with tails, 3.6e-8 on the samples; 40 antennas 2.7,
+// 2.5 and 2.5e-8; 64 antennas 2.6, 2.5 and 2.5e-8, where G and B with the FP16 model end at 3.0e-8 with and
+// without tails and the tails' bytes take 13.0 instead of 10.3 ms.  The plain diagonal form's tails, 48 B a
+// slot, cost 2% and are always kept.
+static constexpr int SUMS_TAILS_ANT = 64;
 
 // The route of a solved term: from sums when the caller asks for it (qc_opts.moments), or by itself
 // where that is the cheaper way to the same steps; sets B.sums and sizes its workspace.
@@ -1182,9 +1199,24 @@ int qc_ctx::plan_sums(const qc_term *terms, int n_terms, int n, const qc_opts *o
         const double sample_bytes = (m16 ? 64.0 : 80.0) * (double)n_strip_rows * n_chan;
         if (2.0 * 4.0 * mom_words(form) * (double)slots > 0.5 * sample_bytes) return QC_OK;
     }
-    const size_t sums_bytes = ((nbytes<float>(slots * mom_words(form)) + 15) / 16) * 16;
+    // an interval several times long: the rows inside each chunk keep a lane's key (units of a strip
+    // x one chunk); else a row's chunks inside each row (units of whole rows), so that an interval
+    // one time long flushes once per row.  The rows are cut into blocks until there are about four
+    // units per resident warp, down to 8 rows inside a chunk (a block's end is a flush)
+    SumsPlan P;
+    P.chunk_major = t.n_tint < n_time ? 1 : 0;
+    const long max_strip = std::max(1, max_strip_rows), n_chunks = (n_chan + 31) / 32;
+    const long strips = std::max(1L, (long)n_strips * (P.chunk_major ? n_chunks : 1));
+    const long blocks = std::max(1L, (4L * sm_count * 12 + strips - 1) / strips);
+    P.rb = (int)std::min(max_strip, std::max(P.chunk_major ? 8L : 1L, (max_strip + blocks - 1) / blocks));
+    P.n_rb = (int)((max_strip + P.rb - 1) / P.rb);
+    P.tails = form == FORM_D || n_ant < SUMS_TAILS_ANT;
+    P.wide = !slots_once(t, form, P);
+    const size_t words = slots * mom_words(form);
+    P.cnt_off = nbytes<float>((P.tails ? 2 : 1) * words);
+    P.mom64_off = P.cnt_off + ((nbytes<long long>(nb) + 15) / 16) * 16;
     int rc;
-    rc = ensure(B.mom, sums_bytes + nbytes<long long>(nb));
+    rc = ensure(B.mom, P.mom64_off + (P.wide ? nbytes<double>(words) : 0));
     if (!rc) rc = size_mom_rows();
     if (rc) {
         if (asked || rc != QC_ENOMEM) return rc;
@@ -1192,11 +1224,54 @@ int qc_ctx::plan_sums(const qc_term *terms, int n_terms, int n, const qc_opts *o
         err.clear();
         return QC_OK;
     }
-    B.sums.form = form;
-    B.sums.ok = ok;
-    B.sums.asked = asked;
-    B.sums.one_launch = one_launch;
+    P.form = form;
+    P.ok = ok;
+    P.asked = asked;
+    P.one_launch = one_launch;
+    B.sums = P;
     return QC_OK;
+}
+
+// Whether the pass adds to each slot of a term at most once: then the additions are exact in FP32.  What
+// follows is the order of mom_pass_kernel's steps and the rule by which it flushes.
+bool qc_ctx::slots_once(const qc_term &t, int form, const SumsPlan &P) const
+{
+    if (!pair_time_once) return false;
+    const int every = form == FORM_FULL ? mom_flush_every(m16) : INT32_MAX;
+    std::vector<int> n_of(t.n_tint, 0);
+    for (int i = 0; i < n_time; ++i) ++n_of[t.t_map[i]];
+    const int deepest = n_time ? *std::max_element(n_of.begin(), n_of.end()) : 0;
+    // a chunk's lanes in one interval, or each in its own: else the parts of an interval are added one by one
+    for (int c0 = 0; c0 < n_chan; c0 += 32) {
+        const int n = std::min(32, n_chan - c0), k = t.f_map[c0 + n - 1] - t.f_map[c0];
+        if (k == 0) continue;
+        for (int l = 1; l < n; ++l)
+            if (t.f_map[c0 + l] == t.f_map[c0 + l - 1]) return false;
+    }
+    if (P.chunk_major) {
+        // a strip's rows inside one chunk: the pair in one strip, the strip in one unit, the interval's times
+        // in a row and no more of them than the lanes keep, the interval's channels in one chunk
+        if (n_up != n_strips || P.n_rb != 1 || deepest > every) return false;
+        for (int i = 1; i < n_time; ++i)
+            if (t.t_map[i] < t.t_map[i - 1]) return false;
+        for (int ch = 32; ch < n_chan; ch += 32)
+            if (t.f_map[ch] == t.f_map[ch - 1]) return false;
+        return true;
+    }
+    // a row's chunks: one row an interval, and no flush between an interval's chunks
+    if (deepest > 1) return false;
+    int run = 0;
+    std::vector<int> cur(32, -1);
+    for (int c0 = 0; c0 < n_chan; c0 += 32) {
+        const int n = std::min(32, n_chan - c0);
+        bool flush = c0 == 0;
+        for (int l = 0; l < n; ++l) flush = flush || t.f_map[c0 + l] != cur[l];
+        if (!flush && ++run < every) continue;
+        if (c0 && t.f_map[c0] == t.f_map[c0 - 1]) return false;
+        run = 0;
+        for (int l = 0; l < 32; ++l) cur[l] = l < n ? t.f_map[c0 + l] : -1;
+    }
+    return true;
 }
 
 // Counters of the term solves pending together from the call's `first`-th one on: max_iter + 1 each.
@@ -1377,21 +1452,15 @@ int qc_ctx::sums_args(const qc_term *terms, int n_terms, int n, const Chain &cha
     ma.n_strips = n_strips;
     ma.n_time = n_time;
     ma.n_chunks = (n_chan + 31) / 32;
-    // an interval several times long: the rows inside each chunk keep a lane's key (units of a strip
-    // x one chunk); else a row's chunks inside each row (units of whole rows), so that an interval
-    // one time long flushes once per row.  The rows are cut into blocks until there are about four
-    // units per resident warp, down to 8 rows inside a chunk (a block's end is a flush)
-    ma.chunk_major = t.n_tint < n_time ? 1 : 0;
-    const long max_strip = std::max(1, max_strip_rows);
-    const long want_units = 4L * sm_count * 12;
+    ma.chunk_major = B.sums.chunk_major;
     ma.group = ma.chunk_major ? 1 : ma.n_chunks;
-    const long strips = std::max(1L, (long)n_strips * (ma.chunk_major ? ma.n_chunks : 1));
-    const long blocks = std::max(1L, (want_units + strips - 1) / strips);
-    ma.rb = (int)std::min(max_strip, std::max(ma.chunk_major ? 8L : 1L, (max_strip + blocks - 1) / blocks));
-    ma.n_rb = (int)((max_strip + ma.rb - 1) / ma.rb);
+    ma.rb = B.sums.rb;
+    ma.n_rb = B.sums.n_rb;
     ma.tn = chain.t[n];
     ma.to = n_terms == 2 ? chain.t[1 - n] : chain.t[n];
     ma.mom = (float *)B.mom.ptr;
+    ma.tail = B.sums.tails ? ma.mom + term_nbins(t) * n_up * mom_words(B.sums.form) : nullptr;
+    ma.mom64 = B.sums.wide ? (double *)((char *)B.mom.ptr + B.sums.mom64_off) : nullptr;
     mn.n_bins = (int)term_nbins(t);
     mn.n_ant = n_ant;
     mn.n_up = n_up;
@@ -1399,6 +1468,7 @@ int qc_ctx::sums_args(const qc_term *terms, int n_terms, int n, const Chain &cha
     mn.form = B.sums.form;
     mn.upair = d_upair;
     mn.mom = ma.mom;
+    mn.tail = ma.tail;
     mn.params = (const double *)B.params.ptr;
     mn.tab = (const float4 *)B.tab.ptr;
     mn.n_fint = t.n_fint;
@@ -1435,9 +1505,12 @@ int qc_ctx::solve_term_sums(const qc_term *terms, int n_terms, int n, const Chai
     int *cnt = (int *)sums_cnt.ptr + P.off;
     if (pending.empty()) CK(cudaMemsetAsync(cnt, 0, nbytes<int>(sums_window(sums_done)), st));
     ++sums_done;
-    CK(cudaMemsetAsync(B.mom.ptr, 0, nbytes<float>((size_t)P.n_bins * n_up * mom_words(B.sums.form)), st));
+    const size_t words = (size_t)P.n_bins * n_up * mom_words(B.sums.form);
+    if (ma.mom64) CK(cudaMemsetAsync(ma.mom64, 0, nbytes<double>(words), st));
+    else CK(cudaMemsetAsync(ma.mom, 0, nbytes<float>((ma.tail ? 2 : 1) * words), st));
     CK(cudaEventRecord(ev[0], st));
     CK(mom_launch_pass(ma, B.sums.form, B.sums.ok, sm_count, st));
+    if (ma.mom64) CK(mom_launch_split(words, ma.mom64, ma.mom, ma.tail, sm_count, st));
     CK(cudaEventRecord(ev[1], st));
     mi.params = (double *)B.params.ptr;
     mi.tab = (float4 *)B.tab.ptr;
@@ -1455,7 +1528,7 @@ int qc_ctx::solve_term_sums(const qc_term *terms, int n_terms, int n, const Chai
     mi.tol = t.tol;
     CK(mom_launch_iterate(mi, st));
     CK(cudaEventRecord(ev[2], st));
-    launches += 2;
+    launches += ma.mom64 ? 3 : 2;
     pending.push_back(P);
     return QC_OK;
 }
@@ -1913,7 +1986,7 @@ int qc_ctx::solve_term(const qc_term *terms, int n_terms, int n, Chain chain, co
     MomNormArgs mn;
     const int mom_n = mom ? mom_words(B.sums.form) : 0;
     const size_t mom_words_all = (size_t)nb * n_up * mom_n;
-    const size_t mom_cnt_off = ((nbytes<float>(mom_words_all) + 15) / 16) * 16;
+    const size_t mom_cnt_off = B.sums.cnt_off;
     if (mom) {
         int rc_ = sums_args(terms, n_terms, n, chain, st, ma, mn);
         if (rc_) return rc_;
@@ -1974,12 +2047,14 @@ int qc_ctx::solve_term(const qc_term *terms, int n_terms, int n, Chain chain, co
                 CK(dd_launch_acc(dda, ts, grid, st));
             } else if (mom) {
                 if (k == 1) {
-                    CK(cudaMemsetAsync(B.mom.ptr, 0, nbytes<float>(mom_words_all), st));
+                    if (ma.mom64) CK(cudaMemsetAsync(ma.mom64, 0, nbytes<double>(mom_words_all), st));
+                    else CK(cudaMemsetAsync(ma.mom, 0, nbytes<float>((ma.tail ? 2 : 1) * mom_words_all), st));
                     CK(mom_launch_bytes(nb, (const long long *)B.nvis.ptr + 2 * (size_t)nb, mom_iter_bytes,
                                         (long long *)((char *)B.mom.ptr + mom_cnt_off), ua.acc_bytes, st));
                     CK(cudaEventRecordWithFlags(events[ev_pass], st, rec_flags));
                     ma.n_active = cnt;
                     CK(mom_launch_pass(ma, B.sums.form, B.sums.ok, sm_count, st));
+                    if (ma.mom64) CK(mom_launch_split(mom_words_all, ma.mom64, ma.mom, ma.tail, sm_count, st));
                     CK(cudaEventRecordWithFlags(events[ev_pass + 1], st, rec_flags));
                 }
                 mn.n_active = cnt + (k - 1);
@@ -2081,7 +2156,7 @@ int qc_ctx::solve_term(const qc_term *terms, int n_terms, int n, Chain chain, co
     } else {
         if ((rc = enqueue())) return rc;
     }
-    launches += 1 + (delay[n] && psums && !dsum ? 4 : 3) * (long long)max_iter + (mom ? 3 : 0);
+    launches += 1 + (delay[n] && psums && !dsum ? 4 : 3) * (long long)max_iter + (mom ? 3 + (ma.mom64 ? 1 : 0) : 0);
     // iteration bookkeeping: which accumulate launches did work, and their device time
     std::vector<int> hcnt(max_iter + 1);
     int herr = 0;

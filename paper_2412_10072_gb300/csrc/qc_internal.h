@@ -52,6 +52,7 @@ cudaError_t mom_launch_bytes(int n_bins, const long long *bin_nbytes, long long 
 cudaError_t mom_launch_rows(long n, const int *strip_rows, const int4 *rows, const uint8_t *row_live,
                             const int *up_of_bl, const float *bl_scale, int4 *out, float *scale, int n_strips,
                             const int *strip_off, int4 *live, float *live_scale, int *strip_end, cudaStream_t st);
+cudaError_t mom_launch_split(size_t words, const double *src, float *dst, float *tail, int sm_count, cudaStream_t st);
 cudaError_t mom_launch_iterate(const qc::MomIterArgs &a, cudaStream_t st);
 cudaError_t dd_launch_residual(const qc::DDArgs &a, int grid, cudaStream_t st);
 
@@ -66,6 +67,10 @@ struct SumsPlan {
     int ok = 0;                // KIND_* of the fixed term
     bool asked = false;        // by qc_opts.moments (else the route was chosen by its cost)
     bool one_launch = false;   // every iteration in one launch (mom_iterate_kernel)
+    bool tails = false;        // slots as head and tail
+    bool wide = false;         // slots added to several times: FP64 additions, split at the end
+    int chunk_major = 0, rb = 1, n_rb = 1;   // units of the pass (MomArgs)
+    size_t cnt_off = 0, mom64_off = 0;   // offsets in TermBufs::mom (heads, tails, bytes per interval, FP64 slots)
 };
 
 // Device buffers of one chain position, reused across calls while large enough.
@@ -99,7 +104,7 @@ struct TermBufs {
     Buf ws_sb;     // warp-specialised kernel, strip tiles: uint32 [n_chunks][words] active-entry bits
     Buf div;       // divergence flagging: double [bins][ant][2] first / last relative updates
     Buf params0;   // divergence flagging: the FP64 parameters before the solve
-    Buf mom;       // a term solved from sums: FP32 sums per (interval, unordered pair), bytes per interval
+    Buf mom;       // a term solved from sums: sums per (interval, unordered pair), bytes per interval
     SumsPlan sums; // the route of the current call
     Buf dsum_t;    // delay terms solved from products: T [n_tint][chunks][pairs][2][32] float4
     Buf dsum_h;    //   double [bins][ant][KG_HSUM]
@@ -181,6 +186,7 @@ struct qc_ctx {
     long n_strip_rows = 0;            // rows in the baseline strips (cross-correlations)
     int max_strip_rows = 0;           // rows of the longest strip
     bool full_grid = false;           // every pair in one orientation, each with one row per data time
+    bool pair_time_once = false;      // no antenna pair (either orientation) has two rows of one data time
     bool m16 = false, has_flag = false;
     const float4 *d_vis = nullptr, *d_model = nullptr, *d_weight = nullptr;
     const uint8_t *d_flag = nullptr;
@@ -269,6 +275,7 @@ struct qc_ctx {
     int pick_order(const qc_term &t, const qc_opts *o) const;
     int plan_sums(const qc_term *terms, int n_terms, int n, const qc_opts *o);
     size_t sums_window(long long first) const;
+    bool slots_once(const qc_term &t, int form, const SumsPlan &P) const;
     int plan_counters(const qc_term *terms, int n_terms, int n_epochs);
     int size_mom_rows();
     int ensure_mom_rows(cudaStream_t st);

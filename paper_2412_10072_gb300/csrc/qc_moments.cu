@@ -24,15 +24,19 @@
 // Plain diagonal form: any other diagonal or phase-only solved term (the other term diagonal, or to
 // its right).  With X = O_p M O_q^H: S_kj = sum w_kj |X_kj|^2, T_kj = sum w_kj conj(X_kj) D_kj (12 words),
 //     JHJ_p[k][k] += sum_j |g_q,j|^2 S_kj,  b_p[k] += sum_j g_q,j T_kj,  and conjugated for q.
-// In all of them JHr = b - JHJ vec(g).  One pass over the data per term solve forms the sums in
-// FP32 (mom_pass_kernel: per-lane register sums, added to the slots by FP32 atomics, a few per
-// slot: a warp covers a whole row, or a strip of one chunk).  The intervals are independent from
-// there on, so one CTA per interval runs all of its iterations (mom_iterate_kernel): an iteration
-// reads 400, 112 or 48 B per (interval, pair) and side out of L2 instead of 80 B per sample out of
-// HBM, with no launch in between.  Measured on the two-term chain (64 antennas, 300 x 512, three
-// epochs of 20 iterations a term): 663 ms with the iterations on the samples, 47.0 ms from sums (passes 6.3
-// ms for G, 6.8 ms for B, 20 iterations 1.5 and 0.9 ms); 27 antennas, 61 x 131, intervals of 5 x 17: 3.80
-// -> 0.36 ms; 7 antennas, 60 x 16: 1.03 -> 0.28 ms.
+// In all of them JHr = b - JHJ vec(g).  One pass over the data per term solve forms the sums
+// (mom_pass_kernel): FP32 register sums of a lane's 8 samples (short forms, kept as head and tail beyond
+// that) or 16 to 32 (full form), added up over the lanes with the last levels' rounding kept, and
+// then to the slots, exactly where a slot takes one addition and in FP64 where it takes several.
+// The intervals are independent from there on, so one CTA per interval runs all of its iterations
+// (mom_iterate_kernel): an iteration reads 400, 112 or 96 B per (interval, pair) and side out of L2
+// (800 and 224 B with tails) instead of 80 B per sample out of HBM, with no launch in between; the
+// products and sums over the pairs are compensated.  Error of the gains against FP64 (rms, relative;
+// rounding the result alone 2.4e-8), then the iterations on the samples: 7 antennas, 4 x 4 intervals
+// 3.8e-8 and 3.8e-8, one interval of 150 x 512 3.1e-8 and 3.0e-8, full-Jones 2.7e-8 and 2.6e-8; 20
+// antennas 3.6e-8 and 3.9e-8; 64 antennas, G and B, 3.0e-8 and 3.0e-8.  Time, two-term chain (64
+// antennas, 300 x 512, three epochs of 20 iterations a term): 660 ms on the samples, 46.2 ms from sums; 27
+// antennas, 61 x 131, intervals of 5 x 17: 3.78 and 0.35 ms; 7 antennas, 60 x 16: 1.02 and 0.25 ms.
 #include "qc_internal.h"
 
 #include <algorithm>
@@ -163,65 +167,114 @@ __device__ __forceinline__ void mom_add_e(float (&acc)[MOM_EW], const J2 &D, con
     for (int u = 0; u < 4; ++u) cacc_conj(acc[16 + 2 * u], acc[17 + 2 * u], m[u], zv[u]);
 }
 
-// Add the warp's register sums (NW words, the slot's order) to the sums of each lane's key
-// (-1: nothing) and zero them:
+// One word of a slot, x + tail.  A slot that takes one addition (mom64 null) keeps it as head and
+// tail, both exact (many antennas: rounded to the head, tail null); where a slot is added to several times the additions are FP64, split into head and tail at the
+// end (mom_split_kernel).  FP32 additions there grew the gains' error with the interval: 2.0e-7 for
+// one interval of 7 antennas over 150 x 512, 3.0e-8 like this.
+__device__ __forceinline__ void slot_add(const MomArgs &a, size_t i, float x, float tail)
+{
+    if (a.mom64) {
+        atomicAdd(a.mom64 + i, (double)x + (double)tail);
+    } else {
+        const float h = x + tail, l = tail - (h - x);
+        atomicAdd(a.mom + i, h);
+        if (a.tail && isfinite(h) && l != 0.f) atomicAdd(a.tail + i, l);   // an infinite or NaN head has no tail
+    }
+}
+
+// Add the warp's register sums (NW words, the slot's order; heads acc, tails lo(v)) to the sums of each
+// lane's key (-1: nothing, sums of zero) and zero them:
 //  - one key for the warp: a reduce-scatter of 32 words at a time (after the halvings at lane
-//    offsets 16 .. 1 lane L holds word L of the group), then one coalesced atomic per group;
+//    offsets 16 .. 1 lane L holds word L of the group), then one coalesced access per group; the
+//    last three levels, whose roundings no longer average out, carry their tails;
 //  - 32 distinct keys: each lane adds its own words;
 //  - otherwise: a segmented reduction per word over the run of equal keys (channel intervals
-//    are contiguous, so a run is a range of lanes), added by the run's first lane.
-template <int NW>
-__device__ __forceinline__ void mom_flush(float (&acc)[NW], int key, int lane, float *mom, int stride)
+//    are contiguous, so a run is a range of lanes), stopped at parts of a quarter of the longest run,
+//    whose first lanes add them (to FP64 slots, see slots_once).
+template <int NW, typename LO>
+__device__ __forceinline__ void mom_flush(float (&acc)[NW], LO &&lo, int key, int lane, const MomArgs &a)
 {
     constexpr int F = (NW + 31) / 32, P = 32;    // groups of 32 words, one exchange tree each
-    const int k0 = __shfl_sync(FULL_MASK, key, 0);
-    if (__all_sync(FULL_MASK, key == k0)) {
+    constexpr int stride = NW == MOM_FW ? MOM_N : (NW == MOM_EW ? MOM_E : MOM_D);
+    const int k0 = __reduce_max_sync(FULL_MASK, key);
+    if (__all_sync(FULL_MASK, key == k0 || key < 0)) {
         if (k0 >= 0) {
             // in place, group by group: after the halving at offset o the live words are [0 .. h)
-            float *dst = mom + (size_t)k0 * stride + lane;
+            const size_t at = (size_t)k0 * stride + lane;
+#pragma unroll
+            for (int v = 0; v < NW; ++v) acc[v] += lo(v);
 #pragma unroll
             for (int f = 0; f < F; ++f) {
+                float t[4] = { 0.f, 0.f, 0.f, 0.f };
 #pragma unroll
                 for (int h = P / 2, o = 16; o >= 1; h >>= 1, o >>= 1) {
                     const bool up = (lane & o) != 0;
 #pragma unroll
                     for (int i = 0; i < h; ++i) {
-                        const float lo = 32 * f + i < NW ? acc[32 * f + i] : 0.f;
-                        const float hi = 32 * f + i + h < NW ? acc[32 * f + i + h] : 0.f;
-                        const float send = up ? lo : hi;
-                        const float keep = up ? hi : lo;
-                        if (32 * f + i < NW) acc[32 * f + i] = keep + __shfl_xor_sync(FULL_MASK, send, o);
+                        const float w0 = 32 * f + i < NW ? acc[32 * f + i] : 0.f;
+                        const float w1 = 32 * f + i + h < NW ? acc[32 * f + i + h] : 0.f;
+                        const float send = up ? w0 : w1;
+                        const float keep = up ? w1 : w0;
+                        if (32 * f + i >= NW) continue;
+                        const float got = __shfl_xor_sync(FULL_MASK, send, o);
+                        if (h > 4) {
+                            acc[32 * f + i] = keep + got;
+                        } else {
+                            float e;
+                            two_sum(keep, got, acc[32 * f + i], e);
+                            if (h < 4) {
+                                const float ts = up ? t[i] : t[i + h];
+                                e += (up ? t[i + h] : t[i]) + __shfl_xor_sync(FULL_MASK, ts, o);
+                            }
+                            t[i] = e;
+                        }
                     }
                 }
-                if (32 * f + lane < NW) atomicAdd(dst + 32 * f, acc[32 * f]);
+                if (32 * f + lane < NW) slot_add(a, at + 32 * f, acc[32 * f], t[0]);
             }
         }
     } else {
         const unsigned m = __match_any_sync(FULL_MASK, key);
-        if (__all_sync(FULL_MASK, m == (1u << lane))) {
+        const size_t at = (size_t)(key >= 0 ? key : 0) * stride;
+        const int len = key >= 0 ? __popc(m) : 0;
+        const int longest = __reduce_max_sync(FULL_MASK, len);
+        if (longest <= 1) {
             if (key >= 0) {
-                float *dst = mom + (size_t)key * stride;
 #pragma unroll
-                for (int v = 0; v < NW; ++v) atomicAdd(dst + v, acc[v]);
+                for (int v = 0; v < NW; ++v) slot_add(a, at + v, acc[v], lo(v));
             }
         } else {
-            const int seg_end = 32 - __clz(m);
-            const bool head = lane == __ffs(m) - 1;
-            float *dst = mom + (size_t)(key >= 0 ? key : 0) * stride;
+            const int first = __ffs(m) - 1, end = 32 - __clz(m);
+            // lanes of a part: the largest power of two up to a quarter of the longest run
+            const int step = 1 << (31 - __clz(max(1, longest >> 2)));
+            const int part_end = min(end, first + ((lane - first) / step + 1) * step);
+            const bool head = key >= 0 && (lane - first) % step == 0;
 #pragma unroll
             for (int v = 0; v < NW; ++v) {
-                float x = acc[v];
-#pragma unroll
-                for (int d = 1; d < 32; d <<= 1) {
+                float x = acc[v] + lo(v);
+                for (int d = 1; d < step; d <<= 1) {
                     const float o = __shfl_down_sync(FULL_MASK, x, d);
-                    if (lane + d < seg_end) x += o;
+                    if (lane + d < part_end) x += o;
                 }
-                if (head && key >= 0) atomicAdd(dst + v, x);
+                if (head) slot_add(a, at + v, x, 0.f);
             }
         }
     }
 #pragma unroll
     for (int v = 0; v < NW; ++v) acc[v] = 0.f;
+}
+
+// FP64 slots to heads and tails
+static __global__ void mom_split_kernel(long n2, const double2 *__restrict__ src, float2 *__restrict__ dst,
+                                        float2 *__restrict__ tail)
+{
+    for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n2; i += (long)gridDim.x * blockDim.x) {
+        const double2 v = src[i];
+        const float2 h = make_float2((float)v.x, (float)v.y);
+        dst[i] = h;
+        if (tail) tail[i] = make_float2(isfinite(h.x) ? (float)(v.x - (double)h.x) : 0.f,
+                                        isfinite(h.y) ? (float)(v.y - (double)h.y) : 0.f);
+    }
 }
 
 // The rows of the baseline strips in strip order, as the pass reads them: {row (-1: no usable
@@ -282,19 +335,23 @@ template <int FORM, int OK, bool M16> struct MomRing {
     static constexpr int OFF_OP = OFF_W + 32, OFF_OQ = OFF_OP + 32 * NO, OFF_KEY = OFF_OQ + 32 * NO;
     static constexpr int OFF_META = OFF_KEY + 8;
     static constexpr int STAGE = OFF_META + 1;               // float4 per stage
-    // three CTAs of 4 warps per SM (the full form's 100 register sums fit 168 registers); ring
+    // three CTAs of 4 warps per SM (the full form's 96 register sums fit 168 registers); ring
     // depth as the shared memory of three CTAs allows
     static constexpr int PER_SM = 3;
     static constexpr int DEPTH = NO == 2 ? 3 : (NO == 1 ? 4 : 6);
     static constexpr size_t SMEM = (size_t)4 * DEPTH * STAGE * sizeof(float4);
     // A lane's sums over a long strip are FP32 sums of terms of one sign, whose rounding grows with
-    // the number of terms and moves the fixed point of all antennas the same way.  The short slots keep
-    // a second set of registers that takes the first one's sums every 8 steps; the full form, which
-    // has no registers left, goes to its slot every 32 (16 with the FP16 model).  Measured over three
-    // epochs of G and B (64 antennas, 40 integrations): B's error against FP64 1.7e-7 without, 3.7e-8
-    // with sums of 8, 3.2e-8 for the iterations on the samples.
+    // the number of terms and moves the fixed point of all antennas the same way.  The short slots keep a
+    // head and a tail that take the sums every LIFT steps, the rounding of the head going to the
+    // tail (kept in shared memory where the registers are taken); the full form, which has neither,
+    // goes to its slot every 32 steps (16 with the FP16 model).
     static constexpr bool TWO_LEVEL = FORM != FORM_FULL;
-    static constexpr int FLUSH_EVERY = TWO_LEVEL ? 1 << 30 : (M16 ? 16 : 32);
+    static constexpr bool TAIL_SMEM = FORM == FORM_E;
+    static constexpr int LIFT = 8;
+    static constexpr int FLUSH_EVERY = TWO_LEVEL ? 1 << 30 : mom_flush_every(M16);
+    static constexpr size_t TAIL = TAIL_SMEM ? (size_t)128 * MOM_EW * sizeof(float) : 0;
+    // integrations whose time maps fit beside the rings (and tails) of three CTAs
+    static constexpr int MAX_STAGED = TAIL_SMEM ? 512 : 1024;
 };
 
 constexpr int MOM_END = 2;       // meta: the warp's steps have run out (bit 0: conjugate baseline)
@@ -471,22 +528,31 @@ static __global__ void __launch_bounds__(128, MomRing<FORM, OK, M16>::PER_SM) mo
     extern __shared__ float4 mom_ring[];
     const int lane = threadIdx.x & 31;
     float4 *ring = mom_ring + (size_t)(threadIdx.x >> 5) * R::DEPTH * R::STAGE;
-    constexpr int stride = mom_words(FORM);
-    float acc[NW], hi[R::TWO_LEVEL ? NW : 1];
+    float acc[NW], hi[R::TWO_LEVEL ? NW : 1], lo_reg[R::TWO_LEVEL && !R::TAIL_SMEM ? NW : 1];
+    float *lo_smem = reinterpret_cast<float *>(mom_ring + (size_t)4 * R::DEPTH * R::STAGE) + threadIdx.x;
+    auto tail = [&](int v) -> float & {
+        if constexpr (R::TAIL_SMEM) return lo_smem[128 * v];
+        else return lo_reg[R::TWO_LEVEL ? v : 0];
+    };
 #pragma unroll
     for (int v = 0; v < NW; ++v) {
         acc[v] = 0.f;
-        if constexpr (R::TWO_LEVEL) hi[v] = 0.f;
+        if constexpr (R::TWO_LEVEL) { hi[v] = 0.f; tail(v) = 0.f; }
     }
     auto lift = [&]() {
         if constexpr (R::TWO_LEVEL) {
 #pragma unroll
-            for (int v = 0; v < NW; ++v) { hi[v] += acc[v]; acc[v] = 0.f; }
+            for (int v = 0; v < NW; ++v) {
+                float e;
+                two_sum(hi[v], acc[v], hi[v], e);
+                tail(v) += e;
+                acc[v] = 0.f;
+            }
         }
     };
     const int *tmap_n = a.tn.t_map, *tmap_o = a.to.t_map;
     if (a.stage_maps) {
-        int *s_map = reinterpret_cast<int *>(mom_ring + (size_t)4 * R::DEPTH * R::STAGE);
+        int *s_map = reinterpret_cast<int *>(reinterpret_cast<char *>(mom_ring) + R::SMEM + R::TAIL);
         for (int i = threadIdx.x; i < a.n_time; i += blockDim.x) {
             s_map[i] = __ldg(a.tn.t_map + i);
             s_map[a.n_time + i] = __ldg(a.to.t_map + i);
@@ -583,16 +649,19 @@ static __global__ void __launch_bounds__(128, MomRing<FORM, OK, M16>::PER_SM) mo
                 peek(stage, meta, key);
             }
             if (meta & MOM_END) { done = true; break; }
-            if (__any_sync(FULL_MASK, key != key_cur) || ++run == R::FLUSH_EVERY) break;
-            if (R::TWO_LEVEL && (run & 7) == 0) lift();
+            // lanes past the last channel keep the key they had: they add nothing
+            if (__any_sync(FULL_MASK, key != key_cur && key >= 0) || ++run == R::FLUSH_EVERY) break;
+            if (R::TWO_LEVEL && run % R::LIFT == 0) lift();
             add(st, meta);
             stage = next;
         }
         if constexpr (R::TWO_LEVEL) {
             lift();
-            mom_flush<NW>(hi, key_cur, lane, a.mom, stride);
+            mom_flush<NW>(hi, tail, key_cur, lane, a);
+#pragma unroll
+            for (int v = 0; v < NW; ++v) tail(v) = 0.f;
         } else {
-            mom_flush<NW>(acc, key_cur, lane, a.mom, stride);
+            mom_flush<NW>(acc, [](int) { return 0.f; }, key_cur, lane, a);
         }
         if (done) break;
         run = 0;
@@ -633,8 +702,11 @@ template <int FORM> struct NormSums {
 // antenna's gain row (g0, g1): with u = 2l + m,
 //   h[l][l2] += sum_m sum_m2 g_m conj(g_m2) S[(l,m)][(l2,m2)],  b[l] += sum_m g_m T[(l,m)].
 // The q side takes conj(S[(m,l)][(m2,l2)]) and conj(T[(m,l)]): indices 1 and 2 exchanged, conjugated.
+// EXACT: exact products, h heads and e tails of the sums (few antennas have few pairs over which the
+// roundings of plain products average out); else plain, e unused.
+template <bool EXACT>
 __device__ __forceinline__ void pair_block(const float4 *__restrict__ sv, const float4 *__restrict__ tv, bool p_side,
-                                           float2 g0, float2 g1, float *h)
+                                           float2 g0, float2 g1, float *h, float *e)
 {
     const float4 a0 = __ldg(sv), a1 = __ldg(sv + 1), a2 = __ldg(sv + 2), a3 = __ldg(sv + 3);
     const float4 t0 = __ldg(tv), t1 = __ldg(tv + 1);
@@ -651,23 +723,67 @@ __device__ __forceinline__ void pair_block(const float4 *__restrict__ sv, const 
     float2 u1 = p_side ? make_float2(t0.z, t0.w) : make_float2(t1.x, t1.y);
     float2 u2 = p_side ? make_float2(t1.x, t1.y) : make_float2(t0.z, t0.w);
     u0.y *= sg; u1.y *= sg; u2.y *= sg; u3.y *= sg;
-    const float n0 = cnorm2(g0), n1 = cnorm2(g1);
-    const float2 x = cmulc(g0, g1);                         // g_0 conj(g_1)
-    h[0] += fmaf(n0, a0.x, fmaf(n1, d1, 2.f * fmaf(x.x, s01.x, -x.y * s01.y)));
-    h[1] += fmaf(n0, d2, fmaf(n1, a0.w, 2.f * fmaf(x.x, s23.x, -x.y * s23.y)));
-    // n0 S02 + n1 S13 + x S03 + conj(x) S12
-    h[2] += fmaf(n0, s02.x, fmaf(n1, s13.x, fmaf(x.x, s03.x + s12.x, x.y * (s12.y - s03.y))));
-    h[3] += fmaf(n0, s02.y, fmaf(n1, s13.y, fmaf(x.x, s03.y + s12.y, x.y * (s03.x - s12.x))));
-    h[4] += fmaf(g0.x, u0.x, fmaf(-g0.y, u0.y, fmaf(g1.x, u1.x, -g1.y * u1.y)));
-    h[5] += fmaf(g0.x, u0.y, fmaf(g0.y, u0.x, fmaf(g1.x, u1.y, g1.y * u1.x)));
-    h[6] += fmaf(g0.x, u2.x, fmaf(-g0.y, u2.y, fmaf(g1.x, u3.x, -g1.y * u3.y)));
-    h[7] += fmaf(g0.x, u2.y, fmaf(g0.y, u2.x, fmaf(g1.x, u3.y, g1.y * u3.x)));
+    if constexpr (EXACT) {
+        const HT n0 = dot2(g0.x, g0.x, g0.y, g0.y), n1 = dot2(g1.x, g1.x, g1.y, g1.y);
+        const HT xr = dot2(g0.x, g1.x, g0.y, g1.y), xi = dot2(g0.y, g1.x, -g0.x, g1.y);   // g_0 conj(g_1)
+        const HT xr2 = { 2.f * xr.hi, 2.f * xr.lo }, xi2 = { -2.f * xi.hi, -2.f * xi.lo };
+        dot_add(h[0], e[0], n0, a0.x);
+        dot_add(h[0], e[0], n1, d1);
+        dot_add(h[0], e[0], xr2, s01.x);
+        dot_add(h[0], e[0], xi2, s01.y);
+        dot_add(h[1], e[1], n0, d2);
+        dot_add(h[1], e[1], n1, a0.w);
+        dot_add(h[1], e[1], xr2, s23.x);
+        dot_add(h[1], e[1], xi2, s23.y);
+        // n0 S02 + n1 S13 + x S03 + conj(x) S12
+        dot_add(h[2], e[2], n0, s02.x);
+        dot_add(h[2], e[2], n1, s13.x);
+        dot_add(h[2], e[2], xr, s03.x);
+        dot_add(h[2], e[2], xr, s12.x);
+        dot_add(h[2], e[2], xi, s12.y);
+        dot_add(h[2], e[2], neg(xi), s03.y);
+        dot_add(h[3], e[3], n0, s02.y);
+        dot_add(h[3], e[3], n1, s13.y);
+        dot_add(h[3], e[3], xr, s03.y);
+        dot_add(h[3], e[3], xr, s12.y);
+        dot_add(h[3], e[3], xi, s03.x);
+        dot_add(h[3], e[3], neg(xi), s12.x);
+        dot_add(h[4], e[4], g0.x, u0.x);
+        dot_add(h[4], e[4], -g0.y, u0.y);
+        dot_add(h[4], e[4], g1.x, u1.x);
+        dot_add(h[4], e[4], -g1.y, u1.y);
+        dot_add(h[5], e[5], g0.x, u0.y);
+        dot_add(h[5], e[5], g0.y, u0.x);
+        dot_add(h[5], e[5], g1.x, u1.y);
+        dot_add(h[5], e[5], g1.y, u1.x);
+        dot_add(h[6], e[6], g0.x, u2.x);
+        dot_add(h[6], e[6], -g0.y, u2.y);
+        dot_add(h[6], e[6], g1.x, u3.x);
+        dot_add(h[6], e[6], -g1.y, u3.y);
+        dot_add(h[7], e[7], g0.x, u2.y);
+        dot_add(h[7], e[7], g0.y, u2.x);
+        dot_add(h[7], e[7], g1.x, u3.y);
+        dot_add(h[7], e[7], g1.y, u3.x);
+    } else {
+        const float n0 = cnorm2(g0), n1 = cnorm2(g1);
+        const float2 x = cmulc(g0, g1);                         // g_0 conj(g_1)
+        h[0] += fmaf(n0, a0.x, fmaf(n1, d1, 2.f * fmaf(x.x, s01.x, -x.y * s01.y)));
+        h[1] += fmaf(n0, d2, fmaf(n1, a0.w, 2.f * fmaf(x.x, s23.x, -x.y * s23.y)));
+        // n0 S02 + n1 S13 + x S03 + conj(x) S12
+        h[2] += fmaf(n0, s02.x, fmaf(n1, s13.x, fmaf(x.x, s03.x + s12.x, x.y * (s12.y - s03.y))));
+        h[3] += fmaf(n0, s02.y, fmaf(n1, s13.y, fmaf(x.x, s03.y + s12.y, x.y * (s03.x - s12.x))));
+        h[4] += fmaf(g0.x, u0.x, fmaf(-g0.y, u0.y, fmaf(g1.x, u1.x, -g1.y * u1.y)));
+        h[5] += fmaf(g0.x, u0.y, fmaf(g0.y, u0.x, fmaf(g1.x, u1.y, g1.y * u1.x)));
+        h[6] += fmaf(g0.x, u2.x, fmaf(-g0.y, u2.y, fmaf(g1.x, u3.x, -g1.y * u3.y)));
+        h[7] += fmaf(g0.x, u2.y, fmaf(g0.y, u2.x, fmaf(g1.x, u3.y, g1.y * u3.x)));
+    }
 }
 
 // The contribution of pair (a, o) to antenna a's register sums; gains of o from g (full: the two
 // float4 of its table entry; else one, (g_XX, g_YY)).
-template <int FORM>
-__device__ __forceinline__ void pair_add(const float *__restrict__ slot, bool p_side, const float4 *g, float *h)
+template <int FORM, bool EXACT>
+__device__ __forceinline__ void pair_add(const float *__restrict__ slot, bool p_side, const float4 *g, float *h,
+                                         float *e)
 {
     const float4 *s = reinterpret_cast<const float4 *>(slot);
     if constexpr (FORM == FORM_FULL) {
@@ -677,26 +793,28 @@ __device__ __forceinline__ void pair_add(const float *__restrict__ slot, bool p_
 #pragma unroll
             for (int k = 0; k < 2; ++k) {
                 const int blk = p_side ? 2 * k + j : 2 * j + k;
-                pair_block(s + 4 * blk, s + MOM_T / 4 + 2 * blk, p_side, make_float2(g[j].x, g[j].y),
-                           make_float2(g[j].z, g[j].w), h + NE_WORDS * k);
+                pair_block<EXACT>(s + 4 * blk, s + MOM_T / 4 + 2 * blk, p_side, make_float2(g[j].x, g[j].y),
+                           make_float2(g[j].z, g[j].w), h + NE_WORDS * k, e + NE_WORDS * k);
             }
     } else if constexpr (FORM == FORM_E) {
-        pair_block(s, s + MOM_ET / 4, p_side, make_float2(g[0].x, g[0].y), make_float2(g[0].z, g[0].w), h);
+        pair_block<EXACT>(s, s + MOM_ET / 4, p_side, make_float2(g[0].x, g[0].y), make_float2(g[0].z, g[0].w), h, e);
     } else {
-        diag_pair_add(__ldg(s), __ldg(s + 1), __ldg(s + 2), p_side, g[0], h);
+        if constexpr (EXACT) diag_pair_add(__ldg(s), __ldg(s + 1), __ldg(s + 2), p_side, g[0], h, e);
+        else diag_pair_add(__ldg(s), __ldg(s + 1), __ldg(s + 2), p_side, g[0], h);
     }
 }
 
 // One warp: antenna a's normal equations of an interval over the other antennas (lanes), in FP32;
 // the totals to out[NWORD].  Antenna o's gains (full: two float4, else one) at gains + o * gstride.
-template <int FORM>
-__device__ __forceinline__ void antenna_sums(const MomNormArgs &A, const float *__restrict__ bin_sums, int a, int lane,
+// TAIL: the slots' tails as well (the sums are linear in the slots: the tails' plain sums go to e).
+template <int FORM, bool TAIL>
+__device__ __forceinline__ void antenna_sums(const MomNormArgs &A, size_t bin_off, int a, int lane,
                                              const float4 *gains, size_t gstride, double *out)
 {
     constexpr int N = NormSums<FORM>::NWORD;
-    float h[N];
+    float h[N], e[N];
 #pragma unroll
-    for (int i = 0; i < N; ++i) h[i] = 0.f;
+    for (int i = 0; i < N; ++i) h[i] = e[i] = 0.f;
     for (int o = lane; o < A.n_ant; o += 32) {
         if (o == a) continue;
         const int up = __ldg(A.upair + (size_t)a * A.n_ant + o);
@@ -704,16 +822,18 @@ __device__ __forceinline__ void antenna_sums(const MomNormArgs &A, const float *
         float4 g[2];
         g[0] = gains[o * gstride];
         if constexpr (FORM == FORM_FULL) g[1] = gains[o * gstride + 1];
-        pair_add<FORM>(bin_sums + (size_t)up * mom_words(FORM), a < o, g, h);   // the smaller index is the sums' p
+        const size_t at = bin_off + (size_t)up * mom_words(FORM);
+        pair_add<FORM, true>(A.mom + at, a < o, g, h, e);                          // the smaller index is the sums' p
+        if constexpr (TAIL) pair_add<FORM, false>(A.tail + at, a < o, g, e, nullptr);
     }
-    const double v = reduce_words<N>(h, lane);
+    const double v = reduce_words<N>(h, e, lane);
     if (lane % (32 / N) == 0) out[lane / (32 / N)] = v;
 }
 
 // Per-iteration form (more antennas than the one-launch kernel takes, divergence flagging, an
 // allreduce before the update): one warp per (interval, antenna); JHr = b - JHJ vec(G_a) in FP64,
 // written in the update kernel's accumulator layout.
-template <int FORM>
+template <int FORM, bool TAIL>
 static __global__ void __launch_bounds__(128) mom_normal_kernel(const MomNormArgs A)
 {
     constexpr int N = NormSums<FORM>::NWORD, NF4 = FORM == FORM_FULL ? 2 : 1;
@@ -725,8 +845,9 @@ static __global__ void __launch_bounds__(128) mom_normal_kernel(const MomNormArg
     const int bin = (int)(w / A.n_ant), a = (int)(w % A.n_ant);
     if (!A.active[bin]) return;
     const int tint = bin / A.n_fint, fint = bin - tint * A.n_fint;
-    antenna_sums<FORM>(A, A.mom + (size_t)bin * A.n_up * mom_words(FORM), a, lane,
-                       A.tab + NF4 * ((size_t)tint * A.n_ant * A.n_fint + fint), (size_t)NF4 * A.n_fint, s_out[warp]);
+    const size_t bin_off = (size_t)bin * A.n_up * mom_words(FORM), gstride = (size_t)NF4 * A.n_fint;
+    const float4 *gains = A.tab + NF4 * ((size_t)tint * A.n_ant * A.n_fint + fint);
+    antenna_sums<FORM, TAIL>(A, bin_off, a, lane, gains, gstride, s_out[warp]);
     __syncwarp();
     if (lane != 0) return;
     double2 G[4];
@@ -799,7 +920,7 @@ __device__ __forceinline__ int solve_blocks(const double (&h00)[NB], const doubl
 // or grid-wide counter stands between two iterations.  Per iteration the warps form the antennas'
 // normal equations from the sums (L2), one thread per antenna solves and updates in FP64 exactly as
 // update_kernel does, and the FP64 relative change of the interval ends the loop.
-template <int FORM>
+template <int FORM, bool TAIL>
 static __global__ void __launch_bounds__(256, 2) mom_iterate_kernel(const MomIterArgs a)
 {
     constexpr bool GFULL = FORM == FORM_FULL;
@@ -814,7 +935,7 @@ static __global__ void __launch_bounds__(256, 2) mom_iterate_kernel(const MomIte
     __shared__ int s_done;
     const int bin = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
     const int tint = bin / A.n_fint, fint = bin - tint * A.n_fint;
-    const float *bin_sums = A.mom + (size_t)bin * A.n_up * mom_words(FORM);
+    const size_t bin_off = (size_t)bin * A.n_up * mom_words(FORM);
     auto tab_at = [&](int i) { return a.tab + NF4 * (((size_t)tint * A.n_ant + i / NF4) * A.n_fint + fint) + i % NF4; };
     for (int i = tid; i < A.n_ant * NF4; i += blockDim.x) g32[i] = *tab_at(i);
     // phase-only: (phi_X, phi_Y) in the first entry; diagonal: entries 0 and 3 of the four kept
@@ -828,7 +949,7 @@ static __global__ void __launch_bounds__(256, 2) mom_iterate_kernel(const MomIte
     int k = 1;
     for (;; ++k) {
         for (int ant = warp; ant < A.n_ant; ant += nw)
-            antenna_sums<FORM>(A, bin_sums, ant, lane, g32, NF4, sums + (size_t)ant * N);
+            antenna_sums<FORM, TAIL>(A, bin_off, ant, lane, g32, NF4, sums + (size_t)ant * N);
         __syncthreads();
         const double alpha = a.alternate ? ((k % 2 == 0) ? 0.5 : 1.0) : a.damping;
         double num = 0, den = 0;
@@ -944,10 +1065,9 @@ static cudaError_t launch_pass(const qc::MomArgs &a, int sm_count, cudaStream_t 
 {
     using R = qc::MomRing<FORM, OK, M16>;
     // the raised shared-memory limit belongs to the device's copy of the kernel: set on every launch
-    // time maps of up to 1024 integrations fit beside the rings of three CTAs
     qc::MomArgs b = a;
-    b.stage_maps = a.n_time <= 1024;
-    const int smem = (int)R::SMEM + (b.stage_maps ? 2 * a.n_time * (int)sizeof(int) : 0);
+    b.stage_maps = a.n_time <= R::MAX_STAGED;
+    const int smem = (int)(R::SMEM + R::TAIL) + (b.stage_maps ? 2 * a.n_time * (int)sizeof(int) : 0);
     const cudaError_t e = cudaFuncSetAttribute(qc::mom_pass_kernel<FORM, OK, M16>,
                                                cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
@@ -981,6 +1101,14 @@ cudaError_t mom_launch_pass(const qc::MomArgs &a, int form, int ok, int sm_count
     return a.model16 ? launch_pass_any<true>(a, form, ok, sm_count, st) : launch_pass_any<false>(a, form, ok, sm_count, st);
 }
 
+cudaError_t mom_launch_split(size_t words, const double *src, float *dst, float *tail, int sm_count, cudaStream_t st)
+{
+    const long n2 = (long)(words / 2);              // a slot is a whole number of 16-byte vectors
+    const int grid = (int)std::max(1L, std::min((n2 + 255) / 256, (long)sm_count * 16));
+    qc::mom_split_kernel<<<grid, 256, 0, st>>>(n2, (const double2 *)src, (float2 *)dst, (float2 *)tail);
+    return cudaGetLastError();
+}
+
 cudaError_t mom_launch_bytes(int n_bins, const long long *bin_nbytes, long long per_iter, long long *iter_nbytes,
                              unsigned long long *acc_bytes, cudaStream_t st)
 {
@@ -990,8 +1118,9 @@ cudaError_t mom_launch_bytes(int n_bins, const long long *bin_nbytes, long long 
 
 template <int FORM> static cudaError_t launch_normal(const qc::MomNormArgs &a, cudaStream_t st)
 {
-    const long warps = (long)a.n_bins * a.n_ant;
-    qc::mom_normal_kernel<FORM><<<(unsigned)((warps + 3) / 4), 128, 0, st>>>(a);
+    const unsigned grid = (unsigned)(((long)a.n_bins * a.n_ant + 3) / 4);
+    if (a.tail) qc::mom_normal_kernel<FORM, true><<<grid, 128, 0, st>>>(a);
+    else qc::mom_normal_kernel<FORM, false><<<grid, 128, 0, st>>>(a);
     return cudaGetLastError();
 }
 
@@ -1002,18 +1131,24 @@ cudaError_t mom_launch_normal(const qc::MomNormArgs &a, cudaStream_t st)
     return launch_normal<qc::FORM_D>(a, st);
 }
 
-template <int FORM> static cudaError_t launch_iterate(const qc::MomIterArgs &a, cudaStream_t st)
+template <int FORM, bool TAIL> static cudaError_t launch_iterate(const qc::MomIterArgs &a, cudaStream_t st)
 {
     const int n_ant = a.n.n_ant;
     const int block = n_ant > 16 ? 256 : (n_ant > 8 ? 128 : 64);
     constexpr int NB = FORM == qc::FORM_FULL ? 2 : 1;
     const size_t smem = (size_t)n_ant * (NB * sizeof(float4) + qc::NormSums<FORM>::NWORD * sizeof(double) + 2 * NB * sizeof(double2));
     if (smem > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(qc::mom_iterate_kernel<FORM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        const cudaError_t e = cudaFuncSetAttribute(qc::mom_iterate_kernel<FORM, TAIL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   (int)smem);
         if (e != cudaSuccess) return e;
     }
-    qc::mom_iterate_kernel<FORM><<<a.n.n_bins, block, smem, st>>>(a);
+    qc::mom_iterate_kernel<FORM, TAIL><<<a.n.n_bins, block, smem, st>>>(a);
     return cudaGetLastError();
+}
+
+template <int FORM> static cudaError_t launch_iterate(const qc::MomIterArgs &a, cudaStream_t st)
+{
+    return a.n.tail ? launch_iterate<FORM, true>(a, st) : launch_iterate<FORM, false>(a, st);
 }
 
 cudaError_t mom_launch_iterate(const qc::MomIterArgs &a, cudaStream_t st)

@@ -7,10 +7,10 @@
 
 namespace qc {
 
-constexpr int MOM_N = 100;          // FP32 words per (interval, pair), full form: S 64, T 32, U 4
+constexpr int MOM_N = 100;          // FP32 words per (interval, pair), full form: S 64, T 32, four of padding
 constexpr int MOM_T = 64;
-// diagonal form (a diagonal or phase-only solved term with a term to its left): S' 16 (4x4
-// Hermitian packed as S), T' 8, U 1, three words of padding (slots of whole 16-byte vectors)
+// left-full form (a diagonal or phase-only solved term with a full term to its left): S' 16 (4x4
+// Hermitian packed as S), T' 8, four words of padding (slots of whole 16-byte vectors)
 constexpr int MOM_E = 28;
 constexpr int MOM_ET = 16;
 // plain diagonal form (a diagonal or phase-only solved term, the other term diagonal or to its
@@ -21,6 +21,9 @@ __host__ __device__ constexpr int mom_words(int form)
 {
     return form == FORM_FULL ? MOM_N : (form == FORM_E ? MOM_E : MOM_D);
 }
+
+// steps after which the full form's lanes go to the slots
+__host__ __device__ constexpr int mom_flush_every(bool m16) { return m16 ? 16 : 32; }
 
 // Hermitian pairs (u, v), u < v, of the 4x4 S blocks: packed as 4 diagonal reals then 6 (re, im)
 __host__ __device__ constexpr int mom_pair(int u, int v)
@@ -49,7 +52,8 @@ struct MomArgs {
     int chunk_major;                     // 1: a unit's rows inside each chunk; 0: a row's chunks inside it
     DevTerm tn;                          // the solved term (maps)
     DevTerm to;                          // the fixed other term of a two-term chain (tables)
-    float *mom;                          // [bins][n_up][mom_words(form)]
+    float *mom, *tail;                   // [bins][n_up][mom_words(form)], heads and tails (or null) of the sums
+    double *mom64;                       // the same in FP64, added to instead, or null: one store a slot
     const int *n_active;                 // or null: always
 };
 
@@ -58,6 +62,7 @@ struct MomNormArgs {
     int form;                            // FORM_*
     const int *upair;                    // [n_ant][n_ant] unordered pair index or -1
     const float *mom;                    // [bins][n_up][mom_words(form)]
+    const float *tail;                   // their tails, or null
     const double *params;                // FP64 gains of the solved term
     const float4 *tab;                   // their FP32 table [n_tint][n_ant][n_fint] x (1 | 2)
     int n_fint;
