@@ -1344,18 +1344,29 @@ int qc_ctx::ensure_mom_rows(cudaStream_t st)
 // other one to the right or diagonal).  The rule: an iteration on T reads 1 KB per (time interval,
 // pair, 32 channels), one on the samples 80 B (64 B with the FP16 model) a sample; T is taken when it is at most 0.6 of that, which leaves the pass that forms
 // it paid for after two iterations (measured on 64 antennas, 75 x 512: pass 1.9 iterations on the
-// samples, an iteration on T 0.3).  That also bounds T to 0.6 of the samples' bytes.
+// samples, an iteration on T 0.3).  That also bounds T to 0.6 of the samples' bytes; where a slot takes
+// several additions, T with its FP64 sums (three times T).
+// Whether every product of a delay term gets one sample: a time an interval, a row a pair and time.
+bool qc_ctx::products_once(const qc_term &t) const
+{
+    std::vector<char> seen(t.n_tint, 0);
+    for (int i = 0; i < n_time; ++i)
+        if (seen[t.t_map[i]]++) return false;
+    return pair_time_once;
+}
+
 int qc_ctx::plan_delay_sums(const qc_term *terms, int n_terms, int n, const qc_opts *o, bool &use)
 {
     use = false;
     const qc_term &t = terms[n];
     TermBufs &B = tb[n];
-    if (!delay[n] || n_terms > 2 || n_dir > 1 || n_up == 0 || n_ant > 256 || t.reduce || t.max_iter < 3)
+    if (!delay[n] || n_terms > 2 || n_dir > 1 || n_up == 0 || n_ant > DSUM_MAX_ANT || t.reduce || t.max_iter < 3)
         return QC_OK;
     if (o->kernel != 0 || o->order != -1 || o->block_threads != 0 || o->ctas_per_sm != 0) return QC_OK;
     if (n == 1 && kind_of_range(terms, 0, 1) == KIND_FULL) return QC_OK;
     const size_t n_chunks = (n_chan + 31) / 32;
-    const size_t t_bytes = (size_t)t.n_tint * n_chunks * n_up * 1024;
+    // the products, and the FP64 ones where a slot takes several additions
+    const size_t t_bytes = (size_t)t.n_tint * n_chunks * n_up * (products_once(t) ? 1024 : 3 * 1024);
     const double sample = m16 ? 64.0 : 80.0;
     if ((double)t_bytes > 0.6 * sample * (double)n_strip_rows * n_chan) return QC_OK;
     int rc = ensure(B.dsum_t, t_bytes);
@@ -1406,6 +1417,7 @@ DelaySumsArgs qc_ctx::delay_sums_args(const qc_term *terms, int n_terms, int n, 
     a.fmap = (const int *)B.dfmap.ptr;
     a.omega = (const float *)B.domega.ptr;
     a.T = (float4 *)B.dsum_t.ptr;
+    a.T64 = products_once(t) ? nullptr : (double *)((char *)B.dsum_t.ptr + (size_t)t.n_tint * a.n_chunks * n_up * 1024);
     a.hsum = (double *)B.dsum_h.ptr;
     a.n_tint = t.n_tint;
     a.upair = d_upair;
@@ -2027,9 +2039,11 @@ int qc_ctx::solve_term(const qc_term *terms, int n_terms, int n, Chain chain, co
                 dsa_.n_active = cnt + (k - 1);
                 if (k == 1) {
                     CK(cudaMemsetAsync(B.dsum_h.ptr, 0, nbytes<double>((size_t)nbu * n_ant * KG_HSUM), st));
-                    if (!dsa_.store)
-                        CK(cudaMemsetAsync(B.dsum_t.ptr, 0, (size_t)t.n_tint * dsa_.n_chunks * n_up * 1024, st));
+                    const size_t words = (size_t)t.n_tint * dsa_.n_chunks * n_up * 256;
+                    if (dsa_.T64) CK(cudaMemsetAsync(dsa_.T64, 0, nbytes<double>(words), st));
+                    else if (!dsa_.store) CK(cudaMemsetAsync(dsa_.T, 0, nbytes<float>(words), st));
                     CK(dsum_launch_pass(dsa_, lk != KIND_NONE ? lk : rk, sm_count, st));
+                    if (dsa_.T64) CK(dsum_launch_round(words, dsa_.T64, dsa_.T, sm_count, st));
                 }
                 CK(dsum_launch_iter(dsa_, st));
             } else if (dds) {

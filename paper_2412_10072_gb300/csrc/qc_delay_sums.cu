@@ -33,8 +33,9 @@ __device__ __forceinline__ void red_add_v4(float4 *p, float4 v)
 // The pass: each warp walks units (a block of rows of one baseline strip, its 32-channel chunks
 // inside each row or, with chunk_major, its rows inside one chunk), DEPTH - 1 steps ahead through a
 // cp.async ring.  A lane (one channel) keeps T of its slot until the time interval or chunk
-// changes and H until its parameter interval or the pair changes.  HBM-bound: it reads the samples once
-// and writes T (80 + 32 B a sample with one integration an interval).
+// changes (then added to the slot, in FP64 where the slot takes several additions) and H until its
+// parameter interval or the pair changes.  HBM-bound: it reads the samples once and writes T (80 +
+// 32 B a sample with one integration an interval).
 template <int OK, bool M16>
 static __global__ void __launch_bounds__(128, 4) delay_sums_pass_kernel(const DelaySumsArgs a)
 {
@@ -132,6 +133,10 @@ static __global__ void __launch_bounds__(128, 4) delay_sums_pass_kernel(const De
             if (a.store) {
                 dst[0] = lo;
                 dst[32] = hi;
+            } else if (a.T64) {
+                double *d = a.T64 + ((size_t)cur_slot * 64 + lane) * 4;
+#pragma unroll
+                for (int i = 0; i < 8; ++i) atomicAdd(d + (i < 4 ? i : 128 + i - 4), (double)t[i]);
             } else {
                 red_add_v4(dst, lo);
                 red_add_v4(dst + 32, hi);
@@ -214,18 +219,28 @@ static __global__ void __launch_bounds__(128, 4) delay_sums_pass_kernel(const De
     cp_async_wait<0>();
 }
 
+// FP64 products to the FP32 ones that the iterations read (four a thread)
+static __global__ void delay_round_kernel(long n4, const double2 *__restrict__ src, float4 *__restrict__ dst)
+{
+    for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += (long)gridDim.x * blockDim.x) {
+        const double2 a = src[2 * i], b = src[2 * i + 1];
+        dst[i] = make_float4((float)a.x, (float)a.y, (float)b.x, (float)b.y);
+    }
+}
+
 // One iteration's right-hand sides: a CTA per (time interval, 32-channel chunk), lanes over the
 // channels.  The antennas' gains at those channels are evaluated once into shared memory; the pairs
 // are walked in 8 x 8 tiles of antennas handed out to the warps, so that the eight q sums of a row of
-// a tile stay in registers and only their totals go to the shared sums.  T streams at 1 KB a
-// pair with eight 16-byte loads a lane in flight; nothing else comes from DRAM.
+// a tile stay in registers and only their totals go to the shared sums (FP64: the FP32 terms of 8
+// pairs at most).  T streams at 1 KB a pair with eight 16-byte loads a lane in flight; nothing else
+// comes from DRAM.
 constexpr int DT = 8;                       // antennas of a tile's side
 
 static __global__ void __launch_bounds__(256, 2) delay_sums_iter_kernel(const DelaySumsArgs a)
 {
     if (__ldg(a.n_active) == 0) return;
     extern __shared__ float4 s_gains[];     // [n_ant][32] (g_X, g_Y)
-    float2 *s_r = reinterpret_cast<float2 *>(s_gains + (size_t)a.n_ant * 32);   // [n_ant][32] (r_X, r_Y)
+    double *s_r = reinterpret_cast<double *>(s_gains + (size_t)a.n_ant * 32);   // [n_ant][2][32] r_X, r_Y
     __shared__ int s_tile;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const int tint = blockIdx.x / a.n_chunks, chunk = blockIdx.x % a.n_chunks, na = a.n_ant;
@@ -240,7 +255,7 @@ static __global__ void __launch_bounds__(256, 2) delay_sums_iter_kernel(const De
             const double *u = a.params + ((size_t)bin * na + i) * 4;
             const float2 gx = delay_gain_f32(u[0], u[1], w), gy = delay_gain_f32(u[2], u[3], w);
             s_gains[i * 32 + lane] = make_float4(gx.x, gx.y, gy.x, gy.y);
-            s_r[i * 32 + lane] = make_float2(0.f, 0.f);
+            s_r[i * 64 + lane] = s_r[i * 64 + 32 + lane] = 0.0;
         }
     }
     if (threadIdx.x == 0) s_tile = 0;
@@ -291,14 +306,14 @@ static __global__ void __launch_bounds__(256, 2) delay_sums_iter_kernel(const De
                     rq[h + j].y -= z01 + z11;
                 }
             }
-            atomicAdd(&s_r[p * 32 + lane].x, rp.x);
-            atomicAdd(&s_r[p * 32 + lane].y, rp.y);
+            atomicAdd(&s_r[p * 64 + lane], (double)rp.x);
+            atomicAdd(&s_r[p * 64 + 32 + lane], (double)rp.y);
         }
 #pragma unroll
         for (int j = 0; j < DT; ++j)
             if (q0 + j < na) {
-                atomicAdd(&s_r[(q0 + j) * 32 + lane].x, rq[j].x);
-                atomicAdd(&s_r[(q0 + j) * 32 + lane].y, rq[j].y);
+                atomicAdd(&s_r[(q0 + j) * 64 + lane], (double)rq[j].x);
+                atomicAdd(&s_r[(q0 + j) * 64 + 32 + lane], (double)rq[j].y);
             }
     }
     __syncthreads();
@@ -308,14 +323,20 @@ static __global__ void __launch_bounds__(256, 2) delay_sums_iter_kernel(const De
     const int b0 = __shfl_sync(WARP_ALL, bin, __ffs(acts) - 1);
     const bool one = __all_sync(WARP_ALL, !act || bin == b0);
     for (int i = warp; i < na; i += nw) {
-        const float2 r = act ? s_r[i * 32 + lane] : make_float2(0.f, 0.f);
-        float v[4] = { r.x, r.x * om, r.y, r.y * om };
+        const double rx = act ? s_r[i * 64 + lane] : 0.0, ry = act ? s_r[i * 64 + 32 + lane] : 0.0;
+        const double w[4] = { rx, rx * om, ry, ry * om };
+        float v[4], tail[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            v[e] = (float)w[e];
+            tail[e] = isfinite(v[e]) ? (float)(w[e] - (double)v[e]) : 0.f;
+        }
         if (one) {
-            const double tot = reduce_words<4>(v, lane);
+            const double tot = reduce_words<4>(v, tail, lane);
             if ((lane & 7) == 0) atomicAdd(a.acc + ((size_t)b0 * na + i) * KG_SUMS + 6 + (lane >> 3), tot);
         } else if (act) {
 #pragma unroll
-            for (int e = 0; e < 4; ++e) atomicAdd(a.acc + ((size_t)bin * na + i) * KG_SUMS + 6 + e, (double)v[e]);
+            for (int e = 0; e < 4; ++e) atomicAdd(a.acc + ((size_t)bin * na + i) * KG_SUMS + 6 + e, w[e]);
         }
     }
 }
@@ -350,9 +371,17 @@ cudaError_t dsum_launch_pass(const qc::DelaySumsArgs &a, int ok, int sm_count, c
     return launch_dsum_pass_ok<qc::KIND_FULL>(a, sm_count, st);
 }
 
+cudaError_t dsum_launch_round(size_t words, const double *src, float4 *dst, int sm_count, cudaStream_t st)
+{
+    const long n4 = (long)(words / 4);
+    const int grid = (int)std::max(1L, std::min((n4 + 255) / 256, (long)sm_count * 16));
+    qc::delay_round_kernel<<<grid, 256, 0, st>>>(n4, (const double2 *)src, dst);
+    return cudaGetLastError();
+}
+
 cudaError_t dsum_launch_iter(const qc::DelaySumsArgs &a, cudaStream_t st)
 {
-    const int smem = a.n_ant * 32 * (int)(sizeof(float4) + sizeof(float2));
+    const int smem = a.n_ant * 32 * (int)(sizeof(float4) + 2 * sizeof(double));
     const cudaError_t e = cudaFuncSetAttribute(qc::delay_sums_iter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     qc::delay_sums_iter_kernel<<<a.n_tint * a.n_chunks, 256, smem, st>>>(a);

@@ -6,6 +6,8 @@
 
 namespace qc {
 
+// antennas whose gains and right-hand sides of 32 channels fit a CTA's shared memory (1 KB each)
+constexpr int DSUM_MAX_ANT = 220;
 constexpr int KG_HSUM = 6;           // FP64 words of the constant sums per (interval, antenna)
 
 struct DelaySumsArgs {
@@ -26,6 +28,7 @@ struct DelaySumsArgs {
     const int *fmap;                 // [n_chan] parameter interval of each channel
     const float *omega;              // [n_chan] 2 pi nu - omega_ref
     float4 *T;                       // [n_tint][n_chunks][n_up][2][32]
+    double *T64;                     // the same in FP64, added to instead, or null (one addition a slot)
     double *hsum;                    // [bins][n_ant][KG_HSUM]
     // iterations
     int n_tint;
@@ -39,4 +42,5 @@ struct DelaySumsArgs {
 } // namespace qc
 
 cudaError_t dsum_launch_pass(const qc::DelaySumsArgs &a, int ok, int sm_count, cudaStream_t st);
+cudaError_t dsum_launch_round(size_t words, const double *src, float4 *dst, int sm_count, cudaStream_t st);
 cudaError_t dsum_launch_iter(const qc::DelaySumsArgs &a, cudaStream_t st);

@@ -106,7 +106,7 @@ struct TermBufs {
     Buf params0;   // divergence flagging: the FP64 parameters before the solve
     Buf mom;       // a term solved from sums: sums per (interval, unordered pair), bytes per interval
     SumsPlan sums; // the route of the current call
-    Buf dsum_t;    // delay terms solved from products: T [n_tint][chunks][pairs][2][32] float4
+    Buf dsum_t;    // delay terms solved from products: T [n_tint][chunks][pairs][2][32] float4 (then in FP64)
     Buf dsum_h;    //   double [bins][ant][KG_HSUM]
     Buf dfmap;     // delay terms: int [n_chan] parameter interval of each channel
     Buf dfr;       // delay terms: int2 [n_fint] first and last channel of each interval
@@ -279,6 +279,7 @@ struct qc_ctx {
     int plan_counters(const qc_term *terms, int n_terms, int n_epochs);
     int size_mom_rows();
     int ensure_mom_rows(cudaStream_t st);
+    bool products_once(const qc_term &t) const;
     int plan_delay_sums(const qc_term *terms, int n_terms, int n, const qc_opts *o, bool &use);
     qc::DelaySumsArgs delay_sums_args(const qc_term *terms, int n_terms, int n, const qc::Chain &chain);
     int sums_args(const qc_term *terms, int n_terms, int n, const qc::Chain &chain, cudaStream_t st, qc::MomArgs &ma,

@@ -10,7 +10,7 @@ import pytest
 
 import oracle as O
 import test_gpu_moments as tmo
-from paper_2412_10072_gb300 import qc
+from paper_2412_10072_gb300 import qc, synth
 
 pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
@@ -101,3 +101,54 @@ def test_sums_hold_their_precision(shape, m16):
     O.solve(P, [o], damping_mode=1)
     err = np.linalg.norm(np.asarray(T.gains, dtype=o.params.dtype) - o.params) / np.linalg.norm(o.params)
     assert err < 6e-8, err
+
+
+def _delay_case(seed, n_ant, n_time, n_chan, t_int, twice=False):
+    """A delay term over intervals of t_int times, with truth as start: data, terms of both sides."""
+    rng = np.random.default_rng(seed)
+    p, q = synth.baselines(n_ant)
+    ant1, ant2 = np.tile(p, n_time), np.tile(q, n_time)
+    tidx = np.repeat(np.arange(n_time, dtype=np.int32), p.size)
+    if twice:                                       # a second row of every pair and time, the other way round
+        ant1, ant2, tidx = np.concatenate([ant1, ant2]), np.concatenate([ant2, ant1]), np.tile(tidx, 2)
+    nu = np.linspace(0.9, 1.7, n_chan)
+    tm = synth.interval_map(n_time, t_int)
+    nt = int(tm[-1]) + 1
+    par = np.zeros((nt, 1, n_ant, 4), np.float32)
+    par[..., 0::2] = rng.uniform(-1, 1, (nt, 1, n_ant, 2))
+    par[..., 1::2] = rng.uniform(-0.1, 0.1, (nt, 1, n_ant, 2))
+    ph = par[tm, 0][:, None, :, 0::2] + 2 * np.pi * nu[None, :, None, None] * par[tm, 0][:, None, :, 1::2]
+    g = np.exp(1j * ph)                             # [time][chan][ant][2]
+    shp = (ant1.size, n_chan, 4)
+    model = np.ones(shp) * rng.uniform(0.5, 1.5, shp)
+    gp, gq = g[tidx, :, ant1], g[tidx, :, ant2].conj()
+    data = model * (gp[..., [0, 0, 1, 1]] * gq[..., [0, 1, 0, 1]])
+    start = (par + rng.normal(0, 1, par.shape) * [0.1, 0.01, 0.1, 0.01]).astype(np.float32)
+    args = (data.astype(np.complex64), model.astype(np.complex64), rng.uniform(0.5, 1.5, shp).astype(np.float32),
+            np.zeros(shp[:2], np.uint8), ant1.astype(np.int32), ant2.astype(np.int32), tidx, n_ant, n_time)
+    fm = np.zeros(n_chan, np.int32)
+    G = lambda: qc.Term("delay", tm, fm, nt, 1, n_ant, gains=start, max_iter=8, tol=0.0, chan_freq=nu)  # noqa: E731
+    o = O.OracleTerm("delay", tm, fm, nt, 1, n_ant, params=start.astype(np.float64), chan_freq=nu, max_iter=8, tol=0.0)
+    O.solve_term(O.OracleProblem(*args), [o], 0, damping_mode=1)
+
+    def phases(u):                                  # at every channel, against antenna 0
+        v = np.asarray(u, np.float64)[:, 0][:, None, :, 0::2] + \
+            2 * np.pi * nu[None, :, None, None] * np.asarray(u, np.float64)[:, 0][:, None, :, 1::2]
+        return v - v[:, :, :1]
+    return args, G, phases(o.params), phases
+
+
+@pytest.mark.parametrize("n_ant,n_time,n_chan,t_int,twice", [(3, 20000, 4, 20000, False), (5, 300, 33, 100, True),
+                                                             (9, 64, 40, 2, False), (9, 16, 40, 1, True),
+                                                             (220, 4, 3, 2, False), (221, 4, 3, 2, False)])
+def test_delay_products_hold_their_precision(n_ant, n_time, n_chan, t_int, twice):
+    """Products of many samples and of few, rows of both orientations, antennas at the limit of a
+    CTA's shared memory and beyond it.  A phase at a channel carries the rounding of its two float32
+    parameters, 2^-25 of 1 and of 10.7 x 0.1, and that of antenna 0: 7e-8 (rms); 1e-7."""
+    args, G, want, phases = _delay_case(11, n_ant, n_time, n_chan, t_int, twice)
+    S = qc.Solver(*args)
+    T = G()
+    S.solve([T])
+    S.close()
+    err = np.sqrt(np.mean((phases(T.gains) - want) ** 2))
+    assert err < 1e-7, err
