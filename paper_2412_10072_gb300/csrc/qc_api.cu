@@ -590,27 +590,29 @@ int qc_ctx::expand_terms(const qc_term *terms, int n_terms, std::vector<qc_term>
         if ((rc = ensure(B.dfmap, nbytes<int>(std::max(1, n_chan))))) return rc;
         if ((rc = ensure(B.dfr, nbytes<int2>(t.n_fint)))) return rc;
         if ((rc = ensure(B.dnu, nbytes<double>(std::max(1, n_chan))))) return rc;
-        if ((rc = ensure(B.domega, nbytes<float>(std::max(1, n_chan))))) return rc;
+        if ((rc = ensure(B.domega, nbytes<float>(2 * (size_t)std::max(1, n_chan))))) return rc;
         B.hufmap.assign(t.f_map, t.f_map + n_chan);
         double mean_nu = 0;
         for (int ch = 0; ch < n_chan; ++ch) mean_nu += t.chan_freq[ch];
         B.omega_ref = n_chan ? DELAY_TWO_PI * (mean_nu / n_chan) : 0.0;
-        std::vector<float> om(n_chan);
+        std::vector<float> om(2 * (size_t)n_chan);      // heads, then tails
         B.hom_sums.assign(t.n_fint, make_double2(0.0, 0.0));
-        B.om_max = 0.f;
+        B.om_max = 0.0;
         for (int ch = 0; ch < n_chan; ++ch) {
-            om[ch] = (float)(DELAY_TWO_PI * t.chan_freq[ch] - B.omega_ref);
-            B.om_max = std::max(B.om_max, std::fabs(om[ch]));
+            const double w = DELAY_TWO_PI * t.chan_freq[ch] - B.omega_ref;
+            om[ch] = (float)w;
+            om[n_chan + ch] = (float)(w - (double)om[ch]);
+            B.om_max = std::max(B.om_max, std::fabs(w));
             double2 &m = B.hom_sums[t.f_map[ch]];
-            m.x += om[ch];
-            m.y += (double)om[ch] * om[ch];
+            m.x += w;
+            m.y += w * w;
         }
         if ((rc = ensure(B.dom_sums, nbytes<double2>(t.n_fint)))) return rc;
         CK(to_device(B.dom_sums.ptr, B.hom_sums.data(), nbytes<double2>(t.n_fint), st));
         if (n_chan) {
             CK(to_device(B.dfmap.ptr, t.f_map, nbytes<int>(n_chan), st));
             CK(to_device(B.dnu.ptr, t.chan_freq, nbytes<double>(n_chan), st));
-            CK(to_device(B.domega.ptr, om.data(), nbytes<float>(n_chan), st));
+            CK(to_device(B.domega.ptr, om.data(), nbytes<float>(om.size()), st));
         }
         CK(to_device(B.dfr.ptr, B.hfr.data(), nbytes<int2>(t.n_fint), st));
         xt[j].type = QC_TERM_DIAG;
@@ -1987,6 +1989,7 @@ int qc_ctx::solve_term(const qc_term *terms, int n_terms, int n, Chain chain, co
         if (dsum) {
             dua.hsum = (const double *)B.dsum_h.ptr;
             dua.omega = (const float *)B.domega.ptr;
+            dua.omega_lo = dua.omega + n_chan;
             dua.om_sums = (const double2 *)B.dom_sums.ptr;
             dua.om_max = B.om_max;
         }

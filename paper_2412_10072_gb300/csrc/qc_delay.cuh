@@ -15,6 +15,7 @@
 // parameters, re-evaluates the channel table and tests convergence on the gains.
 #pragma once
 #include "qc_kernels.cuh"
+#include "qc_sums.cuh"
 
 namespace qc {
 
@@ -106,9 +107,9 @@ struct DelayUpdArgs {
     // a term solved from products (qc_delay_sums.cu): the h sums [bins][n_ant][6], the same for every
     // iteration (else null: they are in acc); the channel table is then left to the end of the solve
     const double *hsum;
-    const float *omega;       // [n_chan] omega' = 2 pi nu - omega_ref (with hsum)
+    const float *omega, *omega_lo;   // [n_chan] omega' = 2 pi nu - omega_ref as head and tail (with hsum)
     const double2 *om_sums;   // [n_fint] sum of omega', of omega'^2 over the interval's channels (with hsum)
-    float om_max;             // largest |omega'|
+    double om_max;            // largest |omega'|
 };
 
 // One block per parameter interval (time interval x frequency interval), threads over antennas.
@@ -140,6 +141,21 @@ __device__ __forceinline__ int delay_solve_pair(double a0, double a1, double a2,
     y[2] = (c2 * r2 - c1 * r3) * ic;
     y[3] = (c0 * r3 - c1 * r2) * ic;
     return 0;
+}
+
+__device__ __forceinline__ float4 delay_split(double a, double b)
+{
+    const float x = (float)a, y = (float)b;
+    return make_float4(x, (float)(a - (double)x), y, (float)(b - (double)y));
+}
+
+// a + b om, each as head and tail, rounded to float once
+__device__ __forceinline__ float delay_phase(float4 ab, float2 om)
+{
+    const float p = __fmul_rn(ab.z, om.x), r = __fmaf_rn(ab.z, om.x, -p);
+    float s, e;
+    two_sum(ab.x, p, s, e);
+    return s + (e + (r + fmaf(ab.z, om.y, fmaf(ab.w, om.x, ab.y))));
 }
 
 // Counts and convergence of an interval, by the whole block (one thread adding up the counts of 512
@@ -286,46 +302,51 @@ static __global__ void __launch_bounds__(128) delay_update_kernel(const DelayUpd
     }
     if (SUMS && !u.hsum) return;       // delay_chan_kernel follows
     if (SUMS) {
-        // the change of the gains, (antenna, channel) by (antenna, channel) over the block's threads.
-        // The phase change (d0 + d1 w_ref) + d1 (w - w_ref) is formed in FP64 at the band's centre
-        // and in FP32 away from it: 0.84 ms a launch with FP64 phases and the channel table on the
-        // 300 x 512 x 64 grid
+        // the change of the gains, (antenna, channel) by (antenna, channel) over the block's threads: the
+        // phase change of a channel from the FP64 changes as head and tail (an ulp of float, as an FP64
+        // phase rounded to it; 64 antennas, 75 x 512: 10.5 ms a solve with FP64 phases)
         __syncthreads();
         const int nch = fr.y - fr.x + 1;
         for (int a0 = 0; a0 < d.n_ant; a0 += 128) {
-            __shared__ float4 s_e[128];
+            __shared__ float4 s_f[128][2];          // head and tail of the change at the centre, of its slope
             const int na = min(128, d.n_ant - a0);
-            if ((int)threadIdx.x < na) {
-                double *A = u.acc + ((size_t)bin * d.n_ant + a0 + threadIdx.x) * KG_SUMS;
-                s_e[threadIdx.x] = make_float4((float)(A[0] + A[1] * d.omega_ref), (float)A[1],
-                                               (float)(A[2] + A[3] * d.omega_ref), (float)A[3]);
-                A[0] = A[1] = A[2] = A[3] = 0.0;
-            }
-            __syncthreads();
-            // phase changes below 1e-3 over the whole interval (all but the first iterations): 4 sin^2
-            // of half the change is its square to 1e-7, and the sum over the channels is closed
             bool small = true;
+            double e[4] = { 0, 0, 0, 0 };
             if ((int)threadIdx.x < na) {
-                const float4 e = s_e[threadIdx.x];
-                const float wmax = u.om_max;
-                small = fabsf(e.x) + fabsf(e.y) * wmax < 1e-3f && fabsf(e.z) + fabsf(e.w) * wmax < 1e-3f;
+                // about the band's centre: A0 + A1 w = (A0 + A1 w_ref) + A1 w'
+                double *A = u.acc + ((size_t)bin * d.n_ant + a0 + threadIdx.x) * KG_SUMS;
+                e[0] = A[0] + A[1] * d.omega_ref;
+                e[1] = A[1];
+                e[2] = A[2] + A[3] * d.omega_ref;
+                e[3] = A[3];
+                A[0] = A[1] = A[2] = A[3] = 0.0;
+                s_f[threadIdx.x][0] = delay_split(e[0], e[1]);
+                s_f[threadIdx.x][1] = delay_split(e[2], e[3]);
+                // changes below 5e-4 over the whole interval (all but the first iterations): 4 sin^2 of half
+                // the change is its square to 2e-8, and the sum over the channels is closed
+                small = fabs(e[0]) + fabs(e[1]) * u.om_max < 5e-4 && fabs(e[2]) + fabs(e[3]) * u.om_max < 5e-4;
             }
             if (__syncthreads_and(small)) {
                 if ((int)threadIdx.x < na) {
-                    const float4 e = s_e[threadIdx.x];
                     const double2 m = u.om_sums[fu];
-                    const double x0 = e.x, x1 = e.y, y0 = e.z, y1 = e.w;
-                    num += x0 * x0 * nch + 2.0 * x0 * x1 * m.x + x1 * x1 * m.y;
-                    num += y0 * y0 * nch + 2.0 * y0 * y1 * m.x + y1 * y1 * m.y;
+                    num += e[0] * e[0] * nch + 2.0 * e[0] * e[1] * m.x + e[1] * e[1] * m.y;
+                    num += e[2] * e[2] * nch + 2.0 * e[2] * e[3] * m.x + e[3] * e[3] * m.y;
                 }
                 continue;
             }
             for (int i = threadIdx.x; i < na * nch; i += blockDim.x) {
                 const int ant = i / nch, c = fr.x + (i - ant * nch);
-                const float4 e = s_e[ant];
-                const float om = __ldg(u.omega + c);
-                const float s0 = sinf(0.5f * fmaf(e.y, om, e.x)), s1 = sinf(0.5f * fmaf(e.w, om, e.z));
-                num += 4.0 * (double)fmaf(s0, s0, s1 * s1);
+                const float2 om = make_float2(__ldg(u.omega + c), __ldg(u.omega_lo + c));
+                const float4 x = s_f[ant][0], y = s_f[ant][1];
+                const float px = delay_phase(x, om), py = delay_phase(y, om);
+                if (fabsf(px) < 8.f && fabsf(py) < 8.f) {
+                    const float s0 = sinf(0.5f * px), s1 = sinf(0.5f * py);
+                    num += 4.0 * ((double)s0 * s0 + (double)s1 * s1);
+                } else {
+                    const double w = (double)om.x + (double)om.y;
+                    num += delay_change2(((double)x.x + x.y) + ((double)x.z + x.w) * w) +
+                           delay_change2(((double)y.x + y.y) + ((double)y.z + y.w) * w);
+                }
             }
             __syncthreads();
         }

@@ -111,10 +111,10 @@ struct TermBufs {
     Buf dfmap;     // delay terms: int [n_chan] parameter interval of each channel
     Buf dfr;       // delay terms: int2 [n_fint] first and last channel of each interval
     Buf dnu;       // delay terms: double [n_chan] channel frequencies
-    Buf domega;    // delay terms: float [n_chan] 2 pi nu - omega_ref
+    Buf domega;    // delay terms: float [2][n_chan] 2 pi nu - omega_ref as head and tail
     Buf dom_sums;  // delay terms: double2 [n_fint] sums of omega' and omega'^2 over the channels
     std::vector<double2> hom_sums;
-    float om_max = 0;
+    double om_max = 0;
     double omega_ref = 0;     // delay terms: 2 pi times the mean channel frequency
     std::vector<int2> hfr;    // host copy of dfr (its size is the term's n_fint)
     std::vector<int> hufmap;  // delay terms: host copy of the term's own f_map

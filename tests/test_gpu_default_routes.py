@@ -103,7 +103,7 @@ def test_sums_hold_their_precision(shape, m16):
     assert err < 6e-8, err
 
 
-def _delay_case(seed, n_ant, n_time, n_chan, t_int, twice=False):
+def _delay_case(seed, n_ant, n_time, n_chan, t_int, twice=False, oracle=True):
     """A delay term over intervals of t_int times, with truth as start: data, terms of both sides."""
     rng = np.random.default_rng(seed)
     p, q = synth.baselines(n_ant)
@@ -129,7 +129,8 @@ def _delay_case(seed, n_ant, n_time, n_chan, t_int, twice=False):
     fm = np.zeros(n_chan, np.int32)
     G = lambda: qc.Term("delay", tm, fm, nt, 1, n_ant, gains=start, max_iter=8, tol=0.0, chan_freq=nu)  # noqa: E731
     o = O.OracleTerm("delay", tm, fm, nt, 1, n_ant, params=start.astype(np.float64), chan_freq=nu, max_iter=8, tol=0.0)
-    O.solve_term(O.OracleProblem(*args), [o], 0, damping_mode=1)
+    if oracle:
+        O.solve_term(O.OracleProblem(*args), [o], 0, damping_mode=1)
 
     def phases(u):                                  # at every channel, against antenna 0
         v = np.asarray(u, np.float64)[:, 0][:, None, :, 0::2] + \
@@ -152,3 +153,22 @@ def test_delay_products_hold_their_precision(n_ant, n_time, n_chan, t_int, twice
     S.close()
     err = np.sqrt(np.mean((phases(T.gains) - want) ** 2))
     assert err < 1e-7, err
+
+
+@pytest.mark.parametrize("n_ant,tol", [(7, 1e-2), (7, 1e-4), (7, 1e-6), (130, 1e-3), (130, 1e-5)])
+def test_delay_convergence(n_ant, tol):
+    """The iterations of every interval, and with them the convergence test on the change of the
+    gains (more antennas than the block of the update takes at once, large and small changes), are
+    those of the chain rule per sample."""
+    args, G, _, phases = _delay_case(12, n_ant, 24, 50, 1 if n_ant < 100 else 6, oracle=False)
+    out = []
+    for kernel in (0, 3):
+        S = qc.Solver(*args)
+        T = G()
+        T.max_iter, T.tol = 12, tol
+        S.solve([T], kernel=kernel)
+        S.close()
+        out.append(T)
+    assert np.array_equal(out[0].iters, out[1].iters)
+    assert 1 < out[0].iters.min() and out[0].iters.max() < 12
+    assert np.sqrt(np.mean((phases(out[0].gains) - phases(out[1].gains)) ** 2)) < 2e-7
