@@ -15,12 +15,25 @@ __device__ __forceinline__ int mad_digit(unsigned key, int level)
 // the digits above a level
 __device__ __forceinline__ unsigned mad_above(int level) { return level == 0 ? 0u : (level == 1 ? 0x7ff00000u : 0x7ffffc00u); }
 
-// s + e += x, the rounding error of s carried in e
-__device__ __forceinline__ void comp_add(float &s, float &e, float x)
+// tot += the eight terms, summed as head and tail: exact to the last bits of the tail, two conversions to
+// FP64 instead of eight.  Where the head overflows (or a term is infinite or NaN), term by term.
+__device__ __forceinline__ void add_terms(double &tot, const float4 &a, const float4 &b)
 {
-    float r;
-    two_sum(s, x, s, r);
-    e += r;
+    float s = a.x, e = 0.f;
+    const float t[7] = { a.y, a.z, a.w, b.x, b.y, b.z, b.w };
+#pragma unroll
+    for (int i = 0; i < 7; ++i) {
+        float r;
+        two_sum(s, t[i], s, r);
+        e += r;
+    }
+    if (isfinite(s) && isfinite(e)) {
+        tot += (double)s + (double)e;
+    } else {
+        tot += (double)a.x;
+#pragma unroll
+        for (int i = 0; i < 7; ++i) tot += (double)t[i];
+    }
 }
 
 // A warp per row, two 32-channel chunks in flight: the chunks' data, model, weights and flags are
@@ -28,9 +41,9 @@ __device__ __forceinline__ void comp_add(float &s, float &e, float x)
 // the sample's key -- the bits of z = sqrt(sum_c w_c |r_c|^2), every operation rounded, in a fixed
 // order, so that the residual (32 B a sample) is neither written nor read again.  (Counting the
 // first digit here too doubled the kernel: most keys share a few bins; a pass over the keys, 4 B a
-// sample, takes 65 us of the 1.3 ms.)  chi^2 is carried per lane as an FP32 head and tail and joined in FP64 per
-// row: converting every term to FP64 took longer than the memory (FP64 runs at 2 lanes a
-// cycle and SM).  64 antennas, 60 x 509, residual written: 1.79 ms a call before, 1.52 now (the kernel
+// sample, takes 65 us of the 1.3 ms.)  chi^2 is summed in FP64 per lane, the eight
+// terms of two samples at a time (add_terms): converting every term to FP64 took longer than the
+// memory (FP64 runs at 2 lanes a cycle and SM).  64 antennas, 60 x 509, residual written: 1.79 ms a call before, 1.52 now (the kernel
 // 1.34, 5.2 TB/s).
 template <bool M16, bool MAD, int NT>
 static __global__ void __launch_bounds__(256, 2) residual_kernel(const ResArgs a, unsigned *__restrict__ keys, MadState *state)
@@ -56,7 +69,6 @@ static __global__ void __launch_bounds__(256, 2) residual_kernel(const ResArgs a
 #pragma unroll
         for (int j = 0; j < NT; ++j) tint[j] = cross && j < C.n_terms ? __ldg(C.t[j].t_map + meta.z) : 0;
         const float sc = M16 && cross ? __ldg(D.bl_scale + meta.w) : 1.f;
-        float hi = 0.f, lo = 0.f;
         auto load = [&](int c) {
             Samp x;
             x.ok = false;
@@ -76,7 +88,9 @@ static __global__ void __launch_bounds__(256, 2) residual_kernel(const ResArgs a
             }
             return x;
         };
+        float4 chi = make_float4(0, 0, 0, 0);     // the last sample's terms of chi^2
         auto finish = [&](int c, const Samp &x) {
+            if constexpr (!MAD) chi = make_float4(0, 0, 0, 0);
             if (c >= D.n_chan) return;
             const size_t s = base + c;
             if (!x.ok) {
@@ -117,10 +131,8 @@ static __global__ void __launch_bounds__(256, 2) residual_kernel(const ResArgs a
                 keys[s] = __float_as_uint(__fsqrt_rn(acc));
                 ++used;
             } else {
-                comp_add(hi, lo, __fmul_rn(w.x, cnorm2(r.a)));
-                comp_add(hi, lo, __fmul_rn(w.y, cnorm2(r.b)));
-                comp_add(hi, lo, __fmul_rn(w.z, cnorm2(r.c)));
-                comp_add(hi, lo, __fmul_rn(w.w, cnorm2(r.d)));
+                chi = make_float4(__fmul_rn(w.x, cnorm2(r.a)), __fmul_rn(w.y, cnorm2(r.b)), __fmul_rn(w.z, cnorm2(r.c)),
+                                  __fmul_rn(w.w, cnorm2(r.d)));
                 if (a.resid) {
                     __stcs(a.resid + 2 * s, make_float4(r.a.x, r.a.y, r.b.x, r.b.y));
                     __stcs(a.resid + 2 * s + 1, make_float4(r.c.x, r.c.y, r.d.x, r.d.y));
@@ -131,10 +143,10 @@ static __global__ void __launch_bounds__(256, 2) residual_kernel(const ResArgs a
             const Samp x0 = load(c);
             const Samp x1 = load(c + 32);
             finish(c, x0);
+            const float4 t0 = chi;
             finish(c + 32, x1);
+            if constexpr (!MAD) add_terms(tot, t0, chi);
         }
-        // an infinite or NaN head has no tail
-        if constexpr (!MAD) tot += isfinite(hi) ? (double)hi + (double)lo : (double)hi;
     }
     if constexpr (MAD) {
         for (int d = 16; d > 0; d >>= 1) used += __shfl_down_sync(0xffffffffu, used, d);

@@ -172,3 +172,34 @@ def test_delay_convergence(n_ant, tol):
     assert np.array_equal(out[0].iters, out[1].iters)
     assert 1 < out[0].iters.min() and out[0].iters.max() < 12
     assert np.sqrt(np.mean((phases(out[0].gains) - phases(out[1].gains)) ** 2)) < 2e-7
+
+
+@pytest.mark.parametrize("n_chan", [1, 33, 70])
+def test_chi2_beyond_float(n_chan):
+    """chi^2 is a 64-bit sum of float32 terms: finite where a row's terms together exceed the largest
+    float32, with every term itself representable; NaN and infinite terms stay what they are."""
+    rng = np.random.default_rng(n_chan)
+    n_ant, n_time = 4, 3
+    p, q = synth.baselines(n_ant)
+    ant1, ant2 = np.tile(p, n_time).astype(np.int32), np.tile(q, n_time).astype(np.int32)
+    tidx = np.repeat(np.arange(n_time, dtype=np.int32), p.size)
+    shp = (ant1.size, n_chan, 4)
+    data = ((1 + rng.random(shp)) * 1e16 * np.exp(1j * rng.uniform(0, 6, shp))).astype(np.complex64)
+    weight = rng.uniform(2e5, 8e5, shp).astype(np.float32)           # terms of 2e37 to 3.2e38
+
+    def chi2(d, w):
+        S = qc.Solver(d, np.zeros(shp, np.complex64), w, np.zeros(shp[:2], np.uint8), ant1, ant2, tidx, n_ant, n_time)
+        T = qc.Term("diag", np.zeros(n_time, np.int32), np.zeros(n_chan, np.int32), 1, 1, n_ant, solve=False)
+        v = S.residual([T])
+        S.close()
+        return v
+
+    term = weight * (data.real.astype(np.float32) ** 2 + data.imag.astype(np.float32) ** 2)
+    assert np.isfinite(term).all() and (n_chan == 1 or term.sum(dtype=np.float64) > 4e39)
+    want = float((weight.astype(np.float64) * np.abs(data.astype(np.complex128)) ** 2).sum())
+    assert abs(chi2(data, weight) - want) <= 2e-7 * want             # four float32 roundings a term, averaged
+    bad = data.copy()
+    bad[5, n_chan // 2, 1] = np.nan
+    assert np.isnan(chi2(bad, weight))
+    bad[5, n_chan // 2, 1] = np.inf
+    assert np.isinf(chi2(bad, weight)) or np.isnan(chi2(bad, weight))
