@@ -148,7 +148,6 @@ int grid_for(long n, int block, int sm)
 qc_ctx::~qc_ctx()
 {
     for (auto &b : tb) if (b.exec) cudaGraphExecDestroy(b.exec);
-    if (pin_open && pin_stream) cudaStreamSynchronize(pin_stream);
     for (void *p : owned) qc_dev_free(p);
     for (auto &b : pin_blocks) cudaFreeHost(b.ptr);
     for (auto e : events) cudaEventDestroy(e);
@@ -156,15 +155,21 @@ qc_ctx::~qc_ctx()
     if (own_stream) cudaStreamDestroy(own_stream);
 }
 
-cudaError_t qc_ctx::pin_begin(cudaStream_t st)
+void qc_ctx::pin_begin()
 {
-    cudaError_t e = cudaSuccess;
-    if (pin_open) e = cudaStreamSynchronize(pin_stream);
     pin_block = pin_used = 0;
     pin_outs.clear();
     pin_open = true;
-    pin_stream = st;
-    return e;
+}
+
+// A call that ends before pin_end has its copies finished here, while its stream still exists: the stream
+// is the caller's, and nothing keeps its handle beyond the call.
+PinScope::~PinScope()
+{
+    if (!c->pin_open) return;
+    cudaStreamSynchronize(st);
+    c->pin_outs.clear();
+    c->pin_open = false;
 }
 
 void *qc_ctx::pin_get(size_t bytes)
@@ -730,7 +735,7 @@ extern "C" int qc_residual(qc_ctx *c, const qc_term *terms, int32_t n_terms, voi
     int rc = c->validate_terms(terms, n_terms, false);
     if (rc) return rc;
     cudaStream_t st = c->own_stream;
-    CK(c->pin_begin(st));
+    PinScope pins(c, st);
     std::vector<qc_term> xt;
     if ((rc = c->expand_terms(terms, n_terms, xt, st))) return rc;
     Chain chain;
@@ -930,7 +935,7 @@ extern "C" int qc_solve(qc_ctx *c, qc_term *terms, int32_t n_terms, const qc_opt
     cudaEvent_t ev0, ev1;
     if ((rc = c->get_event(0, ev0)) || (rc = c->get_event(1, ev1))) return rc;
     CK(cudaEventRecord(ev0, st));
-    CK(c->pin_begin(st));
+    PinScope pins(c, st);
     std::vector<qc_term> xt;     // the kernels' view of the terms (delay terms per channel)
     if ((rc = c->expand_terms(terms, n_terms, xt, st))) return rc;
     Chain chain;
@@ -1054,7 +1059,7 @@ extern "C" int qc_solve(qc_ctx *c, qc_term *terms, int32_t n_terms, const qc_opt
                     if ((rc = c->copy_pending(st))) return rc;
                     CK(cudaStreamSynchronize(st));
                     c->pin_end();
-                    CK(c->pin_begin(st));
+                    c->pin_begin();
                     if ((rc = c->collect_sums(S, n_iter_max))) return rc;
                 }
                 continue;
@@ -2230,7 +2235,7 @@ extern "C" int qc_mad_flag(qc_ctx *c, const qc_term *terms, int32_t n_terms, dou
     int rc = c->validate_terms(terms, n_terms, false);
     if (rc) return rc;
     cudaStream_t st = c->own_stream;
-    CK(c->pin_begin(st));
+    PinScope pins(c, st);
     std::vector<qc_term> xt;
     if ((rc = c->expand_terms(terms, n_terms, xt, st))) return rc;
     Chain chain;

@@ -237,10 +237,9 @@ struct qc_ctx {
     struct PinOut { void *dst; const void *src; size_t bytes; };
     std::vector<PinBlock> pin_blocks;
     size_t pin_block = 0, pin_used = 0, pin_total = 0;
-    bool pin_open = false;            // a call that did not reach its end left copies on pin_stream
-    cudaStream_t pin_stream = nullptr;
+    bool pin_open = false;            // staged copies may be in flight on the call's stream
     std::vector<PinOut> pin_outs;
-    cudaError_t pin_begin(cudaStream_t st);
+    void pin_begin();
     void *pin_get(size_t bytes);
     cudaError_t to_device(void *dst, const void *src, size_t bytes, cudaStream_t st);
     cudaError_t to_host(void *dst, const void *src, size_t bytes, cudaStream_t st);   // valid after pin_end
@@ -291,3 +290,12 @@ struct qc_ctx {
     int solve_term(const qc_term *terms, int n_terms, int n, qc::Chain chain, const qc_opts *o, cudaStream_t st,
                    int *it_max, double *acc_ms, long long *acc_launches, double *pass_ms);
 };
+
+// The pinned staging of one call on stream st.
+struct PinScope {
+    qc_ctx *c;
+    cudaStream_t st;
+    PinScope(qc_ctx *ctx, cudaStream_t stream) : c(ctx), st(stream) { c->pin_begin(); }
+    ~PinScope();
+};
+

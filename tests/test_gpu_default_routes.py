@@ -203,3 +203,35 @@ def test_chi2_beyond_float(n_chan):
     assert np.isnan(chi2(bad, weight))
     bad[5, n_chan // 2, 1] = np.inf
     assert np.isinf(chi2(bad, weight)) or np.isnan(chi2(bad, weight))
+
+
+def test_failed_call_keeps_no_stream():
+    """A call that fails half-way on a caller's stream leaves nothing of that stream behind: the
+    stream is destroyed before the next call and before the solver is closed."""
+    lib = qc.load()
+    obs = tmo._chain_obs(7, ("diag",), n_ant=6, n_time=8, n_chan=20, t_int=(4,), f_int=(20,))
+    want = _terms(obs, (5,))
+    S = qc.Solver.from_obs(obs)
+    S.solve(want)
+
+    def failing(buffer, n, stream, user):
+        return 1
+
+    for fails in ("allocation", "allreduce"):
+        for _ in range(2):
+            st = C.c_void_p()
+            assert lib.cudaStreamCreate(C.byref(st)) == 0
+            F = qc.Solver.from_obs(obs)
+            with pytest.raises(qc.QCError):
+                if fails == "allocation":
+                    lib.qc_test_fail_alloc(3)
+                    F.solve(_terms(obs, (5,)), stream=st.value, kernel=3)
+                else:
+                    F.solve(_terms(obs, (5,), reduce=True), stream=st.value, allreduce=failing)
+            lib.qc_test_fail_alloc(0)
+            assert lib.cudaStreamDestroy(st) == 0
+            got = _terms(obs, (5,))
+            F.solve(got)
+            F.close()
+            assert _rel(got[0].gains, want[0].gains) < 1e-6
+    S.close()
