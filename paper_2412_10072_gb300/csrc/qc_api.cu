@@ -149,7 +149,8 @@ qc_ctx::~qc_ctx()
 {
     for (auto &b : tb) if (b.exec) cudaGraphExecDestroy(b.exec);
     for (void *p : owned) qc_dev_free(p);
-    for (auto &b : pin_blocks) cudaFreeHost(b.ptr);
+    if (pin_ptr) cudaFreeHost(pin_ptr);
+    if (pin_next) cudaFreeHost(pin_next);
     for (auto e : events) cudaEventDestroy(e);
     for (auto e : sums_events) cudaEventDestroy(e);
     if (own_stream) cudaStreamDestroy(own_stream);
@@ -157,7 +158,7 @@ qc_ctx::~qc_ctx()
 
 void qc_ctx::pin_begin()
 {
-    pin_block = pin_used = 0;
+    pin_used = pin_want = 0;
     pin_outs.clear();
     pin_open = true;
 }
@@ -175,23 +176,26 @@ PinScope::~PinScope()
 void *qc_ctx::pin_get(size_t bytes)
 {
     bytes = (bytes + 63) / 64 * 64;
-    for (; pin_block < pin_blocks.size(); ++pin_block, pin_used = 0)
-        if (pin_used + bytes <= pin_blocks[pin_block].bytes) {
-            void *p = pin_blocks[pin_block].ptr + pin_used;
-            pin_used += bytes;
-            return p;
-        }
-    const size_t size = std::max<size_t>(bytes, 256u << 10);
-    if (pin_total + size > PIN_MAX) return nullptr;
+    pin_want += bytes;
+    if (pin_used + bytes > pin_size) return nullptr;
+    void *p = pin_ptr + pin_used;
+    pin_used += bytes;
+    return p;
+}
+
+// Room for what this call has asked for and will ask for (`more`), for the calls to come: allocated (0.1 ms)
+// by a solve once its iterations are on the stream, which hide it; a call that finds no room copies directly.
+void qc_ctx::pin_reserve(size_t more)
+{
+    const size_t want = pin_want + more, size = (want + (64u << 10) - 1) / (64u << 10) * (64u << 10);
+    if (want <= pin_size || size > PIN_MAX || pin_next) return;
     void *p = nullptr;
     if (cudaHostAlloc(&p, size, cudaHostAllocDefault) != cudaSuccess) {
         cudaGetLastError();
-        return nullptr;
+        return;
     }
-    pin_blocks.push_back({ (char *)p, size });
-    pin_total += size;
-    pin_used = bytes;
-    return p;
+    pin_next = (char *)p;
+    pin_next_size = size;
 }
 
 cudaError_t qc_ctx::to_device(void *dst, const void *src, size_t bytes, cudaStream_t st)
@@ -213,6 +217,12 @@ void qc_ctx::pin_end()
     for (const PinOut &o : pin_outs) memcpy(o.dst, o.src, o.bytes);
     pin_outs.clear();
     pin_open = false;
+    if (pin_next) {                 // nothing of the old block is in flight any more
+        if (pin_ptr) cudaFreeHost(pin_ptr);
+        pin_ptr = pin_next;
+        pin_size = pin_next_size;
+        pin_next = nullptr;
+    }
 }
 
 int qc_ctx::fail(int code, const std::string &msg)
@@ -1098,6 +1108,14 @@ extern "C" int qc_solve(qc_ctx *c, qc_term *terms, int32_t n_terms, const qc_opt
         CK(c->to_host(&S.chi2_after, d_chi2, sizeof(double), st));
     }
     // write back solved gains, flags, iteration counts
+    size_t out_bytes = 64;
+    for (const auto &P : c->pending) out_bytes += nbytes<int>(P.max_iter + 1) + 64;
+    for (int j = 0; j < n_terms; ++j)
+        if (terms[j].solve && terms[j].memory == QC_MEM_HOST) {
+            const size_t nb = term_nbins(terms[j]);
+            out_bytes += nb * c->term_nat(terms[j]) * 33 + nbytes<int>(nb) + 3 * 64;
+        }
+    c->pin_reserve(out_bytes);
     for (int j = 0; j < n_terms; ++j) {
         if (!terms[j].solve) continue;
         qc_term &t = terms[j];

@@ -229,18 +229,19 @@ struct qc_ctx {
     std::vector<int> sums_iters;      // max_iter of an epoch's one-launch term solves, in their order
     long long sums_total = 0, sums_done = 0;   // one-launch term solves of the call, those enqueued so far
     // Pinned staging of one call's small copies: a copy from or to pageable memory holds the host
-    // until it is done, and a small solve makes about ten.  Blocks are kept for the context's life
-    // (at most PIN_MAX in all; larger copies go directly); a call ends synchronised, so the next one
-    // starts from the beginning.
+    // until it is done, and a small solve makes about ten (256 us with, 232 us without, 7 antennas).  One
+    // block of up to PIN_MAX, kept for the context's life and allocated by its first solve behind the
+    // kernels: in front of them it cost the first call 0.13 ms, twice a small residual.
+    // Larger copies go directly; a call ends synchronised, so the next one starts from the beginning.
     static constexpr size_t PIN_MAX = 16u << 20;
-    struct PinBlock { char *ptr; size_t bytes; };
     struct PinOut { void *dst; const void *src; size_t bytes; };
-    std::vector<PinBlock> pin_blocks;
-    size_t pin_block = 0, pin_used = 0, pin_total = 0;
+    char *pin_ptr = nullptr, *pin_next = nullptr;     // the block, the one that replaces it at the call's end
+    size_t pin_size = 0, pin_next_size = 0, pin_used = 0, pin_want = 0;
     bool pin_open = false;            // staged copies may be in flight on the call's stream
     std::vector<PinOut> pin_outs;
     void pin_begin();
     void *pin_get(size_t bytes);
+    void pin_reserve(size_t more);
     cudaError_t to_device(void *dst, const void *src, size_t bytes, cudaStream_t st);
     cudaError_t to_host(void *dst, const void *src, size_t bytes, cudaStream_t st);   // valid after pin_end
     void pin_end();                   // after the synchronisation: the staged results to the caller

@@ -235,3 +235,21 @@ def test_failed_call_keeps_no_stream():
             F.close()
             assert _rel(got[0].gains, want[0].gains) < 1e-6
     S.close()
+
+
+def test_staging_limit():
+    """Host gains beyond the pinned block's limit (16 MB) go directly; the first call, which has no
+    block yet, and the next ones agree, also when a call needs a larger block than the one before."""
+    n_ant, n_time, n_chan = 4, 700, 256
+    obs = tmo._chain_obs(8, ("diag",), n_ant=n_ant, n_time=n_time, n_chan=n_chan, t_int=(1,), f_int=(1,), flag_frac=0.0)
+    small = [synth.TermSpec("diag", synth.interval_map(n_time, 350), synth.interval_map(n_chan, 128), 2, 2)]
+    assert obs.terms[0].truth.size * 8 > 16 << 20
+    S = qc.Solver.from_obs(obs)
+    seen = {}
+    for kind in ("small", "large", "small", "large", "small"):
+        T = qc.Term.from_spec((small if kind == "small" else obs.terms)[0], n_ant, max_iter=4, tol=0.0)
+        S.solve([T])
+        assert (T.iters == 4).all()
+        g = seen.setdefault(kind, T.gains)
+        assert _rel(T.gains, g) < 1e-6 and _rel(g, np.ones(1)) > 1e-3
+    S.close()
