@@ -1180,7 +1180,7 @@ int qc_ctx::get_event(int i, cudaEvent_t &ev)
 // ---------------------------------------------------------------------------
 
 // Antennas up to which one CTA keeps an interval's gains and normal equations in shared memory
-// (256 x (32 + 128) B = 40 KB) and walks all of its pairs itself.
+// (256 x (32 + 128 + 64) B = 56 KB) and walks all of its pairs itself.
 static constexpr int SUMS_ONE_LAUNCH_ANT = 256;
 // Antennas from which the full and left-full forms' slots are rounded to their heads: a slot's rounding
 // averages out over the pairs.  Error of three chains and single terms against FP64 (rounding the result
@@ -1190,6 +1190,25 @@ static constexpr int SUMS_ONE_LAUNCH_ANT = 256;
 // slot, cost 2% and are always kept.
 static constexpr int SUMS_TAILS_ANT = 64;
 
+// Whether all iterations of a term go in one launch, a CTA an interval, or in a launch an iteration, a warp
+// an antenna and interval.  Time of an iteration (us, measured, nb intervals of 20 samples a pair):
+//   one launch    a + c pairs ceil(nb / CTAs)     a = 5, 10, 8 and c = 0.0057, 0.0197, 0.0070 (plain diagonal, full,
+//                                                 left-full form), two CTAs an SM
+//   one each      f + m pairs nb                  f = 46, 78, 46 and m = 0.000065, 0.00021, 0.00009
+// and the one launch has about 0.65 of m pairs nb to read as well.  20 iterations in ms, one launch and one
+// each: 64 antennas, 1 interval: 0.40 and 0.92, 1.10 and 1.61, 0.51 and 0.94; 128 antennas, 1 interval: 1.14 and
+// 1.02, 3.56 and 1.90, 1.39 and 1.05; 152 intervals: 2.35 and 2.90, 6.7 and 7.4, 3.2 and 3.5; 256 antennas,
+// 1 interval: 3.9 and 1.3, 13.2 and 3.0, 4.8 and 1.3 (on the samples 2.0, 4.1 and 2.4); 152 intervals: 9.2
+// and 7.7, 27 and 24, 12.1 and 10.2.
+bool qc_ctx::sums_one_launch(int form, size_t nb) const
+{
+    if (n_ant > SUMS_ONE_LAUNCH_ANT) return false;
+    static const double a[3] = { 10, 8, 5 }, c[3] = { 0.0197, 0.0070, 0.0057 };        // FORM_FULL, FORM_E, FORM_D
+    static const double f[3] = { 78, 46, 46 }, m[3] = { 0.00021, 0.00009, 0.000065 };
+    const double pairs = n_up, ctas = 2.0 * sm_count;
+    return a[form] + c[form] * pairs * std::ceil((double)nb / ctas) < f[form] + 0.35 * m[form] * pairs * (double)nb;
+}
+
 // The route of a solved term: from sums when the caller asks for it (qc_opts.moments), or by itself
 // where that is the cheaper way to the same steps; sets B.sums and sizes its workspace.
 //
@@ -1198,7 +1217,9 @@ static constexpr int SUMS_TAILS_ANT = 64;
 // iterations, and then 2 x 4 x words B per (interval, pair) and iteration, mostly out of L2.  The
 // rule takes the sums when an iteration on them moves at most half the bytes of one on the
 // samples, i.e. from 2.4 (plain diagonal form), 5.6 (E form) or 20 (full form) samples per slot
-// on, and a term may take three iterations or more.  It also bounds the workspace to a quarter of
+// on, and a term may take three iterations or more.  There and beyond the sums were never the slower
+// ones (32 to 256 antennas, 1 to 320 intervals, 4 to 256 samples a slot; 20 iterations on 64 antennas and
+// two intervals of 4 samples a pair: 0.41 against 0.98 ms).  It also bounds the workspace to a quarter of
 // the samples' bytes.  The options that name an accumulate kernel, its tiles or launch shape,
 // divergence flagging and an allreduce (whose buffers are documented per iteration) keep the
 // iterations on the samples.
@@ -1217,10 +1238,10 @@ int qc_ctx::plan_sums(const qc_term *terms, int n_terms, int n, const qc_opts *o
     else if (lk == KIND_NONE) { form = FORM_FULL; ok = rk; }
     else return QC_OK;
     const bool asked = o->moments && d_model != nullptr;
-    const bool one_launch = n_ant <= SUMS_ONE_LAUNCH_ANT && !t.reduce && !(o->div_flag && t.max_iter >= 4);
+    const bool one_launch = sums_one_launch(form, nb) && !t.reduce && !(o->div_flag && t.max_iter >= 4);
     if (!asked) {
         const bool plain = o->kernel == 0 && o->order == -1 && o->block_threads == 0 && o->ctas_per_sm == 0;
-        if (!plain || !one_launch || o->div_flag || t.max_iter < 3) return QC_OK;
+        if (!plain || n_ant > SUMS_ONE_LAUNCH_ANT || t.reduce || o->div_flag || t.max_iter < 3) return QC_OK;
         const double sample_bytes = (m16 ? 64.0 : 80.0) * (double)n_strip_rows * n_chan;
         if (2.0 * 4.0 * mom_words(form) * (double)slots > 0.5 * sample_bytes) return QC_OK;
     }

@@ -275,6 +275,7 @@ struct qc_ctx {
     int pick_order(const qc_term &t, const qc_opts *o) const;
     int plan_sums(const qc_term *terms, int n_terms, int n, const qc_opts *o);
     size_t sums_window(long long first) const;
+    bool sums_one_launch(int form, size_t nb) const;
     bool slots_once(const qc_term &t, int form, const SumsPlan &P) const;
     int plan_counters(const qc_term *terms, int n_terms, int n_epochs);
     int size_mom_rows();

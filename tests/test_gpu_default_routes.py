@@ -253,3 +253,29 @@ def test_staging_limit():
         g = seen.setdefault(kind, T.gains)
         assert _rel(T.gains, g) < 1e-6 and _rel(g, np.ones(1)) > 1e-3
     S.close()
+
+
+@pytest.mark.parametrize("kinds,n_ant,t_int", [(("diag",), 100, 8), (("diag",), 160, 8), (("diag",), 160, 1), (("full",), 70, 8),
+                                               (("full",), 110, 8), (("phase",), 160, 8), (("full", "diag"), 130, 8),
+                                               (("diag",), 257, 8)])
+def test_many_antennas(kinds, n_ant, t_int):
+    """Few intervals of many antennas: a launch for all iterations or one each (and beyond 256
+    antennas the samples), against the samples; statistics of either count the same iterations, and
+    asking for the sums is no other result."""
+    n_time, n_chan = 8, 16
+    obs = tmo._chain_obs(90, kinds, n_ant=n_ant, n_time=n_time, n_chan=n_chan, t_int=(t_int, n_time), f_int=(n_chan, n_chan))
+    rng = np.random.default_rng(2)
+    start = [tmo._start(s, rng) for s in obs.terms]
+    S = qc.Solver.from_obs(obs)
+    out = []
+    for kw in (dict(), dict(moments=True), dict(kernel=3)):
+        T = [qc.Term.from_spec(s, n_ant, gains=g, max_iter=4, tol=0.0) for s, g in zip(obs.terms, start)]
+        st = S.solve(T, **kw)
+        assert st.n_iter_max == 4 and st.acc_launches == 4 * len(kinds)
+        out.append((T, st))
+    S.close()
+    assert (out[0][1].acc_bytes < out[2][1].acc_bytes) == (n_ant <= 256)
+    for T, _ in out[:2]:
+        for a, b in zip(T, out[2][0]):
+            assert _rel(a.gains, b.gains) < TOL
+            assert np.array_equal(a.gain_flags, b.gain_flags) and np.array_equal(a.iters, b.iters)
