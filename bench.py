@@ -579,11 +579,9 @@ def run_delay(args):
     init_ms = i0.elapsed_time(i1)
     peaks, peak_src = measured_peaks()
     hbm = float(peaks.get("hbm_gbs", 6800.0))
-    # one pass over the samples of rows with usable data forms per-(interval, pair, channel) products, every
-    # iteration reads those of its active intervals (1 KB per 32 channels)
-    live = (obs["flag"] == 0).any(dim=1)
-    bytes_moved = (80 * int(live.sum().item()) * args.n_chan * len(stats)
-                   + 1024 * ((args.n_chan + 31) // 32) * vis_iters / args.n_chan)
+    # the library's own count: one pass over the samples forms per-(interval, pair, channel) products, every
+    # iteration reads those of its active intervals
+    bytes_moved = sum(s.acc_bytes for s in stats)
     achieved = (bytes_moved / (acc_ms / 1000.0)) / 1e9 if acc_ms > 0 else None
     roofline = {"bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s",
                 "frac": (achieved / hbm) if achieved else None, "traffic": None,

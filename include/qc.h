@@ -150,7 +150,8 @@ typedef struct {
  *                 default options iterates on per-(time interval, pair,
  *                 channel) products formed in one pass, where those are at most
  *                 0.6 of the samples and the other term is diagonal or to its
- *                 right; else (or with kernel 3) a streaming kernel applies the
+ *                 right (qc_stats.acc_bytes then counts the samples' bytes once
+ *                 and 32 B per pair and channel of the intervals iterated on); else (or with kernel 3) a streaming kernel applies the
  *                 chain rule per sample; otherwise the accumulate kernels form
  *                 diagonal blocks per (time interval, channel) bin and the
  *                 update reduces them over the interval's channels.

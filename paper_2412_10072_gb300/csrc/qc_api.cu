@@ -2036,6 +2036,7 @@ int qc_ctx::solve_term(const qc_term *terms, int n_terms, int n, Chain chain, co
             dua.omega_lo = dua.omega + n_chan;
             dua.om_sums = (const double2 *)B.dom_sums.ptr;
             dua.om_max = B.om_max;
+            dua.prod_bytes = 32 * n_up;
         }
     }
     DelaySumsArgs dsa_;

@@ -110,6 +110,7 @@ struct DelayUpdArgs {
     const float *omega, *omega_lo;   // [n_chan] omega' = 2 pi nu - omega_ref as head and tail (with hsum)
     const double2 *om_sums;   // [n_fint] sum of omega', of omega'^2 over the interval's channels (with hsum)
     double om_max;            // largest |omega'|
+    int prod_bytes;           // bytes of a channel's products over the pairs (with hsum)
 };
 
 // One block per parameter interval (time interval x frequency interval), threads over antennas.
@@ -167,7 +168,9 @@ __device__ __forceinline__ void delay_finish(const DelayUpdArgs &u, int bin, int
     unsigned long long nv = 0, nb = 0;
     for (int c = fr.x + (int)threadIdx.x; c <= fr.y; c += blockDim.x) {
         nv += (unsigned long long)u.bin_nvis[cb0 + c];
-        nb += (unsigned long long)u.bin_nbytes[cb0 + c];
+        // from products: the samples once, then the products of the interval
+        nb += u.hsum ? (unsigned long long)u.prod_bytes + (u.k == 1 ? (unsigned long long)u.bin_nbytes[cb0 + c] : 0ull)
+                     : (unsigned long long)u.bin_nbytes[cb0 + c];
     }
     if (nv) atomicAdd(u.vis_iters, nv);
     if (nb) atomicAdd(u.acc_bytes, nb);

@@ -279,3 +279,22 @@ def test_many_antennas(kinds, n_ant, t_int):
         for a, b in zip(T, out[2][0]):
             assert _rel(a.gains, b.gains) < TOL
             assert np.array_equal(a.gain_flags, b.gain_flags) and np.array_equal(a.iters, b.iters)
+
+
+@pytest.mark.parametrize("t_int,n_chan", [(1, 60), (3, 64)])
+def test_delay_bytes_tell_the_route(t_int, n_chan):
+    """qc_stats.acc_bytes of a delay term from products: the samples once (80 B unflagged, a byte of
+    flags each), then 32 B per pair and channel of the intervals iterated on; on the samples all of them
+    an iteration.  Intervals of one time on a full grid are stored, the others added."""
+    args, G, _, _ = _delay_case(13, 8, 12, n_chan, t_int, oracle=False)
+    st = []
+    for kernel in (0, 3):
+        S = qc.Solver(*args)
+        T = G()
+        st.append(S.solve([T], kernel=kernel))
+        S.close()
+    n_pair, n_int, its = 28, 12 // t_int, 8
+    samples = 12 * n_pair * n_chan * 81
+    assert st[0].acc_bytes == samples + its * 32 * n_pair * n_chan * n_int
+    assert st[1].acc_bytes == its * samples
+    assert st[0].vis_iters == st[1].vis_iters == its * 12 * n_pair * n_chan
