@@ -1391,7 +1391,11 @@ int qc_ctx::ensure_mom_rows(cudaStream_t st)
 // pair, 32 channels), one on the samples 80 B (64 B with the FP16 model) a sample; T is taken when it is at most 0.6 of that, which leaves the pass that forms
 // it paid for after two iterations (measured on 64 antennas, 75 x 512: pass 1.9 iterations on the
 // samples, an iteration on T 0.3).  That also bounds T to 0.6 of the samples' bytes; where a slot takes
-// several additions, T with its FP64 sums (three times T).
+// several additions, T with its FP64 sums (three times T).  Few intervals of many antennas leave most SMs
+// without a CTA: time of an iteration in us, measured, 30 + 0.023 to 0.037 per pair and wave of CTAs on
+// products, 82 + 0.024 per 1000 samples on the samples (20 iterations, products and samples: 64 antennas, 1 x
+// 512: 2.1 and 2.1 ms; 75 x 512: 10.0 and 25; 128 antennas, 1 x 64: 4.7 and 2.0; 1 x 512: 6.5 and 3.5; 3 x
+// 512: 6.8 and 7.3; 200 antennas, 2 x 512: 14.4 and 10.2; 3 x 512: 14.8 and 16.0).
 // Whether every product of a delay term gets one sample: a time an interval, a row a pair and time.
 bool qc_ctx::products_once(const qc_term &t) const
 {
@@ -1414,7 +1418,11 @@ int qc_ctx::plan_delay_sums(const qc_term *terms, int n_terms, int n, const qc_o
     // the products, and the FP64 ones where a slot takes several additions
     const size_t t_bytes = (size_t)t.n_tint * n_chunks * n_up * (products_once(t) ? 1024 : 3 * 1024);
     const double sample = m16 ? 64.0 : 80.0;
-    if ((double)t_bytes > 0.6 * sample * (double)n_strip_rows * n_chan) return QC_OK;
+    const double samples = (double)n_strip_rows * n_chan;
+    if ((double)t_bytes > 0.6 * sample * samples) return QC_OK;
+    // an iteration on T is a CTA per (time interval, chunk), which walks all pairs
+    const double waves = std::ceil((double)t.n_tint * (double)n_chunks / (2.0 * sm_count));
+    if (30 + 0.04 * n_up * waves > 82 + 3e-7 * sample * samples) return QC_OK;
     int rc = ensure(B.dsum_t, t_bytes);
     if (!rc) rc = ensure(B.dsum_h, nbytes<double>((size_t)t.n_tint * B.hfr.size() * n_ant * KG_HSUM));
     if (!rc) rc = size_mom_rows();

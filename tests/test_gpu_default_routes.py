@@ -298,3 +298,19 @@ def test_delay_bytes_tell_the_route(t_int, n_chan):
     assert st[0].acc_bytes == samples + its * 32 * n_pair * n_chan * n_int
     assert st[1].acc_bytes == its * samples
     assert st[0].vis_iters == st[1].vis_iters == its * 12 * n_pair * n_chan
+
+
+@pytest.mark.parametrize("n_ant,n_time,n_chan,products", [(8, 1, 64, True), (128, 1, 64, False), (128, 8, 512, True)])
+def test_delay_route_of_few_intervals(n_ant, n_time, n_chan, products):
+    """One CTA per time interval and 32 channels walks all pairs: few of them with many antennas
+    iterate on the samples (qc_stats.acc_bytes tells), with the same result."""
+    args, G, _, phases = _delay_case(14, n_ant, n_time, n_chan, 1, oracle=False)
+    out = []
+    for kernel in (0, 3):
+        S = qc.Solver(*args)
+        T = G()
+        T.max_iter = 3
+        out.append((T, S.solve([T], kernel=kernel).acc_bytes))
+        S.close()
+    assert (out[0][1] < out[1][1]) == products
+    assert np.sqrt(np.mean((phases(out[0][0].gains) - phases(out[1][0].gains)) ** 2)) < 2e-7
