@@ -518,7 +518,7 @@ int qc_batch_create(const qc_batch_problem *p, qc_batch **out);
 
 /*
  * Solve every problem of the batch with Algorithm 1.  With default launch
- * options, no tuned shape for the batch's class, no fallback start, max_iter >= 3
+ * options, no tuned shape that beats them (see qc_batch_autotune), no fallback start, max_iter >= 3
  * and about two samples or more per antenna pair, from sums as
  * qc_batch_solve_moments does (any number of antennas); stats then report the
  * grid of one CTA per problem, depth 0, and the one data pass in `bytes`.
@@ -572,8 +572,12 @@ int qc_batch_solve_moments(qc_batch *b, void *gains, int8_t *gain_flags, int32_t
  * which problems go to a concurrent class of small CTAs, threads in {64, 128}
  * and {4, 8} per SM.  Results are cached for the process per device and shape
  * class of the batch (problem count, FP16 model, log2 size histogram): another
- * batch of the same class uses them without tuning.  best (nullable) receives
- * the chosen shape and its time; `n_tried` (nullable) the candidates timed.
+ * batch of the same class uses them without tuning.  The solve from sums is timed
+ * beside the winner: where it is faster, default solves of the class keep taking
+ * it, and the shape is for the solves that do not (use_graph = 0, which asks for the
+ * shape's own launch; a fallback start; fewer than three iterations).  best
+ * (nullable) receives the chosen shape and its time; `n_tried` (nullable) the shapes
+ * timed.
  */
 int qc_batch_autotune(qc_batch *b, const qc_batch_opts *base, qc_batch_stats *best, int32_t *n_tried);
 

@@ -1115,7 +1115,8 @@ struct qc_batch {
     // A launch shape: CTA size, residency, schedule, copy depth; with split > 0 the problems
     // with fewer samples than split form a second class launched concurrently with its own
     // CTA size and residency (tile = threads consecutive samples per CTA step).
-    struct Shape { int threads, per_sm, schedule, depth; double ms; long long split; int s_threads, s_per_sm; };
+    // sums: the autotuner found the solve from sums faster than this shape
+    struct Shape { int threads, per_sm, schedule, depth; double ms; long long split; int s_threads, s_per_sm; bool sums; };
     std::string shape_key;
     struct GraphKey { int threads, per_sm, schedule, depth, max_iter, damping_mode; double damping, tol; bool m16;
                       void *gains; void *flags; void *iters; cudaStream_t st; const void *fb_gains, *fb_chi2;
@@ -1571,17 +1572,18 @@ static int enqueue_sums(qc_batch *b, const BatchArgs &a, cudaStream_t st)
     return QC_OK;
 }
 
-// Whether qc_batch_solve takes the sums by itself: no launch option of the persistent kernel named or
-// tuned, no fallback start (its bound comes from the caller's chi^2), three iterations or more, and
+// Whether qc_batch_solve takes the sums by itself: no launch option of the persistent kernel named, no
+// tuned shape that the autotuner found faster (or whose launch use_graph = 0 asks for), no fallback start (its bound comes from the caller's chi^2), three iterations or more, and
 // room for the sums in half the samples' bytes (about two samples a pair).  The persistent kernel
 // reads every sample each iteration and flushes its register sums to shared memory at each change
 // of baseline: 180 ms for 1024 problems of up to 64 antennas (2.0e8 samples) against 3.5 from sums.
 static bool sums_pay(const qc_batch *b, const qc_batch_opts *o)
 {
     qc_batch::Shape t;
+    if (tuned_shape(b, t) && !(t.sums && o->use_graph)) return false;
     return o->threads == 0 && o->ctas_per_sm == 0 && o->schedule == QC_SCHED_AUTO && o->depth == 0 && o->split == 0 &&
            o->small_threads == 0 && o->small_ctas_per_sm == 0 && !o->fallback_gains && o->max_iter >= 3 &&
-           4.0 * MOM_W * (double)b->n_pairs <= 0.5 * 80.0 * (double)b->n_vis && !tuned_shape(b, t);
+           4.0 * MOM_W * (double)b->n_pairs <= 0.5 * 80.0 * (double)b->n_vis;
 }
 
 static int batch_solve_sums(qc_batch *b, void *gains, int8_t *gain_flags, int32_t *iters, int32_t mem,
@@ -1825,7 +1827,7 @@ extern "C" int qc_batch_autotune(qc_batch *b, const qc_batch_opts *base, qc_batc
     cudaError_t e = qc_dev_malloc((void **)&g, (size_t)b->total_ant * 2 * sizeof(float2));
     if (e != cudaSuccess) return b->cuda_fail(e, "cudaMalloc");
     std::vector<float2> unit((size_t)b->total_ant * 2, make_float2(1.f, 0.f));
-    qc_batch::Shape win{ 0, 0, 0, 0, 1e30, 0, 0, 0 };
+    qc_batch::Shape win{ 0, 0, 0, 0, 1e30, 0, 0, 0, false };
     int tried = 0, rc = QC_OK;
     qc_batch_stats ws;
     memset(&ws, 0, sizeof ws);
@@ -1846,7 +1848,7 @@ extern "C" int qc_batch_autotune(qc_batch *b, const qc_batch_opts *base, qc_batc
         if (o.split > 0 && s.small_ctas_per_sm != o.small_ctas_per_sm) return QC_OK;
         if (s.ms < win.ms) {
             win = { o.threads, o.ctas_per_sm, o.schedule, o.depth, s.ms, o.split > 0 ? o.split : 0,
-                    o.split > 0 ? o.small_threads : 0, o.split > 0 ? o.small_ctas_per_sm : 0 };
+                    o.split > 0 ? o.small_threads : 0, o.split > 0 ? o.small_ctas_per_sm : 0, false };
             ws = s;
         }
         return QC_OK;
@@ -1884,6 +1886,28 @@ extern "C" int qc_batch_autotune(qc_batch *b, const qc_batch_opts *base, qc_batc
                     o.small_ctas_per_sm = sper;
                     rc = trial(o);
                 }
+    }
+    // the solve from sums beside the winner (the second of two runs: the first one stages its tables)
+    qc_batch_opts def = *base;
+    def.threads = def.ctas_per_sm = def.depth = def.small_threads = def.small_ctas_per_sm = 0;
+    def.split = 0;
+    def.schedule = QC_SCHED_AUTO;
+    def.fallback_gains = nullptr;
+    def.fallback_chi2 = nullptr;
+    def.use_graph = 1;
+    if (!rc && win.threads && sums_pay(b, &def)) {
+        for (int run = 0; run < 2 && !rc; ++run) {
+            e = cudaMemcpy(g, unit.data(), unit.size() * sizeof(float2), cudaMemcpyHostToDevice);
+            qc_batch_stats s;
+            rc = e == cudaSuccess ? stage_sums(b) : b->cuda_fail(e, "cudaMemcpy");
+            if (!rc) rc = batch_solve_sums(b, g, nullptr, nullptr, QC_MEM_DEVICE, &def, &s);
+            win.sums = !rc && s.ms < win.ms;
+        }
+        if (rc == QC_ENOMEM) {                       // no room for the sums: the shape stands
+            cudaGetLastError();
+            b->err.clear();
+            rc = QC_OK;
+        }
     }
     qc_dev_free(g);
     if (rc) return rc;

@@ -314,3 +314,25 @@ def test_delay_route_of_few_intervals(n_ant, n_time, n_chan, products):
         S.close()
     assert (out[0][1] < out[1][1]) == products
     assert np.sqrt(np.mean((phases(out[0][0].gains) - phases(out[1][0].gains)) ** 2)) < 2e-7
+
+
+def test_autotune_keeps_the_faster_route():
+    """Tuning the persistent kernel does not take the default solves of the shape class from the sums
+    where those are faster; asking for the shape's own launch does, and a second batch of the class
+    behaves like the first."""
+    import test_gpu_batch as tb
+    b = tb.small_batch(n=40, seed_base=4200)
+    S = tb.solver_of(b)
+    g0, f0, i0, st0 = S.solve(max_iter=6, tol=0.0)
+    assert st0.depth == 0                                # from sums
+    best, _ = S.autotune()
+    S2 = tb.solver_of(b)
+    for solver in (S, S2):
+        g1, f1, i1, st1 = solver.solve(max_iter=6, tol=0.0)
+        g2, f2, i2, st2 = solver.solve(max_iter=6, tol=0.0, use_graph=False)
+        assert st1.depth == 0 or st1.depth == best.depth and best.ms < st0.ms
+        assert st2.depth == best.depth and st2.bytes > st0.bytes
+        assert _rel(g1, g0) < TOL and _rel(g2, g0) < TOL
+        assert np.array_equal(f1, f0) and np.array_equal(f2, f0) and np.array_equal(i1, i0)
+    S.close()
+    S2.close()
