@@ -1056,8 +1056,7 @@ __global__ void __launch_bounds__(256) batch_iterate_kernel(const SumsArgs s)
         if (tid == 0) {
             double tn = 0, td = 0;
             for (int i = 0; i < n_warps; ++i) { tn += red[0][i]; td += red[1][i]; }
-            // sqrt(tn / td) < tol without the root and the division; 0 where there are no gains
-            s_done = (td > 0 ? tn < a.tol * a.tol * td : 0.0 < a.tol) ? 1 : 0;
+            s_done = converged(tn, td, a.tol) ? 1 : 0;
         }
         __syncthreads();
         if (s_done) break;

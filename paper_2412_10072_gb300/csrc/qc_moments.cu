@@ -1022,8 +1022,7 @@ static __global__ void __launch_bounds__(256, 2) mom_iterate_kernel(const MomIte
         if (tid == 0) {
             double tn = 0, td = 0;
             for (int i = 0; i < nw; ++i) { tn += s_num[i]; td += s_den[i]; }
-            // sqrt(tn / td) < tol without the root and the division; 0 where there are no gains
-            const bool conv = td > 0 ? tn < a.tol * a.tol * td : 0.0 < a.tol;
+            const bool conv = converged(tn, td, a.tol);
             if (!conv) atomicAdd(a.cnt + k, 1);                      // still active after iteration k
             s_done = conv || k == a.max_iter;
         }

@@ -4,6 +4,13 @@
 
 namespace qc {
 
+// sqrt(tn / td) < tol without the root and the division; 0 where there are no gains (td = 0).  A change of
+// exactly zero is below any tolerance but zero, also one whose square underflows.
+__device__ __forceinline__ bool converged(double tn, double td, double tol)
+{
+    return td > 0 && tn != 0 ? tn < tol * tol * td : 0.0 < tol;
+}
+
 // Transposed warp reduction of N = 4, 8 or 16 values per lane: each halving exchanges half of the
 // values a lane holds; the lanes from 32 / N * i on end with the total of value i.  The sum over
 // the lanes is carried as head and tail (Knuth's two-sum, one exact step per level), so the total over

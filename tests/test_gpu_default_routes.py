@@ -336,3 +336,26 @@ def test_autotune_keeps_the_faster_route():
         assert np.array_equal(f1, f0) and np.array_equal(f2, f0) and np.array_equal(i1, i0)
     S.close()
     S2.close()
+
+
+@pytest.mark.parametrize("kinds", [("diag",), ("full",), ("full", "diag")])
+def test_unchanged_gains_converge_at_any_tolerance(kinds):
+    """An interval without data does not change its gains: that is below a tolerance whose square
+    underflows, so one iteration is all, as on the samples; a tolerance of zero takes them all."""
+    obs = tmo._chain_obs(21, kinds, n_ant=6, n_time=8, n_chan=33, t_int=(4, 8), f_int=(33, 33))
+    obs.flag = np.ones_like(obs.flag)
+    for tol, its in ((1e-200, 1), (0.0, 5)):
+        for kw in (dict(), dict(kernel=3)):
+            S = qc.Solver.from_obs(obs)
+            T = [qc.Term.from_spec(s, obs.n_ant, max_iter=5, tol=tol) for s in obs.terms]
+            S.solve(T, **kw)
+            S.close()
+            assert all((t.iters == its).all() for t in T), (tol, kw)
+    import test_gpu_batch as tb
+    b = tb.small_batch(n=5, seed_base=77)
+    b.flag = np.ones_like(np.array(b.flag))
+    S = tb.solver_of(b)
+    for kw in (dict(), dict(threads=256)):
+        _, _, it, _ = S.solve(max_iter=5, tol=1e-200, **kw)
+        assert (it == 1).all()
+    S.close()
