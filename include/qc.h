@@ -233,8 +233,14 @@ typedef struct {
  * itself, with either model, where an iteration on the sums moves at most half the bytes of
  * one on the samples, unless the options name an accumulate kernel, a tile order or a launch
  * shape, or ask for divergence flagging or an allreduce.  The steps are the same either way.
+ * The workspace of a default route stays with the context until qc_destroy: up to the
+ * samples' own bytes for sums (a quarter for heads, a quarter for tails below 64 antennas and in the
+ * plain diagonal form, half where slots are added to several times), up to 0.6 for the products
+ * of a delay term.  A route is left for the iterations on the samples where its workspace would
+ * take more than half of the device's free memory, so that as much again stays free for the
+ * caller, or where an allocation of it fails (which gives back the others).
  * Other solves (a full-Jones term with a term to its left, longer chains, sums of 2^31 or
- * more slots, or more than the device has room for) ignore the option.  qc_stats.vis_iters
+ * more slots) ignore the option.  qc_stats.vis_iters
  * counts the samples of the active intervals per iteration however a term was solved; from
  * sums, qc_stats.acc_bytes counts the pass (the samples' bytes, once) and, per iteration and
  * active interval, the sums read on both sides and the accumulators written;
@@ -412,6 +418,8 @@ int qc_residual_noalloc(int32_t n_row, int32_t n_chan, int32_t n_ant, int32_t n_
  *       returns QC_ENOMEM and releases what it had allocated.  n <= 0 disarms.
  *   qc_test_live_allocs(): device allocations of the library not yet freed
  *       (contexts, batches and their temporary buffers).
+ *   qc_test_free_bytes(n): the free device memory that the default routes see when
+ *       they decide on their workspace (n < 0: the device's own figure).
  *   qc_test_wait_limit(limit_ns, stall): wall-time limit of each bounded wait
  *       on a ring-stage barrier of the bulk-copy accumulate kernels (default
  *       2 s; limit_ns <= 0 restores it).  With stall >= 0, every warp's
@@ -423,6 +431,7 @@ int qc_residual_noalloc(int32_t n_row, int32_t n_chan, int32_t n_ant, int32_t n_
  */
 void qc_test_fail_alloc(int64_t n);
 int64_t qc_test_live_allocs(void);
+void qc_test_free_bytes(int64_t bytes);
 void qc_test_wait_limit(int64_t limit_ns, int32_t stall);
 
 /* Message of the last failed call on `c` ("" if none); with c == NULL, of the last failed qc_create. */

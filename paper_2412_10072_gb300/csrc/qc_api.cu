@@ -240,6 +240,7 @@ int qc_ctx::cuda_fail(cudaError_t e, const char *what)
 namespace {
 std::atomic<long long> g_alloc_countdown{0};   // > 0: the allocation that brings it to 0 fails
 std::atomic<long long> g_live_allocs{0};
+std::atomic<long long> g_free_bytes{-1};       // >= 0: what qc_dev_spare takes for the free memory
 std::atomic<unsigned long long> g_wait_limit_ns{2000000000ull};
 std::atomic<int> g_wait_stall{-1};
 } // namespace
@@ -255,6 +256,17 @@ cudaError_t qc_dev_malloc(void **p, size_t bytes)
     return e;
 }
 
+// Whether `bytes` more of workspace that a route can do without leave as much again for the caller's own
+// allocations.
+bool qc_dev_spare(size_t bytes)
+{
+    size_t avail = 0, total = 0;
+    const long long forced = g_free_bytes.load();
+    if (forced >= 0) avail = (size_t)forced;
+    else if (cudaMemGetInfo(&avail, &total) != cudaSuccess) { cudaGetLastError(); return true; }
+    return bytes <= avail / 2;
+}
+
 void qc_dev_free(void *p)
 {
     if (!p) return;
@@ -266,6 +278,7 @@ uint64_t qc_wait_limit_ns() { return g_wait_limit_ns.load(); }
 int qc_wait_stall_stage() { return g_wait_stall.load(); }
 
 extern "C" void qc_test_fail_alloc(int64_t n) { g_alloc_countdown.store(n > 0 ? n : 0); }
+extern "C" void qc_test_free_bytes(int64_t bytes) { g_free_bytes.store(bytes >= 0 ? bytes : -1); }
 extern "C" int64_t qc_test_live_allocs(void) { return g_live_allocs.load(); }
 extern "C" void qc_test_wait_limit(int64_t limit_ns, int32_t stall_stage)
 {
@@ -285,6 +298,12 @@ void qc_ctx::release(void *p)
 {
     auto it = std::find(owned.begin(), owned.end(), p);
     if (it != owned.end()) { qc_dev_free(p); owned.erase(it); }
+}
+
+void qc_ctx::drop(Buf &b)
+{
+    if (b.ptr) release(b.ptr);
+    b = Buf();
 }
 
 int qc_ctx::ensure(Buf &b, size_t bytes)
@@ -1219,8 +1238,8 @@ bool qc_ctx::sums_one_launch(int form, size_t nb) const
 // samples, i.e. from 2.4 (plain diagonal form), 5.6 (E form) or 20 (full form) samples per slot
 // on, and a term may take three iterations or more.  There and beyond the sums were never the slower
 // ones (32 to 256 antennas, 1 to 320 intervals, 4 to 256 samples a slot; 20 iterations on 64 antennas and
-// two intervals of 4 samples a pair: 0.41 against 0.98 ms).  It also bounds the workspace to a quarter of
-// the samples' bytes.  The options that name an accumulate kernel, its tiles or launch shape,
+// two intervals of 4 samples a pair: 0.41 against 0.98 ms).  It also bounds the heads to a quarter of
+// the samples' bytes, the whole workspace to as many; it has to leave as much free memory (qc_dev_spare).  The options that name an accumulate kernel, its tiles or launch shape,
 // divergence flagging and an allreduce (whose buffers are documented per iteration) keep the
 // iterations on the samples.
 int qc_ctx::plan_sums(const qc_term *terms, int n_terms, int n, const qc_opts *o)
@@ -1261,13 +1280,16 @@ int qc_ctx::plan_sums(const qc_term *terms, int n_terms, int n, const qc_opts *o
     const size_t words = slots * mom_words(form);
     P.cnt_off = nbytes<float>((P.tails ? 2 : 1) * words);
     P.mom64_off = P.cnt_off + ((nbytes<long long>(nb) + 15) / 16) * 16;
-    int rc;
-    rc = ensure(B.mom, P.mom64_off + (P.wide ? nbytes<double>(words) : 0));
+    const size_t bytes = P.mom64_off + (P.wide ? nbytes<double>(words) : 0);
+    const bool grows = B.mom.bytes < bytes || mom_end.ptr == nullptr;
+    if (!asked && grows && !qc_dev_spare(bytes - std::min(bytes, B.mom.bytes))) return QC_OK;
+    int rc = ensure(B.mom, bytes);
     if (!rc) rc = size_mom_rows();
     if (rc) {
         if (asked || rc != QC_ENOMEM) return rc;
         cudaGetLastError();                    // no room for the sums: iterate on the samples
         err.clear();
+        drop(B.mom);
         return QC_OK;
     }
     P.form = form;
@@ -1349,6 +1371,7 @@ int qc_ctx::plan_counters(const qc_term *terms, int n_terms, int n_epochs)
         for (int j = 0; j < n_terms; ++j)
             if (terms[j].solve && tb[j].sums.one_launch && !tb[j].sums.asked) {
                 tb[j].sums = SumsPlan();
+                drop(tb[j].mom);
                 left = true;
             }
         if (!left) return rc;
@@ -1423,12 +1446,15 @@ int qc_ctx::plan_delay_sums(const qc_term *terms, int n_terms, int n, const qc_o
     // an iteration on T is a CTA per (time interval, chunk), which walks all pairs
     const double waves = std::ceil((double)t.n_tint * (double)n_chunks / (2.0 * sm_count));
     if (30 + 0.04 * n_up * waves > 82 + 3e-7 * sample * samples) return QC_OK;
+    if (B.dsum_t.bytes < t_bytes && !qc_dev_spare(t_bytes - B.dsum_t.bytes)) return QC_OK;
     int rc = ensure(B.dsum_t, t_bytes);
     if (!rc) rc = ensure(B.dsum_h, nbytes<double>((size_t)t.n_tint * B.hfr.size() * n_ant * KG_HSUM));
     if (!rc) rc = size_mom_rows();
     if (rc == QC_ENOMEM) {
         cudaGetLastError();                    // no room for the products: iterate on the samples
         err.clear();
+        drop(B.dsum_t);
+        drop(B.dsum_h);
         return QC_OK;
     }
     use = rc == QC_OK;

@@ -27,6 +27,7 @@
 
 cudaError_t qc_dev_malloc(void **p, size_t bytes);   // counted allocation (qc_api.cu)
 void qc_dev_free(void *p);
+bool qc_dev_spare(size_t bytes);
 #include "qc_jones.cuh"
 #include "qc_sums.cuh"
 
@@ -1601,7 +1602,7 @@ static int batch_solve_impl(qc_batch *b, void *gains, int8_t *gain_flags, int32_
     if (o->damping_mode != QC_DAMP_CONST && o->damping_mode != QC_DAMP_ALTERNATE) return b->fail(QC_EINVAL, "damping_mode");
     qc_batch::Shape sh;
     int rc;
-    if (!tuning && sums_pay(b, o)) {
+    if (!tuning && sums_pay(b, o) && (b->sums || qc_dev_spare(sizeof(float) * MOM_W * (size_t)b->n_pairs))) {
         rc = stage_sums(b);
         if (rc == QC_OK) return batch_solve_sums(b, gains, gain_flags, iters, mem, o, stats);
         if (rc != QC_ENOMEM) return rc;

@@ -46,6 +46,7 @@ struct DDArgs {
 cudaError_t dd_launch_acc(const qc::DDArgs &a, int ts, int grid_x, cudaStream_t st);
 // Single-term chains from per-(interval, baseline) sums (qc_moments.cu).
 cudaError_t mom_launch_pass(const qc::MomArgs &a, int form, int ok, int sm_count, cudaStream_t st);
+bool qc_dev_spare(size_t bytes);
 cudaError_t mom_launch_normal(const qc::MomNormArgs &a, cudaStream_t st);
 cudaError_t mom_launch_bytes(int n_bins, const long long *bin_nbytes, long long per_iter, long long *iter_nbytes,
                              unsigned long long *acc_bytes, cudaStream_t st);
@@ -273,6 +274,7 @@ struct qc_ctx {
     qc::Data data_desc() const;
     int run_residual(const qc::Chain &chain, float4 *dres, double *d_chi2, cudaStream_t st);
     int pick_order(const qc_term &t, const qc_opts *o) const;
+    void drop(Buf &b);
     int plan_sums(const qc_term *terms, int n_terms, int n, const qc_opts *o);
     size_t sums_window(long long first) const;
     bool sums_one_launch(int form, size_t nb) const;

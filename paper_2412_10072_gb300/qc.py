@@ -104,6 +104,8 @@ def load(build_if_missing: bool = True):
         lib.qc_test_fail_alloc.restype = None
         lib.qc_test_live_allocs.argtypes = []
         lib.qc_test_live_allocs.restype = C.c_int64
+        lib.qc_test_free_bytes.argtypes = [C.c_int64]
+        lib.qc_test_free_bytes.restype = None
         lib.qc_test_wait_limit.argtypes = [C.c_int64, i32]
         lib.qc_test_wait_limit.restype = None
         _lib = lib

@@ -359,3 +359,83 @@ def test_unchanged_gains_converge_at_any_tolerance(kinds):
         _, _, it, _ = S.solve(max_iter=5, tol=1e-200, **kw)
         assert (it == 1).all()
     S.close()
+
+
+@pytest.fixture
+def lib():
+    lib = qc.load()
+    yield lib
+    lib.qc_test_fail_alloc(0)
+    if hasattr(lib, "qc_test_free_bytes"):
+        lib.qc_test_free_bytes(-1)
+
+
+def test_routes_leave_room(lib):
+    """A default route whose workspace would take more than half of the free memory is left for the
+    iterations on the samples; asking for the sums is not refused."""
+    import test_gpu_batch as tb
+    obs = tmo._chain_obs(31, ("diag",), n_ant=8, n_time=40, n_chan=64, t_int=(8,), f_int=(64,))
+    args, G, _, _ = _delay_case(15, 8, 12, 64, 1, oracle=False)
+    b = tb.small_batch(n=6, seed_base=92)
+
+    def routes():
+        S = qc.Solver.from_obs(obs)
+        r = [S.solve(_terms(obs, (4,))).acc_bytes]
+        S.close()
+        S = qc.Solver(*args)
+        r.append(S.solve([G()]).acc_bytes)
+        S.close()
+        S = tb.solver_of(b)
+        r.append(S.solve(max_iter=4, tol=0.0)[3].bytes)
+        S.close()
+        return r
+
+    free = routes()
+    lib.qc_test_free_bytes(1000)
+    full = routes()
+    assert all(a < c for a, c in zip(free, full))
+    S = qc.Solver.from_obs(obs)
+    assert S.solve(_terms(obs, (4,)), moments=True).acc_bytes == free[0]
+    S.close()
+
+
+@pytest.mark.parametrize("what", ["sums", "delay"])
+def test_failed_workspace_falls_back(lib, what):
+    """Each allocation of a default solve failing in turn: QC_ENOMEM where the samples need it too, else
+    the samples, with the result and the statistics of kernel 3, and nothing is lost."""
+    if what == "sums":
+        obs = tmo._chain_obs(32, ("diag", "full"), n_ant=6, n_time=24, n_chan=40, t_int=(8, 24), f_int=(40, 40))
+        make, terms = (lambda: qc.Solver.from_obs(obs)), (lambda: _terms(obs, (4, 3)))
+    else:
+        args, G, _, _ = _delay_case(16, 6, 12, 64, 1, oracle=False)
+        make, terms = (lambda: qc.Solver(*args)), (lambda: [G()])
+    base = lib.qc_test_live_allocs()
+    S = make()
+    want = terms()
+    ref = S.solve(want, kernel=3)
+    S.close()
+    fell = 0
+    for n in range(1, 60):
+        S = make()
+        T = terms()
+        lib.qc_test_fail_alloc(n)
+        try:
+            st = S.solve(T)
+        except qc.QCError as e:
+            assert e.code == qc.QC_ENOMEM
+            lib.qc_test_fail_alloc(0)
+            st = S.solve(terms())                        # the context still works
+            assert st.n_iter_max == ref.n_iter_max
+            S.close()
+            assert lib.qc_test_live_allocs() == base
+            continue
+        lib.qc_test_fail_alloc(0)
+        S.close()
+        assert lib.qc_test_live_allocs() == base
+        assert st.n_iter_max == ref.n_iter_max
+        for a, c in zip(T, want):
+            assert _rel(a.gains, c.gains) < TOL and np.array_equal(a.iters, c.iters)
+        fell += st.acc_bytes > 0.9 * ref.acc_bytes
+        if n > 40:
+            break
+    assert fell >= 2, fell
