@@ -439,3 +439,20 @@ def test_failed_workspace_falls_back(lib, what):
         if n > 40:
             break
     assert fell >= 2, fell
+
+
+@pytest.mark.parametrize("kinds,n_time", [(("diag",), 1100), (("full", "diag"), 600), (("diag", "full"), 1100)])
+def test_long_time_maps(kinds, n_time):
+    """Time maps longer than the pass keeps in shared memory (512 integrations behind a full term, 1024
+    elsewhere)."""
+    obs = tmo._chain_obs(41, kinds, n_ant=3, n_time=n_time, n_chan=20, t_int=(50, n_time), f_int=(20, 10))
+    out = []
+    for kernel in (0, 3):
+        S = qc.Solver.from_obs(obs)
+        T = _terms(obs, (4, 4))
+        st = S.solve(T, kernel=kernel)
+        S.close()
+        out.append((T, st.acc_bytes))
+    assert out[0][1] < out[1][1]
+    for a, b in zip(out[0][0], out[1][0]):
+        assert _rel(a.gains, b.gains) < TOL
