@@ -236,7 +236,7 @@ typedef struct {
  * The workspace of a default route stays with the context until qc_destroy: up to the
  * samples' own bytes for sums (a quarter for heads, a quarter for tails below 64 antennas and in the
  * plain diagonal form, half where slots are added to several times), up to 0.6 for the products
- * of a delay term.  A route is left for the iterations on the samples where its workspace would
+ * of a delay term (1.8 on grids with holes or uneven intervals).  A route is left for the iterations on the samples where its workspace would
  * take more than half of the device's free memory, so that as much again stays free for the
  * caller, or where an allocation of it fails (which gives back the others).
  * Other solves (a full-Jones term with a term to its left, longer chains, sums of 2^31 or

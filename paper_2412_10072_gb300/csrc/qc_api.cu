@@ -1414,14 +1414,28 @@ int qc_ctx::ensure_mom_rows(cudaStream_t st)
 // pair, 32 channels), one on the samples 80 B (64 B with the FP16 model) a sample; T is taken when it is at most 0.6 of that, which leaves the pass that forms
 // it paid for after two iterations (measured on 64 antennas, 75 x 512: pass 1.9 iterations on the
 // samples, an iteration on T 0.3).  That also bounds T to 0.6 of the samples' bytes; where a slot takes
-// several additions, T with its FP64 sums (three times T).  Few intervals of many antennas leave most SMs
+// several additions, its FP64 sums take twice T beside it.  Few intervals of many antennas leave most SMs
 // without a CTA: time of an iteration in us, measured, 30 + 0.023 to 0.037 per pair and wave of CTAs on
 // products, 82 + 0.024 per 1000 samples on the samples (20 iterations, products and samples: 64 antennas, 1 x
 // 512: 2.1 and 2.1 ms; 75 x 512: 10.0 and 25; 128 antennas, 1 x 64: 4.7 and 2.0; 1 x 512: 6.5 and 3.5; 3 x
 // 512: 6.8 and 7.3; 200 antennas, 2 x 512: 14.4 and 10.2; 3 x 512: 14.8 and 16.0).
-// Whether every product of a delay term gets one sample: a time an interval, a row a pair and time.
+// Times of an interval of a delay term on a full grid whose intervals are all of one length (the last
+// one may be shorter) up to what a lane adds up in FP32: its blocks of rows then end where intervals do.
+// Else 0.
+int qc_ctx::products_depth(const qc_term &t) const
+{
+    int d = 1;
+    while (d < n_time && t.t_map[d] == t.t_map[0]) ++d;
+    bool even = full_grid && n_time > 0 && d <= 32 && t.n_tint == (n_time + d - 1) / d;
+    for (int i = 0; i < n_time && even; ++i) even = t.t_map[i] == i / d;
+    return even ? d : 0;
+}
+
+// Whether every product of a delay term takes one addition: such a grid, or a time an interval and a row
+// a pair and time.
 bool qc_ctx::products_once(const qc_term &t) const
 {
+    if (products_depth(t)) return true;
     std::vector<char> seen(t.n_tint, 0);
     for (int i = 0; i < n_time; ++i)
         if (seen[t.t_map[i]]++) return false;
@@ -1438,11 +1452,12 @@ int qc_ctx::plan_delay_sums(const qc_term *terms, int n_terms, int n, const qc_o
     if (o->kernel != 0 || o->order != -1 || o->block_threads != 0 || o->ctas_per_sm != 0) return QC_OK;
     if (n == 1 && kind_of_range(terms, 0, 1) == KIND_FULL) return QC_OK;
     const size_t n_chunks = (n_chan + 31) / 32;
+    const size_t iter_bytes = (size_t)t.n_tint * n_chunks * n_up * 1024;
     // the products, and the FP64 ones where a slot takes several additions
-    const size_t t_bytes = (size_t)t.n_tint * n_chunks * n_up * (products_once(t) ? 1024 : 3 * 1024);
+    const size_t t_bytes = iter_bytes * (products_once(t) ? 1 : 3);
     const double sample = m16 ? 64.0 : 80.0;
     const double samples = (double)n_strip_rows * n_chan;
-    if ((double)t_bytes > 0.6 * sample * samples) return QC_OK;
+    if ((double)iter_bytes > 0.6 * sample * samples) return QC_OK;
     // an iteration on T is a CTA per (time interval, chunk), which walks all pairs
     const double waves = std::ceil((double)t.n_tint * (double)n_chunks / (2.0 * sm_count));
     if (30 + 0.04 * n_up * waves > 82 + 3e-7 * sample * samples) return QC_OK;
@@ -1487,12 +1502,13 @@ DelaySumsArgs qc_ctx::delay_sums_args(const qc_term *terms, int n_terms, int n, 
     const long strips = std::max(1L, (long)n_strips * (a.chunk_major ? a.n_chunks : 1));
     const long blocks = std::max(1L, (want + strips - 1) / strips);
     a.rb = (int)std::min(max_strip, std::max(a.chunk_major ? 8L : 1L, (max_strip + blocks - 1) / blocks));
+    // a block ends where an interval does: every slot is written once
+    const int depth = products_depth(t);
+    if (depth) a.rb = (a.rb + depth - 1) / depth * depth;
     a.n_rb = (int)((max_strip + a.rb - 1) / a.rb);
     a.t_map = chain.t[n].t_map;
     a.to = n_terms == 2 ? chain.t[1 - n] : chain.t[n];
-    // one row per (interval, pair): every slot is written exactly once
-    a.store = full_grid && t.n_tint == n_time;
-    for (int i = 0; i < n_time && a.store; ++i) a.store = t.t_map[i] == i;
+    a.store = depth > 0;
     a.active = (const uint8_t *)B.active.ptr;
     a.fmap = (const int *)B.dfmap.ptr;
     a.omega = (const float *)B.domega.ptr;

@@ -282,6 +282,7 @@ struct qc_ctx {
     int plan_counters(const qc_term *terms, int n_terms, int n_epochs);
     int size_mom_rows();
     int ensure_mom_rows(cudaStream_t st);
+    int products_depth(const qc_term &t) const;
     bool products_once(const qc_term &t) const;
     int plan_delay_sums(const qc_term *terms, int n_terms, int n, const qc_opts *o, bool &use);
     qc::DelaySumsArgs delay_sums_args(const qc_term *terms, int n_terms, int n, const qc::Chain &chain);

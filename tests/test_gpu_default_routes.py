@@ -141,6 +141,7 @@ def _delay_case(seed, n_ant, n_time, n_chan, t_int, twice=False, oracle=True):
 
 @pytest.mark.parametrize("n_ant,n_time,n_chan,t_int,twice", [(3, 20000, 4, 20000, False), (5, 300, 33, 100, True),
                                                              (9, 64, 40, 2, False), (9, 16, 40, 1, True),
+                                                             (6, 50, 64, 3, False), (5, 70, 40, 33, False),
                                                              (220, 4, 3, 2, False), (221, 4, 3, 2, False)])
 def test_delay_products_hold_their_precision(n_ant, n_time, n_chan, t_int, twice):
     """Products of many samples and of few, rows of both orientations, antennas at the limit of a
