@@ -1634,7 +1634,7 @@ int qc_ctx::solve_term_sums(const qc_term *terms, int n_terms, int n, const Chai
     mi.alternate = o->damping_mode == QC_DAMP_ALTERNATE;
     mi.damping = o->damping > 0 ? o->damping : 1.0;
     mi.tol = t.tol;
-    CK(mom_launch_iterate(mi, st));
+    CK(mom_launch_iterate(mi, sm_count, st));
     CK(cudaEventRecord(ev[2], st));
     launches += ma.mom64 ? 3 : 2;
     pending.push_back(P);

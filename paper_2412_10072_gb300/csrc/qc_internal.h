@@ -54,7 +54,7 @@ cudaError_t mom_launch_rows(long n, const int *strip_rows, const int4 *rows, con
                             const int *up_of_bl, const float *bl_scale, int4 *out, float *scale, int n_strips,
                             const int *strip_off, int4 *live, float *live_scale, int *strip_end, cudaStream_t st);
 cudaError_t mom_launch_split(size_t words, const double *src, float *dst, float *tail, int sm_count, cudaStream_t st);
-cudaError_t mom_launch_iterate(const qc::MomIterArgs &a, cudaStream_t st);
+cudaError_t mom_launch_iterate(const qc::MomIterArgs &a, int sm_count, cudaStream_t st);
 cudaError_t dd_launch_residual(const qc::DDArgs &a, int grid, cudaStream_t st);
 
 struct Buf {

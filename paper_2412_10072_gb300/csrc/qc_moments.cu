@@ -921,7 +921,7 @@ __device__ __forceinline__ int solve_blocks(const double (&h00)[NB], const doubl
 // normal equations from the sums (L2), one thread per antenna solves and updates in FP64 exactly as
 // update_kernel does, and the FP64 relative change of the interval ends the loop.
 template <int FORM, bool TAIL>
-static __global__ void __launch_bounds__(256, 2) mom_iterate_kernel(const MomIterArgs a)
+static __global__ void __launch_bounds__(512, 1) mom_iterate_kernel(const MomIterArgs a)
 {
     constexpr bool GFULL = FORM == FORM_FULL;
     constexpr int N = NormSums<FORM>::NWORD, NB = GFULL ? 2 : 1, NF4 = NB;
@@ -931,7 +931,7 @@ static __global__ void __launch_bounds__(256, 2) mom_iterate_kernel(const MomIte
     double *sums = reinterpret_cast<double *>(s_mem + (size_t)A.n_ant * NF4);  // [n_ant][N]
     double2 *g64 = reinterpret_cast<double2 *>(sums + (size_t)A.n_ant * N);    // [n_ant][2 NB] the FP64 master
     const bool phase = !GFULL && A.type == QC_TERM_PHASE;
-    __shared__ double s_num[8], s_den[8];
+    __shared__ double s_num[16], s_den[16];
     __shared__ int s_done;
     const int bin = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
     const int tint = bin / A.n_fint, fint = bin - tint * A.n_fint;
@@ -1130,10 +1130,11 @@ cudaError_t mom_launch_normal(const qc::MomNormArgs &a, cudaStream_t st)
     return launch_normal<qc::FORM_D>(a, st);
 }
 
-template <int FORM, bool TAIL> static cudaError_t launch_iterate(const qc::MomIterArgs &a, cudaStream_t st)
+template <int FORM, bool TAIL> static cudaError_t launch_iterate(const qc::MomIterArgs &a, int sm_count, cudaStream_t st)
 {
+    // a warp an antenna and round: 16 warps where every interval has an SM to itself, else two CTAs of 8
     const int n_ant = a.n.n_ant;
-    const int block = n_ant > 16 ? 256 : (n_ant > 8 ? 128 : 64);
+    const int block = n_ant > 16 ? (a.n.n_bins <= sm_count ? 512 : 256) : (n_ant > 8 ? 128 : 64);
     constexpr int NB = FORM == qc::FORM_FULL ? 2 : 1;
     const size_t smem = (size_t)n_ant * (NB * sizeof(float4) + qc::NormSums<FORM>::NWORD * sizeof(double) + 2 * NB * sizeof(double2));
     if (smem > 48 * 1024) {
@@ -1145,16 +1146,16 @@ template <int FORM, bool TAIL> static cudaError_t launch_iterate(const qc::MomIt
     return cudaGetLastError();
 }
 
-template <int FORM> static cudaError_t launch_iterate(const qc::MomIterArgs &a, cudaStream_t st)
+template <int FORM> static cudaError_t launch_iterate(const qc::MomIterArgs &a, int sm_count, cudaStream_t st)
 {
-    return a.n.tail ? launch_iterate<FORM, true>(a, st) : launch_iterate<FORM, false>(a, st);
+    return a.n.tail ? launch_iterate<FORM, true>(a, sm_count, st) : launch_iterate<FORM, false>(a, sm_count, st);
 }
 
-cudaError_t mom_launch_iterate(const qc::MomIterArgs &a, cudaStream_t st)
+cudaError_t mom_launch_iterate(const qc::MomIterArgs &a, int sm_count, cudaStream_t st)
 {
-    if (a.n.form == qc::FORM_FULL) return launch_iterate<qc::FORM_FULL>(a, st);
-    if (a.n.form == qc::FORM_E) return launch_iterate<qc::FORM_E>(a, st);
-    return launch_iterate<qc::FORM_D>(a, st);
+    if (a.n.form == qc::FORM_FULL) return launch_iterate<qc::FORM_FULL>(a, sm_count, st);
+    if (a.n.form == qc::FORM_E) return launch_iterate<qc::FORM_E>(a, sm_count, st);
+    return launch_iterate<qc::FORM_D>(a, sm_count, st);
 }
 
 cudaError_t mom_launch_rows(long n, const int *strip_rows, const int4 *rows, const uint8_t *row_live,
