@@ -781,6 +781,7 @@ extern "C" int qc_residual(qc_ctx *c, const qc_term *terms, int32_t n_terms, voi
         }
     }
     if ((rc = c->run_residual(chain, dres, d_chi2, st))) return rc;
+    if (++c->pin_calls >= c->PIN_CALLS) c->pin_reserve(64);
     CK(c->to_host(chi2, d_chi2, sizeof(double), st));
     if (resid && resid_memory != QC_MEM_DEVICE)
         CK(cudaMemcpyAsync(resid, dres, nbytes<float4>(2 * n_vis), cudaMemcpyDeviceToHost, st));
@@ -2366,6 +2367,7 @@ extern "C" int qc_mad_flag(qc_ctx *c, const qc_term *terms, int32_t n_terms, dou
         CK(mad_global_launch(n_vis, keys, factor, state, dout, c->sm_count, st));
     }
     unsigned long long hc = 0;
+    if (++c->pin_calls >= c->PIN_CALLS) c->pin_reserve(64);
     if (out_memory == QC_MEM_HOST) CK(cudaMemcpyAsync(flags_out, dout, (size_t)n_vis, cudaMemcpyDeviceToHost, st));
     CK(c->to_host(&hc, &state->n_flagged, sizeof hc, st));
     CK(cudaStreamSynchronize(st));

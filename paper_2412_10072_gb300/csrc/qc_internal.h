@@ -232,9 +232,12 @@ struct qc_ctx {
     // Pinned staging of one call's small copies: a copy from or to pageable memory holds the host
     // until it is done, and a small solve makes about ten (256 us with, 232 us without, 7 antennas).  One
     // block of up to PIN_MAX, kept for the context's life and allocated by its first solve behind the
-    // kernels: in front of them it cost the first call 0.13 ms, twice a small residual.
+    // kernels (in front of them it cost the first call 0.13 ms, twice a small residual), or by the
+    // PIN_CALLS-th residual or flagging call, which by then have lost as much to direct copies.
     // Larger copies go directly; a call ends synchronised, so the next one starts from the beginning.
     static constexpr size_t PIN_MAX = 16u << 20;
+    static constexpr int PIN_CALLS = 8;
+    int pin_calls = 0;
     struct PinOut { void *dst; const void *src; size_t bytes; };
     char *pin_ptr = nullptr, *pin_next = nullptr;     // the block, the one that replaces it at the call's end
     size_t pin_size = 0, pin_next_size = 0, pin_used = 0, pin_want = 0;

@@ -254,6 +254,13 @@ def test_staging_limit():
         g = seen.setdefault(kind, T.gains)
         assert _rel(T.gains, g) < 1e-6 and _rel(g, np.ones(1)) > 1e-3
     S.close()
+    # residuals and flags alone: direct copies first, the block from the eighth call on
+    R = qc.Solver.from_obs(obs)
+    fixed = _terms(obs, (1,), solve=False)
+    chi2 = [R.residual(fixed) for _ in range(10)]
+    flags = [R.mad_flag(fixed)[1] for _ in range(3)]
+    R.close()
+    assert max(chi2) - min(chi2) <= 1e-12 * chi2[0] and len(set(flags)) == 1
 
 
 @pytest.mark.parametrize("kinds,n_ant,t_int", [(("diag",), 100, 8), (("diag",), 160, 8), (("diag",), 160, 1), (("full",), 70, 8),
