@@ -1215,11 +1215,11 @@ static constexpr int SUMS_TAILS_ANT = 64;
 //   one launch    a + c pairs ceil(nb / CTAs)     a = 5, 10, 8 and c = 0.0057, 0.0197, 0.0070 (plain diagonal, full,
 //                                                 left-full form), two CTAs an SM
 //   one each      f + m pairs nb                  f = 46, 78, 46 and m = 0.000065, 0.00021, 0.00009
-// and the one launch has about 0.65 of m pairs nb to read as well.  20 iterations in ms, one launch and one
-// each: 64 antennas, 1 interval: 0.40 and 0.92, 1.10 and 1.61, 0.51 and 0.94; 128 antennas, 1 interval: 1.14 and
-// 1.02, 3.56 and 1.90, 1.39 and 1.05; 152 intervals: 2.35 and 2.90, 6.7 and 7.4, 3.2 and 3.5; 256 antennas,
-// 1 interval: 3.9 and 1.3, 13.2 and 3.0, 4.8 and 1.3 (on the samples 2.0, 4.1 and 2.4); 152 intervals: 9.2
-// and 7.7, 27 and 24, 12.1 and 10.2.
+// and the one launch has about 0.65 of m pairs nb to read as well; c with 8 warps a CTA (16, where every
+// interval has an SM, take 0.85 of it).  20 iterations in ms, one launch and one each: 64 antennas, 1 interval: 0.34
+// and 0.90, 0.99 and 1.58, 0.43 and 0.91; 128 antennas, 1 interval, 8 warps: 1.14 and 1.02, 3.56 and 1.90, 1.39 and
+// 1.05; 152 intervals: 2.0 and 2.8, 6.7 and 7.4, 2.7 and 3.4; 256 antennas, 1 interval, 8 warps: 3.9 and 1.3, 13.2
+// and 3.0, 4.8 and 1.3 (on the samples 2.0, 4.1 and 2.4); 152 intervals: 9.2 and 7.7, 27 and 24, 12.1 and 10.2.
 bool qc_ctx::sums_one_launch(int form, size_t nb) const
 {
     if (n_ant > SUMS_ONE_LAUNCH_ANT) return false;
