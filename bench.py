@@ -970,8 +970,21 @@ def run_batched(args):
     else:
         vis_all = float(vis_iters)
     value = vis_all / (ms / 1e3)
-    # the same solves from per-baseline sufficient statistics (one data pass, iterations on the sums)
-    moments = None
+    # the autotuned persistent kernel by itself (the default solve takes the sums where they are faster), and
+    # the solve from per-baseline sums asked for (one data pass, iterations on the sums)
+    from_sums = stats[-1].depth == 0
+    moments = persistent = None
+    if not dist:
+        gk = unit.clone()
+        S.solve(unit.clone(), stream=stream, use_graph=False)
+        p0, p1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        p0.record(stream)
+        ps = S.solve(gk, stream=stream, use_graph=False)[3]
+        p1.record(stream)
+        torch.cuda.synchronize()
+        ms_p = p0.elapsed_time(p1)
+        persistent = {"value": ps.vis_iters / (ms_p / 1e3), "unit": UNIT, "ms": ms_p, "threads": ps.threads,
+                      "ctas_per_sm": ps.ctas_per_sm, "depth": ps.depth, "split": ps.split}
     if not dist:
         gm = [unit.clone() for _ in range(args.steps + 1)]
         S.solve(gm[-1], stream=stream, moments=True)
@@ -983,15 +996,15 @@ def run_batched(args):
         torch.cuda.synchronize()
         ms_m = m0.elapsed_time(m1)
         moments = {"value": sum(x.vis_iters for x in mstats) / (ms_m / 1e3), "unit": UNIT,
-                   "ms_per_step": ms_m / args.steps, "speedup_over_sample_solve": ms / ms_m,
+                   "ms_per_step": ms_m / args.steps, "speedup_over_sample_solve": persistent["ms"] * args.steps / ms_m,
                    "bytes_per_step": sum(x.bytes for x in mstats) / args.steps,
                    "mean_iters": mstats[-1].mean_iters,
                    "note": "qc_batch_solve_moments: one pass forms per-baseline sums, iterations use them"}
     peaks, src = measured_peaks()
     hbm = float(peaks.get("hbm_gbs", 6800.0))
-    # algorithmic bytes: 81 B per vis-iteration (every sample of every iteration); the kernel skips
-    # copying flagged samples, but they share DRAM bursts with read neighbours
-    achieved = 81.0 * vis_iters / (ms / 1e3) / 1e9
+    # from sums: the one data pass; the persistent kernel: 81 B per vis-iteration (every sample of every
+    # iteration; it skips copying flagged samples, but they share DRAM bursts with read neighbours)
+    achieved = (float(byts) if from_sums else 81.0 * vis_iters) / (ms / 1e3) / 1e9
     # looped plain launches on a sample of the same problems
     rng = np.random.default_rng(0)
     idx = np.sort(rng.choice(b.n_prob, size=min(args.looped, b.n_prob), replace=False))
@@ -1024,22 +1037,24 @@ def run_batched(args):
             "warmup": args.warmup, "ms_per_step": ms / args.steps, "higher_is_better": True, "scaling": "weak",
             "vs_baseline": None, "dtype": "c64", "data": "synthetic",
             "config": {"workload": f"batched: {args.n_prob} independent diagonal-gain intervals, ant U{{7..64}}, "
-                                   "times U{1..16}, chans U{1..64}, flags U(0,0.5), one persistent launch",
+                                   "times U{1..16}, chans U{1..64}, flags U(0,0.5)",
                        "n_vis": b.n_vis, "input_bytes_per_gpu": int(b.n_vis * 81),
                        "l2": "inputs larger than L2 (129 MB); a small problem may stay in L2 across its iterations",
                        "parallelism": f"replicas x{world}" if world > 1 else "1 GPU", "gen_s": round(t_gen, 1)},
             "autotune": {"threads": best.threads, "ctas_per_sm": best.ctas_per_sm, "schedule": best.schedule,
                          "candidates": n_tried, "best_ms": best.ms},
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s", "frac": achieved / hbm,
-                         "traffic": None, "kernel": "batch_kernel (persistent, whole solve)",
-                         "bytes_per_vis_iteration": 81, "unflagged_read_bytes": byts,
+                         "traffic": None,
+                         "kernel": "batch_sums_kernel and batch_iterate_kernel (sums once, iterations on them)"
+                         if from_sums else "batch_kernel (persistent, whole solve)",
+                         "bytes_per_vis_iteration": None if from_sums else 81, "unflagged_read_bytes": byts,
                          "peak_source": f"{src} hbm_gbs (MEASURED_PEAKS.json)",
                          "mean_iters": stats[-1].mean_iters},
             "looped_plain": {"problems": int(idx.size), "value": loop_value, "unit": UNIT, "seconds": dt_loop,
                              "speedup_of_batched": value / loop_value},
-            "moments": moments,
+            "moments": moments, "persistent_kernel": persistent,
             "cpu_baseline": cpu, "e2e": None, "clocks": clock_info,
-            "gpu_launches": args.steps, "vis_iters": int(vis_all)}), flush=True)
+            "gpu_launches": args.steps * (2 if from_sums else 1), "vis_iters": int(vis_all)}), flush=True)
     S.close()
     if dist:
         dist.destroy_process_group()
@@ -1111,13 +1126,14 @@ def run_warmstart(args):
         res = {}
         for tol in ladder:
             for _ in range(max(1, args.warmup)):       # warm the launch path
-                solver.solve(unit.clone(), max_iter=20, tol=tol, stream=stream, moments=mom)
+                solver.solve(unit.clone(), max_iter=20, tol=tol, stream=stream, moments=mom, use_graph=mom)
 
             def run():
                 if start == "mlp":
                     return ws.warm_solve(solver, net, gp, max_iter=40, tol=tol, stream=stream, moments=mom)
                 g0 = unit.clone() if start == "unit" else gp.clone()
-                g, _, it, st = solver.solve(g0, max_iter=40, tol=tol, stream=stream, moments=mom)
+                # (use_graph = False: the tuned persistent kernel also where the sums are faster)
+                g, _, it, st = solver.solve(g0, max_iter=40, tol=tol, stream=stream, moments=mom, use_graph=mom)
                 return g, it, st, 0
 
             (g, it, st, n_fb), ms = timed(run)

@@ -243,7 +243,7 @@ typedef struct {
  * more slots) ignore the option.  qc_stats.vis_iters
  * counts the samples of the active intervals per iteration however a term was solved; from
  * sums, qc_stats.acc_bytes counts the pass (the samples' bytes, once) and, per iteration and
- * active interval, the sums read on both sides and the accumulators written;
+ * active interval, the sums' heads read on both sides and the accumulators written;
  * qc_stats.pass_ms is the passes' device time when qc_opts.moments asked for them.
  */
 
