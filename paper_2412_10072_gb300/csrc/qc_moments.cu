@@ -36,7 +36,7 @@
 // 3.8e-8 and 3.8e-8, one interval of 150 x 512 3.1e-8 and 3.0e-8, full-Jones 2.7e-8 and 2.6e-8; 20
 // antennas 3.6e-8 and 3.9e-8; 64 antennas, G and B, 3.0e-8 and 3.0e-8.  Time, two-term chain (64
 // antennas, 300 x 512, three epochs of 20 iterations a term): 660 ms on the samples, 46.2 ms from sums; 27
-// antennas, 61 x 131, intervals of 5 x 17: 3.78 and 0.35 ms; 7 antennas, 60 x 16: 1.02 and 0.25 ms.
+// antennas, 61 x 131, intervals of 5 x 17: 3.78 and 0.37 ms; 7 antennas, 60 x 16: 1.02 and 0.23 ms.
 #include "qc_internal.h"
 
 #include <algorithm>
@@ -1132,9 +1132,15 @@ cudaError_t mom_launch_normal(const qc::MomNormArgs &a, cudaStream_t st)
 
 template <int FORM, bool TAIL> static cudaError_t launch_iterate(const qc::MomIterArgs &a, int sm_count, cudaStream_t st)
 {
-    // a warp an antenna and round: 16 warps where every interval has an SM to itself, else two CTAs of 8
+    // a warp an antenna and round: 16 warps where every interval has an SM to itself, else two CTAs of 8;
+    // fewer for few antennas, unless a turn is long (the forms with 4x4 blocks) or all of them have one (10
+    // antennas, full and left-full form, 120 intervals: 0.70 ms with 4 warps, 0.58 with 10; 7 antennas, 60
+    // intervals: 0.27 with 2, 0.24 with 7; 16 antennas, plain diagonal form: 0.32 with 4, 0.33 with 16)
     const int n_ant = a.n.n_ant;
-    const int block = n_ant > 16 ? (a.n.n_bins <= sm_count ? 512 : 256) : (n_ant > 8 ? 128 : 64);
+    const bool alone = a.n.n_bins <= sm_count;
+    const int block = alone && (FORM != qc::FORM_D || n_ant <= 8) ? 32 * std::min(16, std::max(2, n_ant))
+                      : n_ant > 16                                ? (alone ? 512 : 256)
+                                                                  : (n_ant > 8 ? 128 : 64);
     constexpr int NB = FORM == qc::FORM_FULL ? 2 : 1;
     const size_t smem = (size_t)n_ant * (NB * sizeof(float4) + qc::NormSums<FORM>::NWORD * sizeof(double) + 2 * NB * sizeof(double2));
     if (smem > 48 * 1024) {
